@@ -143,8 +143,10 @@ def _ptr(t) -> Optional[int]:
 
 def _stream_ptr(stream) -> Optional[int]:
     if stream is None:
+        # the current stream's handle without building a Stream object for it: 0.2 instead of 3.2 us per call, where a
+        # whole decode call takes 7
         import torch
-        stream = torch.cuda.current_stream()
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
     return stream.cuda_stream or None
 
 
