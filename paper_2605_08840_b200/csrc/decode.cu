@@ -233,10 +233,14 @@ cudaError_t launch_decode(const Problem& p, const void* q, const void* Kc, const
                       ? launch_partial_g<__nv_bfloat16>(p, q, Kc, Vc, n_rows, part, splits, st)
                       : launch_partial_g<float>(p, q, Kc, Vc, n_rows, part, splits, st);
   if (e != cudaSuccess) return e;
+  *n_launches = 2;
+  return launch_decode_combine(p, part, splits, out, lse, st);
+}
+
+cudaError_t launch_decode_combine(const Problem& p, const float* part, int splits, float* out, float* lse, cudaStream_t st) {
   const int threads = ((p.d + 31) / 32) * 32;
   dim3 grid(p.Hq, p.batch);
   decode_combine_kernel<<<grid, threads, 0, st>>>(p.Hq, p.G, p.d, splits, part, out, lse);
-  *n_launches = 2;
   return cudaGetLastError();
 }
 

@@ -11,6 +11,7 @@ struct restkv_handle {
   int sm_count;
   unsigned int* dev_status;   // 256-byte device block, word 0 = sticky status bits
   void* tc_state;
+  int decode_clusters[5];     // clusters of 1, 2, 4, 8, 16 CTAs of the decode kernel that the device holds at once
   long long launches;
   int last_cuda_error;
   int kernel_path;            // 0 auto, 1 SIMT, 2 tensor core required, 3 tensor core in its head-sequential form
@@ -311,7 +312,9 @@ restkv_status restkv_create(restkv_handle** out) {
   if (e == cudaSuccess) e = cudaMemset(h->dev_status, 0, 256);
   if (e != cudaSuccess) { delete h; return RESTKV_ERR_CUDA; }
   h->tc_state = nullptr;
-  if (tc_init(&h->tc_state) != cudaSuccess || tc_fused_init() != cudaSuccess) h->tc_state = nullptr;
+  if (tc_init(&h->tc_state) != cudaSuccess || tc_fused_init() != cudaSuccess ||
+      decode_mma_init(h->decode_clusters) != cudaSuccess)
+    h->tc_state = nullptr;
   h->wait_limit = 2000000000ll;
   h->fused_select = true;
   h->last_evict_fused = false;
@@ -558,7 +561,19 @@ restkv_status restkv_decode(restkv_handle* h, const restkv_shape* shape, const v
   if (s != RESTKV_OK) return s;
   if (!workspace || ((uintptr_t)workspace & 255u) != 0) return RESTKV_ERR_WORKSPACE;
   Call c{h, (cudaStream_t)stream};
-  // bf16, head_dim 128: the decode step is plain attention of up to 128 query rows per KV head, i.e. phases A and B
+  // bf16, head_dim 128, up to 16 query heads per KV head: a kernel of its own, one cluster of CTAs per KV head, which
+  // needs scratch only where several clusters share one
+  if (h->tc_state && h->kernel_path != 1 && p.dtype == RESTKV_BF16 && p.d == 128 && p.G <= kDecodeMmaMaxG) {
+    int cluster, splits;
+    decode_mma_plan(h->decode_clusters, p.BH, p.G, n_rows, workspace_bytes, &cluster, &splits);
+    RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE,
+                  launch_decode_mma(h->tc_state, p, q, Kc, Vc, n_rows, out, lse, (float*)workspace, cluster, splits,
+                                    h->wait_limit, h->dev_status, c.st), 1);
+    if (splits > 1)
+      RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE, launch_decode_combine(p, (const float*)workspace, splits, out, lse, c.st), 1);
+    return RESTKV_OK;
+  }
+  // more query heads per KV head: the decode step is plain attention of up to 128 query rows per KV head, i.e. phases A and B
   // of the tensor-core score kernel with the group's queries padded to its 128 rows.  It needs about 10 MB of
   // workspace (any restkv_workspace_bytes result has that); with less, or for other shapes, the SIMT kernels run.
   bool tc_ws_too_small = false;

@@ -94,6 +94,14 @@ cudaError_t launch_compact(const Problem& p, const void* K, const void* V, const
                            void* K_out, void* V_out, unsigned int* dev_status, cudaStream_t st);
 cudaError_t launch_decode(const Problem& p, const void* q, const void* Kc, const void* Vc, int n_rows, float* out,
                           float* lse, float* part, int splits, cudaStream_t st, int* n_launches);
+cudaError_t launch_decode_combine(const Problem& p, const float* part, int splits, float* out, float* lse, cudaStream_t st);
+// bf16, head_dim 128, at most 16 query heads per KV head (decode_mma.cu).  clusters_of: [5], filled at init.
+constexpr int kDecodeMmaMaxG = 16;
+cudaError_t decode_mma_init(int* clusters_of);
+void decode_mma_plan(const int* clusters_of, int BH, int G, int n_rows, size_t scratch_bytes, int* cluster, int* splits);
+cudaError_t launch_decode_mma(void* state, const Problem& p, const void* q, const void* Kc, const void* Vc, int n_rows,
+                              float* out, float* lse, float* part, int cluster, int splits, long long wait_limit,
+                              unsigned int* dev_status, cudaStream_t st);
 cudaError_t launch_adaptive_params(const Problem& p, const Workspace& ws, int budget, float beta, int base_width,
                                    cudaStream_t st, int* n_launches);
 

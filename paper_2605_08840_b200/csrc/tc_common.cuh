@@ -118,8 +118,8 @@ constexpr float kHeavyA = 0.125f;             // attention weight above which ||
 
 // ------------------------------------------------------------------------------------------------
 inline CUresult encode_tiles(TcState* st, CUtensorMap* map, const void* base, int rank, const cuuint64_t* dims,
-                      const cuuint64_t* strides_bytes) {
-  cuuint32_t box[4] = {64, 128, 1, 1};
+                      const cuuint64_t* strides_bytes, cuuint32_t box_rows = 128) {
+  cuuint32_t box[4] = {64, box_rows, 1, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   return st->encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims,
                     strides_bytes, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,

@@ -490,6 +490,33 @@ def test_decode_matches_oracle(handle, spec):
     np.testing.assert_allclose(lse.cpu().numpy(), ref_lse, rtol=1e-5, atol=1e-5)
 
 
+@pytest.mark.parametrize("spec", [(1, 4, 1, 1), (1, 32, 8, 15), (3, 12, 4, 17), (1, 16, 1, 127), (2, 48, 3, 2049),
+                                  (1, 9, 1, 20001), (1, 4, 1, 131072), (40, 8, 4, 300), (1, 34, 2, 257)])
+def test_decode_cluster_kernel(handle, spec):
+    """bf16, head_dim 128: rows around the 16-row tile and the split over warps, CTAs and clusters; 1 to 17 query heads per
+    KV head (17: the padded path); one cluster and several per head, more heads than SMs."""
+    import torch
+    b, Hq, Hkv, rows = spec
+    rng = np.random.default_rng(rows)
+
+    def draw(shape):
+        bits = round_to_bf16_bits(rng.standard_normal(shape).astype(np.float32))
+        return (bits.astype(np.uint32) << 16).view(np.float32), torch_dev(bits.view(np.int16), "bf16")
+
+    q, qd = draw((b, Hq, 128))
+    K, Kd = draw((b, Hkv, rows, 128))
+    V, Vd = draw((b, Hkv, rows, 128))
+    ref, ref_lse = oracle.decode(q, K, V)
+    shape = shape_of(Case("dec", b, Hq, Hkv, 128, rows, 1, dtype="bf16"))
+    out = torch.full((b, Hq, 128), float("nan"), device="cuda")
+    lse = torch.full((b, Hq), float("nan"), device="cuda")
+    ws = torch.empty(handle.workspace_bytes(shape, 0), dtype=torch.uint8, device="cuda")
+    handle.decode(shape, qd, Kd, Vd, rows, out, ws, lse=lse)
+    torch.cuda.synchronize()
+    assert_decode_close(out.cpu().numpy(), ref, q, K, V, "bf16")
+    np.testing.assert_allclose(lse.cpu().numpy(), ref_lse, rtol=1e-5, atol=1e-5)
+
+
 def test_decode_over_compacted_cache_of_config2(handle):
     import torch
     inp = make_inputs(CONFIGS["cfg2"])
