@@ -46,64 +46,6 @@ __device__ __forceinline__ void mma_tile_kk(uint32_t tmem_d, uint32_t a_smem, ui
   }
 }
 
-// Exact ||o - v||^2 for the rare entries whose attention weight is large (the expansion ||o||^2 + ||v||^2 - 2 o.v
-// cancels when o approaches v).  Computed by a whole warp: lane L takes elements 4L .. 4L+3, the partial sums meet by butterfly exchange (every
-// lane returns the full sum).
-__device__ __forceinline__ float exact_dist2_warp(const float* __restrict__ o_row, const __nv_bfloat16* __restrict__ v_row,
-                                                  int lane) {
-  const float4 o = *reinterpret_cast<const float4*>(o_row + lane * 4);
-  const uint2 vv = *reinterpret_cast<const uint2*>(v_row + lane * 4);
-  const float d0 = o.x - __uint_as_float(vv.x << 16), d1 = o.y - __uint_as_float(vv.x & 0xFFFF0000u);
-  const float d2 = o.z - __uint_as_float(vv.y << 16), d3 = o.w - __uint_as_float(vv.y & 0xFFFF0000u);
-  float ss = (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-  return ss;
-}
-
-// The same under the output projection: (o - v)^T Mt (o - v) = (o - v) . (Mt o - Mt v), Mt symmetric [128 x 128] fp32,
-// Mt o given (op_row).  Row k of Mt is read by the whole warp (coalesced) and weighted with v_k, which lane k / 4 holds.
-__device__ __forceinline__ float exact_proj_dist2_warp(const float* __restrict__ o_row, const float* __restrict__ op_row,
-                                                       const __nv_bfloat16* __restrict__ v_row,
-                                                       const float* __restrict__ Mt, int lane) {
-  const float4 o = *reinterpret_cast<const float4*>(o_row + lane * 4);
-  const float4 op = *reinterpret_cast<const float4*>(op_row + lane * 4);
-  const uint2 vv = *reinterpret_cast<const uint2*>(v_row + lane * 4);
-  const float v[4] = {__uint_as_float(vv.x << 16), __uint_as_float(vv.x & 0xFFFF0000u), __uint_as_float(vv.y << 16),
-                      __uint_as_float(vv.y & 0xFFFF0000u)};
-  float4 mv = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
-  for (int src = 0; src < 32; ++src) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float vk = __shfl_sync(0xffffffffu, v[e], src);
-      const float4 m = __ldg(reinterpret_cast<const float4*>(Mt + (src * 4 + e) * kHeadDim + lane * 4));
-      mv.x = fmaf(m.x, vk, mv.x); mv.y = fmaf(m.y, vk, mv.y); mv.z = fmaf(m.z, vk, mv.z); mv.w = fmaf(m.w, vk, mv.w);
-    }
-  }
-  float ss = ((o.x - v[0]) * (op.x - mv.x) + (o.y - v[1]) * (op.y - mv.y)) +
-             ((o.z - v[2]) * (op.z - mv.z) + (o.w - v[3]) * (op.w - mv.w));
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-  return fmaxf(ss, 0.f);
-}
-
-// The expansion o^T Mt o - 2 (Mt o) . v + v^T Mt v in fp32 with exact dot products (vmv = v^T Mt v given): accurate
-// as long as the three terms do not nearly cancel, i.e. while o stays away from v.
-__device__ __forceinline__ float expanded_proj_dist2_warp(const float* __restrict__ o_row, const float* __restrict__ op_row,
-                                                          const __nv_bfloat16* __restrict__ v_row, float vmv, int lane) {
-  const float4 o = *reinterpret_cast<const float4*>(o_row + lane * 4);
-  const float4 op = *reinterpret_cast<const float4*>(op_row + lane * 4);
-  const uint2 vv = *reinterpret_cast<const uint2*>(v_row + lane * 4);
-  const float v0 = __uint_as_float(vv.x << 16), v1 = __uint_as_float(vv.x & 0xFFFF0000u);
-  const float v2 = __uint_as_float(vv.y << 16), v3 = __uint_as_float(vv.y & 0xFFFF0000u);
-  // o . (Mt o) - 2 v . (Mt o) = (o - 2 v) . (Mt o)
-  float ss = ((o.x - 2.f * v0) * op.x + (o.y - 2.f * v1) * op.y) + ((o.z - 2.f * v2) * op.z + (o.w - 2.f * v3) * op.w);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-  return fmaxf(ss + vmv, 0.f);
-}
-
 // After a wait has failed: wait (bounded, whatever the abort flag says) for a bulk copy or an MMA that this thread
 // itself set in motion, so that nothing is still writing this CTA's shared or tensor memory when it returns.
 __device__ __forceinline__ void wait_issued(uint64_t* bar, uint32_t parity) {

@@ -28,6 +28,8 @@ static_assert(kFFirstWorker * kFRegsControl + kFWorkerWarps * kFRegsWorker <= (k
               "the register split must fit the pool the CTA is launched with");
 constexpr int kFRing = 4;                         // 32 KB tile slots after Q | O' | aug | ones
 constexpr size_t kFSmem = 2 * kTileBytes + kAugBytes + kOnesBytes + kFRing * kTileBytes + 1024;
+// A row's weights add up to 1, so that at most 8 tokens of a head (7 but for rounding) exceed kHeavyA = 1/8 in it.
+constexpr int kMaxHeavy = 8 * kRows;
 constexpr int kFVSlots = 3;                       // phase A: V slots = ring 2, ring 3 and the (then unused) O' tile
 
 struct FusedArgs {
@@ -54,8 +56,10 @@ struct FusedArgs {
   float* I_hat;                      // [BH, n]
   float* I_raw;                      // [BH, 128, n] or null: the per-query indicators, for the adaptive window of
                                      //  Eq. 10-12; every tile then takes the slower epilogue that holds them
+  const __nv_bfloat16* Q;            // [BH, 128, 128]
+  const __nv_bfloat16* K;
   const __nv_bfloat16* V;
-  long long vsb, vsh, vsn;
+  long long ksb, ksh, ksn, vsb, vsh, vsn;
   // Output projection of Eq. 4 (all null without one): Eq. 7's squared norm becomes the quadratic form of Mt, the
   // per-head matrices [Hq, 128, 128]; vmv [BH, G, n_kv] holds the tokens' own terms v^T Mt v (in place of ||v||^2),
   // O_proj [BH, 128, 128] receives Mt o of the window rows.
@@ -72,8 +76,6 @@ struct FusedArgs {
   int32_t* sel_indices;              // [BH, keep]
   unsigned int* sel_hist;            // [BH, 4, 256] digit histograms of the group, zero at launch
   unsigned int* sel_sfx;             // [CTA, 4, kSfxStride] per CTA: suffix sums of its own digit histograms
-  const __nv_bfloat16* K;
-  long long ksb, ksh, ksn;
   __nv_bfloat16* K_out;              // [BH, keep, 128]
   __nv_bfloat16* V_out;
 };
@@ -121,7 +123,7 @@ __device__ void init_bars(FusedBars* B, bool first, bool from_lse) {
     mbar_init(&B->pv_done[i], 1);
     mbar_init(&B->kv_full[i], 1);
     mbar_init(&B->kv_empty[i], from_lse ? 3 : 1);   // MMA commit (+ the two ||v||^2 warps, which read the V tile)
-    mbar_init(&B->acc_full[i], 1);
+    mbar_init(&B->acc_full[i], from_lse ? 1 : 2);   // MMA commit (+ the warp that tells which tiles may hold a large weight)
     mbar_init(&B->acc_empty[i], kFWorkerWarps);
   }
   for (int i = 0; i < kFVSlots; ++i) {
@@ -171,7 +173,9 @@ struct Ctx {
   FusedBars* B;
   int* abort_flag;
   float* sm_stats;         // [6][128] floats: row maxima of the column halves [slot][half], then (m, l) hand-over
+  volatile int* look;      // [2] whether a weight of the tile in accumulator set s may exceed kHeavyA
   float* vn_s;             // [4][128] ||v||^2 of the last four tiles of phase C (from_lse only)
+  int* heavy;              // (over sm_stats, which phase A no longer needs) [0]: count, then the tokens of this CTA's share that have a weight above kHeavyA in some row
   int warp, lane;
 };
 
@@ -699,6 +703,30 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
         wait_issued(&B->drain, 0);
       }
     }
+  } else if (!kLse && warp == 2) {
+    // ---- which tiles need their logits looked at: some row's largest logit reaches that row's M2 - log2(1 / kHeavyA).
+    //      Told with the accumulators' barrier, so that the epilogue warps spend neither loads nor registers on it. ----
+    const int nt_all = (a.n_kv + kTile - 1) / kTile;
+    const float* tm = a.tile_max + ((long long)bh * nt_all + tile0) * kRows + lane;
+    float m2r[4], next[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      m2r[k] = a.row_M2[(long long)bh * kRows + k * 32 + lane] - log2f(1.f / kHeavyA);
+      next[k] = T > 0 ? tm[(long long)(T - 1) * kRows + k * 32] : -INFINITY;
+    }
+    for (int it = 0; it < T; ++it) {
+      const int s = it & 1;
+      const bool any = __any_sync(0xffffffffu, next[0] > m2r[0] || next[1] > m2r[1] || next[2] > m2r[2] || next[3] > m2r[3]);
+      if (it + 1 < T) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) next[k] = tm[(long long)(T - 2 - it) * kRows + k * 32];
+      }
+      if (it >= 2 && !mbar_wait(&B->acc_empty[s], ((it >> 1) - 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit)) break;
+      if (lane == 0) {
+        cx.look[s] = any;
+        mbar_arrive(&B->acc_full[s]);
+      }
+    }
   } else if (kLse) {
     // ---- ||v||^2 of the tile's tokens from the V tile in shared memory (phase A, which computes it otherwise, does
     //      not run): warp 2 takes tokens 0-63, warp 3 tokens 64-127, a lane two rows; ring of four tiles ----
@@ -735,6 +763,134 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
         mbar_arrive(&B->kv_empty[s]);
       }
     }
+  }
+}
+
+// Eight values per lane -> sums over the warp: lane L returns the sum of value L / 4 (three exchanges halve the values,
+// two finish).
+__device__ __forceinline__ float reduce8_warp(float* v, int lane) {
+#pragma unroll
+  for (int half = 4; half > 0; half >>= 1) {
+    const int bit = half * 4;
+    const bool up = (lane & bit) != 0;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const float send = up ? v[i] : v[i + half], keep = up ? v[i + half] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+    }
+  }
+  float r = v[0];
+  r += __shfl_xor_sync(0xffffffffu, r, 2);
+  return r + __shfl_xor_sync(0xffffffffu, r, 1);
+}
+
+// The tokens that phase C has noted (a weight above kHeavyA in some window row: an attention sink has one in nearly every
+// row) are scored again from K, V, Q and O themselves: the expansion ||o||^2 + ||v||^2 - 2 o.v cancels when o approaches v,
+// and 1 / (1 - A) amplifies what is left.  All sixteen worker warps take one token together, eight rows each with their
+// loads side by side, so that a token costs about two L2 round trips; done inside the tile's epilogue, a row after the
+// other, a sink took the CTA that owned it 17 us.  After the loop over the tiles, so that none of it takes registers there.
+// Under the output projection the expansion (o - 2 v) . (Mt o) + v^T Mt v from exact dot products serves up to A = 0.9,
+// the full form (o - v) . (Mt o - Mt v) beyond.
+template <int kW, bool kProj>
+__device__ void heavy_pass(const Ctx& cx, const FusedArgs& a, int bh) {
+  constexpr int kG = kRows / kW;
+  const int lane = cx.lane, wq = cx.warp - kFFirstWorker;
+  named_barrier_sync(1, kFWorkerWarps * 32);   // every warp has noted its tokens, and I_hat of the share is written
+  const int count = min(cx.heavy[0], kMaxHeavy);
+  if (count > 0) {
+    const int b = bh / a.Hkv, h = bh % a.Hkv;
+    const float c2 = a.scale * kLog2e;
+    const bool group_max = a.group_max != 0;
+    const __nv_bfloat16* Kh = a.K + (long long)b * a.ksb + (long long)h * a.ksh + lane * 4;
+    const __nv_bfloat16* Vh = a.V + (long long)b * a.vsb + (long long)h * a.vsh + lane * 4;
+    const int row0 = wq * 8, g = row0 / kW;
+    const long long off0 = ((long long)bh * kRows + row0) * kHeadDim + lane * 4;
+    const float M2 = a.row_M2[(long long)bh * kRows + row0 + (lane >> 2)];
+    int done = 0;
+    for (int e = 0; e < count; ++e) {
+      const int j = cx.heavy[1 + e];
+      bool seen = false;   // several warpgroups note the same token
+      for (int k = lane; k < e; k += 32) seen |= cx.heavy[1 + k] == j;
+      if (__any_sync(0xffffffffu, seen)) continue;
+      auto unpack = [](uint2 u) {
+        return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                           __uint_as_float(u.y & 0xFFFF0000u));
+      };
+      const float4 kj = unpack(*reinterpret_cast<const uint2*>(Kh + (long long)j * a.ksn));
+      const float4 vj = unpack(*reinterpret_cast<const uint2*>(Vh + (long long)j * a.vsn));
+      float part[8];
+      float4 o[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) o[i] = *reinterpret_cast<const float4*>(a.O_f32 + off0 + i * kHeadDim);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float4 q = unpack(*reinterpret_cast<const uint2*>(a.Q + off0 + i * kHeadDim));
+        part[i] = (q.x * kj.x + q.y * kj.y) + (q.z * kj.z + q.w * kj.w);
+      }
+      const float u = ex2_approx(M2 - c2 * reduce8_warp(part, lane));   // 1 / A of row row0 + lane / 4
+      float x;
+      if (!kProj) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float d0 = o[i].x - vj.x, d1 = o[i].y - vj.y, d2 = o[i].z - vj.z, d3 = o[i].w - vj.w;
+          part[i] = (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
+        }
+        x = reduce8_warp(part, lane);
+      } else {
+        const bool extreme = __any_sync(0xffffffffu, u < 1.f / 0.9f);
+        float4 mv = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (extreme) {
+          const float* Mt = a.proj_Mt + (long long)(h * kG + g) * kHeadDim * kHeadDim + lane * 4;
+#pragma unroll 4
+          for (int k = 0; k < kHeadDim; ++k) {
+            const float own = (k & 3) == 0 ? vj.x : (k & 3) == 1 ? vj.y : (k & 3) == 2 ? vj.z : vj.w;
+            const float vk = __shfl_sync(0xffffffffu, own, k >> 2);
+            const float4 m = __ldg(reinterpret_cast<const float4*>(Mt + k * kHeadDim));
+            mv.x = fmaf(m.x, vk, mv.x); mv.y = fmaf(m.y, vk, mv.y); mv.z = fmaf(m.z, vk, mv.z); mv.w = fmaf(m.w, vk, mv.w);
+          }
+        }
+        const float vs = extreme ? 1.f : 2.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float4 op = *reinterpret_cast<const float4*>(a.O_proj + off0 + i * kHeadDim);
+          part[i] = (fmaf(-vs, vj.x, o[i].x) * (op.x - mv.x) + fmaf(-vs, vj.y, o[i].y) * (op.y - mv.y)) +
+                    (fmaf(-vs, vj.z, o[i].z) * (op.z - mv.z) + fmaf(-vs, vj.w, o[i].w) * (op.w - mv.w));
+        }
+        x = reduce8_warp(part, lane);
+        if (!extreme) x += a.vmv[((long long)bh * kG + g) * a.n_kv + j];
+        x = fmaxf(x, 0.f);
+      }
+      const float um = u - 1.f;
+      const float I = x * rsqrt_approx(fmaf(x * um, um, 1e-36f));
+      float* buf = cx.sm_stats + 1 + kMaxHeavy + (done & 1) * kRows;
+      if ((lane & 3) == 0) {
+        buf[row0 + (lane >> 2)] = I;
+        if (a.I_raw) a.I_raw[((long long)bh * kRows + row0 + (lane >> 2)) * a.n + j] = I;
+      }
+      named_barrier_sync(1, kFWorkerWarps * 32);
+      if (wq == (done & (kFWorkerWarps - 1))) {   // one warp adds the token up; the others go on to the next one
+        float r[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int row = k * 32 + lane, i = row % kW;
+          r[k] = buf[row] * powf(a.t_decay, (float)(kW - 1 - i)) * (i == 0 ? a.t_seed_first : 1.f) *
+                 (i == kW - 1 ? a.t_seed_last : 1.f);
+#pragma unroll
+          for (int off = 1; off < 32; off <<= 1) {
+            const float other = __shfl_xor_sync(0xffffffffu, r[k], off);
+            r[k] = (off >= kW && group_max) ? fmaxf(r[k], other) : r[k] + other;   // over a query head's window, then over heads
+          }
+        }
+        float tot;
+        if (!group_max || kW == 128) tot = (r[0] + r[1]) + (r[2] + r[3]);
+        else if (kW == 64) tot = fmaxf(r[0] + r[1], r[2] + r[3]);
+        else tot = fmaxf(fmaxf(r[0], r[1]), fmaxf(r[2], r[3]));
+        if (lane == 0) a.I_hat[(long long)bh * a.n + j] = tot * a.t_scale / (group_max ? 1.f : (float)kG);
+      }
+      ++done;
+    }
+    named_barrier_sync(1, kFWorkerWarps * 32);
+    if (wq == 0 && lane == 0) cx.heavy[0] = 0;
   }
 }
 
@@ -781,36 +937,13 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
     if (kW == 64) return fmaxf(r0 + r1, r2 + r3);
     return fmaxf(fmaxf(r0, r1), fmaxf(r2, r3));
   };
-  const float* O_head = a.O_f32 + (long long)bh * kRows * kHeadDim;
-  const __nv_bfloat16* V_head = a.V + (long long)b * a.vsb + (long long)h * a.vsh;
   // with the output projection the token's own term is v^T Mt v of the query head that this warpgroup's 32 columns
-  // belong to (w >= 32 there), and the exact distances go through that head's Mt
+  // belong to (w >= 32 there)
   const int g_cols = (cgp * 32) / kW;
   const float* vn_head = kProj ? a.vmv + ((long long)bh * kG + g_cols) * a.n_kv : a.vnorm + (long long)bh * a.n_kv;
-  const float* Mt_g = kProj ? a.proj_Mt + (long long)(h * kG + g_cols) * kHeadDim * kHeadDim : nullptr;
-  const float* Op_head = kProj ? a.O_proj + (long long)bh * kRows * kHeadDim : nullptr;
-  // S' above this <=> A > 0.9: under the projection only those entries take the exact quadratic form; the others
-  // above kHeavyA take its expansion in fp32 from exact dot products, which is accurate while 1 - A is not small
-  const float extreme_thr = log2f(1.f / 0.9f) / neg_c2;
-  auto exact_dist2 = [&](int row, int js, bool extreme) {
-    const __nv_bfloat16* v_row = V_head + (long long)js * a.vsn;
-    if (!kProj) return exact_dist2_warp(O_head + row * kHeadDim, v_row, lane);
-    if (extreme) return exact_proj_dist2_warp(O_head + row * kHeadDim, Op_head + row * kHeadDim, v_row, Mt_g, lane);
-    return expanded_proj_dist2_warp(O_head + row * kHeadDim, Op_head + row * kHeadDim, v_row, vn_head[js], lane);
-  };
   float* I_head = a.I_hat + (long long)bh * n;
   float* raw_head = (a.I_raw && !kLse) ? a.I_raw + (long long)bh * kRows * n : nullptr;
   bool ok = true;
-  const int nt_all = (a.n_kv + kTile - 1) / kTile;
-  // a tile needs exact distances iff some row's largest logit in it reaches that row's M2 - log2(1 / kHeavyA);
-  // every warp checks all 128 rows (lane = rows lane, lane + 32, ...) so that no synchronisation is needed
-  const float* tm_head = a.tile_max + (long long)bh * nt_all * kRows;
-  float m2r[4], tm_next[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    m2r[k] = a.row_M2[(long long)bh * kRows + k * 32 + lane] - log2f(1.f / kHeavyA);
-    tm_next[k] = -INFINITY;
-  }
   float vn_next = 0.f;
   // from_lse: no phase A has left ||v||^2 and the tiles' row maxima behind; ||v||^2 comes from the control warps
   // through shared memory and a warp finds out from the logits themselves whether its part of a tile is heavy
@@ -820,19 +953,12 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
     const int j = (tile0 + T - 1) * kTile + t;
     vn_next = (j < n) ? vn_head[j] : 1.f;
   }
-  if (T > 0 && !from_lse) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) tm_next[k] = tm_head[(long long)(tile0 + T - 1) * kRows + k * 32 + lane];
-  }
 
   for (int it = 0; it < T; ++it) {
     const int s = it & 1;
     const uint32_t par = (uint32_t)(it >> 1) & 1u;
     float vn = vn_next;
     // only Eq. 7 has the factor 1 / (1 - A) and the distance that need the exact form near A = 1
-    const bool tile_heavy = raw_head != nullptr ||
-                            (kEq7 && __any_sync(0xffffffffu, tm_next[0] > m2r[0] || tm_next[1] > m2r[1] ||
-                                                                      tm_next[2] > m2r[2] || tm_next[3] > m2r[3]));
     if (from_lse) {
       ok = ok && mbar_wait(&B->vn_full[it & 3], (uint32_t)(it >> 2) & 1u, abort_flag, dev_status, kDevTimeout, a.wait_limit);
       const int jv = (tile0 + T - 1 - it) * kTile + t;
@@ -841,10 +967,6 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
     if (it + 1 < T && vn_global) {   // next tile's ||v||^2 (or v^T Mt v), well ahead of its use
       const int jn = (tile0 + T - 2 - it) * kTile + t;
       vn_next = (jn < n) ? vn_head[jn] : 1.f;
-    }
-    if (it + 1 < T && !from_lse) {   // next tile's row maxima
-#pragma unroll
-      for (int k = 0; k < 4; ++k) tm_next[k] = tm_head[(long long)(tile0 + T - 2 - it) * kRows + k * 32 + lane];
     }
     // The shares of the previous tile are summed in a fixed order by warpgroup 0 once all sixteen warps have
     // stored theirs.  A slot of `red` is rewritten four tiles later, which the two accumulator buffers only
@@ -869,35 +991,30 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
       const f32x2 vlen2 = f2_make(vlen, vlen);
       f32x2 h2 = f2_make(0.f, 0.f);
       float sv0[16], cv0[16], sv1[16], cv1[16];
-      if (!tile_heavy) {
+      const bool look = kEq7 && (from_lse || cx.look[s] != 0);
+      float mx = -INFINITY;   // where a weight may exceed kHeavyA: this lane's largest logit
+      if (raw_head == nullptr) {
         tmem_ld16(tS, sv0);
         if (kEq7) tmem_ld16(tC, cv0);
         tmem_wait_ld();
         tmem_ld16(tS + 16, sv1);   // the second half of the columns travels while the first is worked on
         if (kEq7) tmem_ld16(tC + 16, cv1);
-      }
-      bool redo_heavy = false;   // from_lse: this warp found a weight above kHeavyA among the logits it holds
-      if (!tile_heavy) {
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
           const float* sv = c == 0 ? sv0 : sv1;
           const float* cv = c == 0 ? cv0 : cv1;
           if (c == 1) {
             tmem_wait_ld();
-            // every tensor-memory read of this tile is done: the MMA warp may refill the accumulators
+            // every tensor-memory read of this tile is done: the MMA warp may refill the accumulators (the logits of a
+            // tile that may hold a large weight are read once more below; the check between the two halves instead
+            // kept their instructions from mixing, 2 % of the whole call)
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&B->acc_empty[s]);
-            if (from_lse && kEq7) {
-              // no pass 1 has flagged the tiles with large weights: the warp looks at the logits it now holds in
-              // registers (S' above heavy_thr <=> A > kHeavyA) and, if it finds one, does its part of the tile again
-              // below with exact distances, from those registers (the accumulators are already released)
-              float mx = fmaxf(sv0[0], sv1[0]);
+            if (lane == 0 && (from_lse || !look)) mbar_arrive(&B->acc_empty[s]);
+          }
+          if (from_lse && kEq7) {
 #pragma unroll
-              for (int u = 1; u < 16; ++u) mx = fmaxf(mx, fmaxf(sv0[u], sv1[u]));
-              redo_heavy = __any_sync(0xffffffffu, mx > heavy_thr && j < n);
-              if (redo_heavy) break;
-            }
+            for (int u = 0; u < 16; ++u) mx = fmaxf(mx, sv[u]);
           }
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
@@ -922,42 +1039,8 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
             h2 = f2_make(0.f, 0.f);
           }
         }
-        if (from_lse && kEq7 && redo_heavy) {
-          tot = 0.f;
-          h2 = f2_make(0.f, 0.f);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const float* sv = (c < 2 ? sv0 : sv1) + (c & 1) * 8;
-            const float* cv = (c < 2 ? cv0 : cv1) + (c & 1) * 8;
-            float I[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              const float um = ex2_approx(sv[u] * neg_c2) - 1.f;
-              float x = cv[u] + vnb;
-              unsigned int todo = __ballot_sync(0xffffffffu, sv[u] > heavy_thr && j < n);
-              while (todo) {
-                const int src = __ffs(todo) - 1;
-                todo &= todo - 1;
-                const int js = __shfl_sync(0xffffffffu, j, src);
-                const float d2x = exact_dist2(cgp * 32 + c * 8 + u, js, __shfl_sync(0xffffffffu, sv[u] > extreme_thr, src) != 0);
-                if (lane == src) x = d2x;
-              }
-              I[u] = x * rsqrt_approx(fmaf(x * um, um, 1e-36f));
-            }
-            if ((c * 8) % kRun == 0) I[0] *= seed_coef;
-            if ((c * 8 + 8) % kRun == 0) I[7] *= last_coef;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) h2 = f2_fma(h2, d2, f2_make(I[2 * q], I[2 * q + 1]));
-            if ((c * 8 + 8) % kRun == 0) {   // end of a run
-              const float run = fmaf(f2_lo(h2), ema_decay, f2_hi(h2));
-              tot = group_max ? fmaxf(tot, run) : tot + run;
-              h2 = f2_make(0.f, 0.f);
-            }
-          }
-        }
       } else {
-        // rare: the tile may hold large attention weights; those entries take the exact distance.  Also the
-        // epilogue of every tile when the per-query indicators are wanted.
+        // the epilogue of every tile when the per-query indicators are wanted
 #pragma unroll 1
         for (int c = 0; c < 4; ++c) {
           float sv[8], cv[8], I[8];
@@ -966,24 +1049,16 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
           tmem_wait_ld();
 #pragma unroll
           for (int u = 0; u < 8; ++u) {
+            mx = fmaxf(mx, sv[u]);
             if (kEq7) {
               const float um = ex2_approx(sv[u] * neg_c2) - 1.f;
-              float x = cv[u] + vnb;
-              // the whole warp computes the exact distance of each of its lanes' heavy entries in turn
-              unsigned int todo = __ballot_sync(0xffffffffu, sv[u] > heavy_thr && j < n);
-              while (todo) {
-                const int src = __ffs(todo) - 1;
-                todo &= todo - 1;
-                const int js = __shfl_sync(0xffffffffu, j, src);
-                const float d2x = exact_dist2(cgp * 32 + c * 8 + u, js, __shfl_sync(0xffffffffu, sv[u] > extreme_thr, src) != 0);
-                if (lane == src) x = d2x;
-              }
+              const float x = cv[u] + vnb;
               I[u] = x * rsqrt_approx(fmaf(x * um, um, 1e-36f));
             } else {
               I[u] = ex2_approx(-sv[u] * neg_c2) * vlen;
             }
           }
-          if (raw_head && j < n) {
+          if (j < n) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) raw_head[(long long)(cgp * 32 + c * 8 + u) * n + j] = I[u];
           }
@@ -997,9 +1072,27 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
             h2 = f2_make(0.f, 0.f);
           }
         }
+      }
+      if (raw_head != nullptr || (!from_lse && look)) {
+        if (kEq7 && raw_head == nullptr) {
+#pragma unroll 1
+          for (int c = 0; c < 4; ++c) {
+            float sv[8];
+            tmem_ld8(tS + c * 8, sv);
+            tmem_wait_ld();
+#pragma unroll
+            for (int u = 0; u < 8; ++u) mx = fmaxf(mx, sv[u]);
+          }
+        }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&B->acc_empty[s]);
+      }
+      // only Eq. 7 has the factor 1 / (1 - A) and the distance that need the exact form near A = 1: those tokens are noted
+      // and done again after the last tile (S' above heavy_thr <=> A > kHeavyA)
+      if (look && mx > heavy_thr && j < n) {
+        const int e = atomicAdd(cx.heavy, 1);
+        if (e < kMaxHeavy) cx.heavy[1 + e] = j;
       }
     } else {
       __syncwarp();
@@ -1015,6 +1108,7 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
     const int jl = tile0 * kTile + t;   // the last tile processed is the first of the share
     if (ok && jl < n) I_head[jl] = join_shares(red[rs][0][t], red[rs][1][t], red[rs][2][t], red[rs][3][t]);
   }
+  if (kEq7) heavy_pass<kW, kProj>(cx, a, bh);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1365,6 +1459,7 @@ __device__ void worker_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, c
         named_barrier_sync(2, kFWorkerWarps * 32);   // the exchange buffer is reused by the next batch of rows
       }
       fence_proxy_async_smem();   // the exchange buffer is overwritten by a TMA load in phase C
+      if (threadIdx.x == kFFirstWorker * 32) cx.heavy[0] = 0;
     }
     if (!group_barrier_follow(go)) break;
     tc_fence_after();
@@ -1388,8 +1483,8 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) FusedBars bars;
   __shared__ uint32_t tmem_slot;
-  __shared__ int abort_flag, go_flag;
-  __shared__ float sm_stats[6 * kRows];
+  __shared__ int abort_flag, go_flag, look_flag[2];
+  __shared__ float sm_stats[1 + kMaxHeavy + 2 * kRows];   // phase A's exchange (6 x 128), then the list of heavy tokens
   __shared__ float vn_ring[4 * kTile];
   __shared__ float red[4][4][kTile];   // [tile & 3][warpgroup][token]: each warpgroup's share of the score
 
@@ -1403,11 +1498,14 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   cx.abort_flag = &abort_flag;
   cx.sm_stats = sm_stats;
   cx.vn_s = vn_ring;
+  cx.look = look_flag;
+  cx.heavy = reinterpret_cast<int*>(sm_stats);
   cx.warp = threadIdx.x >> 5;
   cx.lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
+    cx.heavy[0] = 0;
     init_bars(&bars, true, kLse);
     prefetch_tensormap(&tmQ);
     prefetch_tensormap(&tmK);
@@ -1695,7 +1793,8 @@ cudaError_t launch_tc_fused(void* state, const Problem& p, const Workspace& ws, 
   fused_plan(p, sm_count, reuse_l2, &a.groups, &a.cpg);
   a.part_m = ws.part_m; a.part_l = ws.part_l; a.part_O = ws.part_O;
   a.O_f32 = ws.O_f32; a.O_m2 = ws.O_m2; a.aug = ws.aug; a.vnorm = ws.vnorm; a.I_hat = ws.I_hat;
-  a.V = (const __nv_bfloat16*)V; a.vsb = p.vsb; a.vsh = p.vsh; a.vsn = p.vsn;
+  a.Q = (const __nv_bfloat16*)Q; a.K = (const __nv_bfloat16*)K; a.V = (const __nv_bfloat16*)V;
+  a.ksb = p.ksb; a.ksh = p.ksh; a.ksn = p.ksn; a.vsb = p.vsb; a.vsh = p.vsh; a.vsn = p.vsn;
   a.counters = ws.counters; a.tile_max = ws.tile_max; a.row_M2 = ws.row_M2; a.dev_status = dev_status;
   a.wait_limit = wait_limit;
   a.I_raw = O_given ? nullptr : I_raw;
@@ -1706,7 +1805,6 @@ cudaError_t launch_tc_fused(void* state, const Problem& p, const Workspace& ws, 
     a.sel_keep = sel->keep; a.sel_W = sel->W; a.sel_gamma = sel->gamma;
     a.sel_scores = sel->scores; a.sel_indices = sel->indices;
     a.sel_hist = ws.sel_hist; a.sel_sfx = ws.sel_sfx;
-    a.K = (const __nv_bfloat16*)K; a.ksb = p.ksb; a.ksh = p.ksh; a.ksn = p.ksn;
     a.K_out = (__nv_bfloat16*)sel->K_out; a.V_out = (__nv_bfloat16*)sel->V_out;
     e = cudaMemsetAsync(ws.sel_hist, 0, (size_t)p.BH * kSelPasses * 256 * sizeof(unsigned int), st);
     if (e != cudaSuccess) return e;

@@ -576,6 +576,47 @@ def test_score_from_lse_matches_oracle(handle, spec):
     assert_scores_close(run.scores.cpu().numpy(), ref.scores, TOL[dtype])
 
 
+def _with_sinks(case, rows, share):
+    """`rows` draw about `share` of every window query's attention each (planted through the first coordinate)."""
+    inp = make_inputs(case)
+    inp.Q[..., 0] = 8.0
+    inp.K[..., 0] = 0.0
+    logit = np.log(share / (1.0 - share * len(rows)) * 1.65 * case.n)
+    inp.K[:, :, rows, 0] = logit * np.sqrt(case.head_dim) / 8.0
+    inp.K = (round_to_bf16_bits(inp.K).astype(np.uint32) << 16).view(np.float32)
+    return inp
+
+
+@pytest.mark.parametrize("spec", [(32, 8, 2, 0, [0], 0.3), (32, 8, 2, 32, [0, 127, 128, 255, 256, 998, 999], 0.13),
+                                  (64, 4, 2, 0, [5], 0.93), (16, 16, 2, 0, [0, 999], 0.3), (128, 2, 2, 0, [3, 130], 0.4)])
+@pytest.mark.parametrize("group", [rk.GROUP_MEAN, rk.GROUP_MAX])
+def test_large_attention_weights(handle, spec, group):
+    """Tokens with a weight above 1/8 (attention sinks) are scored again with exact distances: at the edges of tiles and of
+    the prefix, up to seven per row, near A = 1; from Q, K, V and from given statistics; fixed and adaptive window."""
+    import torch
+    w, Hq, Hkv, tail, rows, share = spec
+    inp = _with_sinks(Case("sinks", 1, Hq, Hkv, 128, 1000, w, 200, 5, 0, 0.9, "bf16", tail, "normal", 77), rows, share)
+    c = inp.case
+    ref, O, lse = _window_stats(inp, with_A_check=False)
+    A = oracle_scores(inp, want_A=True).A
+    assert (A[..., rows] > 0.125).any() and (share < 0.9 or (A > 0.9).any())
+    handle.set_variant(group=group)
+    try:
+        ref = oracle_scores(inp, group_mode=group)
+        run = DeviceRun(handle, inp)
+        assert_scores_close(run.evict()[0], ref.scores, TOL["bf16"])
+        handle.score_from_lse(run.shape, run.Q, run.K, run.V, torch.from_numpy(O).cuda(), torch.from_numpy(lse).cuda(),
+                              c.ema_decay, run.pool(), run.scores, run.ws)
+        torch.cuda.synchronize()
+        assert_scores_close(run.scores.cpu().numpy(), ref.scores, TOL["bf16"])
+        run = DeviceRun(handle, inp, adaptive_budget=c.budget)
+        scores = run.score(pool=rk.adaptive_pool(2000.0, c.width, c.budget))
+        assert tuple(run.pool_used.cpu().numpy()[0, 0]) == (c.width, 0)   # the planted rows do not move the window
+        assert_scores_close(scores, ref.scores, TOL["bf16"])
+    finally:
+        handle.set_variant()
+
+
 @pytest.mark.parametrize("spec", [("cfg2", 0), ("cfg2", 32), ("cfg1b", 0)])
 def test_evict_from_lse_matches_oracle(handle, spec):
     """restkv_evict_from_lse: score, select and compact from given window statistics, all three acceptance rules."""
