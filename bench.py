@@ -311,7 +311,6 @@ def main():
         flush.zero_()
         step()
     barrier()
-    fused = handle.last_evict_fused_select()
     launches0 = handle.launch_count()
     sampler = ClockSampler(local)
     if rank == 0:
@@ -330,8 +329,8 @@ def main():
 
     # Per-kernel durations in passes of their own (the event records between the launches would sit inside the
     # timed region otherwise): CUDA events recorded by the library right around each launch, on the call's stream.
-    # On the tensor-core path with a fixed window one persistent launch does everything (pass 1, merge, pass 2,
-    # pooling, selection, gather); a second pass with the selection as its own kernel gives the split.
+    # On the tensor-core path with a fixed window a step is two launches: the score kernel (pass 1, merge, pass 2) and the
+    # selection (pooling, top-B, gather), which is chained to it except in these passes.
     def kernel_pass(kernel_ids, reps):
         prof = {}
         for name in kernel_ids:
@@ -352,18 +351,7 @@ def main():
             handle.set_profile_events(kid, None, None)
         return {k: float(np.mean(v)) for k, v in ms.items()}
 
-    split_ids = {"score": rk.KERNEL_PASS2, "pool_select_compact": rk.KERNEL_SELECT}
-    if case.batch * case.n_kv_heads * 8 > 148:      # many rows: the gather runs as its own kernel
-        split_ids = {"score": rk.KERNEL_PASS2, "pool_select": rk.KERNEL_SELECT, "compact": rk.KERNEL_COMPACT}
-    reps = max(3, min(args.steps, 20))
-    kmean_split = None
-    if fused:
-        kmean = kernel_pass({"score_pool_select_compact": rk.KERNEL_PASS2}, reps)
-        handle.set_fused_select(False)
-        kmean_split = kernel_pass(split_ids, reps)
-        handle.set_fused_select(True)
-    else:
-        kmean = kernel_pass(split_ids, reps)
+    kmean = kernel_pass({"score": rk.KERNEL_PASS2, "pool_select_compact": rk.KERNEL_SELECT}, max(3, min(args.steps, 20)))
     clocks = sampler.stop() if rank == 0 else None      # sampled through the timed steps and the per-kernel passes
     assert handle.poll_status() == rk.RESTKV_OK
 
@@ -578,7 +566,8 @@ def main():
                 torch.cuda.synchronize()
                 if it >= 3:
                     tp.append(ev0.elapsed_time(ev1))
-            pk = kernel_pass({"value_forms": rk.KERNEL_PASS1, "score_pool_select_compact": rk.KERNEL_PASS2}, 5)
+            pk = kernel_pass({"value_forms": rk.KERNEL_PASS1, "score": rk.KERNEL_PASS2,
+                              "pool_select_compact": rk.KERNEL_SELECT}, 5)
         finally:
             handle.set_output_projection(None)
         assert handle.poll_status() == rk.RESTKV_OK
@@ -635,15 +624,12 @@ def main():
     peaks = load_peaks()
     kv_bytes, out_bytes = algorithmic_bytes(case, keep)
     flops = algorithmic_flops(case)
-    dominant = "score_pool_select_compact" if fused else "score"
-    # algorithmic bytes of the dominant kernel: K and V once plus 4 B of score per token and head, and, when it also
-    # selects and gathers, the indices and the compacted cache written
+    dominant = "score"
+    # algorithmic bytes of the dominant kernel: K and V once plus 4 B of score per token and head
     dom_bytes = kv_bytes + 4 * case.batch * case.n_kv_heads * case.n_kv
-    if fused:
-        dom_bytes += out_bytes + 4 * case.batch * case.n_kv_heads * keep
     achieved = dom_bytes / (kmean[dominant] * 1e-3) / 1e9
     roofline = {"bound": "hbm",
-                "kernel": "tc_fused_kernel (pass 1 + merge + pass 2%s)" % (" + pooling + selection + gather" if fused else ""),
+                "kernel": "tc_fused_kernel (pass 1 + merge + pass 2)",
                 "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"],
                 "traffic": measured_traffic(args.workload) if args.path == 0 else None,
                 "peak_source": peaks["source"], "algorithmic_bytes_per_launch": dom_bytes,
@@ -659,7 +645,7 @@ def main():
         "config": workload_config(case, l2="flushed between steps (256 MiB write); inputs 537 MB > 126 MB L2"),
         "clocks": clocks, "e2e": e2e, "gpu_launches": int(launches),
         "roofline": roofline, "path_roofline": path_roofline, "kernels_ms": kmean,
-        "kernels_ms_selection_as_own_kernel": kmean_split, "decode": decode, "from_lse": from_lse,
+        "decode": decode, "from_lse": from_lse,
         "variants": variants, "adaptive_window": adaptive, "reevict": reevict, "output_projection": projection,
     }
     if not args.no_cpu_baseline and world == 1:

@@ -82,8 +82,8 @@ typedef struct {
   int budget;     /* ADAPTIVE: B of Eq. 10 (per-query top-B whose mean index gives D_front / D_rear) */
 } restkv_pool_params;
 
-/* Creates a handle for the CURRENT device: queries its properties and allocates a 256-byte
- * device status block (the only allocation the library ever makes).  Host pointer out. */
+/* Creates a handle for the CURRENT device: queries its properties and allocates a device block of
+ * 1280 bytes for status and barrier counters (the only allocation the library ever makes).  Host pointer out. */
 restkv_status restkv_create(restkv_handle** out);
 restkv_status restkv_destroy(restkv_handle* h);
 
@@ -248,7 +248,8 @@ const char* restkv_error_string(restkv_status s);
  * single kernels of the fused path with CUDA events.  start/stop are cudaEvent_t handles created by the caller
  * with timing enabled; passing NULL for both clears the pair.  On the tensor-core path pass 1, the merge and pass 2
  * are one launch, recorded as RESTKV_KERNEL_PASS2 (PASS1 and COMBINE fire on the SIMT path only); in restkv_evict
- * the pooling and the gather run inside the select kernel, recorded as RESTKV_KERNEL_SELECT. */
+ * the pooling and the gather run inside the select kernel, recorded as RESTKV_KERNEL_SELECT (events around it keep it from
+ * being chained to the kernel before). */
 typedef enum {
   RESTKV_KERNEL_NONE = 0, RESTKV_KERNEL_PASS1 = 1, RESTKV_KERNEL_COMBINE = 2, RESTKV_KERNEL_PASS2 = 3,
   RESTKV_KERNEL_POOL = 4, RESTKV_KERNEL_SELECT = 5, RESTKV_KERNEL_COMPACT = 6
@@ -262,12 +263,12 @@ restkv_status restkv_set_profile_events(restkv_handle* h, int which, void* start
  * barriers per head; the slower of the two on today's shapes). */
 restkv_status restkv_set_kernel_path(restkv_handle* h, int path);
 
-/* restkv_evict on the tensor-core path with a fixed window lets the score kernel itself pool (Eq. 13), select and
- * gather (Eq. 14) each head, with the head's own thread blocks, as soon as the head's scores are complete (default:
- * on).  With 0 the pooling, selection and gather always run as the separate kernel that other paths use; the results
- * are the same.  Meant for timing the two against each other. */
+/* The launch of restkv_evict that pools (Eq. 13), selects and gathers (Eq. 14) is chained to the score kernel: its blocks
+ * may be scheduled while the last blocks of that kernel run (default: on).  With 0 it is an ordinary launch in stream
+ * order; the results are the same.  Meant for timing the two against each other. */
 restkv_status restkv_set_fused_select(restkv_handle* h, int on);
-int restkv_last_evict_fused_select(const restkv_handle* h);   /* 1 if the last restkv_evict ran them inside the score kernel */
+int restkv_last_evict_fused_select(const restkv_handle* h);   /* 1 if the last restkv_evict ran with a fixed window on the
+                                                                 tensor-core path with that launch chained */
 
 /* Bound of every device-side wait of the persistent kernels, in SM clocks (default 2e9, about a second).  A wait
  * that runs out sets the sticky status (RESTKV_ERR_TIMEOUT from restkv_poll_status), the kernel stops issuing
@@ -284,7 +285,7 @@ restkv_status restkv_set_wait_limit(restkv_handle* h, long long sm_clocks);
  *   indices      device int32 [batch, n_kv_heads, S]: the kept rows of a head ascending, then -1 up to S
  *   K_out, V_out device [batch, n_kv_heads, S, head_dim]: rows past a head's count are left untouched
  *   scores_out, workspace (restkv_workspace_bytes[_adaptive](shape, max_budget)), pool, errors: as restkv_evict.
- * The selection and the gather run in the cluster select kernel (never inside the score kernel).
+ * The selection and the gather run in the same select kernel.
  */
 restkv_status restkv_evict_budgets(restkv_handle* h, const restkv_shape* shape, const void* Q_obs, const void* K,
                                    const void* V, float ema_decay, const restkv_pool_params* pool,

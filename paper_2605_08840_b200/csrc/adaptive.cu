@@ -2,46 +2,38 @@
 // top-B rows of the raw indicator over the first and second half of the window queries; the box
 // width and shift follow from their difference.
 #include "restkv_common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace restkv {
 
 namespace {
 
-__global__ void zero_sums_kernel(unsigned long long* sums, int count) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < count) sums[i] = 0ull;
-}
-
-// grid = batch*Hq*w rows of idx [rows, Bp]; adds each row's index sum to its KV head's front or rear total.
-__global__ void index_sum_kernel(int Hq, int G, int w, int Bp, const int32_t* __restrict__ idx,
-                                 unsigned long long* __restrict__ sums) {
-  const int row = blockIdx.x;            // (b, hq, i)
-  const int i = row % w;
-  const int bhq = row / w;
-  const int b = bhq / Hq, hq = bhq % Hq;
-  const int Hkv = Hq / G;
-  const int bh = b * Hkv + hq / G;
-  unsigned long long s = 0;
-  for (int k = threadIdx.x; k < Bp; k += blockDim.x) s += (unsigned long long)idx[(long long)row * Bp + k];
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  __shared__ unsigned long long red[32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long t = 0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += red[k];
-    atomicAdd(&sums[2 * bh + (i < w / 2 ? 0 : 1)], t);
-  }
-}
-
-__global__ void window_params_kernel(int BH, int G, int w, int Bp, double beta, int base_width,
+// grid BH, block 128: the index sums of the head's w * G rows (front and rear half of the window apart), `parts` values per
+// row, and from them the head's window.
+__global__ void window_params_kernel(int G, int w, int Bp, int parts, double beta, int base_width,
                                      const unsigned long long* __restrict__ sums, int* __restrict__ pool) {
-  const int bh = blockIdx.x * blockDim.x + threadIdx.x;
-  if (bh >= BH) return;
+  ptx::grid_dependency_wait();
+  const int bh = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  unsigned long long front = 0, rear = 0;
+  for (int e = threadIdx.x; e < G * w * parts; e += blockDim.x) {
+    const unsigned long long s = sums[(long long)bh * G * w * parts + e];
+    if ((e / parts) % w < w / 2) front += s;
+    else rear += s;
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    front += __shfl_xor_sync(0xffffffffu, front, off);
+    rear += __shfl_xor_sync(0xffffffffu, rear, off);
+  }
+  __shared__ unsigned long long red[4][2];
+  if (lane == 0) { red[wid][0] = front; red[wid][1] = rear; }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int k = 1; k < 4; ++k) { front += red[k][0]; rear += red[k][1]; }
   const long long cnt_front = (long long)G * (w / 2) * Bp;
   const long long cnt_rear = (long long)G * (w - w / 2) * Bp;
-  const double D_rear = (double)sums[2 * bh + 1] / (double)cnt_rear;
-  const double D_front = cnt_front ? (double)sums[2 * bh] / (double)cnt_front : D_rear;
+  const double D_rear = (double)rear / (double)cnt_rear;
+  const double D_front = cnt_front ? (double)front / (double)cnt_front : D_rear;
   const double x = (D_front - D_rear) / beta;
   const int Ws = 2 * (int)floor(fabs(x)) + 1;   // Eq. 11
   const int gamma = (int)trunc(x);              // Eq. 12, truncating toward zero
@@ -52,21 +44,26 @@ __global__ void window_params_kernel(int BH, int G, int w, int Bp, double beta, 
 }  // namespace
 
 cudaError_t launch_adaptive_params(const Problem& p, const Workspace& ws, int budget, float beta, int base_width,
-                                   cudaStream_t st, int* n_launches) {
+                                   const int* clusters_of, unsigned int* dev_status, cudaStream_t st, int* n_launches) {
   int Bp = budget - p.tail;
   if (Bp > p.n) Bp = p.n;
   const int rows = p.batch * p.Hq * p.w;
   *n_launches = 0;
-  cudaError_t e = launch_select(rows, p.n, p.n, Bp, nullptr, nullptr, nullptr, 1, 0, false, ws.I_raw, ws.adaptive_idx, nullptr, nullptr, nullptr,
-                                nullptr, nullptr, nullptr, st);
+  cudaError_t e = launch_select(rows, p.n, p.n, Bp, nullptr, nullptr, nullptr, 1, 0, false, ws.I_raw, nullptr, ws.adaptive_sums,
+                                nullptr, nullptr, nullptr, nullptr, nullptr, clusters_of, dev_status, true, st);
   if (e != cudaSuccess) return e;
-  ++*n_launches;
-  zero_sums_kernel<<<(2 * p.BH + 127) / 128, 128, 0, st>>>(ws.adaptive_sums, 2 * p.BH);
-  index_sum_kernel<<<rows, 256, 0, st>>>(p.Hq, p.G, p.w, Bp, ws.adaptive_idx, ws.adaptive_sums);
-  window_params_kernel<<<(p.BH + 127) / 128, 128, 0, st>>>(p.BH, p.G, p.w, Bp, (double)beta, base_width,
-                                                           ws.adaptive_sums, ws.pool);
-  *n_launches += 3;
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned int)p.BH);
+  cfg.blockDim = dim3(128);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  *n_launches = 2;
+  return cudaLaunchKernelEx(&cfg, window_params_kernel, p.G, p.w, Bp, select_cluster(rows, p.n, clusters_of), (double)beta,
+                            base_width, (const unsigned long long*)ws.adaptive_sums, ws.pool);
 }
 
 }  // namespace restkv

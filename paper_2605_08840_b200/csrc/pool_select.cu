@@ -2,6 +2,7 @@
 #include <cooperative_groups.h>
 
 #include "restkv_common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace restkv {
 
@@ -24,7 +25,7 @@ __device__ __forceinline__ float box_mean(const float* __restrict__ src, int n, 
     return s;
   }
   for (int t = lo; t <= hi; ++t) s += src[t];
-  return s / (float)W;
+  return s * (1.f / (float)W);
 }
 
 // grid (ceil(n_kv/256), BH).  The window (W, gamma) comes from `pool` (per head, device) when it is non-null.
@@ -42,7 +43,7 @@ __global__ void pool_kernel(int n, int n_kv, const float* __restrict__ I_hat, co
 // Radix select.  Scores map to unsigned keys whose order matches the float order.
 __device__ __forceinline__ unsigned int float_key(float x) {
   const unsigned int u = __float_as_uint(x);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  return u ^ ((unsigned int)((int)u >> 31) | 0x80000000u);
 }
 
 // Optional gather fused into the select kernel (all pointers null: indices only).  K, V addressed by element strides;
@@ -56,363 +57,398 @@ struct GatherArgs {
   int Hkv, esize, row_chunks;
 };
 
-constexpr int kSelThreads = 1024;
-constexpr int kSelBins = 256;                // 8-bit digits
-constexpr int kSelMaxSmemKeys = 44 * 1024;   // keys of one CTA's slice kept in shared memory (176 KB)
-constexpr int kSelMaxStagedWidth = 65;       // widest box whose taps are staged in shared memory
+struct SelectArgs {
+  int n, n_kv, keep;            // keep: entries per row, also the row stride of the outputs
+  const int* keep_rows;         // non-null: row r keeps min(max(keep_rows[r], 1), keep), the rest of its indices is -1
+  const float* I_hat;           // non-null: pool first (Eq. 13) and write the pooled scores; null: read `scores`
+  const int* pool;              // per row (W, gamma) on the device, or null: W, gamma below
+  int W, gamma, pool_max;
+  float* scores;
+  int32_t* indices;
+  unsigned long long* index_sums;   // non-null: the sum of each row's kept indices instead of the indices
+  int parts;                    // blocks per row: the cluster's, or (no cluster) blocks that each select from the whole row
+  int per;                      // keys of one block's slice
+  int held;                     // 1: the slice's keys stay in shared memory; 0: they are formed again from the scores
+  int room;                     // floats of shared memory behind the keys: the taps, later the indices this block gathers and
+                                //  the rows on their way
+  int copy_rows;                // rows that a warp copies at a time
+  int own_idx;                  // 1: the indices fit there
+  unsigned int* dev_status;
+  GatherArgs ga;
+};
 
-// Inclusive scan over the 1024 threads of the block, in thread order.
-__device__ __forceinline__ unsigned int block_inclusive_scan(unsigned int v, unsigned int* warp_sums) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const unsigned int t = __shfl_up_sync(0xffffffffu, v, off);
-    if (lane >= off) v += t;
-  }
-  if (lane == 31) warp_sums[wid] = v;
-  __syncthreads();
-  if (wid == 0) {
-    unsigned int w = warp_sums[lane];
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const unsigned int t = __shfl_up_sync(0xffffffffu, w, off);
-      if (lane >= off) w += t;
+constexpr int kSelBins = 2048;               // 11-bit digits
+constexpr unsigned int kInfKey = 0xFF800000u;
+
+// Bounded wait for a bulk copy.
+__device__ __forceinline__ void wait_copy(uint64_t* bar, uint32_t parity, unsigned int* dev_status) {
+  const long long t0 = clock64();
+  while (!ptx::mbar_try_wait(bar, parity))
+    if (clock64() - t0 > 4000000000ll) {
+      atomicOr(dev_status, (unsigned int)kDevTimeout);
+      return;
     }
-    warp_sums[lane] = w;   // inclusive over warps
-  }
-  __syncthreads();
-  if (wid > 0) v += warp_sums[wid - 1];
-  __syncthreads();   // warp_sums may be reused by the caller
-  return v;
 }
 
-// Box means of one CTA's slice from its staged taps (staged[t - s_lo] = I_hat[t] for t in [s_lo, s_hi]), summed in
-// the same order as box_mean; writes the pooled scores and their keys.  kWidth = 0: width known only at run time.
-template <int kWidth>
-__device__ __forceinline__ void pool_staged(const float* __restrict__ staged, int s_lo, int s_hi, int n, int j0, int cnt,
-                                            int W, int gamma, float* __restrict__ srow, unsigned int* __restrict__ skeys) {
-  const int width = kWidth ? kWidth : W;
-  const int half = width / 2;
-  const float fw = (float)width;
-  for (int jj = threadIdx.x; jj < cnt; jj += kSelThreads) {
-    const int j = j0 + jj;
-    float out = INFINITY;
-    if (j < n) {
-      const long long a64 = (long long)j - half + gamma, b64 = (long long)j + half + gamma;
-      float acc = 0.f;
-      if (a64 >= s_lo && b64 <= s_hi) {   // the whole window is staged: fixed trip count
-        const float* p = staged + (int)(a64 - s_lo);
-        if (kWidth) {
+// Box means of rows [0, scored) of a slice from its staged taps (row jj: taps[jj .. jj + W - 1]), +inf for the rows from
+// there to cnt; f(jj, score) for each.  kW = 0: the width is known only at run time, pool_max: the maximum instead.
+template <int kThreads, int kW, typename F>
+__device__ __forceinline__ void pool_slice(const float* taps, int W, bool pool_max, int scored, int cnt, F&& f) {
+  const float inv = 1.f / (float)(kW ? kW : W);
+#pragma unroll 2
+  for (int jj = threadIdx.x; jj < cnt; jj += kThreads) {
+    float acc = 0.f;
+    if (kW) {
 #pragma unroll
-          for (int k = 0; k < kWidth; ++k) acc += p[k];
-        } else {
-          for (int k = 0; k < width; ++k) acc += p[k];
-        }
-      } else {
-        const int a = a64 < s_lo ? s_lo : (int)(a64 <= s_hi ? a64 : s_hi + 1), b = b64 > s_hi ? s_hi : (int)(b64 >= s_lo ? b64 : s_lo - 1);
-        for (int t = a; t <= b; ++t) acc += staged[t - s_lo];
-      }
-      out = acc / fw;
+      for (int t = 0; t < kW; ++t) acc += taps[jj + t];
+    } else if (pool_max) {
+      for (int t = 0; t < W; ++t) acc = fmaxf(acc, taps[jj + t]);
+    } else {
+#pragma unroll 4
+      for (int t = 0; t < W; ++t) acc += taps[jj + t];
     }
-    srow[jj] = out;
-    skeys[jj] = float_key(out);
+    f(jj, jj < scored ? ((!kW && pool_max) ? acc : acc * inv) : INFINITY);
   }
 }
 
-// One thread-block cluster per row; CTA `rank` of the cluster owns the contiguous slice [rank*per, (rank+1)*per)
-// of the row.  With I_hat non-null the kernel first applies the box mean of Eq. 13 and writes the pooled scores;
-// otherwise it reads `scores`.  The keys of the slice stay in shared memory (use_smem) or are re-read from
-// `scores`.  The cluster first agrees on the smallest and largest key: the bits they share are common to every
-// key and are skipped.  The remaining bits are resolved 8 at a time from the top: every warp counts into its own
-// 256-bin histogram (no contention between warps), the CTA sums them, the cluster sums the CTAs' histograms
-// through distributed shared memory, and one warp finds the bin that holds the keep-th largest key.  That yields
-// the key T of the keep-th largest score and how many scores equal to T are kept; an ordered pass then writes,
-// in ascending index order, every index whose key is > T plus the first kept ones whose key equals T (lower
-// index wins ties).
-// keep_rows non-null: row r keeps min(max(keep_rows[r], 1), keep) entries instead of `keep` (non-uniform budgets);
-// its outputs still have a row stride of `keep`, the unused tail of its indices is set to -1.
-__global__ void __launch_bounds__(kSelThreads, 1)
-select_kernel(int n, int n_kv, int keep, const int* __restrict__ keep_rows, const float* __restrict__ I_hat, const int* __restrict__ pool, int W,
-              int gamma, int pool_max, float* scores, int32_t* __restrict__ indices, int32_t* __restrict__ pool_used,
-              int per, int use_smem, int stage_taps, GatherArgs ga) {
+// Top-B of one row by its blocks, with the pooling before it and the gather behind it.
+//
+// What bounds it: a row's scores are a few hundred KB at most and come from L2, so the kernel is a chain of latencies:
+// global loads, block-wide and cluster-wide synchronisations, shared-memory atomics, and instructions fetched for the first
+// time (so the loops are kept short; with keys in registers and the loops over them unrolled the 128k workload took 48 us,
+// most of it for fetching straight-line code).  Hence:
+//   - long rows: one cluster per row, CTA `part` owns the slice [part * per, (part + 1) * per).  Short rows: no cluster;
+//     every block of the row selects from the whole row by itself, which takes no longer than the cluster's exchanges would,
+//     and the blocks share the gather only;
+//   - the slice's keys stay in shared memory; a warp owns a contiguous run of them, so that the ordered emit needs only
+//     ballots;
+//   - the smallest key and the largest finite one are agreed on first; keys count as offsets from the smallest, +inf as one
+//     past the largest.  The first 11-bit digit then spreads the scores over about a thousand bins, so that one histogram
+//     serves all warps without contention, and the bin that holds the keep-th largest key is narrow: the passes end as soon
+//     as the rest of that bin is kept as a whole, usually after the second digit;
+//   - what the CTAs of a cluster tell one another (extremes, counts, positions of the kept rows) is put straight into the
+//     shared memory of whoever needs it, with one cluster barrier per exchange.
+// Measured (8 rows, gather included, timed alone): 131072 rows / 2048 kept 51 -> 31 us, 16384 / 1024 29 -> 14 us, 3032 / 1056
+// 10 us; 64 rows of 32768 / 2048 kept 73 (two kernels) -> 38 us.
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kernel(const __grid_constant__ SelectArgs a) {
   cg::cluster_group cluster = cg::this_cluster();
-  const unsigned int CS = cluster.num_blocks(), rank = cluster.block_rank();
-  const int row = blockIdx.x / CS;
-  extern __shared__ unsigned int skeys[];
-  __shared__ unsigned int wh[32][kSelBins];    // per-warp histograms
-  __shared__ unsigned int hist[2][kSelBins];   // the CTA's histogram of the current pass (double-buffered)
-  __shared__ unsigned int tot[kSelBins];       // the cluster's histogram
+  const int CS = (int)cluster.num_blocks();
+  const int row = (int)blockIdx.x / a.parts, part = (int)blockIdx.x % a.parts;
+  constexpr int kWarps = kThreads / 32, kBpt = kSelBins / kThreads;
+  extern __shared__ __align__(16) unsigned int skeys[];   // [per rounded up to 4] keys (if held), then [room]
+  float* const room = reinterpret_cast<float*>(skeys + (a.held ? (a.per + 3) & ~3 : 0));
+  __shared__ __align__(16) unsigned int hist[2][kSelBins];   // double-buffered: peers read one while the other is prepared
+  __shared__ unsigned int tot[kSelBins];                     // the cluster's histogram
   __shared__ unsigned int warp_a[32], warp_b[32];
-  __shared__ unsigned int s_digit, s_remaining;
-  __shared__ unsigned int cta_counts[2];
-  __shared__ unsigned int cta_minmax[2];
+  __shared__ unsigned int s_digit, s_remaining, s_count;
+  __shared__ unsigned int s_min, s_max, s_gt, s_eq;          // s_gt, s_eq: totals of the CTAs before this one
+  __shared__ __align__(8) uint64_t tap_bar, copy_bar[kWarps][2];
 
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const long long j0 = (long long)rank * per;
-  const int cnt = (int)max(0ll, min((long long)n_kv, j0 + per) - j0);
-  float* srow = scores + (long long)row * n_kv;
-  const int out_stride = keep;
-  int32_t* dst = indices + (long long)row * out_stride;
-  if (keep_rows) {
-    keep = min(max(keep_rows[row], 1), out_stride);
-    if (rank == 0)
-      for (int pos = keep + tid; pos < out_stride; pos += kSelThreads) dst[pos] = -1;
-  }
+  auto csync = [&]() { if (CS > 1) cluster.sync(); else __syncthreads(); };
+  auto in_cta = [&](auto* p, int r) { return CS > 1 ? cluster.map_shared_rank(p, r) : p; };
 
-  // ---- keys of the slice ----
-  if (I_hat) {
-    if (pool) { W = pool[2 * row]; gamma = pool[2 * row + 1]; }
-    if (pool_used && rank == 0 && tid == 0) { pool_used[2 * row] = W; pool_used[2 * row + 1] = gamma; }
-    const float* src = I_hat + (long long)row * n;
-    if (stage_taps && !pool_max && W <= kSelMaxStagedWidth && cnt > 0) {
-      // the taps of the whole slice (slice + halo) are staged in shared memory once, then summed from there in
-      // the same order as box_mean does
-      float* staged = reinterpret_cast<float*>(skeys + per);
-      const int half = W / 2;
-      const long long lo64 = j0 - half + gamma, hi64 = j0 + cnt - 1 + half + gamma;
-      const int s_lo = lo64 < 0 ? 0 : (int)(lo64 < n ? lo64 : n), s_hi = hi64 > n - 1 ? n - 1 : (int)(hi64 > -1 ? hi64 : -1);
-      // several loads in flight per thread
-      for (int t0 = s_lo + tid; t0 <= s_hi; t0 += 8 * kSelThreads) {
-        float v[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int t = t0 + k * kSelThreads;
-          v[k] = t <= s_hi ? src[t] : 0.f;
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int t = t0 + k * kSelThreads;
-          if (t <= s_hi) staged[t - s_lo] = v[k];
-        }
-      }
-      __syncthreads();
-      switch (W) {   // the common widths get a compile-time trip count
-        case 1: pool_staged<1>(staged, s_lo, s_hi, n, (int)j0, cnt, W, gamma, srow + j0, skeys); break;
-        case 3: pool_staged<3>(staged, s_lo, s_hi, n, (int)j0, cnt, W, gamma, srow + j0, skeys); break;
-        case 5: pool_staged<5>(staged, s_lo, s_hi, n, (int)j0, cnt, W, gamma, srow + j0, skeys); break;
-        case 7: pool_staged<7>(staged, s_lo, s_hi, n, (int)j0, cnt, W, gamma, srow + j0, skeys); break;
-        case 21: pool_staged<21>(staged, s_lo, s_hi, n, (int)j0, cnt, W, gamma, srow + j0, skeys); break;
-        case 31: pool_staged<31>(staged, s_lo, s_hi, n, (int)j0, cnt, W, gamma, srow + j0, skeys); break;
-        default: pool_staged<0>(staged, s_lo, s_hi, n, (int)j0, cnt, W, gamma, srow + j0, skeys); break;
-      }
-    } else {
-      for (int jj = tid; jj < cnt; jj += kSelThreads) {
-        const float out = box_mean(src, n, (int)(j0 + jj), W, gamma, pool_max != 0);
-        srow[j0 + jj] = out;
-        if (use_smem) skeys[jj] = float_key(out);
-      }
-    }
-  } else if (use_smem) {
-    for (int jj = tid; jj < cnt; jj += kSelThreads) skeys[jj] = float_key(srow[j0 + jj]);
+  for (int b = tid; b < kSelBins; b += kThreads) hist[0][b] = 0u;
+  if (tid == 0) {
+    s_min = 0xFFFFFFFFu;
+    s_max = s_gt = s_eq = 0u;
+    ptx::mbar_init(&tap_bar, 1);
+    for (int w = 0; w < 2 * kWarps; ++w) ptx::mbar_init(&copy_bar[0][0] + w, 1);
+    ptx::fence_mbar_init();
   }
-  __syncthreads();
-  auto key_at = [&](int jj) -> unsigned int { return use_smem ? skeys[jj] : float_key(srow[j0 + jj]); };
-
-  if (keep >= n_kv) {   // budget covers everything: identity (uniform over the cluster)
-    for (int jj = tid; jj < cnt; jj += kSelThreads) dst[j0 + jj] = (int32_t)(j0 + jj);
-    if (ga.K) {
-      const int b = row / ga.Hkv, h = row % ga.Hkv;
-      const unsigned char* Kh = ga.K + ((long long)b * ga.ksb + (long long)h * ga.ksh) * ga.esize;
-      const unsigned char* Vh = ga.V + ((long long)b * ga.vsb + (long long)h * ga.vsh) * ga.esize;
-      const int rc2 = 2 * ga.row_chunks;
-      for (long long e = tid; e < (long long)cnt * rc2; e += kSelThreads) {
-        const long long r = e / rc2;
-        const int c = (int)(e - r * rc2);
-        const bool isV = c >= ga.row_chunks;
-        const int chunk = isV ? c - ga.row_chunks : c;
-        const long long j = j0 + r;
-        const uint4* src = reinterpret_cast<const uint4*>((isV ? Vh + j * ga.vsn * ga.esize : Kh + j * ga.ksn * ga.esize)) + chunk;
-        uint4* out = reinterpret_cast<uint4*>((isV ? ga.V_out : ga.K_out) + ((long long)row * out_stride + j) * ga.row_chunks * 16) + chunk;
-        *out = __ldg(src);
-      }
-    }
-    return;
+  csync();
+  ptx::grid_dependency_wait();
+  const int n = a.n, n_kv = a.n_kv;
+  const int rank = CS > 1 ? part : 0;
+  const long long j0 = (long long)rank * a.per;
+  const int cnt = (int)max(0ll, min((long long)n_kv, j0 + a.per) - j0);
+  float* srow = a.scores + (long long)row * n_kv + j0;
+  int32_t* dst = a.index_sums ? nullptr : a.indices + (long long)row * a.keep;
+  int keep = a.keep;
+  if (a.keep_rows) {
+    keep = min(max(a.keep_rows[row], 1), a.keep);
+    if (part == 0)
+      for (int pos = keep + tid; pos < a.keep; pos += kThreads) dst[pos] = -1;
   }
+  // this warp's run of the slice
+  const int cw = (((a.per + kWarps - 1) / kWarps) + 31) & ~31;
+  const int wbeg = min(cnt, wid * cw), wlen = min(cnt, wbeg + cw) - wbeg;
+  auto key_at = [&](int i) { return a.held ? skeys[wbeg + i] : float_key(srow[wbeg + i]); };   // i: position in the run
 
-  // ---- smallest and largest key of the row ----
+  // ---- keys of the slice, their smallest and largest finite one ----
   unsigned int kmin = 0xFFFFFFFFu, kmax = 0u;
-  for (int jj = tid; jj < cnt; jj += kSelThreads) {
-    const unsigned int key = key_at(jj);
+  auto take = [&](int jj, float score) {
+    const unsigned int key = float_key(score);
     kmin = min(kmin, key);
-    kmax = max(kmax, key);
+    kmax = max(kmax, key < kInfKey ? key : 0u);
+    if (a.held) skeys[jj] = key;
+  };
+  if (a.I_hat) {
+    int W = a.W, gamma = a.gamma;
+    if (a.pool) { W = a.pool[2 * row]; gamma = a.pool[2 * row + 1]; }
+    const float* src = a.I_hat + (long long)row * n;
+    // blocks that all select from the whole row write a share of its pooled scores each
+    const int w_per = CS > 1 ? cnt : (cnt + a.parts - 1) / a.parts, w0 = CS > 1 ? 0 : part * w_per, w1 = min(cnt, w0 + w_per);
+    auto put = [&](int jj, float score) {
+      if (!a.held || (jj >= w0 && jj < w1)) srow[jj] = score;
+      take(jj, score);
+    };
+    if (cnt > 0 && (long long)cnt + W + 6 <= a.room) {
+      // The slice's taps, zeros outside the scored rows: every row then takes the same W taps without a bounds check
+      // (adding 0 changes nothing), in the order of box_mean.  One bulk copy brings them in, from the 16-byte boundary
+      // before the first one to the boundary behind the last one (both inside the workspace that I_hat lies in).
+      const long long lo = j0 - W / 2 + gamma, hi = lo + cnt + W - 1;   // taps [lo, hi)
+      const long long g0 = lo < 0 ? 0 : (lo < n ? lo : n), g1 = hi > n ? n : (hi > 0 ? hi : 0);
+      const int mis = (int)((reinterpret_cast<uintptr_t>(src + g0) >> 2) & 3);   // floats between the boundary and tap g0
+      const int shift = 4 - (int)((g0 - lo + 4 - mis) & 3);                      // so that the boundary is one in here, too
+      float* const taps = room + (shift & 3);                                    // taps[t - lo]
+      if (g1 > g0) {
+        if (tid == 0) {
+          const uint32_t bytes = (uint32_t)(((g1 - g0 + mis) * 4 + 15) & ~15ll);
+          ptx::mbar_arrive_expect_tx(&tap_bar, bytes);
+          ptx::bulk_load(taps + (g0 - lo) - mis, src + g0 - mis, bytes, &tap_bar);
+        }
+        wait_copy(&tap_bar, 0u, a.dev_status);
+      }
+      __syncthreads();   // the copy's edges may hold neighbours: overwritten only once it has landed
+      for (long long t = lo + tid; t < g0 && t < hi; t += kThreads) taps[t - lo] = 0.f;
+      for (long long t = (g1 > lo ? g1 : lo) + tid; t < hi; t += kThreads) taps[t - lo] = 0.f;
+      __syncthreads();
+      const int scored = (int)max(0ll, min((long long)cnt, n - j0));   // rows of the slice before the window's own
+      if (W == 7 && !a.pool_max) pool_slice<kThreads, 7>(taps, W, false, scored, cnt, put);
+      else if (W == 5 && !a.pool_max) pool_slice<kThreads, 5>(taps, W, false, scored, cnt, put);
+      else pool_slice<kThreads, 0>(taps, W, a.pool_max != 0, scored, cnt, put);
+    } else {
+      for (int jj = tid; jj < cnt; jj += kThreads) put(jj, box_mean(src, n, (int)(j0 + jj), W, gamma, a.pool_max != 0));
+    }
+  } else {
+    for (int t0 = tid; t0 < cnt; t0 += 8 * kThreads) {   // several loads in flight per thread
+      float v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = t0 + k * kThreads < cnt ? __ldcg(srow + t0 + k * kThreads) : 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (t0 + k * kThreads < cnt) take(t0 + k * kThreads, v[k]);
+    }
   }
   kmin = __reduce_min_sync(0xffffffffu, kmin);
   kmax = __reduce_max_sync(0xffffffffu, kmax);
-  if (lane == 0) { warp_a[wid] = kmin; warp_b[wid] = kmax; }
-  __syncthreads();
-  if (wid == 0) {
-    kmin = __reduce_min_sync(0xffffffffu, warp_a[lane]);
-    kmax = __reduce_max_sync(0xffffffffu, warp_b[lane]);
-    if (lane == 0) { cta_minmax[0] = kmin; cta_minmax[1] = kmax; }
-  }
-  cluster.sync();
-  kmin = 0xFFFFFFFFu;
-  kmax = 0u;
-  for (unsigned int r = 0; r < CS; ++r) {
-    const unsigned int* mm = cluster.map_shared_rank(cta_minmax, r);
-    kmin = min(kmin, mm[0]);
-    kmax = max(kmax, mm[1]);
-  }
-
-  // ---- radix passes over the bits in which the keys differ ----
-  const unsigned int diff = kmin ^ kmax;
-  int hi = diff ? 32 - __clz(diff) : 0;                                  // bits [hi-1 .. 0] vary
-  unsigned int prefix = hi >= 32 ? 0u : (kmax >> hi) << hi;              // the bits every key shares
-  unsigned int remaining = (unsigned int)keep;
-  int pb = 0;
-#pragma unroll 1
-  while (hi > 0) {
-    const int lo = hi > 8 ? hi - 8 : 0;
-    const unsigned int dmask = (1u << (hi - lo)) - 1u;
-    for (int b = tid; b < 32 * kSelBins; b += kSelThreads) (&wh[0][0])[b] = 0;
-    __syncthreads();
-    for (int jj = tid; jj < cnt; jj += kSelThreads) {
-      const unsigned int key = key_at(jj);
-      if (hi >= 32 || ((key ^ prefix) >> hi) == 0) atomicAdd(&wh[wid][(key >> lo) & dmask], 1u);
-    }
-    __syncthreads();
-    if (tid < kSelBins) {
-      unsigned int h = 0;
-#pragma unroll 8
-      for (int wv = 0; wv < 32; ++wv) h += wh[wv][tid];
-      hist[pb][tid] = h;
-    }
-    cluster.sync();
-    if (tid < kSelBins) {
-      unsigned int h = 0;
-      for (unsigned int r = 0; r < CS; ++r) h += cluster.map_shared_rank(&hist[pb][0], r)[tid];
-      tot[tid] = h;
-    }
+  if (CS > 1) {   // one message to each CTA instead of one from every warp
+    if (lane == 0) { warp_a[wid] = kmin; warp_b[wid] = kmax; }
     __syncthreads();
     if (wid == 0) {
-      // lane L owns bins 255-8L .. 248-8L, so that the lanes walk the bins from the top
-      unsigned int mine[8], sum = 0;
+      kmin = __reduce_min_sync(0xffffffffu, lane < kWarps ? warp_a[lane] : 0xFFFFFFFFu);
+      kmax = __reduce_max_sync(0xffffffffu, lane < kWarps ? warp_b[lane] : 0u);
+    }
+  }
+  if ((CS == 1 || wid == 0) && lane < CS) {
+    atomicMin(in_cta(&s_min, lane), kmin);
+    atomicMax(in_cta(&s_max, lane), kmax);
+  }
+  csync();
+  kmin = s_min;
+  const unsigned int range = s_max >= kmin ? s_max - kmin + 1u : 0u;   // offset of +inf
+  auto offset_of = [&](unsigned int key) { return min(key - kmin, range); };
+
+  // ---- digits from the top ----
+  unsigned int above = kmin, equal = 0u, need_eq = 0u;   // kept: key >= above, and the first need_eq with key == equal
+  if (keep < n_kv) {
+    int hi = 32 - __clz((int)range);        // bits [hi - 1 .. 0] vary
+    unsigned int prefix = 0u, remaining = (unsigned int)keep;
+    int pb = 0;
+    bool whole = false;
+#pragma unroll 1
+    while (hi > 0 && !whole) {
+      const int lo = hi > 11 ? hi - 11 : 0;
+      const unsigned int want = hi >= 32 ? 0u : prefix >> hi, mask = (1u << (hi - lo)) - 1u;
+#pragma unroll 4
+      for (int i = lane; i < wlen; i += 32) {
+        const unsigned int v = offset_of(key_at(i));
+        if (hi >= 32 || (v >> hi) == want) atomicAdd(&hist[pb][(v >> lo) & mask], 1u);
+      }
+      csync();
+      const unsigned int* total = hist[pb];
+      if (CS > 1) {
+        // every CTA adds up its share of the bins over the cluster and hands the sums to all (each CTA reading all bins of
+        // all peers took twice as long)
+        const int bins = kSelBins / CS;
+        for (int b0 = tid; b0 < bins; b0 += kThreads) {
+          const int b = rank * bins + b0;
+          unsigned int v[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) { mine[k] = tot[kSelBins - 1 - 8 * lane - k]; sum += mine[k]; }
+          for (int r = 0; r < 8; ++r) v[r] = r < CS ? *cluster.map_shared_rank(&hist[pb][b], r) : 0u;
+          const unsigned int sum8 = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+#pragma unroll
+          for (int r = 0; r < 8; ++r)
+            if (r < CS) *cluster.map_shared_rank(&tot[b], r) = sum8;
+        }
+        cluster.sync();
+        total = tot;
+      }
+      // this thread's kBpt bins, walked from the top
+      unsigned int own[kBpt], sum = 0u;
+      const int first = kSelBins - kBpt * (tid + 1);
+#pragma unroll
+      for (int i = 0; i < kBpt; ++i) {
+        own[i] = total[first + i];
+        sum += own[i];
+      }
       unsigned int incl = sum;
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
         const unsigned int t = __shfl_up_sync(0xffffffffu, incl, off);
         if (lane >= off) incl += t;
       }
-      unsigned int acc = incl - sum;
-      if (acc < remaining && remaining <= incl) {   // exactly one lane
+      if (lane == 31) warp_a[wid] = incl;
+      // nobody reads the other buffer any more (its readers have passed the synchronisation above): ready it
+      for (int b = tid; b < kSelBins; b += kThreads) hist[pb ^ 1][b] = 0u;
+      __syncthreads();
+      unsigned int acc = __reduce_add_sync(0xffffffffu, lane < wid ? warp_a[lane] : 0u) + incl - sum;
+      if (acc < remaining && remaining <= acc + sum) {   // exactly one thread
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          if (acc < remaining && remaining <= acc + mine[k]) {
-            s_digit = (unsigned int)(kSelBins - 1 - 8 * lane - k);
+        for (int i = kBpt - 1; i >= 0; --i) {
+          if (acc < remaining && remaining <= acc + own[i]) {
+            s_digit = (unsigned int)(first + i);
             s_remaining = remaining - acc;
+            s_count = own[i];
           }
-          acc += mine[k];
+          acc += own[i];
         }
       }
+      __syncthreads();
+      prefix |= s_digit << lo;
+      remaining = s_remaining;
+      whole = s_count == remaining;   // the rest of the bin is kept as a whole
+      hi = lo;
+      pb ^= 1;
     }
-    __syncthreads();
-    prefix |= s_digit << lo;
-    remaining = s_remaining;
-    hi = lo;
-    pb ^= 1;
-    // hist[pb] is rewritten two passes later, after another cluster.sync that every peer reaches only once it
-    // has finished reading this pass's histograms
+    // offsets back to keys; the offset of +inf stands for no other key
+    if (whole) {
+      above = prefix >= range ? kInfKey : kmin + prefix;
+    } else {
+      equal = prefix >= range ? kInfKey : kmin + prefix;
+      above = prefix >= range ? 0xFFFFFFFFu : prefix + 1u >= range ? kInfKey : equal + 1u;
+      need_eq = remaining;
+    }
+    if (range == 0u) { equal = kmin; above = 0xFFFFFFFFu; need_eq = remaining; }   // all keys alike
   }
-  const unsigned int T = prefix;            // key of the keep-th largest score
-  const unsigned int need_eq = remaining;   // how many keys equal to T are kept (>= 1)
 
-  // ---- ordered emit: warp `wid` owns a contiguous run of the slice ----
-  const int cw = (((cnt + 31) / 32) + 31) & ~31;
-  const int wbeg = min(cnt, wid * cw), wend = min(cnt, wbeg + cw);
-  const unsigned int lt_mask = (1u << lane) - 1u;
-  unsigned int cgt = 0, ceq = 0;
-  for (int base = wbeg; base < wend; base += 32) {
-    const int jj = base + lane;
-    const bool valid = jj < wend;
-    const unsigned int key = valid ? key_at(jj) : 0u;
-    cgt += __popc(__ballot_sync(0xffffffffu, valid && key > T));
-    ceq += __popc(__ballot_sync(0xffffffffu, valid && key == T));
+  // ---- ordered emit: ascending indices, of equal keys the lower index ----
+  unsigned int cgt = 0u, ceq = 0u;
+#pragma unroll 4
+  for (int i = lane; i < wlen; i += 32) {
+    const unsigned int v = key_at(i);
+    cgt += v >= above;
+    ceq += v == equal;
   }
+  cgt = __reduce_add_sync(0xffffffffu, cgt);
+  ceq = __reduce_add_sync(0xffffffffu, ceq);
   if (lane == 0) { warp_a[wid] = cgt; warp_b[wid] = ceq; }
   __syncthreads();
-  if (wid == 0) {
-    unsigned int a = warp_a[lane], b = warp_b[lane];
-    const unsigned int a_own = a, b_own = b;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const unsigned int ta = __shfl_up_sync(0xffffffffu, a, off), tb = __shfl_up_sync(0xffffffffu, b, off);
-      if (lane >= off) { a += ta; b += tb; }
+  if (CS > 1) {
+    if (wid == 0) {
+      cgt = __reduce_add_sync(0xffffffffu, lane < kWarps ? warp_a[lane] : 0u);
+      ceq = __reduce_add_sync(0xffffffffu, lane < kWarps ? warp_b[lane] : 0u);
+      if (lane > rank && lane < CS) {
+        atomicAdd(in_cta(&s_gt, lane), cgt);
+        atomicAdd(in_cta(&s_eq, lane), ceq);
+      }
     }
-    warp_a[lane] = a - a_own;   // exclusive over the warps
-    warp_b[lane] = b - b_own;
-    if (lane == 31) { cta_counts[0] = a; cta_counts[1] = b; }
+    cluster.sync();
   }
-  __syncthreads();
-  cluster.sync();
-  unsigned int g_before = 0, e_before = 0;   // totals of the lower ranks of the cluster
-  for (unsigned int r = 0; r < rank; ++r) {
-    const unsigned int* rc = cluster.map_shared_rank(cta_counts, r);
-    g_before += rc[0];
-    e_before += rc[1];
-  }
-  unsigned int run_gt = warp_a[wid] + g_before, run_eq = warp_b[wid] + e_before;
-  for (int base = wbeg; base < wend; base += 32) {
-    const int jj = base + lane;
-    const bool valid = jj < wend;
-    const unsigned int key = valid ? key_at(jj) : 0u;
-    const bool gt = valid && key > T, eq = valid && key == T;
+  unsigned int run_gt = s_gt + __reduce_add_sync(0xffffffffu, lane < wid ? warp_a[lane] : 0u);
+  unsigned int run_eq = s_eq + __reduce_add_sync(0xffffffffu, lane < wid ? warp_b[lane] : 0u);
+  // every block copies an equal share of the rows; the positions of a share go to its block (the taps are used up)
+  const unsigned int share = ((unsigned int)keep + a.parts - 1) / a.parts;
+  const unsigned int first = min((unsigned int)keep, (unsigned int)part * share), last = min((unsigned int)keep, first + share);
+  const bool own_idx = a.own_idx != 0;
+  int32_t* const s_idx = reinterpret_cast<int32_t*>(room);
+  const unsigned int lt_mask = (1u << lane) - 1u;
+  unsigned long long isum = 0ull;
+#pragma unroll 2
+  for (int i0 = 0; i0 < wlen; i0 += 32) {
+    const int i = i0 + lane;
+    const unsigned int v = i < wlen ? key_at(i) : 0u;
+    const bool gt = i < wlen && v >= above, eq = i < wlen && v == equal;
     const unsigned int mgt = __ballot_sync(0xffffffffu, gt), meq = __ballot_sync(0xffffffffu, eq);
-    const unsigned int gt_before = run_gt + __popc(mgt & lt_mask);
-    const unsigned int eq_before = run_eq + __popc(meq & lt_mask);
-    if (gt || (eq && eq_before < need_eq)) {
-      const unsigned int pos = gt_before + min(eq_before, need_eq);
-      if (pos < (unsigned int)keep) dst[pos] = (int32_t)(j0 + jj);
-    }
-    run_gt += __popc(mgt);
-    run_eq += __popc(meq);
-  }
-  if (ga.K) {
-    // ---- gather: every CTA of the cluster takes an equal share of the row's `keep` indices, whoever emitted them
-    //      (the selected rows may all lie in one CTA's slice) ----
-    cluster.sync();   // all indices of the row are written and visible to the cluster
-    const unsigned int share = ((unsigned int)keep + CS - 1) / CS;
-    const unsigned int first = min((unsigned int)keep, rank * share);
-    const unsigned int mine = min((unsigned int)keep, first + share) - first;
-    const int b = row / ga.Hkv, h = row % ga.Hkv;
-    const unsigned char* Kh = ga.K + ((long long)b * ga.ksb + (long long)h * ga.ksh) * ga.esize;
-    const unsigned char* Vh = ga.V + ((long long)b * ga.vsb + (long long)h * ga.vsh) * ga.esize;
-    const long long out_row0 = (long long)row * out_stride;
-    const int rc2 = 2 * ga.row_chunks;
-    // four chunks per thread and round, the index loads first and then the row loads, so that they overlap
-    const unsigned int total = mine * (unsigned int)rc2;
-    for (unsigned int e0 = tid; e0 < total; e0 += 4 * kSelThreads) {
-      long long jj[4];
-      uint4 val[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const unsigned int e = e0 + k * kSelThreads;
-        jj[k] = e < total ? dst[first + e / rc2] : 0;
+    if (mgt | meq) {
+      const unsigned int gt_before = run_gt + __popc(mgt & lt_mask), eq_before = run_eq + __popc(meq & lt_mask);
+      if (gt || (eq && eq_before < need_eq)) {
+        const unsigned int pos = gt_before + min(eq_before, need_eq);
+        const int j = (int)j0 + wbeg + i;
+        if (a.index_sums) isum += (unsigned long long)j;
+        else if (!own_idx) {
+          if (pos < (unsigned int)keep && (CS > 1 || (pos >= first && pos < last))) dst[pos] = j;
+        } else if (CS == 1) {
+          if (pos >= first && pos < last) s_idx[pos - first] = j;
+        } else {
+          const unsigned int to = pos / share;
+          *cluster.map_shared_rank(s_idx + (pos - to * share), to) = j;
+        }
       }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const unsigned int e = e0 + k * kSelThreads;
-        const int c = (int)(e % rc2);
-        const bool isV = c >= ga.row_chunks;
-        const int chunk = isV ? c - ga.row_chunks : c;
-        const uint4* src = reinterpret_cast<const uint4*>((isV ? Vh + jj[k] * ga.vsn * ga.esize : Kh + jj[k] * ga.ksn * ga.esize)) + chunk;
-        if (e < total) val[k] = __ldg(src);
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const unsigned int e = e0 + k * kSelThreads;
-        if (e >= total) continue;
-        const unsigned int r = e / rc2;
-        const int c = (int)(e - r * rc2);
-        const bool isV = c >= ga.row_chunks;
-        const int chunk = isV ? c - ga.row_chunks : c;
-        uint4* out = reinterpret_cast<uint4*>((isV ? ga.V_out : ga.K_out) + (out_row0 + first + r) * ga.row_chunks * 16) + chunk;
-        *out = val[k];
-      }
+      run_gt += __popc(mgt);
+      run_eq += __popc(meq);
     }
   }
-  cluster.sync();   // shared memory stays alive until every peer has read cta_counts
+  if (a.index_sums) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) isum += __shfl_xor_sync(0xffffffffu, isum, off);
+    unsigned long long* sums = reinterpret_cast<unsigned long long*>(&hist[0][0]);   // its readers are done with it
+    if (lane == 0) sums[wid] = isum;
+    __syncthreads();
+    if (tid == 0) {
+      for (int w = 1; w < kWarps; ++w) isum += sums[w];
+      a.index_sums[(long long)row * a.parts + part] = isum;
+    }
+  }
+  if (!a.ga.K) {
+    if (CS > 1) cluster.sync();   // shared memory stays alive until every peer has done with it
+    return;
+  }
+  ptx::fence_proxy_async_smem();   // rows are about to land where keys and taps were
+  csync();   // all positions of this block's share have arrived
+
+  // ---- gather: every warp copies batches of copy_rows rows through its own two buffers, row by row in and as one piece
+  //      out, by bulk copies (with loads and stores the same work took twice as long: 14 k cycles for 256 rows a CTA) ----
+  const int rows = (int)(last - first);
+  if (own_idx)
+    for (int i = tid; i < rows; i += kThreads) dst[first + i] = s_idx[i];
+  const int b = row / a.ga.Hkv, h = row % a.ga.Hkv, es = a.ga.esize, rb = a.ga.row_chunks * 16, R = a.copy_rows;
+  const unsigned char* Kh = a.ga.K + ((long long)b * a.ga.ksb + (long long)h * a.ga.ksh) * es;
+  const unsigned char* Vh = a.ga.V + ((long long)b * a.ga.vsb + (long long)h * a.ga.vsh) * es;
+  const long long out0 = (long long)row * a.keep + first;
+  uint8_t* const stage = reinterpret_cast<uint8_t*>(s_idx) + (own_idx ? ((int)share * 4 + 15) & ~15 : 0) + wid * 4 * R * rb;
+  const int batches = (rows + R - 1) / R, mine = batches > wid ? (batches - wid + kWarps - 1) / kWarps : 0;
+  auto rows_of = [&](int it) { return min(R, rows - (wid + it * kWarps) * R); };
+  for (int it = 0; it <= mine; ++it) {
+    if (it < mine) {
+      const int r0 = (wid + it * kWarps) * R, cr = rows_of(it);
+      uint8_t* buf = stage + (it & 1) * 2 * R * rb;
+      if (lane == 0) {
+        if (it >= 2) ptx::bulk_store_wait_read<0>();   // the buffer's last batch has left
+        ptx::mbar_arrive_expect_tx(&copy_bar[wid][it & 1], (uint32_t)(2 * cr * rb));
+      }
+      __syncwarp();
+      if (lane < 2 * cr) {
+        const bool isV = lane >= cr;
+        const int r = isV ? lane - cr : lane;
+        const long long j = own_idx ? s_idx[r0 + r] : dst[first + r0 + r];
+        const unsigned char* src = isV ? Vh + j * a.ga.vsn * es : Kh + j * a.ga.ksn * es;
+        ptx::bulk_load(buf + (isV ? R * rb : 0) + r * rb, src, (uint32_t)rb, &copy_bar[wid][it & 1]);
+      }
+    }
+    if (it > 0 && lane == 0) {
+      const int p = it - 1, cr = rows_of(p);
+      const long long at = (out0 + (long long)(wid + p * kWarps) * R) * rb;
+      uint8_t* buf = stage + (p & 1) * 2 * R * rb;
+      wait_copy(&copy_bar[wid][p & 1], (uint32_t)(p >> 1) & 1u, a.dev_status);
+      ptx::bulk_store(a.ga.K_out + at, ptx::smem_u32(buf), (uint32_t)(cr * rb));
+      ptx::bulk_store(a.ga.V_out + at, ptx::smem_u32(buf + R * rb), (uint32_t)(cr * rb));
+      ptx::bulk_store_commit();
+    }
+  }
+  if (lane == 0) ptx::bulk_store_wait();
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -453,51 +489,112 @@ cudaError_t launch_pool(const Problem& p, const Workspace& ws, const int* pool_d
   return cudaGetLastError();
 }
 
-// rows x n_kv scores -> rows x min(budget, n_kv) indices.  I_hat non-null: pool first (n scored rows per row of
-// I_hat, window from pool_dev or (W, gamma)) and write the pooled scores.
-cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep_rows, const float* I_hat, const int* pool_dev, int W,
-                          int gamma, bool pool_max, float* scores, int32_t* indices, int32_t* pool_used, const Problem* gather,
-                          const void* K, const void* V, void* K_out, void* V_out, cudaStream_t st) {
-  GatherArgs ga{};
+namespace {
+
+using SelectKernel = void (*)(const SelectArgs);
+constexpr size_t kSelMaxSmem = 200 * 1024;
+
+}  // namespace
+
+// clusters_of: how many clusters of 1, 2, 4 and 8 CTAs of the large kind the device holds at once.
+cudaError_t select_init(int* clusters_of) {
+  cudaError_t e = cudaSuccess;
+  for (SelectKernel kernel : {select_kernel<512>, select_kernel<1024>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelMaxSmem);
+  for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(8);
+    cfg.blockDim = dim3(1024);
+    cfg.dynamicSmemBytes = 64 * 1024;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1u << i;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaOccupancyMaxActiveClusters(&clusters_of[i], select_kernel<1024>, &cfg);
+  }
+  return e;
+}
+
+// CTAs of a row's cluster: as many as let all rows run at once (8 at most: smaller slices no longer shorten the chain of
+// synchronisations); more rows than SMs: as few as let three blocks of 512 threads share an SM's memory, so that one row's
+// loads run under another's passes.  1: no cluster.
+int select_cluster(int rows, int n_kv, const int* clusters_of) {
+  int i = 3;
+  while (i > 0 && (rows > clusters_of[i] || (n_kv >> i) < 256)) --i;
+  if (rows > clusters_of[0])
+    while (i < 3 && (n_kv >> i) > 13000) ++i;
+  return 1 << i;
+}
+
+// Rows up to this length are selected from by every block of the row for itself when the blocks only share the gather: a
+// block of 1024 threads forms 8 keys per thread in about the time that the cluster's four barriers take.
+constexpr int kSelLocalRows = 8192;
+
+// rows x n_kv scores -> rows x min(budget, n_kv) indices (or, with index_sums, the sums of those indices: one value per
+// CTA of the row's cluster, select_cluster of them).  I_hat non-null: pool first (n scored rows per row of I_hat, window
+// from pool_dev or (W, gamma)) and write the pooled scores.  chained: the launch may overlap the end of the kernel
+// before it in the stream (it waits for that kernel's results itself).
+cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep_rows, const float* I_hat, const int* pool_dev,
+                          int W, int gamma, bool pool_max, float* scores, int32_t* indices, unsigned long long* index_sums,
+                          const Problem* gather, const void* K, const void* V, void* K_out, void* V_out,
+                          const int* clusters_of, unsigned int* dev_status, bool chained, cudaStream_t st) {
+  SelectArgs a{};
+  a.dev_status = dev_status;
   if (gather) {
-    ga.K = (const unsigned char*)K; ga.V = (const unsigned char*)V;
-    ga.K_out = (unsigned char*)K_out; ga.V_out = (unsigned char*)V_out;
-    ga.ksb = gather->ksb; ga.ksh = gather->ksh; ga.ksn = gather->ksn;
-    ga.vsb = gather->vsb; ga.vsh = gather->vsh; ga.vsn = gather->vsn;
-    ga.Hkv = gather->Hkv; ga.esize = gather->dtype == RESTKV_BF16 ? 2 : 4; ga.row_chunks = gather->d * ga.esize / 16;
+    a.ga.K = (const unsigned char*)K; a.ga.V = (const unsigned char*)V;
+    a.ga.K_out = (unsigned char*)K_out; a.ga.V_out = (unsigned char*)V_out;
+    a.ga.ksb = gather->ksb; a.ga.ksh = gather->ksh; a.ga.ksn = gather->ksn;
+    a.ga.vsb = gather->vsb; a.ga.vsh = gather->vsh; a.ga.vsn = gather->vsn;
+    a.ga.Hkv = gather->Hkv; a.ga.esize = gather->dtype == RESTKV_BF16 ? 2 : 4; a.ga.row_chunks = gather->d * a.ga.esize / 16;
   }
-  const int keep = budget < n_kv ? budget : n_kv;
-  // CTAs per row: 8 for long rows, fewer when there are so many rows that all clusters would not be resident at
-  // once (two 1024-thread CTAs per SM) and the slices still fit in shared memory
-  int CS = n_kv > 4096 ? 8 : 1;
-  int sms = 148;
-  {
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  a.n = n; a.n_kv = n_kv; a.keep = budget < n_kv ? budget : n_kv; a.keep_rows = keep_rows;
+  a.I_hat = I_hat; a.pool = pool_dev; a.W = W; a.gamma = gamma; a.pool_max = pool_max ? 1 : 0;
+  a.scores = scores; a.indices = indices; a.index_sums = index_sums;
+  int CS = select_cluster(rows, n_kv, clusters_of);
+  a.parts = CS;
+  if (I_hat && gather && n_kv <= kSelLocalRows && rows <= clusters_of[0]) {
+    CS = 1;
+    a.parts = clusters_of[0] / rows;
+    if (a.parts > (a.keep + 31) / 32) a.parts = (a.keep + 31) / 32;   // at least a row per warp to copy
   }
-  while (CS > 1 && (long long)rows * CS > 2ll * sms && (n_kv + CS / 2 - 1) / (CS / 2) <= kSelMaxSmemKeys / 2) CS >>= 1;
-  cudaError_t e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kSelMaxSmemKeys * (int)sizeof(unsigned int));
-  if (e != cudaSuccess) return e;
-  int per = (n_kv + CS - 1) / CS;
-  per = (per + 3) & ~3;
-  const int use_smem = per <= kSelMaxSmemKeys ? 1 : 0;
+  a.per = (n_kv + CS - 1) / CS;
+  const bool small_blocks = rows > clusters_of[0];
+  const int threads = small_blocks ? 512 : 1024;
+  // the taps of a slice (with some margin for a window known on the device only), later the indices the block gathers
+  const long long cap = kSelMaxSmem / 4, per4 = (a.per + 3) & ~3;
+  long long room = I_hat ? (long long)a.per + 7 + (pool_dev ? 256 : W) : 0;
+  long long need = I_hat ? a.per / 2 : 0;   // held keys leave at least this (longer windows then read their taps from memory)
+  if (gather) {   // the indices, and behind them two buffers of copy_rows rows of K and V for every warp
+    const long long buf = (long long)(threads / 32) * a.ga.row_chunks * 16, idx = (((a.keep + a.parts - 1) / a.parts) + 3) & ~3;
+    a.held = per4 + (need > buf ? need : buf) <= cap ? 1 : 0;
+    const long long most = cap - (a.held ? per4 : 0);
+    a.own_idx = idx + buf <= most ? 1 : 0;
+    a.copy_rows = 4;
+    while (a.copy_rows > 1 && (a.own_idx ? idx : 0) + a.copy_rows * buf > most) a.copy_rows >>= 1;
+    const long long copies = (a.own_idx ? idx : 0) + a.copy_rows * buf;
+    if (room < copies) room = copies;
+  } else {
+    a.held = per4 + need <= cap ? 1 : 0;
+  }
+  const long long most = cap - (a.held ? per4 : 0);
+  a.room = (int)(room < most ? room : most);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned int)(rows * CS));
-  cfg.blockDim = dim3(kSelThreads);
-  // with room for it, the pooling taps of the slice (slice + halo) are staged behind the keys
-  const int stage_taps = (I_hat && use_smem && 2 * per + kSelMaxStagedWidth <= kSelMaxSmemKeys) ? 1 : 0;
-  cfg.dynamicSmemBytes = use_smem ? (size_t)(stage_taps ? 2 * per + kSelMaxStagedWidth : per) * sizeof(unsigned int) : 0;
+  cfg.gridDim = dim3((unsigned int)(rows * a.parts));
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = (size_t)(a.room + (a.held ? (a.per + 3) & ~3 : 0)) * sizeof(float);
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = CS;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, select_kernel, n, n_kv, keep, keep_rows, I_hat, pool_dev, W, gamma, pool_max ? 1 : 0, scores, indices,
-                            pool_used, per, use_smem, stage_taps, ga);
+  cfg.numAttrs = chained ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, small_blocks ? select_kernel<512> : select_kernel<1024>, a);
 }
 
 cudaError_t launch_compact(const Problem& p, const void* K, const void* V, const int32_t* indices, int n_sel,

@@ -9,13 +9,14 @@
 struct restkv_handle {
   int device;
   int sm_count;
-  unsigned int* dev_status;   // 256-byte device block, word 0 = sticky status bits
+  unsigned int* dev_status;   // device block: kDevStatusWords (word 0 = sticky status bits), then kDevCounterWords
   void* tc_state;
+  int select_clusters[4];     // clusters of 1, 2, 4, 8 CTAs of the select kernel that the device holds at once
   int decode_clusters[5];     // clusters of 1, 2, 4, 8, 16 CTAs of the decode kernel that the device holds at once
   long long launches;
   int last_cuda_error;
   int kernel_path;            // 0 auto, 1 SIMT, 2 tensor core required, 3 tensor core in its head-sequential form
-  bool fused_select;          // restkv_evict lets the tensor-core score kernel pool, select and gather when it can
+  bool fused_select;          // restkv_evict chains the launch that pools, selects and gathers to the score kernel
   bool last_evict_fused;      // whether the last restkv_evict did
   long long wait_limit;       // SM clocks a device-side wait may last
   restkv_variant variant;     // ablation variant of the score calls (all 0: the method as printed)
@@ -63,11 +64,8 @@ size_t plan_workspace(const Problem& p, int budget, int sm_count, bool adaptive,
   w.part_m = (float*)take(slots * R * sizeof(float));
   w.part_l = (float*)take(slots * R * sizeof(float));
   w.part_O = (float*)take(slots * R * d * sizeof(float));
-  w.counters = (unsigned int*)take(1024);
   w.tile_max = (float*)take(BH * (size_t)((p.n_kv + 127) / 128) * 128 * sizeof(float));
   w.row_M2 = (float*)take(BH * 128 * sizeof(float));
-  w.sel_hist = (unsigned int*)take(tc_fused_select_hist_words(p.BH) * sizeof(unsigned int));
-  w.sel_sfx = (unsigned int*)take(tc_fused_select_sfx_words(sm_count) * sizeof(unsigned int));
   w.q_pad = (__nv_bfloat16*)take(BH * 128 * 128 * sizeof(__nv_bfloat16));
   w.vnorm = (float*)take(BH * (size_t)p.n_kv * sizeof(float));
   w.fin_m = (float*)take(BH * R * sizeof(float));
@@ -82,12 +80,8 @@ size_t plan_workspace(const Problem& p, int budget, int sm_count, bool adaptive,
   w.pool = (int*)take(BH * 2 * sizeof(int));
   w.dec_part = (float*)take(BH * (size_t)kDecodeMaxSplits * p.G * (d + 2) * sizeof(float));
   if (adaptive) {
-    int Bp = budget - p.tail;
-    if (Bp > p.n) Bp = p.n;
-    if (Bp < 1) Bp = 1;
     w.I_raw = (float*)take((size_t)p.batch * p.Hq * p.w * p.n * sizeof(float));
-    w.adaptive_idx = (int32_t*)take((size_t)p.batch * p.Hq * p.w * Bp * sizeof(int32_t));
-    w.adaptive_sums = (unsigned long long*)take(BH * 2 * sizeof(unsigned long long));
+    w.adaptive_sums = (unsigned long long*)take((size_t)p.batch * p.Hq * p.w * 8 * sizeof(unsigned long long));
   }
   w.bytes = off;
   if (ws) *ws = w;
@@ -107,7 +101,6 @@ static size_t plan_decode_tc(int BH, int sm_count, void* base, Workspace* ws) {
   w.part_m = (float*)take(slots * 128 * sizeof(float));
   w.part_l = (float*)take(slots * 128 * sizeof(float));
   w.part_O = (float*)take(slots * 128 * 128 * sizeof(float));
-  w.counters = (unsigned int*)take(1024);
   w.row_M2 = (float*)take(bh * 128 * sizeof(float));
   w.q_pad = (__nv_bfloat16*)take(bh * 128 * 128 * sizeof(__nv_bfloat16));
   w.O_f32 = (float*)take(bh * 128 * 128 * sizeof(float));
@@ -211,8 +204,8 @@ struct Call {
 // null the caller pools (the fused path does it inside the select kernel).
 static restkv_status run_score(Call& c, const Problem& p, const Workspace& ws, const void* Q, const void* K,
                                const void* V, float ema_decay, const restkv_pool_params* pool, float* scores,
-                               int32_t* pool_used, const FusedSelect* sel = nullptr, bool* sel_done = nullptr,
-                               const float* O_given = nullptr, const float* LSE_given = nullptr) {
+                               int32_t* pool_used, const float* O_given = nullptr, const float* LSE_given = nullptr,
+                               bool* on_tc = nullptr) {
   const bool adaptive = pool->mode == RESTKV_POOL_ADAPTIVE;
   // the tensor-core pass 2 carries the temporal weights as an fp32 Horner chain, which Eq. 9 with alpha = 0 and
   // some inverted EMAs do not fit: those run on the SIMT kernels
@@ -225,6 +218,7 @@ static restkv_status run_score(Call& c, const Problem& p, const Workspace& ws, c
   if (c.h->kernel_path == 1) use_tc = false;
   if (c.h->kernel_path >= 2 && !use_tc) return RESTKV_ERR_UNSUPPORTED;
   if (!use_tc && !simt_supported(p)) return RESTKV_ERR_UNSUPPORTED;
+  if (on_tc) *on_tc = use_tc;
   if (p.n_kv == 1 && p.indicator == RESTKV_INDICATOR_RECONSTRUCTION) {
     // A single visible row has A = 1 and nothing to redistribute its weight to: the indicator is
     // 0/0 there and is defined as 0 (Eq. 7 has no value), so no kernel is needed.
@@ -239,12 +233,9 @@ static restkv_status run_score(Call& c, const Problem& p, const Workspace& ws, c
       RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS1,
                     launch_tc_vmv(c.h->tc_state, p, V, ws.vmv, c.h->sm_count, c.h->wait_limit, c.h->dev_status, c.st), 1);
     if (use_tc) {
-      const bool with_sel = sel && c.h->fused_select &&
-                            tc_fused_select_supported(p, c.h->sm_count, false, sel->keep, sel->W, sel->gamma);
       RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS2,
-                    launch_tc_fused(c.h->tc_state, p, ws, Q, K, V, ema_decay, c.h->sm_count, false, false,
-                                    c.h->wait_limit, with_sel ? sel : nullptr, O_given, nullptr, c.h->dev_status, c.st), 1);
-      if (sel_done) *sel_done = with_sel;
+                    launch_tc_fused(c.h->tc_state, p, ws, Q, K, V, ema_decay, c.h->sm_count, false, false, c.h->wait_limit,
+                                    O_given, nullptr, c.h->dev_status + kDevStatusWords, c.h->dev_status, true, c.st), 1);
     } else {
       Workspace wsl = ws;
       wsl.O_f32 = const_cast<float*>(O_given);
@@ -259,13 +250,10 @@ static restkv_status run_score(Call& c, const Problem& p, const Workspace& ws, c
     if (p.proj.M)   // the tokens' own terms under the output projection, by a kernel of its own (timed as "pass 1")
       RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS1,
                     launch_tc_vmv(c.h->tc_state, p, V, ws.vmv, c.h->sm_count, c.h->wait_limit, c.h->dev_status, c.st), 1);
-    const bool with_sel = sel && c.h->fused_select &&
-                          tc_fused_select_supported(p, c.h->sm_count, reuse_l2, sel->keep, sel->W, sel->gamma);
     RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS2,
-                  launch_tc_fused(c.h->tc_state, p, ws, Q, K, V, ema_decay, c.h->sm_count, reuse_l2, false,
-                                  c.h->wait_limit, with_sel ? sel : nullptr, nullptr, adaptive ? ws.I_raw : nullptr,
-                                  c.h->dev_status, c.st), 1);
-    if (sel_done) *sel_done = with_sel;
+                  launch_tc_fused(c.h->tc_state, p, ws, Q, K, V, ema_decay, c.h->sm_count, reuse_l2, false, c.h->wait_limit,
+                                  nullptr, adaptive ? ws.I_raw : nullptr, c.h->dev_status + kDevStatusWords,
+                                  c.h->dev_status, true, c.st), 1);
   } else {
     RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS1, launch_simt_pass1(p, ws, Q, K, V, c.st), 1);
     RESTKV_LAUNCH(c, RESTKV_KERNEL_COMBINE, launch_combine(p, ws, c.st), 1);
@@ -274,7 +262,7 @@ static restkv_status run_score(Call& c, const Problem& p, const Workspace& ws, c
   }
   if (adaptive) {
     int nl = 0;
-    cudaError_t e = launch_adaptive_params(p, ws, pool->budget, pool->beta, pool->base_width, c.st, &nl);
+    cudaError_t e = launch_adaptive_params(p, ws, pool->budget, pool->beta, pool->base_width, c.h->select_clusters, c.h->dev_status, c.st, &nl);
     if (e != cudaSuccess) return c.fail(e);
     c.h->launches += nl;
   }
@@ -308,8 +296,9 @@ restkv_status restkv_create(restkv_handle** out) {
   int major = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, h->device);
   if (e == cudaSuccess && major != 10) { delete h; return RESTKV_ERR_UNSUPPORTED; }   // sm_100a only
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->dev_status, 256);
-  if (e == cudaSuccess) e = cudaMemset(h->dev_status, 0, 256);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&h->dev_status, (kDevStatusWords + kDevCounterWords) * sizeof(unsigned int));
+  if (e == cudaSuccess) e = cudaMemset(h->dev_status, 0, (kDevStatusWords + kDevCounterWords) * sizeof(unsigned int));
+  if (e == cudaSuccess) e = select_init(h->select_clusters);
   if (e != cudaSuccess) { delete h; return RESTKV_ERR_CUDA; }
   h->tc_state = nullptr;
   if (tc_init(&h->tc_state) != cudaSuccess || tc_fused_init() != cudaSuccess ||
@@ -396,7 +385,7 @@ restkv_status restkv_score_from_lse(restkv_handle* h, const restkv_shape* shape,
       RESTKV_OK)
     return s;
   Call c{h, (cudaStream_t)stream};
-  return run_score(c, p, ws, Q_obs, K, V, ema_decay, pool, scores, pool_used, nullptr, nullptr, O_obs, LSE_obs);
+  return run_score(c, p, ws, Q_obs, K, V, ema_decay, pool, scores, pool_used, O_obs, LSE_obs);
 }
 
 restkv_status restkv_select(restkv_handle* h, const restkv_shape* shape, const float* scores, int budget,
@@ -410,7 +399,7 @@ restkv_status restkv_select(restkv_handle* h, const restkv_shape* shape, const f
   Call c{h, (cudaStream_t)stream};
   RESTKV_LAUNCH(c, RESTKV_KERNEL_SELECT,
                 launch_select(p.BH, p.n, p.n_kv, budget, nullptr, nullptr, nullptr, 1, 0, false, const_cast<float*>(scores), indices, nullptr,
-                              nullptr, nullptr, nullptr, nullptr, nullptr, c.st), 1);
+                              nullptr, nullptr, nullptr, nullptr, nullptr, h->select_clusters, h->dev_status, true, c.st), 1);
   return RESTKV_OK;
 }
 
@@ -449,30 +438,16 @@ static restkv_status evict_impl(restkv_handle* h, const restkv_shape* shape, con
   if ((s = check_ws(p, ws_budget, h->sm_count, adaptive, workspace, workspace_bytes, &ws)) != RESTKV_OK) return s;
   Call c{h, (cudaStream_t)stream};
   float* scores = scores_out ? scores_out : ws.scores;
-  // With a fixed window the tensor-core score kernel pools, selects and gathers each head itself, right after the
-  // head's scores are complete and with the head's own CTAs; otherwise the kernels below do.
-  const int keep_rows = budget < p.n_kv ? budget : p.n_kv;
-  FusedSelect sel{keep_rows, pool->width, pool->shift, scores, indices, K_out, V_out};
-  bool sel_done = false;
-  if ((s = run_score(c, p, ws, Q_obs, K, V, ema_decay, pool, nullptr, nullptr, (adaptive || budgets) ? nullptr : &sel,
-                     &sel_done, O_obs, LSE_obs)) != RESTKV_OK)
-    return s;
-  h->last_evict_fused = sel_done;
-  if (sel_done) return RESTKV_OK;
-  // Pooling (Eq. 13) runs inside the select kernel, which also writes the pooled scores.  So does the gather
-  // (Eq. 14) while the select kernel's clusters fit the GPU in one wave; with more (batch, head) rows than that the
-  // stand-alone gather, which spreads over every SM, is the faster one.
-  // (with per-head budgets the index rows have unused tails, which only the select kernel's own gather skips)
-  const bool fuse_gather = p.BH * 8 <= h->sm_count || budgets != nullptr;
+  bool on_tc = false;
+  if ((s = run_score(c, p, ws, Q_obs, K, V, ema_decay, pool, nullptr, nullptr, O_obs, LSE_obs, &on_tc)) != RESTKV_OK) return s;
+  // Pooling (Eq. 13), selection and gather (Eq. 14) in one launch, chained to the kernel before it.  (The score kernel did
+  // this itself for long: six group barriers and four digit passes by 144 CTAs of which each had little to do, half of a
+  // short context's time; a 3000-row prompt went from 54.8 to 40.9 us.)
+  h->last_evict_fused = on_tc && !adaptive && !budgets && h->fused_select;
   RESTKV_LAUNCH(c, RESTKV_KERNEL_SELECT,
                 launch_select(p.BH, p.n, p.n_kv, budget, budgets, ws.I_hat, adaptive ? ws.pool : nullptr, pool->width,
-                              pool->shift, p.spatial == RESTKV_SPATIAL_MAX, scores, indices, nullptr,
-                              fuse_gather ? &p : nullptr, K, V, K_out, V_out, c.st), 1);
-  if (!fuse_gather) {
-    const int n_sel = budget < p.n_kv ? budget : p.n_kv;
-    RESTKV_LAUNCH(c, RESTKV_KERNEL_COMPACT,
-                  launch_compact(p, K, V, indices, n_sel, K_out, V_out, h->dev_status, c.st), 1);
-  }
+                              pool->shift, p.spatial == RESTKV_SPATIAL_MAX, scores, indices, nullptr, &p, K, V, K_out, V_out,
+                              h->select_clusters, h->dev_status, h->fused_select, c.st), 1);
   return RESTKV_OK;
 }
 
@@ -588,7 +563,7 @@ restkv_status restkv_decode(restkv_handle* h, const restkv_shape* shape, const v
       RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE, launch_decode_pad(p, q, ws.q_pad, c.st), 1);
       RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE,
                     launch_tc_fused(h->tc_state, pd, ws, ws.q_pad, Kc, Vc, 0.f, h->sm_count, false, true, h->wait_limit,
-                                    nullptr, nullptr, nullptr, h->dev_status, c.st), 1);
+                                    nullptr, nullptr, h->dev_status + kDevStatusWords, h->dev_status, false, c.st), 1);
       RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE, launch_decode_extract(p, ws.O_f32, ws.row_M2, out, lse, c.st), 1);
       return RESTKV_OK;
     }

@@ -42,11 +42,8 @@ struct Workspace {
   float* part_l;          // [slots, R]      one per CTA in the persistent tensor-core kernel
   float* part_O;          // [slots, R, d]
   float* vnorm;           // [BH, n_kv]  ||v_j||^2 (tensor-core path)
-  unsigned int* counters; // [256] group barrier counters of the persistent score kernel
   float* tile_max;        // [BH, tiles, 128] per-tile row maxima of the persistent score kernel
   float* row_M2;          // [BH, 128] log2 normaliser of each query row
-  unsigned int* sel_hist; // [BH, 4, 256] digit histograms of the selection inside the score kernel
-  unsigned int* sel_sfx;  // [SMs, 4, 260] per-CTA suffix sums of those histograms
   __nv_bfloat16* q_pad;   // [BH, 128, 128] decode queries padded to the kernel's 128 rows
   float* fin_m;           // [BH, R]    row max of the scaled logits (natural units)
   float* fin_l;           // [BH, R]    sum of exp(s - m)
@@ -60,21 +57,14 @@ struct Workspace {
   int* pool;              // [BH, 2] (W, gamma)
   float* dec_part;        // decode partials
   float* I_raw;           // adaptive only: [batch, Hq, w, n]
-  int32_t* adaptive_idx;  // adaptive only: [batch*Hq*w, B_p] per-query top-B_p indices
-  unsigned long long* adaptive_sums;  // adaptive only: [BH, 2] index sums (front, rear)
+  unsigned long long* adaptive_sums;  // adaptive only: [batch*Hq*w, 8] index sums of the per-query top-B_p, a value per CTA of a row
   size_t bytes;
 };
 
 constexpr int kDecodeMaxSplits = 64;
 
-// Pooling window, budget and outputs of the selection that the tensor-core score kernel can run itself.
-struct FusedSelect {
-  int keep, W, gamma;
-  float* scores;          // [BH, n_kv] pooled scores
-  int32_t* indices;       // [BH, keep]
-  void* K_out;            // [BH, keep, d]
-  void* V_out;
-};
+// Words of the handle's device block: status, and the barrier counters of the persistent score kernel (zero between launches).
+constexpr int kDevStatusWords = 64, kDevCounterWords = 256;
 
 int pass1_splits(const Problem& p, int sm_count);
 size_t plan_workspace(const Problem& p, int budget, int sm_count, bool adaptive, void* base, Workspace* ws);
@@ -87,9 +77,12 @@ cudaError_t launch_simt_pass2(const Problem& p, const Workspace& ws, const void*
                               float ema_decay, float* I_raw, cudaStream_t st);
 cudaError_t launch_pool(const Problem& p, const Workspace& ws, const int* pool_dev, int W, int gamma, float* scores,
                         int32_t* pool_used, cudaStream_t st);
-cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep_rows, const float* I_hat, const int* pool_dev, int W,
-                          int gamma, bool pool_max, float* scores, int32_t* indices, int32_t* pool_used, const Problem* gather,
-                          const void* K, const void* V, void* K_out, void* V_out, cudaStream_t st);
+cudaError_t select_init(int* clusters_of);   // [4]
+int select_cluster(int rows, int n_kv, const int* clusters_of);
+cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep_rows, const float* I_hat, const int* pool_dev,
+                          int W, int gamma, bool pool_max, float* scores, int32_t* indices, unsigned long long* index_sums,
+                          const Problem* gather, const void* K, const void* V, void* K_out, void* V_out,
+                          const int* clusters_of, unsigned int* dev_status, bool chained, cudaStream_t st);
 cudaError_t launch_compact(const Problem& p, const void* K, const void* V, const int32_t* indices, int n_sel,
                            void* K_out, void* V_out, unsigned int* dev_status, cudaStream_t st);
 cudaError_t launch_decode(const Problem& p, const void* q, const void* Kc, const void* Vc, int n_rows, float* out,
@@ -103,7 +96,7 @@ cudaError_t launch_decode_mma(void* state, const Problem& p, const void* q, cons
                               float* out, float* lse, float* part, int cluster, int splits, long long wait_limit,
                               unsigned int* dev_status, cudaStream_t st);
 cudaError_t launch_adaptive_params(const Problem& p, const Workspace& ws, int budget, float beta, int base_width,
-                                   cudaStream_t st, int* n_launches);
+                                   const int* clusters_of, unsigned int* dev_status, cudaStream_t st, int* n_launches);
 
 // Output projection (Eq. 4): the caller-owned factor buffer and the per-call projected rows.
 size_t projection_factor_bytes(int n_q_heads, int d);
@@ -118,8 +111,8 @@ cudaError_t tc_init(void** state);   // resolves the driver entry point for tens
 cudaError_t tc_fused_init();
 cudaError_t launch_tc_fused(void* state, const Problem& p, const Workspace& ws, const void* Q, const void* K,
                             const void* V, float ema_decay, int sm_count, bool reuse_l2, bool attention_only,
-                            long long wait_limit, const FusedSelect* sel, const float* O_given, float* I_raw,
-                            unsigned int* dev_status, cudaStream_t st);
+                            long long wait_limit, const float* O_given, float* I_raw, unsigned int* counters,
+                            unsigned int* dev_status, bool chained, cudaStream_t st);
 // Given the window rows' outputs O [BH, R, d] and log-sum-exps LSE [BH, R] (natural log): what the score kernels read
 // instead of the results of pass 1 and the merge.  tensor_core: -2 bf16(O), the constant strip, the rows' log2
 // normalisers; otherwise fin_m = LSE, fin_l = 1.
@@ -131,9 +124,6 @@ cudaError_t launch_tc_vmv(void* state, const Problem& p, const void* V, float* o
                           unsigned int* dev_status, cudaStream_t st);
 // Whether the tensor-core kernel's temporal chain can carry the variant's weights for this decay and window.
 bool tc_variant_supported(const Problem& p, float ema_decay);
-bool tc_fused_select_supported(const Problem& p, int sm_count, bool reuse_l2, int keep, int W, int gamma);
-size_t tc_fused_select_sfx_words(int sm_count);
-size_t tc_fused_select_hist_words(int BH);
 cudaError_t launch_decode_pad(const Problem& p, const void* q, __nv_bfloat16* q_pad, cudaStream_t st);
 cudaError_t launch_decode_extract(const Problem& p, const float* O_f32, const float* row_M2, float* out, float* lse,
                                   cudaStream_t st);

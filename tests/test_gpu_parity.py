@@ -413,6 +413,17 @@ def test_evict_host_matches_oracle(handle):
 
 
 # ------------------------------------------------------------------ unit: select, compact, decode
+@pytest.mark.parametrize("spec", [(1, 1, 1, 1), (1, 31, 7, 5), (2, 255, 254, 7), (3, 1025, 40, 33), (2, 8160, 3000, 7), (2, 8161, 3000, 5),
+                                  (20, 8161, 77, 7), (40, 9000, 700, 3), (160, 1500, 64, 7), (150, 26001, 100, 5),
+                                  (1, 65537, 513, 301), (1, 300007, 70000, 7)])
+def test_selection_kernel_edges(handle, spec):
+    """One block, blocks that each select from the whole row, and clusters; every row length around its limits, many rows,
+    a window wider than the staged taps, a slice that does not stay in shared memory."""
+    heads, n, budget, width = spec
+    inp = make_inputs(Case("sel", 1, heads, heads, 16, n, 2, budget, width, 1, 0.5, "f32", 2, "normal", n))
+    full_check(handle, inp)
+
+
 def test_select_matches_stable_sort_with_ties_and_inf(handle):
     import torch
     rng = np.random.default_rng(3)
