@@ -30,9 +30,9 @@ namespace restkv {
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 int pass1_splits(const Problem& p, int sm_count) {
-  // one wave of (batch, head, split) blocks over the SMs, at least one 128-token tile per split
-  int splits = sm_count / p.BH;
-  const int tiles = (p.n_kv + 127) / 128;
+  // two blocks of the SIMT pass 1 (a token split, a (batch, KV head), 64 query rows) per SM, at least one 32-token tile each
+  int splits = 2 * sm_count / (p.BH * ((p.R + 63) / 64));
+  const int tiles = (p.n_kv + 31) / 32;
   if (splits > tiles) splits = tiles;
   if (splits < 1) splits = 1;
   return splits;

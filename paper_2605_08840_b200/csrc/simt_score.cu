@@ -1,257 +1,468 @@
 // fp32 SIMT kernels of the score path: used for RESTKV_F32 inputs and for every shape the
 // tensor-core kernels do not cover.  Same two-pass structure as the tensor-core path:
-//   pass 1   per (batch, KV head, token split): online softmax statistics (m, l) and the
-//            unnormalised window outputs of all w*G query rows           (Eq. 3)
-//   combine  merge the splits: m, l, O, plus the quantities the tensor-core pass 2 wants
+//   pass 1   per (batch, KV head, token split, block of 64 query rows): online softmax statistics (m, l) and the
+//            unnormalised window outputs                                  (Eq. 3)
+//   combine  merge the splits: m, l, O
 //   pass 2   per token: A = exp(s - m) / l, I = A / (1 - A) * ||o - v||  (Eq. 7),
-//            EMA recursion over the window queries                        (Eq. 8-9),
+//            weighted over the window queries                             (Eq. 8-9),
 //            mean over the query heads of the group
+// What bounds them: FFMA issue on long caches, launches and the latency of each kernel's chain on the short ones that
+// single precision is used for.  Tiles of K, V, Q, O lie row-major in shared memory, rows padded by 16 bytes (their pitch
+// is then an odd multiple of 16 bytes, so that 128-bit loads from eight different rows do not collide), and a thread works
+// on a small block of (row, token) pairs, four dims per load.  Measured on 1024 rows, 2 KV heads of 4 queries, d = 64,
+// against one thread per query row (pass 1) and per token and head (pass 2) before: 198 + 8 + 115 -> 8.5 + 8 + 13 us; the
+// launches are chained, the whole eviction of that cache takes 30 us instead of 265.
 #include "restkv_common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace restkv {
 
 namespace {
 
-constexpr int kP1Tile = 32;   // tokens per shared-memory tile in pass 1
-constexpr int kP2Tile = 64;   // tokens per block in pass 2
+constexpr int kThreads = 256;
+constexpr int kP1Tile = 32;   // tokens per tile of pass 1
+constexpr int kP1Rows = 64;   // query rows per block of pass 1
+constexpr int kP2Rows = 64;   // query rows per step of pass 2
 
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+  const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                     __uint_as_float(u.y & 0xFFFF0000u));
+}
+
+// rows x d elements as fp32 into rows of pitch d + 4; rows from rows_valid on are zero.  fp32 travels by asynchronous
+// copies (all of a kernel's tiles are then in flight together: the short caches this path is used for are bound by such
+// latencies), bf16 through registers, four loads at a time.  load_wait: the copies of this thread have landed.
+__device__ __forceinline__ void load_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 template <typename T>
-__device__ __forceinline__ void load_tile_f32(float* dst, int dst_stride, const T* src, long long row_stride,
-                                              int rows, int rows_valid, int d) {
-  // rows x d elements, converted to fp32; rows >= rows_valid are zero-filled
-  for (int e = threadIdx.x; e < rows * d; e += blockDim.x) {
-    int r = e / d, k = e - r * d;
-    dst[r * dst_stride + k] = (r < rows_valid) ? to_f32<T>(src[(long long)r * row_stride + k]) : 0.f;
+__device__ __forceinline__ void load_rows(float* dst, const T* src, long long row_stride, int rows, int rows_valid, int d) {
+  // q four-element pieces per row; the row of piece e by a reciprocal (e < 2^16 here, so the rounding cannot reach a whole)
+  const int q = d >> 2, total = rows * q, ld = d + 4;
+  const float inv_q = 1.f / (float)q;
+  for (int e0 = threadIdx.x; e0 < total; e0 += 4 * kThreads) {
+    float4 v[4];
+    int at[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int e = e0 + k * kThreads, r = (int)(((float)e + 0.5f) * inv_q), c = (e - r * q) * 4;
+      at[k] = r * ld + c;
+      const bool in = e < total && r < rows_valid;
+      if constexpr (sizeof(T) == 4) {
+        if (e < total)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(dst + at[k])),
+                       "l"(src + (in ? r * row_stride + c : 0)), "r"(in ? 16 : 0)
+                       : "memory");
+      } else {
+        v[k] = in ? load4(src + r * row_stride + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+    if constexpr (sizeof(T) != 4) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (e0 + k * kThreads < total) *reinterpret_cast<float4*>(dst + at[k]) = v[k];
+    }
   }
 }
 
+__device__ __forceinline__ float dot4(float4 a, float4 b, float acc) {
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
+}
+
 // ------------------------------------------------------------------------------------------------
-// Pass 1.  grid (splits, BH), block = R rounded up to a warp multiple.  Thread r owns query row r.
-// Shared memory: Qs [R][d+1], Os [R][d+1], Kt [32][d], Vt [32][d] (fp32).
-template <typename T>
-__global__ void simt_pass1_kernel(Problem p, const T* __restrict__ Q, const T* __restrict__ K,
-                                  const T* __restrict__ V, float* __restrict__ part_m, float* __restrict__ part_l,
-                                  float* __restrict__ part_O, int splits) {
-  extern __shared__ float smem[];
-  const int d = p.d, R = p.R, ld = d + 1;
+// Pass 1.  grid (splits, BH, blocks of 64 rows), block 256.  For the logits a thread owns rows tid / 8 and tid / 8 + 32 and
+// every eighth token of the tile; for P V rows tid / 16 + 16 i and the columns 4 (tid % 16) + 64 c, c < kCols.
+// Shared memory: Q [64][d+4], K [32][d+4], V [32][d+4], P [64][36], the rows' rescaling factors [64].
+template <typename T, int kCols>
+__global__ void __launch_bounds__(kThreads) simt_pass1_kernel(Problem p, const T* __restrict__ Q, const T* __restrict__ K,
+                                                              const T* __restrict__ V, float* __restrict__ part_m,
+                                                              float* __restrict__ part_l, float* __restrict__ part_O, int splits) {
+  extern __shared__ __align__(16) float smem[];
+  const int d = p.d, ld = d + 4, R = p.R;
+  constexpr int ldp = kP1Tile + 4;
   float* Qs = smem;
-  float* Os = Qs + (size_t)R * ld;
-  float* Kt = Os + (size_t)R * ld;
-  float* Vt = Kt + (size_t)kP1Tile * d;
-
-  const int split = blockIdx.x, bh = blockIdx.y;
+  float* Ks = Qs + kP1Rows * ld;
+  float* Vs = Ks + kP1Tile * ld;
+  float* Ps = Vs + kP1Tile * ld;
+  float* corr_s = Ps + kP1Rows * ldp;
+  const int split = blockIdx.x, bh = blockIdx.y, row0 = blockIdx.z * kP1Rows;
   const int b = bh / p.Hkv, h = bh % p.Hkv;
-  const int r = threadIdx.x;
-  const bool active = r < R;
-  const int i_q = active ? (r % p.w) : 0;   // window position of this row (row = g*w + i)
-
-  const T* Qh = Q + ((long long)b * p.Hq + (long long)h * p.G) * p.w * d;   // [R, d] contiguous
+  const int tid = threadIdx.x, tr = tid >> 3, tc = tid & 7, pr = tid >> 4, pc = (tid & 15) * 4;
+  const T* Qh = Q + (((long long)b * p.Hq + (long long)h * p.G) * p.w + row0) * d;   // [R, d] contiguous
   const T* Kh = K + (long long)b * p.ksb + (long long)h * p.ksh;
   const T* Vh = V + (long long)b * p.vsb + (long long)h * p.vsh;
+  ptx::grid_dependency_wait();
+  ptx::grid_dependency_launch();
+  load_rows<T>(Qs, Qh, d, kP1Rows, min(kP1Rows, R - row0), d);
 
-  for (int e = threadIdx.x; e < R * d; e += blockDim.x) {
-    int rr = e / d, k = e - rr * d;
-    Qs[rr * ld + k] = to_f32<T>(Qh[(long long)rr * d + k]);
-    Os[rr * ld + k] = 0.f;
-  }
-
-  // contiguous range of 32-token tiles for this split
   const int n_tiles = (p.n_kv + kP1Tile - 1) / kP1Tile;
   const int per = (n_tiles + splits - 1) / splits;
-  const int tile0 = split * per;
-  const int tile1 = min(n_tiles, tile0 + per);
+  const int tile0 = split * per, tile1 = min(n_tiles, tile0 + per);
+  float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
+  float o[4][4 * kCols];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int c = 0; c < 4 * kCols; ++c) o[i][c] = 0.f;
 
-  float m = -INFINITY, l = 0.f;
   for (int tile = tile0; tile < tile1; ++tile) {
-    const int j0 = tile * kP1Tile;
-    const int valid = min(kP1Tile, p.n_kv - j0);
+    const int j0 = tile * kP1Tile, valid = min(kP1Tile, p.n_kv - j0);
+    __syncthreads();   // the tile before has been used
+    load_rows<T>(Ks, Kh + (long long)j0 * p.ksn, p.ksn, kP1Tile, valid, d);
+    load_rows<T>(Vs, Vh + (long long)j0 * p.vsn, p.vsn, kP1Tile, valid, d);
+    load_wait();
     __syncthreads();
-    load_tile_f32<T>(Kt, d, Kh + (long long)j0 * p.ksn, p.ksn, kP1Tile, valid, d);
-    load_tile_f32<T>(Vt, d, Vh + (long long)j0 * p.vsn, p.vsn, kP1Tile, valid, d);
+    float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll 2
+    for (int k = 0; k < d; k += 4) {
+      const float4 q0 = *reinterpret_cast<const float4*>(Qs + tr * ld + k), q1 = *reinterpret_cast<const float4*>(Qs + (tr + 32) * ld + k);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const float4 kv = *reinterpret_cast<const float4*>(Ks + (tc + 8 * t) * ld + k);
+        s[0][t] = dot4(q0, kv, s[0][t]);
+        s[1][t] = dot4(q1, kv, s[1][t]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int r = tr + 32 * i, i_q = (row0 + r) % p.w;   // window position of the row (row = g*w + i)
+      float tmax = -INFINITY;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int j = j0 + tc + 8 * t;
+        // visible: inside the cache, and for trailing (window) rows only those not after this query
+        const bool vis = j < p.n_kv && (j < p.n || (j - p.n) <= i_q);
+        s[i][t] = vis ? s[i][t] * p.scale : -INFINITY;
+        tmax = fmaxf(tmax, s[i][t]);
+      }
+#pragma unroll
+      for (int off = 4; off > 0; off >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, off));
+      const float m_new = fmaxf(m[i], tmax);
+      const float base = m_new == -INFINITY ? 0.f : m_new;   // nothing visible so far: every weight is 0
+      const float corr = expf(m[i] - base);                  // m = -inf gives 0
+      float sum = 0.f;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const float e = expf(s[i][t] - base);
+        sum += e;
+        Ps[r * ldp + tc + 8 * t] = e;
+      }
+#pragma unroll
+      for (int off = 4; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+      l[i] = l[i] * corr + sum;
+      m[i] = m_new;
+      if (tc == 0) corr_s[r] = corr;
+    }
     __syncthreads();
-    if (!active) continue;
-
-    float s[kP1Tile];
 #pragma unroll
-    for (int t = 0; t < kP1Tile; ++t) s[t] = 0.f;
-    for (int k = 0; k < d; ++k) {
-      const float qv = Qs[r * ld + k];
+    for (int i = 0; i < 4; ++i) {
+      const float c = corr_s[pr + 16 * i];
 #pragma unroll
-      for (int t = 0; t < kP1Tile; ++t) s[t] = fmaf(qv, Kt[t * d + k], s[t]);
+      for (int e = 0; e < 4 * kCols; ++e) o[i][e] *= c;
     }
-    float tmax = -INFINITY;
+#pragma unroll 2
+    for (int t = 0; t < kP1Tile; t += 4) {
+      float4 pw[4];
 #pragma unroll
-    for (int t = 0; t < kP1Tile; ++t) {
-      const int j = j0 + t;
-      // visible: inside the cache, and for trailing (window) rows only those not after this query
-      const bool vis = (t < valid) && (j < p.n || (j - p.n) <= i_q);
-      s[t] = vis ? s[t] * p.scale : -INFINITY;
-      tmax = fmaxf(tmax, s[t]);
-    }
-    const float m_new = fmaxf(m, tmax);
-    if (m_new == -INFINITY) continue;   // nothing visible so far
-    const float corr = expf(m - m_new);   // m = -inf gives 0
-    float lsum = 0.f;
+      for (int i = 0; i < 4; ++i) pw[i] = *reinterpret_cast<const float4*>(Ps + (pr + 16 * i) * ldp + t);
 #pragma unroll
-    for (int t = 0; t < kP1Tile; ++t) {
-      s[t] = expf(s[t] - m_new);          // masked entries give 0
-      lsum += s[t];
-    }
-    l = l * corr + lsum;
-    m = m_new;
-    for (int k = 0; k < d; ++k) {
-      float acc = Os[r * ld + k] * corr;
+      for (int u = 0; u < 4; ++u)
 #pragma unroll
-      for (int t = 0; t < kP1Tile; ++t) acc = fmaf(s[t], Vt[t * d + k], acc);
-      Os[r * ld + k] = acc;
+        for (int c = 0; c < kCols; ++c) {
+          if (pc + 64 * c >= d) continue;
+          const float4 v = *reinterpret_cast<const float4*>(Vs + (t + u) * ld + pc + 64 * c);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float w = u == 0 ? pw[i].x : u == 1 ? pw[i].y : u == 2 ? pw[i].z : pw[i].w;
+            o[i][4 * c] = fmaf(w, v.x, o[i][4 * c]);
+            o[i][4 * c + 1] = fmaf(w, v.y, o[i][4 * c + 1]);
+            o[i][4 * c + 2] = fmaf(w, v.z, o[i][4 * c + 2]);
+            o[i][4 * c + 3] = fmaf(w, v.w, o[i][4 * c + 3]);
+          }
+        }
     }
   }
-  if (active) {
-    const long long o = ((long long)bh * splits + split) * R + r;
-    part_m[o] = m;
-    part_l[o] = l;
-    float* Op = part_O + o * d;
-    for (int k = 0; k < d; ++k) Op[k] = Os[r * ld + k];
+  const long long out = ((long long)bh * splits + split) * R + row0;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (tc == 0 && row0 + tr + 32 * i < R) {
+      part_m[out + tr + 32 * i] = m[i];
+      part_l[out + tr + 32 * i] = l[i];
+    }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = pr + 16 * i;
+    if (row0 + r >= R) continue;
+#pragma unroll
+    for (int c = 0; c < kCols; ++c)
+      if (pc + 64 * c < d)
+        *reinterpret_cast<float4*>(part_O + (out + r) * d + pc + 64 * c) = make_float4(o[i][4 * c], o[i][4 * c + 1], o[i][4 * c + 2], o[i][4 * c + 3]);
   }
 }
 
 // ------------------------------------------------------------------------------------------------
-// Combine the token splits.  grid (R, BH), block 128: one block per query row.
-__global__ void combine_kernel(int R, int d, int splits, const float* __restrict__ part_m,
-                               const float* __restrict__ part_l, const float* __restrict__ part_O,
-                               float* __restrict__ fin_m, float* __restrict__ fin_l, float* __restrict__ O_f32) {
-  const int r = blockIdx.x, bh = blockIdx.y;
+// Combine the token splits.  grid (R, BH), block 128: one block per query row; warp w adds up splits w, w + 4, ..., lane =
+// four dims (two times four where d > 128); the four sums are added in a fixed order.
+__global__ void __launch_bounds__(128) combine_kernel(int R, int d, int splits, const float* __restrict__ part_m,
+                                                      const float* __restrict__ part_l, const float* __restrict__ part_O,
+                                                      float* __restrict__ fin_m, float* __restrict__ fin_l,
+                                                      float* __restrict__ O_f32) {
+  ptx::grid_dependency_wait();
+  ptx::grid_dependency_launch();
+  __shared__ __align__(16) float sums[4][256];
+  const int r = blockIdx.x, bh = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const long long base = (long long)bh * splits * R + r;   // + s * R
   float m = -INFINITY;
-  for (int s = 0; s < splits; ++s) m = fmaxf(m, part_m[base + (long long)s * R]);
+  for (int s = lane; s < splits; s += 32) m = fmaxf(m, part_m[base + (long long)s * R]);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
   float l = 0.f;
-  for (int s = 0; s < splits; ++s) {
-    const float ms = part_m[base + (long long)s * R];
-    if (ms != -INFINITY) l += part_l[base + (long long)s * R] * expf(ms - m);
-  }
-  const float inv_l = 1.f / l;
-  for (int k = threadIdx.x; k < d; k += blockDim.x) {
-    float acc = 0.f;
-    for (int s = 0; s < splits; ++s) {
-      const float ms = part_m[base + (long long)s * R];
-      if (ms != -INFINITY) acc += part_O[(base + (long long)s * R) * d + k] * expf(ms - m);
+  for (int s = lane; s < splits; s += 32) l += part_l[base + (long long)s * R] * expf(part_m[base + (long long)s * R] - m);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+  for (int c = lane * 4; c < d; c += 128) {
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int s = wid; s < splits; s += 4) {
+      const float w = expf(part_m[base + (long long)s * R] - m);   // an empty split weighs 0
+      const float4 v = *reinterpret_cast<const float4*>(part_O + (base + (long long)s * R) * d + c);
+      acc.x = fmaf(v.x, w, acc.x); acc.y = fmaf(v.y, w, acc.y); acc.z = fmaf(v.z, w, acc.z); acc.w = fmaf(v.w, w, acc.w);
     }
-    O_f32[((long long)bh * R + r) * d + k] = acc * inv_l;
+    *reinterpret_cast<float4*>(&sums[wid][c]) = acc;
   }
+  __syncthreads();
+  const float inv_l = 1.f / l;
+  for (int k = threadIdx.x; k < d; k += 128)
+    O_f32[((long long)bh * R + r) * d + k] = ((sums[0][k] + sums[1][k]) + (sums[2][k] + sums[3][k])) * inv_l;
   if (threadIdx.x == 0) {
     fin_m[(long long)bh * R + r] = m;
     fin_l[(long long)bh * R + r] = l;
   }
 }
 
+// Eq. 7 for one pair from its scaled logit's weight e = exp(s - m) and the squared distance; vlen: ||v|| for the
+// attention-weight indicators (1 without the value norm).
+__device__ __forceinline__ float indicator_of(int indicator, float e, float l, float ss, float vlen) {
+  if (indicator != RESTKV_INDICATOR_RECONSTRUCTION) return (e / l) * vlen;
+  const float one_minus = fmaxf((l - e) / l, 5.9604645e-8f);   // 1 - A; clamped so that A -> 1 stays finite
+  return (e / l) / one_minus * sqrtf(ss);
+}
+
+// Weight of window position i under the temporal mode (Eq. 8-9 as the closed form of its recursion, Appendix G.2).
+__device__ __forceinline__ float temporal_weight(int mode, float decay, int w, int i) {
+  const float alpha = 1.f - decay;
+  switch (mode) {
+    case RESTKV_TEMPORAL_EMA: return i == 0 ? powf(decay, (float)(w - 1)) : alpha * powf(decay, (float)(w - 1 - i));
+    case RESTKV_TEMPORAL_MEAN: return 1.f / (float)w;
+    case RESTKV_TEMPORAL_INV_EMA: return i == w - 1 ? powf(decay, (float)(w - 1)) : alpha * powf(decay, (float)i);
+    default: return i == w - 1 ? 1.f : 0.f;   // the newest query alone
+  }
+}
+
 // ------------------------------------------------------------------------------------------------
-// Pass 2.  grid (token tiles of 64, BH), block 64 * GP threads: thread = (token, group slot).
-// Shared memory: Kt [64][d+1], Vt [64][d+1], red [GP][64].
+// Pass 2 without an output projection.  grid (blocks of kTB tokens, BH), block 256: a thread owns two rows of each step of
+// 64 and kTB / 8 tokens.  Shared memory: K, V [kTB][d+4], Q, O [held][d+4] (held: a multiple of 64, all rows if they fit), the temporal weights [w], and for the maximum over
+// the query heads the weighted indicators of a step [64][kTB+1] and the heads' sums [G][kTB].
+template <typename T, int kTB>
+__global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T* __restrict__ Q, const T* __restrict__ K,
+                                                              const T* __restrict__ V, const float* __restrict__ fin_m,
+                                                              const float* __restrict__ fin_l, const float* __restrict__ O_f32,
+                                                              float ema_decay, float* __restrict__ I_hat, float* __restrict__ I_raw,
+                                                              int held) {
+  extern __shared__ __align__(16) float smem[];
+  constexpr int kTok = kTB / 8;
+  const int d = p.d, ld = d + 4, R = p.R;
+  float* Ks = smem;
+  float* Vs = Ks + kTB * ld;
+  float* Qh_s = Vs + kTB * ld;
+  float* Oh_s = Qh_s + held * ld;
+  float* wt = Oh_s + held * ld;
+  float* Iw = wt + p.w;
+  float* gsum = Iw + kP2Rows * (kTB + 1);
+  __shared__ float vlen_s[kTB], red[4][kTB];
+  const int bh = blockIdx.y, b = bh / p.Hkv, h = bh % p.Hkv, j0 = blockIdx.x * kTB;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int rl = (wid & 3) * 8 + (lane & 7), tl = (wid >> 2) * 4 + (lane >> 3);
+  const int valid = min(kTB, p.n - j0);
+  const T* Qh = Q + ((long long)b * p.Hq + (long long)h * p.G) * p.w * d;
+  const float* Oh = O_f32 + (long long)bh * R * d;
+  const bool gmax = p.group == RESTKV_GROUP_MAX;
+  for (int i = tid; i < p.w; i += kThreads) wt[i] = temporal_weight(p.temporal, ema_decay, p.w, i);
+  ptx::grid_dependency_wait();
+  ptx::grid_dependency_launch();
+  load_rows<T>(Ks, K + (long long)b * p.ksb + (long long)h * p.ksh + (long long)j0 * p.ksn, p.ksn, kTB, valid, d);
+  load_rows<T>(Vs, V + (long long)b * p.vsb + (long long)h * p.vsh + (long long)j0 * p.vsn, p.vsn, kTB, valid, d);
+  if (gmax)
+    for (int e = tid; e < p.G * kTB; e += kThreads) gsum[e] = 0.f;
+  if (p.indicator == RESTKV_INDICATOR_ATTENTION_VNORM) {
+    load_wait();
+    __syncthreads();
+    if (tid < kTB) {
+      float vv = 0.f;
+      for (int k = 0; k < d; ++k) vv = fmaf(Vs[tid * ld + k], Vs[tid * ld + k], vv);
+      vlen_s[tid] = sqrtf(vv);
+    }
+  } else if (tid < kTB) {
+    vlen_s[tid] = 1.f;
+  }
+  float acc[kTok];
+#pragma unroll
+  for (int t = 0; t < kTok; ++t) acc[t] = 0.f;
+
+  for (int row0 = 0; row0 < R; row0 += kP2Rows) {
+    const int rows = min(kP2Rows, R - row0);
+    if (row0 % held == 0) {   // the next `held` rows of Q and O
+      if (row0 > 0) __syncthreads();   // the rows before have been used
+      load_rows<T>(Qh_s, Qh + (long long)row0 * d, d, held, min(held, R - row0), d);
+      load_rows<float>(Oh_s, Oh + (long long)row0 * d, d, held, min(held, R - row0), d);
+    }
+    const float* Qs = Qh_s + (row0 % held) * ld;
+    const float* Os = Oh_s + (row0 % held) * ld;
+    float fm[2], fl[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int r = rl + 32 * i;
+      fm[i] = r < rows ? fin_m[(long long)bh * R + row0 + r] : 0.f;
+      fl[i] = r < rows ? fin_l[(long long)bh * R + row0 + r] : 1.f;
+    }
+    if (row0 % held == 0) {
+      load_wait();
+      __syncthreads();
+    }
+    float s[2][kTok], ss[2][kTok];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int t = 0; t < kTok; ++t) s[i][t] = ss[i][t] = 0.f;
+#pragma unroll 2
+    for (int k = 0; k < d; k += 4) {
+      float4 q[2], o[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        q[i] = *reinterpret_cast<const float4*>(Qs + (rl + 32 * i) * ld + k);
+        o[i] = *reinterpret_cast<const float4*>(Os + (rl + 32 * i) * ld + k);
+      }
+#pragma unroll
+      for (int t = 0; t < kTok; ++t) {
+        const float4 kv = *reinterpret_cast<const float4*>(Ks + (tl + 8 * t) * ld + k);
+        const float4 v = *reinterpret_cast<const float4*>(Vs + (tl + 8 * t) * ld + k);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          s[i][t] = dot4(q[i], kv, s[i][t]);
+          const float4 df = make_float4(o[i].x - v.x, o[i].y - v.y, o[i].z - v.z, o[i].w - v.w);
+          ss[i][t] = dot4(df, df, ss[i][t]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int r = rl + 32 * i, row = row0 + r;
+      const float weight = r < rows ? wt[row % p.w] : 0.f;
+#pragma unroll
+      for (int t = 0; t < kTok; ++t) {
+        const int tok = tl + 8 * t;
+        const float I = indicator_of(p.indicator, expf(s[i][t] * p.scale - fm[i]), fl[i], ss[i][t], vlen_s[tok]);
+        if (I_raw && r < rows && tok < valid) I_raw[((long long)bh * R + row) * p.n + j0 + tok] = I;
+        const float wI = r < rows ? weight * I : 0.f;
+        if (gmax) Iw[r * (kTB + 1) + tok] = wI;
+        else acc[t] += wI;
+      }
+    }
+    if (gmax) {   // add this step's rows to the sums of their heads, in order
+      __syncthreads();
+      const int g0 = row0 / p.w, g1 = (row0 + rows - 1) / p.w;
+      for (int e = tid; e < (g1 - g0 + 1) * kTB; e += kThreads) {
+        const int g = g0 + e / kTB, tok = e % kTB;
+        const int ra = max(row0, g * p.w) - row0, rb = min(row0 + rows, (g + 1) * p.w) - row0;
+        float sum = gsum[g * kTB + tok];
+        for (int r = ra; r < rb; ++r) sum += Iw[r * (kTB + 1) + tok];
+        gsum[g * kTB + tok] = sum;
+      }
+      __syncthreads();
+    }
+  }
+  if (gmax) {
+    __syncthreads();
+    if (tid < valid) {
+      float best = 0.f;
+      for (int g = 0; g < p.G; ++g) best = fmaxf(best, gsum[g * kTB + tid]);
+      I_hat[(long long)bh * p.n + j0 + tid] = best;
+    }
+    return;
+  }
+#pragma unroll
+  for (int t = 0; t < kTok; ++t) {
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) acc[t] += __shfl_xor_sync(0xffffffffu, acc[t], off);
+    if ((lane & 7) == 0) red[wid & 3][tl + 8 * t] = acc[t];
+  }
+  __syncthreads();
+  if (tid < valid) I_hat[(long long)bh * p.n + j0 + tid] = ((red[0][tid] + red[1][tid]) + (red[2][tid] + red[3][tid])) / (float)p.G;
+}
+
+// ------------------------------------------------------------------------------------------------
+// Pass 2 under the output projection of Eq. 4: (o - v)^T M (o - v) = (o - v) . (M o - M v); M v is formed once per token and
+// query head, M o comes in.  grid (token tiles of 64, BH), block 64 * GP threads: thread = (token, group slot).
+// Shared memory: Kt [64][d+1], Vt [64][d+1], red [GP][64], M v of each thread [GP * 64][d+1].
+constexpr int kP2Tile = 64;
 template <typename T>
-__global__ void simt_pass2_kernel(Problem p, const T* __restrict__ Q, const T* __restrict__ K,
-                                  const T* __restrict__ V, const float* __restrict__ fin_m,
-                                  const float* __restrict__ fin_l, const float* __restrict__ O_f32,
-                                  const float* __restrict__ O_proj, float ema_decay,
-                                  float* __restrict__ I_hat, float* __restrict__ I_raw, int GP) {
-  extern __shared__ float smem[];
+__global__ void simt_pass2_proj_kernel(Problem p, const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V,
+                                       const float* __restrict__ fin_m, const float* __restrict__ fin_l,
+                                       const float* __restrict__ O_f32, const float* __restrict__ O_proj, float ema_decay,
+                                       float* __restrict__ I_hat, float* __restrict__ I_raw, int GP) {
+  extern __shared__ __align__(16) float smem[];
   const int d = p.d, ld = d + 1;
   float* Kt = smem;
   float* Vt = Kt + (size_t)kP2Tile * ld;
   float* red = Vt + (size_t)kP2Tile * ld;
-  float* MVs = red + (size_t)GP * kP2Tile;   // [GP * kP2Tile][ld]: M v_j of each thread, with a projection only
-
+  float* MVs = red + (size_t)GP * kP2Tile;
   const int bh = blockIdx.y, b = bh / p.Hkv, h = bh % p.Hkv;
   const int j0 = blockIdx.x * kP2Tile;
   const int valid = min(kP2Tile, p.n - j0);
   const T* Kh = K + (long long)b * p.ksb + (long long)h * p.ksh + (long long)j0 * p.ksn;
   const T* Vh = V + (long long)b * p.vsb + (long long)h * p.vsh + (long long)j0 * p.vsn;
-  load_tile_f32<T>(Kt, ld, Kh, p.ksn, kP2Tile, valid, d);
-  load_tile_f32<T>(Vt, ld, Vh, p.vsn, kP2Tile, valid, d);
+  ptx::grid_dependency_wait();
+  for (int e = threadIdx.x; e < kP2Tile * d; e += blockDim.x) {
+    const int r = e / d, k = e - r * d;
+    Kt[r * ld + k] = r < valid ? to_f32<T>(Kh[r * p.ksn + k]) : 0.f;
+    Vt[r * ld + k] = r < valid ? to_f32<T>(Vh[r * p.vsn + k]) : 0.f;
+  }
   __syncthreads();
-
   const int t = threadIdx.x % kP2Tile, slot = threadIdx.x / kP2Tile;
   const int j = j0 + t;
-  const float alpha = 1.f - ema_decay;
   const T* Qh = Q + ((long long)b * p.Hq + (long long)h * p.G) * p.w * d;
   const float* Oh = O_f32 + (long long)bh * p.R * d;
   const float* kr = Kt + t * ld;
   const float* vr = Vt + t * ld;
-
-  // variants of Appendix G: p.indicator picks the per-query indicator, p.temporal the weights over the window
-  // queries, p.group the reduction over the query heads of the group
+  float* mv = MVs + (size_t)threadIdx.x * ld;
   const bool gmax = p.group == RESTKV_GROUP_MAX;
   float group_red = 0.f;
   if (t < valid) {
-    float vlen = 1.f;
-    if (p.indicator == RESTKV_INDICATOR_ATTENTION_VNORM) {
-      float vv = 0.f;
-      for (int k = 0; k < d; ++k) vv = fmaf(vr[k], vr[k], vv);
-      vlen = sqrtf(vv);
-    }
     for (int g = slot; g < p.G; g += GP) {
-      float ema = 0.f, pw = 1.f;   // pw = ema_decay^i for the inverted EMA
-      // Eq. 7 with the projection of Eq. 4: (o - v)^T M (o - v) = (o - v) . (M o - M v); M v is formed once per
-      // token and query head, M o comes in
-      float* mv = MVs + (size_t)threadIdx.x * ld;
-      if (p.proj.M && p.indicator == RESTKV_INDICATOR_RECONSTRUCTION) {
-        const float* Mg = p.proj.M + (long long)(h * p.G + g) * d * d;
-        for (int i = 0; i < d; ++i) {
-          float acc = 0.f;
-          for (int k = 0; k < d; ++k) acc = fmaf(Mg[i * d + k], vr[k], acc);
-          mv[i] = acc;
-        }
+      const float* Mg = p.proj.M + (long long)(h * p.G + g) * d * d;
+      for (int i = 0; i < d; ++i) {
+        float acc = 0.f;
+        for (int k = 0; k < d; ++k) acc = fmaf(Mg[i * d + k], vr[k], acc);
+        mv[i] = acc;
       }
+      float sum = 0.f;
       for (int i = 0; i < p.w; ++i) {
         // without temporal smoothing only the newest query counts (the raw indicators still want every query)
         if (p.temporal == RESTKV_TEMPORAL_NONE && i != p.w - 1 && !I_raw) continue;
         const int r = g * p.w + i;
         const T* qr = Qh + (long long)r * d;
         const float* orow = Oh + (long long)r * d;
+        const float* oprow = O_proj + ((long long)bh * p.R + r) * d;
         float s = 0.f, ss = 0.f;
-        if (p.proj.M) {
-          const float* oprow = O_proj + ((long long)bh * p.R + r) * d;
-          for (int k = 0; k < d; ++k) {
-            s = fmaf(to_f32<T>(qr[k]), kr[k], s);
-            ss = fmaf(orow[k] - vr[k], oprow[k] - mv[k], ss);
-          }
-          ss = fmaxf(ss, 0.f);
-        } else {
-          for (int k = 0; k < d; ++k) {
-            s = fmaf(to_f32<T>(qr[k]), kr[k], s);
-            const float df = orow[k] - vr[k];
-            ss = fmaf(df, df, ss);
-          }
+        for (int k = 0; k < d; ++k) {
+          s = fmaf(to_f32<T>(qr[k]), kr[k], s);
+          ss = fmaf(orow[k] - vr[k], oprow[k] - mv[k], ss);
         }
         const long long ri = (long long)bh * p.R + r;
-        const float l = fin_l[ri];
-        const float e = expf(s * p.scale - fin_m[ri]);
-        float I;
-        if (p.indicator == RESTKV_INDICATOR_RECONSTRUCTION) {
-          // 1 - A formed as (l - e) / l; clamped so that A -> 1 stays finite
-          const float one_minus = fmaxf((l - e) / l, 5.9604645e-8f);
-          I = (e / l) / one_minus * sqrtf(ss);
-        } else {
-          I = (e / l) * vlen;
-        }
-        if (I_raw) I_raw[(((long long)b * p.Hq + (long long)h * p.G + g) * p.w + i) * p.n + j] = I;
-        switch (p.temporal) {
-          case RESTKV_TEMPORAL_EMA:   // Eq. 9, oldest query first
-            ema = (i == 0) ? I : fmaf(alpha, I, ema_decay * ema);
-            break;
-          case RESTKV_TEMPORAL_MEAN:
-            ema += I;
-            break;
-          case RESTKV_TEMPORAL_INV_EMA:   // the recursion run backwards: weights alpha d^i, d^(w-1) for the newest
-            ema = fmaf((i == p.w - 1) ? pw : alpha * pw, I, ema);
-            pw *= ema_decay;
-            break;
-          default:
-            if (i == p.w - 1) ema = I;
-            break;
-        }
+        const float I = indicator_of(p.indicator, expf(s * p.scale - fin_m[ri]), fin_l[ri], fmaxf(ss, 0.f), 1.f);
+        if (I_raw) I_raw[ri * p.n + j] = I;
+        sum = fmaf(temporal_weight(p.temporal, ema_decay, p.w, i), I, sum);
       }
-      if (p.temporal == RESTKV_TEMPORAL_MEAN) ema /= (float)p.w;
-      group_red = gmax ? fmaxf(group_red, ema) : group_red + ema;
+      group_red = gmax ? fmaxf(group_red, sum) : group_red + sum;
     }
   }
   red[slot * kP2Tile + t] = group_red;
@@ -263,60 +474,76 @@ __global__ void simt_pass2_kernel(Problem p, const T* __restrict__ Q, const T* _
   }
 }
 
-template <typename KernelT>
-cudaError_t allow_smem(KernelT kernel, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+// A launch chained to the kernel before it in the stream (every kernel here waits for that one's results itself).
+template <typename... KArgs, typename... Args>
+cudaError_t chain(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned int)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+template <typename T>
+cudaError_t pass1(const Problem& p, const Workspace& ws, const void* Q, const void* K, const void* V, cudaStream_t st) {
+  const dim3 grid(ws.splits, p.BH, (p.R + kP1Rows - 1) / kP1Rows);
+  const size_t smem = ((size_t)(kP1Rows + 2 * kP1Tile) * (p.d + 4) + (size_t)kP1Rows * (kP1Tile + 4) + kP1Rows) * sizeof(float);
+  // columns of P V per thread: the accumulators of 64 rows x d, four rows each
+  auto kernel = p.d <= 64 ? simt_pass1_kernel<T, 1> : p.d <= 128 ? simt_pass1_kernel<T, 2> : simt_pass1_kernel<T, 4>;
+  return chain(kernel, grid, kThreads, smem, st, p, (const T*)Q, (const T*)K, (const T*)V, ws.part_m, ws.part_l, ws.part_O, ws.splits);
+}
+
+template <typename T>
+cudaError_t pass2(const Problem& p, const Workspace& ws, const void* Q, const void* K, const void* V, float ema_decay, float* I_raw,
+                  cudaStream_t st) {
+  if (p.proj.M) {
+    const int GP = p.G < 4 ? p.G : 4;
+    const size_t smem = ((size_t)(2 + GP) * kP2Tile * (p.d + 1) + (size_t)GP * kP2Tile) * sizeof(float);
+    return chain(simt_pass2_proj_kernel<T>, dim3((p.n + kP2Tile - 1) / kP2Tile, p.BH), kP2Tile * GP, smem, st, p, (const T*)Q,
+                 (const T*)K, (const T*)V, ws.fin_m, ws.fin_l, ws.O_f32, ws.O_proj, ema_decay, ws.I_hat, I_raw, GP);
+  }
+  const int all = (p.R + kP2Rows - 1) / kP2Rows * kP2Rows;
+  auto floats = [&](int tb, int held) {
+    return (size_t)2 * (tb + held) * (p.d + 4) + p.w +
+           (p.group == RESTKV_GROUP_MAX ? (size_t)kP2Rows * (tb + 1) + (size_t)p.G * tb : 0);
+  };
+  // 32 tokens per block share the loads of Q and O better; 16 where that would leave SMs with a single block, or where 32
+  // do not fit shared memory
+  const bool wide = (long long)(p.n + 31) / 32 * p.BH >= 296 && floats(32, kP2Rows) * sizeof(float) <= 220 * 1024;
+  const int tb = wide ? 32 : 16;
+  // all rows of Q and O stay in shared memory where two blocks of that size fit an SM
+  const int held = floats(tb, all) * sizeof(float) <= 110 * 1024 ? all : kP2Rows;
+  return chain(wide ? simt_pass2_kernel<T, 32> : simt_pass2_kernel<T, 16>, dim3((p.n + tb - 1) / tb, p.BH), kThreads,
+               floats(tb, held) * sizeof(float), st, p, (const T*)Q, (const T*)K, (const T*)V, ws.fin_m, ws.fin_l, ws.O_f32, ema_decay,
+               ws.I_hat, I_raw, held);
 }
 
 }  // namespace
 
 cudaError_t launch_simt_pass1(const Problem& p, const Workspace& ws, const void* Q, const void* K, const void* V,
                               cudaStream_t st) {
-  const int threads = ((p.R + 31) / 32) * 32;
-  const size_t smem = ((size_t)2 * p.R * (p.d + 1) + (size_t)2 * kP1Tile * p.d) * sizeof(float);
-  dim3 grid(ws.splits, p.BH);
-  cudaError_t e;
-  if (p.dtype == RESTKV_BF16) {
-    if ((e = allow_smem(simt_pass1_kernel<__nv_bfloat16>, smem)) != cudaSuccess) return e;
-    simt_pass1_kernel<__nv_bfloat16><<<grid, threads, smem, st>>>(
-        p, (const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, ws.part_m, ws.part_l,
-        ws.part_O, ws.splits);
-  } else {
-    if ((e = allow_smem(simt_pass1_kernel<float>, smem)) != cudaSuccess) return e;
-    simt_pass1_kernel<float><<<grid, threads, smem, st>>>(p, (const float*)Q, (const float*)K, (const float*)V,
-                                                          ws.part_m, ws.part_l, ws.part_O, ws.splits);
-  }
-  return cudaGetLastError();
+  return p.dtype == RESTKV_BF16 ? pass1<__nv_bfloat16>(p, ws, Q, K, V, st) : pass1<float>(p, ws, Q, K, V, st);
 }
 
 cudaError_t launch_combine(const Problem& p, const Workspace& ws, cudaStream_t st) {
-  dim3 grid(p.R, p.BH);
-  combine_kernel<<<grid, 128, 0, st>>>(p.R, p.d, ws.splits, ws.part_m, ws.part_l, ws.part_O, ws.fin_m, ws.fin_l,
-                                       ws.O_f32);
-  return cudaGetLastError();
+  return chain(combine_kernel, dim3(p.R, p.BH), 128, 0, st, p.R, p.d, ws.splits, ws.part_m, ws.part_l, ws.part_O, ws.fin_m,
+               ws.fin_l, ws.O_f32);
 }
 
 cudaError_t launch_simt_pass2(const Problem& p, const Workspace& ws, const void* Q, const void* K, const void* V,
                               float ema_decay, float* I_raw, cudaStream_t st) {
-  int GP = p.G < 4 ? p.G : 4;
-  const int threads = kP2Tile * GP;
-  size_t smem = ((size_t)2 * kP2Tile * (p.d + 1) + (size_t)GP * kP2Tile) * sizeof(float);
-  if (p.proj.M) smem += (size_t)GP * kP2Tile * (p.d + 1) * sizeof(float);
-  dim3 grid((p.n + kP2Tile - 1) / kP2Tile, p.BH);
-  cudaError_t e;
-  if (p.dtype == RESTKV_BF16) {
-    if ((e = allow_smem(simt_pass2_kernel<__nv_bfloat16>, smem)) != cudaSuccess) return e;
-    simt_pass2_kernel<__nv_bfloat16><<<grid, threads, smem, st>>>(
-        p, (const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, ws.fin_m, ws.fin_l, ws.O_f32,
-        ws.O_proj, ema_decay, ws.I_hat, I_raw, GP);
-  } else {
-    if ((e = allow_smem(simt_pass2_kernel<float>, smem)) != cudaSuccess) return e;
-    simt_pass2_kernel<float><<<grid, threads, smem, st>>>(p, (const float*)Q, (const float*)K, (const float*)V,
-                                                          ws.fin_m, ws.fin_l, ws.O_f32, ws.O_proj, ema_decay,
-                                                          ws.I_hat, I_raw, GP);
-  }
-  return cudaGetLastError();
+  return p.dtype == RESTKV_BF16 ? pass2<__nv_bfloat16>(p, ws, Q, K, V, ema_decay, I_raw, st)
+                                : pass2<float>(p, ws, Q, K, V, ema_decay, I_raw, st);
 }
 
 }  // namespace restkv
