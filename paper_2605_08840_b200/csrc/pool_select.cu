@@ -90,6 +90,18 @@ __device__ __forceinline__ void wait_copy(uint64_t* bar, uint32_t parity, unsign
     }
 }
 
+// The block's sum of v to *out, by way of one word per warp in shared memory.
+__device__ __forceinline__ void block_sum_out(unsigned long long v, unsigned long long* words, unsigned long long* out) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  __syncthreads();   // whatever the words held before has been read
+  if ((threadIdx.x & 31) == 0) words[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (unsigned int w = 1; w < blockDim.x / 32; ++w) v += words[w];
+  *out = v;
+}
+
 // Box means of rows [0, scored) of a slice from its staged taps (row jj: taps[jj .. jj + W - 1]), +inf for the rows from
 // there to cnt; f(jj, score) for each.  kW = 0: the width is known only at run time, pool_max: the maximum instead.
 template <int kThreads, int kW, typename F>
@@ -139,7 +151,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
   extern __shared__ __align__(16) unsigned int skeys[];   // [per rounded up to 4] keys (if held), then [room]
   float* const room = reinterpret_cast<float*>(skeys + (a.held ? (a.per + 3) & ~3 : 0));
   __shared__ __align__(16) unsigned int hist[2][kSelBins];   // double-buffered: peers read one while the other is prepared
-  __shared__ unsigned int tot[kSelBins];                     // the cluster's histogram
+  __shared__ __align__(16) unsigned int tot[kSelBins];                     // the cluster's histogram
   __shared__ unsigned int warp_a[32], warp_b[32];
   __shared__ unsigned int s_digit, s_remaining, s_count;
   __shared__ unsigned int s_min, s_max, s_gt, s_eq;          // s_gt, s_eq: totals of the CTAs before this one
@@ -334,6 +346,16 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
     if (range == 0u) { equal = kmin; above = 0xFFFFFFFFu; need_eq = remaining; }   // all keys alike
   }
 
+  if (a.index_sums && need_eq == 0u) {   // no ties at the threshold: the order does not matter
+    unsigned long long isum = 0ull;
+#pragma unroll 4
+    for (int i = lane; i < wlen; i += 32)
+      if (key_at(i) >= above) isum += (unsigned long long)(j0 + wbeg + i);
+    block_sum_out(isum, reinterpret_cast<unsigned long long*>(tot), a.index_sums + (long long)row * a.parts + part);
+    if (CS > 1) cluster.sync();   // shared memory stays alive until every peer has done with it
+    return;
+  }
+
   // ---- ordered emit: ascending indices, of equal keys the lower index ----
   unsigned int cgt = 0u, ceq = 0u;
 #pragma unroll 4
@@ -391,17 +413,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
       run_eq += __popc(meq);
     }
   }
-  if (a.index_sums) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) isum += __shfl_xor_sync(0xffffffffu, isum, off);
-    unsigned long long* sums = reinterpret_cast<unsigned long long*>(&hist[0][0]);   // its readers are done with it
-    if (lane == 0) sums[wid] = isum;
-    __syncthreads();
-    if (tid == 0) {
-      for (int w = 1; w < kWarps; ++w) isum += sums[w];
-      a.index_sums[(long long)row * a.parts + part] = isum;
-    }
-  }
+  if (a.index_sums) block_sum_out(isum, reinterpret_cast<unsigned long long*>(tot), a.index_sums + (long long)row * a.parts + part);
   if (!a.ga.K) {
     if (CS > 1) cluster.sync();   // shared memory stays alive until every peer has done with it
     return;
@@ -518,13 +530,13 @@ cudaError_t select_init(int* clusters_of) {
 }
 
 // CTAs of a row's cluster: as many as let all rows run at once (8 at most: smaller slices no longer shorten the chain of
-// synchronisations); more rows than SMs: as few as let three blocks of 512 threads share an SM's memory, so that one row's
+// synchronisations); more rows than SMs: as few as let two blocks of 512 threads share an SM's memory, so that one row's
 // loads run under another's passes.  1: no cluster.
 int select_cluster(int rows, int n_kv, const int* clusters_of) {
   int i = 3;
   while (i > 0 && (rows > clusters_of[i] || (n_kv >> i) < 256)) --i;
   if (rows > clusters_of[0])
-    while (i < 3 && (n_kv >> i) > 13000) ++i;
+    while (i < 3 && (n_kv >> i) > 22000) ++i;
   return 1 << i;
 }
 
