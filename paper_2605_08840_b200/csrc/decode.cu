@@ -6,6 +6,7 @@
 #include <mutex>
 
 #include "restkv_common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace restkv {
 
@@ -162,6 +163,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(
 // grid (Hq, batch); block d threads (rounded to a warp).  Merges the splits.
 __global__ void decode_combine_kernel(int Hq, int G, int d, int splits, const float* __restrict__ part,
                                       float* __restrict__ out, float* __restrict__ lse) {
+  ptx::grid_dependency_wait();
   const int hq = blockIdx.x, b = blockIdx.y;
   const int Hkv = Hq / G, h = hq / G, g = hq % G;
   const float* base = part + (((long long)b * Hkv + h) * splits) * G * (d + 2) + (long long)g * (d + 2);
@@ -240,8 +242,16 @@ cudaError_t launch_decode(const Problem& p, const void* q, const void* Kc, const
 cudaError_t launch_decode_combine(const Problem& p, const float* part, int splits, float* out, float* lse, cudaStream_t st) {
   const int threads = ((p.d + 31) / 32) * 32;
   dim3 grid(p.Hq, p.batch);
-  decode_combine_kernel<<<grid, threads, 0, st>>>(p.Hq, p.G, p.d, splits, part, out, lse);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};   // chained to the kernel that writes the partials
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned int)threads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, decode_combine_kernel, p.Hq, p.G, p.d, splits, part, out, lse);
 }
 
 }  // namespace restkv

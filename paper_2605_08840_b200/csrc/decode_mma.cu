@@ -97,6 +97,12 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
   if (lane == 0) {
     for (int s = 0; s < kDmStages; ++s) mbar_init(&full[warp][s], 1);
     fence_mbar_init();
+    prefetch_tensormap(&tmK);
+    prefetch_tensormap(&tmV);
+  }
+  grid_dependency_wait();   // nothing above touches what the kernel before may still write
+  grid_dependency_launch();
+  if (lane == 0) {
     for (int i = 0; i < mine && i < kDmStages; ++i) request(i);
   }
   // Q as the A operand: row = query head (zero past G), eight K = 16 steps
@@ -335,12 +341,14 @@ cudaError_t launch_decode_mma(void* state, const Problem& p, const void* q, cons
   cfg.blockDim = dim3(kDmThreads);
   cfg.dynamicSmemBytes = kDmSmem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned int)cluster;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return p.G > 8 ? launch_decode_mma_t<true>(&cfg, tmK, tmV, a) : launch_decode_mma_t<false>(&cfg, tmK, tmV, a);
 }
 
