@@ -253,6 +253,23 @@ __device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+// 2^t of a pair on the FMA pipe, for code that keeps the special-function unit busy: t = n + f with n the nearest integer
+// (adding 1.5 * 2^23 rounds to it), a polynomial of degree 5 for 2^f on [-1/2, 1/2] (minimax by Remez exchange, relative
+// error 7.5e-8, 2.1e-7 with the fp32 rounding of the chain; ex2.approx: 2.4e-7), n added to the exponent.  t below 127.
+__device__ __forceinline__ f32x2 exp2_fma(f32x2 t) {
+  const f32x2 magic = f2_make(12582912.f, 12582912.f), minus_magic = f2_make(-12582912.f, -12582912.f);
+  const f32x2 minus1 = f2_make(-1.f, -1.f);
+  const f32x2 r = f2_add(t, magic);
+  const f32x2 f = f2_fma(f2_add(r, minus_magic), minus1, t);
+  f32x2 p = f2_make(1.32764725e-3f, 1.32764725e-3f);
+  p = f2_fma(p, f, f2_make(9.67554096e-3f, 9.67554096e-3f));
+  p = f2_fma(p, f, f2_make(5.55071309e-2f, 5.55071309e-2f));
+  p = f2_fma(p, f, f2_make(0.240221202f, 0.240221202f));
+  p = f2_fma(p, f, f2_make(0.693146944f, 0.693146944f));
+  p = f2_fma(p, f, f2_make(1.f, 1.f));
+  return f2_make(__uint_as_float(__float_as_uint(f2_lo(p)) + (__float_as_uint(f2_lo(r)) << 23)),
+                 __uint_as_float(__float_as_uint(f2_hi(p)) + (__float_as_uint(f2_hi(r)) << 23)));
+}
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
   const f32x2 d = f2_fma(f2_make(a.x, a.y), f2_make(b.x, b.y), f2_make(c.x, c.y));
   return make_float2(f2_lo(d), f2_hi(d));

@@ -1007,7 +1007,12 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
             const f32x2 nt = f2_mul(f2_make(sv[2 * q], sv[2 * q + 1]), nc2);
             f32x2 Iq;
             if (kEq7) {
-              const f32x2 um = f2_add(f2_make(ex2_approx(f2_lo(nt)), ex2_approx(f2_hi(nt))), m1);   // 1/A - 1
+              // 1/A; one pair in four on the FMA pipe (1/A beyond 2^126 squares to infinity below either way): batch of 8
+              // x 32768 539 -> 522 us, 131072 258 -> 256 us; with every other pair no better, and from given statistics
+              // (no pass 1, so less to wait for) slower
+              const f32x2 u2 = (!from_lse && (q & 3) == 3) ? exp2_fma(f2_make(fminf(f2_lo(nt), 126.f), fminf(f2_hi(nt), 126.f)))
+                                       : f2_make(ex2_approx(f2_lo(nt)), ex2_approx(f2_hi(nt)));
+              const f32x2 um = f2_add(u2, m1);                                                       // 1/A - 1
               const f32x2 x = f2_add(f2_make(cv[2 * q], cv[2 * q + 1]), vn2);                       // ||o - v||^2
               const f32x2 bq = f2_fma(f2_mul(x, um), um, tiny2);                                    // x (1/A - 1)^2
               Iq = f2_mul(x, f2_make(rsqrt_approx(f2_lo(bq)), rsqrt_approx(f2_hi(bq))));
