@@ -52,18 +52,9 @@ cudaError_t launch_adaptive_params(const Problem& p, const Workspace& ws, int bu
   cudaError_t e = launch_select(rows, p.n, p.n, Bp, nullptr, nullptr, nullptr, 1, 0, false, ws.I_raw, nullptr, ws.adaptive_sums,
                                 nullptr, nullptr, nullptr, nullptr, nullptr, clusters_of, dev_status, true, st);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned int)p.BH);
-  cfg.blockDim = dim3(128);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   *n_launches = 2;
-  return cudaLaunchKernelEx(&cfg, window_params_kernel, p.G, p.w, Bp, select_cluster(rows, p.n, clusters_of), (double)beta,
-                            base_width, (const unsigned long long*)ws.adaptive_sums, ws.pool);
+  return launch_chained(window_params_kernel, dim3((unsigned int)p.BH), 128, 0, st, p.G, p.w, Bp, select_cluster(rows, p.n, clusters_of),
+                        (double)beta, base_width, ws.adaptive_sums, ws.pool);
 }
 
 }  // namespace restkv

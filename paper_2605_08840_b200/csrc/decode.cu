@@ -242,16 +242,7 @@ cudaError_t launch_decode(const Problem& p, const void* q, const void* Kc, const
 cudaError_t launch_decode_combine(const Problem& p, const float* part, int splits, float* out, float* lse, cudaStream_t st) {
   const int threads = ((p.d + 31) / 32) * 32;
   dim3 grid(p.Hq, p.batch);
-  cudaLaunchConfig_t cfg = {};   // chained to the kernel that writes the partials
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3((unsigned int)threads);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, decode_combine_kernel, p.Hq, p.G, p.d, splits, part, out, lse);
+  return launch_chained(decode_combine_kernel, grid, threads, 0, st, p.Hq, p.G, p.d, splits, part, out, lse);
 }
 
 }  // namespace restkv

@@ -31,6 +31,8 @@ __device__ __forceinline__ float box_mean(const float* __restrict__ src, int n, 
 // grid (ceil(n_kv/256), BH).  The window (W, gamma) comes from `pool` (per head, device) when it is non-null.
 __global__ void pool_kernel(int n, int n_kv, const float* __restrict__ I_hat, const int* __restrict__ pool, int W,
                             int gamma, bool pool_max, float* __restrict__ scores, int32_t* __restrict__ pool_used) {
+  ptx::grid_dependency_wait();
+  ptx::grid_dependency_launch();
   const int bh = blockIdx.y;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (pool) { W = pool[2 * bh]; gamma = pool[2 * bh + 1]; }
@@ -496,9 +498,8 @@ __global__ void compact_kernel(int Hkv, int n_kv, int n_sel, int row_chunks, lon
 cudaError_t launch_pool(const Problem& p, const Workspace& ws, const int* pool_dev, int W, int gamma, float* scores,
                         int32_t* pool_used, cudaStream_t st) {
   dim3 grid((p.n_kv + 255) / 256, p.BH);
-  pool_kernel<<<grid, 256, 0, st>>>(p.n, p.n_kv, ws.I_hat, pool_dev, W, gamma, p.spatial == RESTKV_SPATIAL_MAX, scores,
-                                    pool_used);
-  return cudaGetLastError();
+  return launch_chained(pool_kernel, grid, 256, 0, st, p.n, p.n_kv, ws.I_hat, pool_dev, W, gamma, p.spatial == RESTKV_SPATIAL_MAX,
+                        scores, pool_used);
 }
 
 namespace {

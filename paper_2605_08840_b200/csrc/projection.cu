@@ -5,6 +5,7 @@
 //     forms belongs to one and the same quadratic form.
 //   per call:  m_r = M o_r for the window rows (SIMT path; the tensor-core kernel does it in its merge).
 #include "restkv_common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace restkv {
 
@@ -132,6 +133,8 @@ __global__ void proj_factor_kernel(int d, const float* __restrict__ M, float* __
 __global__ void proj_rows_kernel(int Hkv, int G, int w, int R, int d, const float* __restrict__ M,
                                  const float* __restrict__ O, float* __restrict__ O_proj) {
   extern __shared__ float orow[];
+  ptx::grid_dependency_wait();
+  ptx::grid_dependency_launch();
   const int r = blockIdx.x, bh = blockIdx.y, i = threadIdx.x;
   const int hq = (bh % Hkv) * G + r / w;
   const float* Mh = M + (long long)hq * d * d;
@@ -180,8 +183,7 @@ cudaError_t launch_projection_prepare(int n_q_heads, int d, int d_model, restkv_
 }
 
 cudaError_t launch_projection_rows(const Problem& p, const float* O, float* O_proj, cudaStream_t st) {
-  proj_rows_kernel<<<dim3(p.R, p.BH), p.d, p.d * sizeof(float), st>>>(p.Hkv, p.G, p.w, p.R, p.d, p.proj.M, O, O_proj);
-  return cudaGetLastError();
+  return launch_chained(proj_rows_kernel, dim3(p.R, p.BH), p.d, p.d * sizeof(float), st, p.Hkv, p.G, p.w, p.R, p.d, p.proj.M, O, O_proj);
 }
 
 }  // namespace restkv

@@ -1293,6 +1293,8 @@ __global__ void from_lse_prep_kernel(int rows, float scale, const float* __restr
                                      float* __restrict__ row_M2, const float* __restrict__ proj_Mt,
                                      float* __restrict__ O_proj, int Hkv, int w) {
   __shared__ float xs[8][kHeadDim];
+  grid_dependency_wait();
+  grid_dependency_launch();
   const int wi = threadIdx.x >> 5;
   const int ri = blockIdx.x * (blockDim.x >> 5) + wi, lane = threadIdx.x & 31;
   if (ri >= rows) return;
@@ -1338,6 +1340,8 @@ __global__ void from_lse_prep_kernel(int rows, float scale, const float* __restr
 // SIMT kernels: A = exp(s * scale - fin_m) / fin_l with fin_m = LSE and fin_l = 1.
 __global__ void from_lse_prep_simt_kernel(int rows, const float* __restrict__ LSE, float* __restrict__ fin_m,
                                           float* __restrict__ fin_l) {
+  grid_dependency_wait();
+  grid_dependency_launch();
   const int ri = blockIdx.x * blockDim.x + threadIdx.x;
   if (ri >= rows) return;
   fin_m[ri] = LSE[ri];
@@ -1371,11 +1375,9 @@ cudaError_t launch_from_lse_prep(const Problem& p, const Workspace& ws, const fl
                                  bool tensor_core, cudaStream_t st) {
   const int rows = p.BH * p.R;
   if (tensor_core)
-    from_lse_prep_kernel<<<(rows + 7) / 8, 256, 0, st>>>(rows, p.scale, O, LSE, ws.O_m2, ws.aug, ws.row_M2, p.proj.Mt,
-                                                         ws.O_proj, p.Hkv, p.w);
-  else
-    from_lse_prep_simt_kernel<<<(rows + 255) / 256, 256, 0, st>>>(rows, LSE, ws.fin_m, ws.fin_l);
-  return cudaGetLastError();
+    return launch_chained(from_lse_prep_kernel, dim3((rows + 7) / 8), 256, 0, st, rows, p.scale, O, LSE, ws.O_m2, ws.aug, ws.row_M2,
+                          p.proj.Mt, ws.O_proj, p.Hkv, p.w);
+  return launch_chained(from_lse_prep_simt_kernel, dim3((rows + 255) / 256), 256, 0, st, rows, LSE, ws.fin_m, ws.fin_l);
 }
 
 bool tc_supported(const Problem& p) {
@@ -1515,20 +1517,12 @@ cudaError_t launch_tc_fused(void* state, const Problem& p, const Workspace& ws, 
   a.wait_limit = wait_limit;
   a.I_raw = O_given ? nullptr : I_raw;
   if (O_given) a.O_f32 = const_cast<float*>(O_given);   // read only in this mode
-  const dim3 grid(a.groups * a.cpg), block(kFThreads);
+  const dim3 grid(a.groups * a.cpg);
   FusedKernel kernel = attention_only ? pick_fused(32, false, 0) : pick_fused(p.w, a.from_lse != 0, a.proj_Mt ? 3 : p.indicator);
   if (!kernel) return cudaErrorInvalidValue;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = kFSmem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, tmQ, tmK, tmV, tmO, tmAug, a);
+  if (chained) return launch_chained(kernel, grid, kFThreads, kFSmem, st, tmQ, tmK, tmV, tmO, tmAug, a);
+  kernel<<<grid, kFThreads, kFSmem, st>>>(tmQ, tmK, tmV, tmO, tmAug, a);
+  return cudaGetLastError();
 }
 
 }  // namespace restkv

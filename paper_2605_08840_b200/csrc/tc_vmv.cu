@@ -50,7 +50,10 @@ vmv_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUte
   const long long per = (total + gridDim.x - 1) / gridDim.x;
   const long long first = (long long)blockIdx.x * per;
   const int cnt = (int)max(0ll, min(total, first + per) - first);
-  if (cnt == 0) return;   // uniform over the CTA
+  if (cnt == 0) {   // uniform over the CTA
+    grid_dependency_wait();
+    return;
+  }
 
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* gen_base = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -86,6 +89,8 @@ vmv_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUte
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
+  grid_dependency_wait();
+  grid_dependency_launch();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -238,8 +243,7 @@ cudaError_t launch_tc_vmv(void* state, const Problem& p, const void* V, float* o
   a.out = out; a.dev_status = dev_status; a.wait_limit = wait_limit;
   const long long total = (long long)a.BH * a.tiles;
   const int grid = (int)(total < sm_count ? total : sm_count);
-  vmv_kernel<<<grid, kVThreads, kVSmem, st>>>(tmV, tmLT, a);
-  return cudaGetLastError();
+  return launch_chained(vmv_kernel, dim3(grid), kVThreads, kVSmem, st, tmV, tmLT, a);
 }
 
 }  // namespace restkv
