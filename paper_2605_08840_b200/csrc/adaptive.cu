@@ -8,16 +8,208 @@ namespace restkv {
 
 namespace {
 
-// grid BH, block 128: the index sums of the head's w * G rows (front and rear half of the window apart), `parts` values per
-// row, and from them the head's window.
-__global__ void window_params_kernel(int G, int w, int Bp, int parts, double beta, int base_width,
-                                     const unsigned long long* __restrict__ sums, int* __restrict__ pool) {
+constexpr int kRsThreads = 1024;
+constexpr int kRsBins = 2048;        // 11-bit digits
+constexpr int kRsList = 1024;        // keys of the last digit that are ranked one by one
+constexpr int kRsMaxSmem = 200 * 1024;
+
+// Sum of the indices of the Bp largest of each row's n values (ties to the lower index), all rows of the raw indicator.
+// What bounds it: the rows come once from HBM or L2; against that stand three walks over a row's keys in shared memory.
+// So one persistent block per SM, the next row on its way by bulk copy while this one is worked on (two buffers; one for
+// rows past 100 KB; longer rows are read again on every walk), and no more than the walks that are needed: the extremes,
+// a histogram of 11-bit digits of the offsets from the smallest (about a thousand bins in use, so one histogram serves all
+// warps without contention), then the sum above the digit that holds the Bp-th largest while that digit's few keys are
+// listed and ranked, a key per warp.  1024 rows of 20011: 62 us as selections in two blocks of 512 threads per SM, 47 us so
+// (10 k cycles per row: 0.8 k extremes, 3 k histogram, 2.6 k the last walk, the rest synchronisation).
+template <bool kHeld>   // false: no buffers, the keys are read from global memory on every walk
+__global__ void __launch_bounds__(kRsThreads, 1)
+row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buffers, unsigned long long* __restrict__ sums,
+                unsigned int* dev_status) {
+  extern __shared__ __align__(16) uint4 rs_buf[];   // `buffers` rows of quads + 1
+  __shared__ __align__(16) unsigned int hist[kRsBins];
+  __shared__ unsigned int list_v[kRsList], list_i[kRsList];
+  __shared__ unsigned int warp_a[32], warp_b[32];
+  __shared__ unsigned long long warp_s[32];
+  __shared__ unsigned int s_digit, s_rest, s_count, s_listed;
+  __shared__ __align__(8) uint64_t bar[2];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int room = (n + 3) / 4 + 1;   // quads of a row, wherever it begins within one
+  if (tid == 0) {
+    ptx::mbar_init(&bar[0], 1);
+    ptx::mbar_init(&bar[1], 1);
+    ptx::fence_mbar_init();
+  }
+  for (int b = tid; b < kRsBins; b += kRsThreads) hist[b] = 0u;
+  __syncthreads();
   ptx::grid_dependency_wait();
+  ptx::grid_dependency_launch();
+  // A row begins `mis` floats behind a 16-byte boundary; the copy takes whole quads (inside the workspace on both sides).
+  auto request = [&](int row, int it) {
+    const int b = it % buffers;
+    const long long at = (long long)row * n;
+    const int mis = (int)(at & 3);
+    const uint32_t bytes = (uint32_t)((mis + n + 3) / 4) * 16u;
+    ptx::mbar_arrive_expect_tx(&bar[b], bytes);
+    ptx::bulk_load(rs_buf + (size_t)b * room, src + at - mis, bytes, &bar[b]);
+  };
+  if (kHeld && tid == 0)
+    for (int it = 0; it < buffers; ++it)
+      if ((int)blockIdx.x + it * (int)gridDim.x < rows) request(blockIdx.x + it * gridDim.x, it);
+  int it = 0;
+  for (int row = blockIdx.x; row < rows; row += gridDim.x, ++it) {
+    const long long at = (long long)row * n;
+    const int mis = (int)(at & 3), quads = (mis + n + 3) / 4;
+    const uint4* quad = kHeld ? rs_buf + (size_t)(it % buffers) * room : reinterpret_cast<const uint4*>(src + at - mis);
+    if (kHeld) {
+      const int b = it % buffers;
+      const long long t0 = clock64();
+      while (!ptx::mbar_try_wait(&bar[b], (uint32_t)(it / buffers) & 1u))
+        if (clock64() - t0 > 4000000000ll) {
+          atomicOr(dev_status, (unsigned int)kDevTimeout);
+          break;
+        }
+    }
+    // f(index, key) for this thread's share of the row: whole quads of the row, then the few keys at its two ends.  The
+    // indicators are not negative, so that their bits are keys as they are.
+    const unsigned int* words = reinterpret_cast<const unsigned int*>(quad);
+    const int q0 = mis ? 1 : 0, q1 = (mis + n) / 4, head = mis ? 4 - mis : 0, tail = q1 >= q0 ? mis + n - 4 * q1 : 0;
+    const int ends = q1 >= q0 ? head + tail : n;   // (a row inside a single quad: all of it)
+    auto each = [&](auto&& f) {
+#pragma unroll 2
+      for (int q = q0 + tid; q < q1; q += kRsThreads) {
+        const uint4 k4 = quad[q];
+        const unsigned int i = (unsigned int)(4 * q - mis);
+        f(i, k4.x);
+        f(i + 1, k4.y);
+        f(i + 2, k4.z);
+        f(i + 3, k4.w);
+      }
+      if (tid < ends) {
+        const int i = tid < head || q1 < q0 ? tid : n - tail + (tid - head);
+        f((unsigned int)i, words[mis + i]);
+      }
+    };
+    // ---- extremes ----
+    unsigned int kmin = 0xFFFFFFFFu, kmax = 0u;
+    each([&](unsigned int, unsigned int key) {
+      kmin = min(kmin, key);
+      kmax = max(kmax, key);
+    });
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) { warp_a[wid] = kmin; warp_b[wid] = kmax; }
+    if (tid == 0) s_listed = 0u;
+    __syncthreads();
+    kmin = __reduce_min_sync(0xffffffffu, warp_a[lane]);
+    kmax = __reduce_max_sync(0xffffffffu, warp_b[lane]);
+    // ---- digits from the top, until the digit's keys fit the list ----
+    int hi = 32 - __clz((int)(kmax - kmin)), lo = hi;   // bits [hi - 1 .. 0] of the offsets vary
+    unsigned int prefix = 0u, rest = (unsigned int)Bp, listed = (unsigned int)n;
+#pragma unroll 1
+    while (lo > 0 && (listed > kRsList || lo == hi)) {
+      const int top = lo;
+      lo = top > 11 ? top - 11 : 0;
+      if (top == hi) each([&](unsigned int, unsigned int key) { atomicAdd(&hist[(key - kmin) >> lo], 1u); });
+      else each([&](unsigned int, unsigned int key) {
+        const unsigned int v = key - kmin;
+        if ((v >> top) == (prefix >> top)) atomicAdd(&hist[(v >> lo) & (kRsBins - 1)], 1u);
+      });
+      __syncthreads();
+      const int first = kRsBins - 2 * (tid + 1);   // this thread's two bins, walked from the top
+      const uint2 own = *reinterpret_cast<const uint2*>(&hist[first]);
+      const unsigned int sum = own.x + own.y;
+      unsigned int incl = sum;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const unsigned int t = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += t;
+      }
+      if (lane == 31) warp_a[wid] = incl;
+      *reinterpret_cast<uint2*>(&hist[first]) = make_uint2(0u, 0u);   // ready for the next time
+      __syncthreads();
+      const unsigned int acc = __reduce_add_sync(0xffffffffu, lane < wid ? warp_a[lane] : 0u) + incl - sum;
+      if (acc < rest && rest <= acc + sum) {   // exactly one thread
+        const bool upper = rest <= acc + own.y;
+        s_digit = (unsigned int)(first + (upper ? 1 : 0));
+        s_rest = rest - acc - (upper ? 0u : own.y);
+        s_count = upper ? own.y : own.x;
+      }
+      __syncthreads();
+      prefix |= s_digit << lo;
+      rest = s_rest;
+      listed = s_count;
+    }
+    // ---- the sum above the digit; the digit's keys [k0, k1] listed (or, more equal keys than the list takes, counted) ----
+    const unsigned int k0 = kmin + prefix, k1 = k0 + ((lo < 32 ? 1u << lo : 0u) - 1u);
+    const bool ties = listed > kRsList;
+    unsigned long long isum = 0ull;
+    each([&](unsigned int i, unsigned int key) {
+      if (key > k1) {
+        isum += i;
+      } else if (key >= k0 && !ties) {
+        const unsigned int slot = atomicAdd(&s_listed, 1u);
+        list_v[slot] = key;
+        list_i[slot] = i;
+      }
+    });
+    __syncthreads();   // the row has been walked for the last time (but for ties), the list is complete
+    if (!ties) {
+      if (kHeld && tid == kRsThreads - 1 && row + (long long)buffers * gridDim.x < rows) request(row + buffers * gridDim.x, it + buffers);
+      // a listed key per warp: the lanes count the keys that come before it
+      for (unsigned int t = wid; t < listed; t += kRsThreads / 32) {
+        const unsigned int v = list_v[t], i = list_i[t];
+        unsigned int before = 0u;
+        for (unsigned int u0 = 0; u0 < listed; u0 += 32) {
+          const unsigned int u = u0 + lane;
+          const unsigned int ov = u < listed ? list_v[u] : 0u, oi = u < listed ? list_i[u] : 0xFFFFFFFFu;
+          before += __popc(__ballot_sync(0xffffffffu, (ov > v) | ((ov == v) & (oi < i))));
+        }
+        if (lane == 0 && before < rest) isum += i;
+      }
+    } else {
+      // more equal keys than the list takes: the first `rest` of them, counted in order (a warp owns a run of the row)
+      const int cw = ((quads * 4 + 31) / 32 + 31) & ~31, wbeg = wid * cw;
+      const unsigned int* keys = reinterpret_cast<const unsigned int*>(quad) + mis;
+      unsigned int eq = 0u;
+      for (int i = wbeg + lane; i < min(n, wbeg + cw); i += 32) eq += keys[i] == k0;
+      eq = __reduce_add_sync(0xffffffffu, eq);
+      if (lane == 0) warp_a[wid] = eq;
+      __syncthreads();
+      unsigned int run = __reduce_add_sync(0xffffffffu, lane < wid ? warp_a[lane] : 0u);
+      for (int i0 = wbeg; i0 < min(n, wbeg + cw); i0 += 32) {
+        const int i = i0 + lane;
+        const bool is = i < min(n, wbeg + cw) && keys[i] == k0;
+        const unsigned int m = __ballot_sync(0xffffffffu, is);
+        if (is && run + __popc(m & ((1u << lane) - 1u)) < rest) isum += (unsigned int)i;
+        run += __popc(m);
+      }
+      __syncthreads();
+      if (kHeld && tid == kRsThreads - 1 && row + (long long)buffers * gridDim.x < rows) request(row + buffers * gridDim.x, it + buffers);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) isum += __shfl_xor_sync(0xffffffffu, isum, off);
+    if (lane == 0) warp_s[wid] = isum;
+    __syncthreads();
+    if (wid == 0) {
+      isum = warp_s[lane];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) isum += __shfl_xor_sync(0xffffffffu, isum, off);
+      if (lane == 0) sums[row] = isum;
+    }
+  }
+}
+
+// grid BH, block 128: the index sums of the head's w * G rows (front and rear half of the window apart) and from them the
+// head's window.
+__global__ void window_params_kernel(int G, int w, int Bp, double beta, int base_width, const unsigned long long* __restrict__ sums,
+                                     int* __restrict__ pool) {
+  ptx::grid_dependency_wait();
+  ptx::grid_dependency_launch();
   const int bh = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   unsigned long long front = 0, rear = 0;
-  for (int e = threadIdx.x; e < G * w * parts; e += blockDim.x) {
-    const unsigned long long s = sums[(long long)bh * G * w * parts + e];
-    if ((e / parts) % w < w / 2) front += s;
+  for (int e = threadIdx.x; e < G * w; e += blockDim.x) {
+    const unsigned long long s = sums[(long long)bh * G * w + e];
+    if (e % w < w / 2) front += s;
     else rear += s;
   }
 #pragma unroll
@@ -43,18 +235,23 @@ __global__ void window_params_kernel(int G, int w, int Bp, int parts, double bet
 
 }  // namespace
 
-cudaError_t launch_adaptive_params(const Problem& p, const Workspace& ws, int budget, float beta, int base_width,
-                                   const int* clusters_of, unsigned int* dev_status, cudaStream_t st, int* n_launches) {
+cudaError_t adaptive_init() {
+  return cudaFuncSetAttribute(row_sums_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsMaxSmem);
+}
+
+cudaError_t launch_adaptive_params(const Problem& p, const Workspace& ws, int budget, float beta, int base_width, int sm_count,
+                                   unsigned int* dev_status, cudaStream_t st, int* n_launches) {
   int Bp = budget - p.tail;
   if (Bp > p.n) Bp = p.n;
   const int rows = p.batch * p.Hq * p.w;
-  *n_launches = 0;
-  cudaError_t e = launch_select(rows, p.n, p.n, Bp, nullptr, nullptr, nullptr, 1, 0, false, ws.I_raw, nullptr, ws.adaptive_sums,
-                                nullptr, nullptr, nullptr, nullptr, nullptr, clusters_of, dev_status, true, st);
-  if (e != cudaSuccess) return e;
+  const size_t room = ((size_t)(p.n + 3) / 4 + 1) * 16;
+  const int buffers = 2 * room <= (size_t)kRsMaxSmem ? 2 : room <= (size_t)kRsMaxSmem ? 1 : 0;
   *n_launches = 2;
-  return launch_chained(window_params_kernel, dim3((unsigned int)p.BH), 128, 0, st, p.G, p.w, Bp, select_cluster(rows, p.n, clusters_of),
-                        (double)beta, base_width, ws.adaptive_sums, ws.pool);
+  const cudaError_t e = launch_chained(buffers ? row_sums_kernel<true> : row_sums_kernel<false>, dim3((unsigned int)(rows < sm_count ? rows : sm_count)), kRsThreads,
+                                       buffers * room, st, rows, p.n, Bp, ws.I_raw, buffers, ws.adaptive_sums, dev_status);
+  if (e != cudaSuccess) return e;
+  return launch_chained(window_params_kernel, dim3((unsigned int)p.BH), 128, 0, st, p.G, p.w, Bp, (double)beta, base_width,
+                        ws.adaptive_sums, ws.pool);
 }
 
 }  // namespace restkv

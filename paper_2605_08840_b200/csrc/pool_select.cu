@@ -42,11 +42,7 @@ __global__ void pool_kernel(int n, int n_kv, const float* __restrict__ I_hat, co
 }
 
 // ------------------------------------------------------------------------------------------------
-// Radix select.  Scores map to unsigned keys whose order matches the float order.
-__device__ __forceinline__ unsigned int float_key(float x) {
-  const unsigned int u = __float_as_uint(x);
-  return u ^ ((unsigned int)((int)u >> 31) | 0x80000000u);
-}
+// Radix select.
 
 // Optional gather fused into the select kernel (all pointers null: indices only).  K, V addressed by element strides;
 // K_out, V_out [rows, keep, row_chunks * 16 bytes] contiguous.
@@ -67,7 +63,6 @@ struct SelectArgs {
   int W, gamma, pool_max;
   float* scores;
   int32_t* indices;
-  unsigned long long* index_sums;   // non-null: the sum of each row's kept indices instead of the indices
   int parts;                    // blocks per row: the cluster's, or (no cluster) blocks that each select from the whole row
   int per;                      // keys of one block's slice
   int held;                     // 1: the slice's keys stay in shared memory; 0: they are formed again from the scores
@@ -90,18 +85,6 @@ __device__ __forceinline__ void wait_copy(uint64_t* bar, uint32_t parity, unsign
       atomicOr(dev_status, (unsigned int)kDevTimeout);
       return;
     }
-}
-
-// The block's sum of v to *out, by way of one word per warp in shared memory.
-__device__ __forceinline__ void block_sum_out(unsigned long long v, unsigned long long* words, unsigned long long* out) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  __syncthreads();   // whatever the words held before has been read
-  if ((threadIdx.x & 31) == 0) words[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  for (unsigned int w = 1; w < blockDim.x / 32; ++w) v += words[w];
-  *out = v;
 }
 
 // Box means of rows [0, scored) of a slice from its staged taps (row jj: taps[jj .. jj + W - 1]), +inf for the rows from
@@ -178,7 +161,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
   const long long j0 = (long long)rank * a.per;
   const int cnt = (int)max(0ll, min((long long)n_kv, j0 + a.per) - j0);
   float* srow = a.scores + (long long)row * n_kv + j0;
-  int32_t* dst = a.index_sums ? nullptr : a.indices + (long long)row * a.keep;
+  int32_t* dst = a.indices + (long long)row * a.keep;
   int keep = a.keep;
   if (a.keep_rows) {
     keep = min(max(a.keep_rows[row], 1), a.keep);
@@ -348,16 +331,6 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
     if (range == 0u) { equal = kmin; above = 0xFFFFFFFFu; need_eq = remaining; }   // all keys alike
   }
 
-  if (a.index_sums && need_eq == 0u) {   // no ties at the threshold: the order does not matter
-    unsigned long long isum = 0ull;
-#pragma unroll 4
-    for (int i = lane; i < wlen; i += 32)
-      if (key_at(i) >= above) isum += (unsigned long long)(j0 + wbeg + i);
-    block_sum_out(isum, reinterpret_cast<unsigned long long*>(tot), a.index_sums + (long long)row * a.parts + part);
-    if (CS > 1) cluster.sync();   // shared memory stays alive until every peer has done with it
-    return;
-  }
-
   // ---- ordered emit: ascending indices, of equal keys the lower index ----
   unsigned int cgt = 0u, ceq = 0u;
 #pragma unroll 4
@@ -389,7 +362,6 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
   const bool own_idx = a.own_idx != 0;
   int32_t* const s_idx = reinterpret_cast<int32_t*>(room);
   const unsigned int lt_mask = (1u << lane) - 1u;
-  unsigned long long isum = 0ull;
 #pragma unroll 2
   for (int i0 = 0; i0 < wlen; i0 += 32) {
     const int i = i0 + lane;
@@ -401,8 +373,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
       if (gt || (eq && eq_before < need_eq)) {
         const unsigned int pos = gt_before + min(eq_before, need_eq);
         const int j = (int)j0 + wbeg + i;
-        if (a.index_sums) isum += (unsigned long long)j;
-        else if (!own_idx) {
+        if (!own_idx) {
           if (pos < (unsigned int)keep && (CS > 1 || (pos >= first && pos < last))) dst[pos] = j;
         } else if (CS == 1) {
           if (pos >= first && pos < last) s_idx[pos - first] = j;
@@ -415,7 +386,6 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
       run_eq += __popc(meq);
     }
   }
-  if (a.index_sums) block_sum_out(isum, reinterpret_cast<unsigned long long*>(tot), a.index_sums + (long long)row * a.parts + part);
   if (!a.ga.K) {
     if (CS > 1) cluster.sync();   // shared memory stays alive until every peer has done with it
     return;
@@ -533,7 +503,7 @@ cudaError_t select_init(int* clusters_of) {
 // CTAs of a row's cluster: as many as let all rows run at once (8 at most: smaller slices no longer shorten the chain of
 // synchronisations); more rows than SMs: as few as let two blocks of 512 threads share an SM's memory, so that one row's
 // loads run under another's passes.  1: no cluster.
-int select_cluster(int rows, int n_kv, const int* clusters_of) {
+static int select_cluster(int rows, int n_kv, const int* clusters_of) {
   int i = 3;
   while (i > 0 && (rows > clusters_of[i] || (n_kv >> i) < 256)) --i;
   if (rows > clusters_of[0])
@@ -545,13 +515,11 @@ int select_cluster(int rows, int n_kv, const int* clusters_of) {
 // block of 1024 threads forms 8 keys per thread in about the time that the cluster's four barriers take.
 constexpr int kSelLocalRows = 8192;
 
-// rows x n_kv scores -> rows x min(budget, n_kv) indices (or, with index_sums, the sums of those indices: one value per
-// CTA of the row's cluster, select_cluster of them).  I_hat non-null: pool first (n scored rows per row of I_hat, window
+// rows x n_kv scores -> rows x min(budget, n_kv) indices.  I_hat non-null: pool first (n scored rows per row of I_hat, window
 // from pool_dev or (W, gamma)) and write the pooled scores.  chained: the launch may overlap the end of the kernel
 // before it in the stream (it waits for that kernel's results itself).
 cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep_rows, const float* I_hat, const int* pool_dev,
-                          int W, int gamma, bool pool_max, float* scores, int32_t* indices, unsigned long long* index_sums,
-                          const Problem* gather, const void* K, const void* V, void* K_out, void* V_out,
+                          int W, int gamma, bool pool_max, float* scores, int32_t* indices, const Problem* gather, const void* K, const void* V, void* K_out, void* V_out,
                           const int* clusters_of, unsigned int* dev_status, bool chained, cudaStream_t st) {
   SelectArgs a{};
   a.dev_status = dev_status;
@@ -564,7 +532,7 @@ cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep
   }
   a.n = n; a.n_kv = n_kv; a.keep = budget < n_kv ? budget : n_kv; a.keep_rows = keep_rows;
   a.I_hat = I_hat; a.pool = pool_dev; a.W = W; a.gamma = gamma; a.pool_max = pool_max ? 1 : 0;
-  a.scores = scores; a.indices = indices; a.index_sums = index_sums;
+  a.scores = scores; a.indices = indices;
   int CS = select_cluster(rows, n_kv, clusters_of);
   a.parts = CS;
   if (I_hat && gather && n_kv <= kSelLocalRows && rows <= clusters_of[0]) {

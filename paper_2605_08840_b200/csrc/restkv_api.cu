@@ -81,7 +81,7 @@ size_t plan_workspace(const Problem& p, int budget, int sm_count, bool adaptive,
   w.dec_part = (float*)take(BH * (size_t)kDecodeMaxSplits * p.G * (d + 2) * sizeof(float));
   if (adaptive) {
     w.I_raw = (float*)take((size_t)p.batch * p.Hq * p.w * p.n * sizeof(float));
-    w.adaptive_sums = (unsigned long long*)take((size_t)p.batch * p.Hq * p.w * 8 * sizeof(unsigned long long));
+    w.adaptive_sums = (unsigned long long*)take((size_t)p.batch * p.Hq * p.w * sizeof(unsigned long long));
   }
   w.bytes = off;
   if (ws) *ws = w;
@@ -262,7 +262,7 @@ static restkv_status run_score(Call& c, const Problem& p, const Workspace& ws, c
   }
   if (adaptive) {
     int nl = 0;
-    cudaError_t e = launch_adaptive_params(p, ws, pool->budget, pool->beta, pool->base_width, c.h->select_clusters, c.h->dev_status, c.st, &nl);
+    cudaError_t e = launch_adaptive_params(p, ws, pool->budget, pool->beta, pool->base_width, c.h->sm_count, c.h->dev_status, c.st, &nl);
     if (e != cudaSuccess) return c.fail(e);
     c.h->launches += nl;
   }
@@ -299,6 +299,7 @@ restkv_status restkv_create(restkv_handle** out) {
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->dev_status, (kDevStatusWords + kDevCounterWords) * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(h->dev_status, 0, (kDevStatusWords + kDevCounterWords) * sizeof(unsigned int));
   if (e == cudaSuccess) e = select_init(h->select_clusters);
+  if (e == cudaSuccess) e = adaptive_init();
   if (e != cudaSuccess) { delete h; return RESTKV_ERR_CUDA; }
   h->tc_state = nullptr;
   if (tc_init(&h->tc_state) != cudaSuccess || tc_fused_init() != cudaSuccess ||
@@ -398,7 +399,7 @@ restkv_status restkv_select(restkv_handle* h, const restkv_shape* shape, const f
   if ((s = check_ws(p, budget, h->sm_count, false, workspace, workspace_bytes, &ws)) != RESTKV_OK) return s;
   Call c{h, (cudaStream_t)stream};
   RESTKV_LAUNCH(c, RESTKV_KERNEL_SELECT,
-                launch_select(p.BH, p.n, p.n_kv, budget, nullptr, nullptr, nullptr, 1, 0, false, const_cast<float*>(scores), indices, nullptr,
+                launch_select(p.BH, p.n, p.n_kv, budget, nullptr, nullptr, nullptr, 1, 0, false, const_cast<float*>(scores), indices,
                               nullptr, nullptr, nullptr, nullptr, nullptr, h->select_clusters, h->dev_status, true, c.st), 1);
   return RESTKV_OK;
 }
@@ -446,7 +447,7 @@ static restkv_status evict_impl(restkv_handle* h, const restkv_shape* shape, con
   h->last_evict_fused = on_tc && !adaptive && !budgets && h->fused_select;
   RESTKV_LAUNCH(c, RESTKV_KERNEL_SELECT,
                 launch_select(p.BH, p.n, p.n_kv, budget, budgets, ws.I_hat, adaptive ? ws.pool : nullptr, pool->width,
-                              pool->shift, p.spatial == RESTKV_SPATIAL_MAX, scores, indices, nullptr, &p, K, V, K_out, V_out,
+                              pool->shift, p.spatial == RESTKV_SPATIAL_MAX, scores, indices, &p, K, V, K_out, V_out,
                               h->select_clusters, h->dev_status, h->fused_select, c.st), 1);
   return RESTKV_OK;
 }

@@ -57,7 +57,7 @@ struct Workspace {
   int* pool;              // [BH, 2] (W, gamma)
   float* dec_part;        // decode partials
   float* I_raw;           // adaptive only: [batch, Hq, w, n]
-  unsigned long long* adaptive_sums;  // adaptive only: [batch*Hq*w, 8] index sums of the per-query top-B_p, a value per CTA of a row
+  unsigned long long* adaptive_sums;  // adaptive only: [batch*Hq*w] index sums of the per-query top-B_p
   size_t bytes;
 };
 
@@ -78,10 +78,8 @@ cudaError_t launch_simt_pass2(const Problem& p, const Workspace& ws, const void*
 cudaError_t launch_pool(const Problem& p, const Workspace& ws, const int* pool_dev, int W, int gamma, float* scores,
                         int32_t* pool_used, cudaStream_t st);
 cudaError_t select_init(int* clusters_of);   // [4]
-int select_cluster(int rows, int n_kv, const int* clusters_of);
 cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep_rows, const float* I_hat, const int* pool_dev,
-                          int W, int gamma, bool pool_max, float* scores, int32_t* indices, unsigned long long* index_sums,
-                          const Problem* gather, const void* K, const void* V, void* K_out, void* V_out,
+                          int W, int gamma, bool pool_max, float* scores, int32_t* indices, const Problem* gather, const void* K, const void* V, void* K_out, void* V_out,
                           const int* clusters_of, unsigned int* dev_status, bool chained, cudaStream_t st);
 cudaError_t launch_compact(const Problem& p, const void* K, const void* V, const int32_t* indices, int n_sel,
                            void* K_out, void* V_out, unsigned int* dev_status, cudaStream_t st);
@@ -96,7 +94,8 @@ cudaError_t launch_decode_mma(void* state, const Problem& p, const void* q, cons
                               float* out, float* lse, float* part, int cluster, int splits, long long wait_limit,
                               unsigned int* dev_status, cudaStream_t st);
 cudaError_t launch_adaptive_params(const Problem& p, const Workspace& ws, int budget, float beta, int base_width,
-                                   const int* clusters_of, unsigned int* dev_status, cudaStream_t st, int* n_launches);
+                                   int sm_count, unsigned int* dev_status, cudaStream_t st, int* n_launches);
+cudaError_t adaptive_init();
 
 // Output projection (Eq. 4): the caller-owned factor buffer and the per-call projected rows.
 size_t projection_factor_bytes(int n_q_heads, int d);
@@ -143,6 +142,12 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, int threa
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// Scores map to unsigned keys whose order matches the float order.
+__device__ __forceinline__ unsigned int float_key(float x) {
+  const unsigned int u = __float_as_uint(x);
+  return u ^ ((unsigned int)((int)u >> 31) | 0x80000000u);
 }
 
 // ---- small device helpers ------------------------------------------------------------------------

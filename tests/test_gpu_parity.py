@@ -424,6 +424,31 @@ def test_selection_kernel_edges(handle, spec):
     full_check(handle, inp)
 
 
+@pytest.mark.parametrize("spec", [(3, 2), (7, 3), (1023, 40), (4099, 4098), (25001, 900), (26000, 900), (51300, 2000)])
+@pytest.mark.parametrize("ties", [False, True])
+def test_adaptive_window_row_lengths(handle, spec, ties):
+    """The index sums behind the adaptive window: rows that begin anywhere within 16 bytes, of a few keys, with two, one and
+    no buffers in shared memory; with all keys of a row equal (the first B_p of them count)."""
+    n, budget = spec
+    inp = make_inputs(Case("adapt", 1, 4, 2, 16, n, 6, budget, 1, 0, 0.5, "f32", 0, "normal", n))
+    if ties:
+        inp.K[...] = inp.K[:, :, :1]
+        inp.V[...] = inp.V[:, :, :1] * np.where(np.arange(n) % 2, 1.0, -1.0).astype(np.float32)[:, None]
+    probe = oracle_scores(inp, pool_mode=1, beta=1e9, base_width=1, budget=budget)
+    delta = np.abs(probe.D[..., 0] - probe.D[..., 1])
+    if not ties and n > 4100:
+        assert delta.min() > 0
+    beta = float(delta.max() / 20.5) if delta.max() > 0 else 1.0     # the mean indices enter with a twentieth of their difference
+    ref = oracle_scores(inp, pool_mode=1, beta=beta, base_width=1, budget=budget)
+    x = (probe.D[..., 0] - probe.D[..., 1]) / beta
+    settled = np.abs(x - np.round(x)) > 0.02
+    run = DeviceRun(handle, inp, adaptive_budget=budget)
+    run.score(pool=rk.adaptive_pool(beta, 1, budget))
+    assert handle.poll_status() == rk.RESTKV_OK
+    if not ties:                                                      # (equal in exact arithmetic only: the order is open)
+        assert np.array_equal(run.pool_used.cpu().numpy()[settled], ref.pool[settled])
+
+
 def test_select_matches_stable_sort_with_ties_and_inf(handle):
     import torch
     rng = np.random.default_rng(3)
