@@ -287,10 +287,11 @@ __global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T
   const float* Oh = O_f32 + (long long)bh * R * d;
   const bool gmax = p.group == RESTKV_GROUP_MAX;
   for (int i = tid; i < p.w; i += kThreads) wt[i] = temporal_weight(p.temporal, ema_decay, p.w, i);
-  ptx::grid_dependency_wait();
-  ptx::grid_dependency_launch();
+  // The kernel before this one (the combine, or what takes its place) lets it start only after its own wait, so that Q, K and V,
+  // which lie further back in the stream, may be read at once; O, m and l may not.
   load_rows<T>(Ks, K + (long long)b * p.ksb + (long long)h * p.ksh + (long long)j0 * p.ksn, p.ksn, kTB, valid, d);
   load_rows<T>(Vs, V + (long long)b * p.vsb + (long long)h * p.vsh + (long long)j0 * p.vsn, p.vsn, kTB, valid, d);
+  load_rows<T>(Qh_s, Qh, d, held, min(held, R), d);
   if (gmax)
     for (int e = tid; e < p.G * kTB; e += kThreads) gsum[e] = 0.f;
   if (p.indicator == RESTKV_INDICATOR_ATTENTION_VNORM) {
@@ -307,12 +308,16 @@ __global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T
   float acc[kTok];
 #pragma unroll
   for (int t = 0; t < kTok; ++t) acc[t] = 0.f;
+  ptx::grid_dependency_wait();
+  ptx::grid_dependency_launch();
 
   for (int row0 = 0; row0 < R; row0 += kP2Rows) {
     const int rows = min(kP2Rows, R - row0);
     if (row0 % held == 0) {   // the next `held` rows of Q and O
-      if (row0 > 0) __syncthreads();   // the rows before have been used
-      load_rows<T>(Qh_s, Qh + (long long)row0 * d, d, held, min(held, R - row0), d);
+      if (row0 > 0) {
+        __syncthreads();   // the rows before have been used
+        load_rows<T>(Qh_s, Qh + (long long)row0 * d, d, held, min(held, R - row0), d);
+      }
       load_rows<float>(Oh_s, Oh + (long long)row0 * d, d, held, min(held, R - row0), d);
     }
     const float* Qs = Qh_s + (row0 % held) * ld;
@@ -507,7 +512,7 @@ cudaError_t pass2(const Problem& p, const Workspace& ws, const void* Q, const vo
            (p.group == RESTKV_GROUP_MAX ? (size_t)kP2Rows * (tb + 1) + (size_t)p.G * tb : 0);
   };
   // 32 tokens per block share the loads of Q and O better; 16 where that would leave SMs with a single block, or where 32
-  // do not fit shared memory
+  // do not fit shared memory (8 were slower even for 1024 rows of 2 heads, one block per SM: 33.8 against 28.6 us)
   const bool wide = (long long)(p.n + 31) / 32 * p.BH >= 296 && floats(32, kP2Rows) * sizeof(float) <= 220 * 1024;
   const int tb = wide ? 32 : 16;
   // all rows of Q and O stay in shared memory where two blocks of that size fit an SM
