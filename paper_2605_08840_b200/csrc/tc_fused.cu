@@ -39,7 +39,6 @@ struct FusedArgs {
   // t_scale * sum_i c_i I_i t_decay^(w-1-i) with c_0 = t_seed_first, c_(w-1) = t_seed_last, c_i = 1 otherwise (w >= 16 here).
   float t_decay, t_seed_first, t_seed_last, t_scale;
   int group_max;                     // 1: maximum over the query heads of a group instead of their mean
-  int pool_max;                      // 1: the selection phase takes the maximum over the box instead of the mean
   int groups, cpg;                   // CTA groups and CTAs per group
   int attention_only;                // 1: stop after the merge (phases A and B): plain attention of the 128 rows
   int from_lse;                      // 1: O and the rows' log-sum-exp are given: phases A and B are skipped, phase C
@@ -1505,7 +1504,6 @@ cudaError_t launch_tc_fused(void* state, const Problem& p, const Workspace& ws, 
     a.proj_Mt = p.proj.Mt; a.vmv = ws.vmv; a.O_proj = ws.O_proj;
   }
   a.group_max = p.group == RESTKV_GROUP_MAX ? 1 : 0;
-  a.pool_max = p.spatial == RESTKV_SPATIAL_MAX ? 1 : 0;
   a.attention_only = attention_only ? 1 : 0;
   a.from_lse = O_given ? 1 : 0;
   fused_plan(p, sm_count, reuse_l2, &a.groups, &a.cpg);
