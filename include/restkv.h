@@ -26,8 +26,10 @@
  *    bounded wait that ran out) set a sticky status word that restkv_poll_status() reads;
  *    kernels never trap.  Check restkv_poll_status() before using the outputs of a call.
  *  - Calls must not overlap on the GPU if they share a workspace.
- *  - The tensor-core kernels behind restkv_score, restkv_evict and restkv_decode (bf16, head_dim 128)
- *    are persistent: their thread blocks wait for one another inside one launch, so each launch
+ *  - Launches are chained: a kernel may be scheduled while the one before it in the stream ends, but waits for its results
+ *    before it touches anything.
+ *  - The tensor-core kernels behind restkv_score and restkv_evict (bf16, head_dim 128), and behind restkv_decode with
+ *    more than 16 query heads per KV head, are persistent: their thread blocks wait for one another inside one launch, so each launch
  *    needs every SM of the device for itself.  Do not let two such calls, or one of them and any
  *    other kernel that occupies SMs, run at the same time (two streams without ordering): order
  *    them on one stream or with events.  If SMs are held by something else the waits are bounded:
@@ -189,9 +191,10 @@ restkv_status restkv_evict_host(restkv_handle* h, const restkv_shape* shape, con
  *   out      device float [batch, n_q_heads, head_dim]
  *   lse      optional device float [batch, n_q_heads] (natural-log sum of exp of the scaled logits)
  * shape->n_kv, w, causal_tail and the strides are ignored.
- * RESTKV_BF16 with head_dim 128 and up to 128 query heads per KV head runs as plain attention on the tensor-core
- * kernel (the softmax weights are rounded to bf16 before they meet V) when the workspace has the ~10 MB it needs,
- * which every restkv_workspace_bytes() result has; everything else runs on fp32 SIMT kernels, which need
+ * RESTKV_BF16 with head_dim 128 and up to 16 query heads per KV head runs on a cluster kernel of its own, up to 128 as
+ * plain attention on the tensor-core kernel when the workspace has the ~10 MB it needs, which every
+ * restkv_workspace_bytes() result has (the softmax weights are rounded to bf16 before they meet V in both);
+ * everything else runs on fp32 SIMT kernels, which need
  * batch * n_kv_heads * 64 * group * (head_dim + 2) floats and take 1, 2, 4 or 8 query heads per KV head and rows of
  * 32, 64, ..., 1024 bytes (head_dim * element size a power of two); other shapes return RESTKV_ERR_UNSUPPORTED.
  */

@@ -19,7 +19,7 @@ constexpr int kRsMaxSmem = 200 * 1024;
 // rows past 100 KB; longer rows are read again on every walk), and no more than the walks that are needed: the extremes,
 // a histogram of 11-bit digits of the offsets from the smallest (about a thousand bins in use, so one histogram serves all
 // warps without contention), then the sum above the digit that holds the Bp-th largest while that digit's few keys are
-// listed and ranked, a key per warp.  1024 rows of 20011: 62 us as selections in two blocks of 512 threads per SM, 47 us so
+// listed and ranked, a key per warp.  1024 rows of 20011: 62 us as selections in two blocks of 512 threads per SM, 43 us so
 // (10 k cycles per row: 0.8 k extremes, 3 k histogram, 2.6 k the last walk, the rest synchronisation).
 template <bool kHeld>   // false: no buffers, the keys are read from global memory on every walk
 __global__ void __launch_bounds__(kRsThreads, 1)
