@@ -145,7 +145,8 @@ restkv_status restkv_evict_from_lse(restkv_handle* h, const restkv_shape* shape,
 /*
  * restkv_select -- Eq. 14's argmax_B: per (batch, KV head) the min(budget, n_kv) largest scores,
  * ties to the lower index, indices written in ascending order.
- *   scores   device float [batch, n_kv_heads, n_kv] (+inf allowed, NaN not)
+ *   scores   device float [batch, n_kv_heads, n_kv] (+inf allowed; a NaN has no rank in Eq. 14 and counts as larger than
+ *            +inf, a negative one as smaller than -inf, so that min(budget, n_kv) distinct rows come out in any case)
  *   indices  device int32 [batch, n_kv_heads, min(budget, n_kv)]
  */
 restkv_status restkv_select(restkv_handle* h, const restkv_shape* shape, const float* scores, int budget,

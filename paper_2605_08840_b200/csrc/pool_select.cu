@@ -77,6 +77,11 @@ struct SelectArgs {
 constexpr int kSelBins = 2048;               // 11-bit digits
 constexpr unsigned int kInfKey = 0xFF800000u;
 
+// The selection's key of a score: any bit pattern has its place, so that exactly `keep` rows come out whatever the scores are
+// (a NaN in a head's V makes all its scores NaN; after a wait that ran out they are anything).  NaNs rank above +inf; the
+// highest key is kept free, as a bound that no row reaches.
+__device__ __forceinline__ unsigned int select_key(float x) { return min(float_key(x), 0xFFFFFFFEu); }
+
 // Bounded wait for a bulk copy.
 __device__ __forceinline__ void wait_copy(uint64_t* bar, uint32_t parity, unsigned int* dev_status) {
   const long long t0 = clock64();
@@ -119,8 +124,8 @@ __device__ __forceinline__ void pool_slice(const float* taps, int W, bool pool_m
 //     and the blocks share the gather only;
 //   - the slice's keys stay in shared memory; a warp owns a contiguous run of them, so that the ordered emit needs only
 //     ballots;
-//   - the smallest key and the largest finite one are agreed on first; keys count as offsets from the smallest, +inf as one
-//     past the largest.  The first 11-bit digit then spreads the scores over about a thousand bins, so that one histogram
+//   - the smallest key and the largest but +inf are agreed on first; keys count as offsets from the smallest, +inf as one
+//     past the largest (or, below a NaN, as itself).  The first 11-bit digit then spreads the scores over about a thousand bins, so that one histogram
 //     serves all warps without contention, and the bin that holds the keep-th largest key is narrow: the passes end as soon
 //     as the rest of that bin is kept as a whole, usually after the second digit;
 //   - what the CTAs of a cluster tell one another (extremes, counts, positions of the kept rows) is put straight into the
@@ -171,14 +176,14 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
   // this warp's run of the slice
   const int cw = (((a.per + kWarps - 1) / kWarps) + 31) & ~31;
   const int wbeg = min(cnt, wid * cw), wlen = min(cnt, wbeg + cw) - wbeg;
-  auto key_at = [&](int i) { return a.held ? skeys[wbeg + i] : float_key(srow[wbeg + i]); };   // i: position in the run
+  auto key_at = [&](int i) { return a.held ? skeys[wbeg + i] : select_key(srow[wbeg + i]); };   // i: position in the run
 
-  // ---- keys of the slice, their smallest and largest finite one ----
+  // ---- keys of the slice, the smallest and the largest but +inf ----
   unsigned int kmin = 0xFFFFFFFFu, kmax = 0u;
   auto take = [&](int jj, float score) {
-    const unsigned int key = float_key(score);
+    const unsigned int key = select_key(score);
     kmin = min(kmin, key);
-    kmax = max(kmax, key < kInfKey ? key : 0u);
+    kmax = max(kmax, key != kInfKey ? key : 0u);
     if (a.held) skeys[jj] = key;
   };
   if (a.I_hat) {
@@ -245,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
   }
   csync();
   kmin = s_min;
-  const unsigned int range = s_max >= kmin ? s_max - kmin + 1u : 0u;   // offset of +inf
+  const unsigned int range = s_max >= kmin ? s_max - kmin + 1u : 0u;   // offset of +inf, unless a NaN lies above it
   auto offset_of = [&](unsigned int key) { return min(key - kmin, range); };
 
   // ---- digits from the top ----
@@ -320,15 +325,15 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
       hi = lo;
       pb ^= 1;
     }
-    // offsets back to keys; the offset of +inf stands for no other key
+    // offsets back to keys; the offset `range` stands for +inf and for no other key
+    const unsigned int edge = prefix >= range ? kInfKey : kmin + prefix;
     if (whole) {
-      above = prefix >= range ? kInfKey : kmin + prefix;
+      above = edge;
     } else {
-      equal = prefix >= range ? kInfKey : kmin + prefix;
-      above = prefix >= range ? 0xFFFFFFFFu : prefix + 1u >= range ? kInfKey : equal + 1u;
+      equal = edge;
+      above = edge + 1u;
       need_eq = remaining;
     }
-    if (range == 0u) { equal = kmin; above = 0xFFFFFFFFu; need_eq = remaining; }   // all keys alike
   }
 
   // ---- ordered emit: ascending indices, of equal keys the lower index ----
@@ -377,7 +382,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
           if (pos < (unsigned int)keep && (CS > 1 || (pos >= first && pos < last))) dst[pos] = j;
         } else if (CS == 1) {
           if (pos >= first && pos < last) s_idx[pos - first] = j;
-        } else {
+        } else if (pos < (unsigned int)keep) {
           const unsigned int to = pos / share;
           *cluster.map_shared_rank(s_idx + (pos - to * share), to) = j;
         }
@@ -417,7 +422,8 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
       if (lane < 2 * cr) {
         const bool isV = lane >= cr;
         const int r = isV ? lane - cr : lane;
-        const long long j = own_idx ? s_idx[r0 + r] : dst[first + r0 + r];
+        // (bounded, should the taps' copy that was given up on have landed over the indices after all)
+        const long long j = min((unsigned int)(own_idx ? s_idx[r0 + r] : dst[first + r0 + r]), (unsigned int)n_kv - 1u);
         const unsigned char* src = isV ? Vh + j * a.ga.vsn * es : Kh + j * a.ga.ksn * es;
         ptx::bulk_load(buf + (isV ? R * rb : 0) + r * rb, src, (uint32_t)rb, &copy_bar[wid][it & 1]);
       }

@@ -472,6 +472,74 @@ def test_select_matches_stable_sort_with_ties_and_inf(handle):
         np.testing.assert_array_equal(got, oracle.select(s.astype(np.float64), B))
 
 
+def _key_order(bits):
+    """Sort keys of float bit patterns: the order of the numbers, NaNs above +inf and below -inf by their sign and payload (the two
+    highest patterns count as one)."""
+    bits = bits.astype(np.uint32)
+    return np.minimum(np.where(bits >> 31 != 0, ~bits, bits | np.uint32(0x80000000)), np.uint32(0xFFFFFFFE)).astype(np.int64)
+
+
+@pytest.mark.parametrize("spec", [(3, 40, 7), (8, 9000, 300), (8, 16384, 1024), (200, 3000, 64), (1, 300007, 2000)])
+@pytest.mark.parametrize("kind", ["all", "most", "few", "payloads", "with_inf", "only_inf"])
+def test_select_with_nan_scores(handle, spec, kind):
+    """Any bit pattern has its place in the order: exactly `budget` distinct ascending indices come out, NaNs ranked above +inf
+    (negative ones below -inf), in one block, in a cluster and with keys that do not stay in shared memory."""
+    import torch
+    heads, n, budget = spec
+    rng = np.random.default_rng(n + heads)
+    s = np.abs(rng.standard_normal((heads, n))).astype(np.float32)
+    nan, inf = np.uint32(0x7FFFFFFF), np.uint32(0x7F800000)
+    bits = s.view(np.uint32)
+    if kind == "all":
+        bits[...] = nan
+    elif kind == "most":
+        bits[rng.random(bits.shape) < 0.9] = nan
+    elif kind == "few":
+        bits[:, rng.permutation(n)[:budget // 2]] = nan
+    elif kind == "payloads":
+        bits[...] = rng.integers(0, 2 ** 32, bits.shape, dtype=np.uint64).astype(np.uint32)
+        bits[:, ::3] = np.where(rng.random((heads, len(range(0, n, 3)))) < 0.5, np.uint32(0x7FC00001), np.uint32(0xFFFFFFFF))
+    elif kind == "with_inf":
+        bits[:, -2 * budget:] = inf
+        bits[:, rng.permutation(n)[:budget // 3]] = nan
+    else:
+        bits[...] = inf
+    shape = rk.make_shape(1, heads, heads, 16, n, 1)
+    ws = torch.empty(handle.workspace_bytes(shape, budget), dtype=torch.uint8, device="cuda")
+    idx = torch.full((1, heads, budget), -7, dtype=torch.int32, device="cuda")
+    handle.select(shape, torch.from_numpy(s).cuda(), budget, idx, ws)
+    assert handle.poll_status() == rk.RESTKV_OK
+    ref = np.sort(np.argsort(-_key_order(bits), axis=-1, kind="stable")[:, :budget], axis=-1)
+    np.testing.assert_array_equal(idx.cpu().numpy()[0], ref)
+
+
+@pytest.mark.parametrize("spec", [("bf16", 32, 8, 128, 1000, 0), ("bf16", 32, 8, 128, 9000, 32), ("bf16", 32, 8, 128, 20000, 0),
+                                  ("f32", 8, 2, 64, 1000, 32), ("f32", 8, 2, 64, 9000, 0)])
+def test_evict_with_a_nan_in_one_head(handle, spec):
+    """A NaN in one head's V makes all scores of that head NaN: its first `budget` rows are kept and copied, the other heads are
+    what they are without it."""
+    import torch
+    dtype, Hq, Hkv, d, n, tail = spec
+    inp = make_inputs(Case("nan", 1, Hq, Hkv, d, n, 32, 300, 7, 0, 0.9, dtype, tail, "normal", 5))
+    clean = [x.copy() for x in DeviceRun(handle, inp).evict()]
+    run = DeviceRun(handle, inp)
+    run.V[0, 1, n // 2, 3] = float("nan")
+    scores, idx, K_out, V_out = run.evict()
+    assert np.isnan(scores[0, 1, :n]).all()
+    np.testing.assert_array_equal(idx[0, 1], np.arange(300))
+    np.testing.assert_array_equal(K_out[0, 1], run._bits(run.K)[0, 1, :300])
+    np.testing.assert_array_equal(V_out[0, 1], run._bits(run.V)[0, 1, :300])
+    for h in range(Hkv):
+        if h != 1:
+            for x, y in zip(clean, (scores, idx, K_out, V_out)):
+                np.testing.assert_array_equal(x[0, h], y[0, h])
+    run = DeviceRun(handle, inp, adaptive_budget=300)
+    run.V[0, 1, n // 2, 3] = float("nan")
+    _, idx, _, _ = run.evict(pool=rk.adaptive_pool(2000.0, 5, 300))
+    np.testing.assert_array_equal(idx[0, 1], np.arange(300))
+    torch.cuda.synchronize()
+
+
 def test_compact_bit_exact_and_bad_index_reported(handle):
     import torch
     case = Case("cmp", 2, 4, 2, 64, 300, 8, dtype="f32")
