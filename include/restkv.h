@@ -34,7 +34,8 @@
  *    other kernel that occupies SMs, run at the same time (two streams without ordering): order
  *    them on one stream or with events.  If SMs are held by something else the waits are bounded:
  *    the kernel gives up after about a second, the outputs of that call are undefined, and
- *    restkv_poll_status() returns RESTKV_ERR_TIMEOUT.
+ *    restkv_poll_status() returns RESTKV_ERR_TIMEOUT.  (Each launch counts its blocks in a set of counters of its own,
+ *    of 64 taken in turn, and 64 more for launches recorded into graphs.)
  */
 #ifndef RESTKV_H_
 #define RESTKV_H_
@@ -85,7 +86,7 @@ typedef struct {
 } restkv_pool_params;
 
 /* Creates a handle for the CURRENT device: queries its properties and allocates a device block of
- * 1280 bytes for status and barrier counters (the only allocation the library ever makes).  Host pointer out. */
+ * 128 KB for status and barrier counters (the only allocation the library ever makes).  Host pointer out. */
 restkv_status restkv_create(restkv_handle** out);
 restkv_status restkv_destroy(restkv_handle* h);
 

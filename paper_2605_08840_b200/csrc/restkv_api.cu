@@ -1,4 +1,5 @@
 // C ABI of librestkv.so: argument checks, workspace carve-up and kernel sequencing.
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <cmath>
@@ -9,7 +10,8 @@
 struct restkv_handle {
   int device;
   int sm_count;
-  unsigned int* dev_status;   // device block: kDevStatusWords (word 0 = sticky status bits), then kDevCounterWords
+  unsigned int* dev_status;   // device block of kDevWords: word 0 = sticky status bits, then the sets of barrier counters
+  std::atomic<unsigned int> counter_turn[2];   // launches so far that took a set: called, recorded into graphs
   void* tc_state;
   int select_clusters[4];     // clusters of 1, 2, 4, 8 CTAs of the select kernel that the device holds at once
   int decode_clusters[5];     // clusters of 1, 2, 4, 8, 16 CTAs of the decode kernel that the device holds at once
@@ -184,6 +186,17 @@ static bool simt_supported(const Problem& p) {
 struct Call {
   restkv_handle* h;
   cudaStream_t st;
+  // the barrier counters of the next persistent launch
+  unsigned int* counters() {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
+      (void)cudaGetLastError();   // the legacy stream beside a capture in another one: the launch itself will say so
+      capture = cudaStreamCaptureStatusNone;
+    }
+    const unsigned int recorded = capture == cudaStreamCaptureStatusNone ? 0u : 1u;
+    const unsigned int turn = h->counter_turn[recorded].fetch_add(1u, std::memory_order_relaxed) % kCounterSets;
+    return h->dev_status + kDevStatusWords + (recorded * kCounterSets + turn) * kDevCounterWords;
+  }
   restkv_status fail(cudaError_t e) {
     h->last_cuda_error = (int)e;
     return RESTKV_ERR_CUDA;
@@ -235,7 +248,7 @@ static restkv_status run_score(Call& c, const Problem& p, const Workspace& ws, c
     if (use_tc) {
       RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS2,
                     launch_tc_fused(c.h->tc_state, p, ws, Q, K, V, ema_decay, c.h->sm_count, false, false, c.h->wait_limit,
-                                    O_given, nullptr, c.h->dev_status + kDevStatusWords, c.h->dev_status, true, c.st), 1);
+                                    O_given, nullptr, nullptr, c.h->dev_status, true, c.st), 1);
     } else {
       Workspace wsl = ws;
       wsl.O_f32 = const_cast<float*>(O_given);
@@ -252,8 +265,7 @@ static restkv_status run_score(Call& c, const Problem& p, const Workspace& ws, c
                     launch_tc_vmv(c.h->tc_state, p, V, ws.vmv, c.h->sm_count, c.h->wait_limit, c.h->dev_status, c.st), 1);
     RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS2,
                   launch_tc_fused(c.h->tc_state, p, ws, Q, K, V, ema_decay, c.h->sm_count, reuse_l2, false, c.h->wait_limit,
-                                  nullptr, adaptive ? ws.I_raw : nullptr, c.h->dev_status + kDevStatusWords,
-                                  c.h->dev_status, true, c.st), 1);
+                                  nullptr, adaptive ? ws.I_raw : nullptr, c.counters(), c.h->dev_status, true, c.st), 1);
   } else {
     RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS1, launch_simt_pass1(p, ws, Q, K, V, c.st), 1);
     RESTKV_LAUNCH(c, RESTKV_KERNEL_COMBINE, launch_combine(p, ws, c.st), 1);
@@ -296,11 +308,17 @@ restkv_status restkv_create(restkv_handle** out) {
   int major = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, h->device);
   if (e == cudaSuccess && major != 10) { delete h; return RESTKV_ERR_UNSUPPORTED; }   // sm_100a only
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->dev_status, (kDevStatusWords + kDevCounterWords) * sizeof(unsigned int));
-  if (e == cudaSuccess) e = cudaMemset(h->dev_status, 0, (kDevStatusWords + kDevCounterWords) * sizeof(unsigned int));
+  h->dev_status = nullptr;
+  if (e == cudaSuccess) e = cudaMalloc((void**)&h->dev_status, kDevWords * sizeof(unsigned int));
+  if (e == cudaSuccess) e = cudaMemset(h->dev_status, 0, kDevWords * sizeof(unsigned int));
   if (e == cudaSuccess) e = select_init(h->select_clusters);
   if (e == cudaSuccess) e = adaptive_init();
-  if (e != cudaSuccess) { delete h; return RESTKV_ERR_CUDA; }
+  if (e != cudaSuccess) {
+    cudaFree(h->dev_status);
+    delete h;
+    return RESTKV_ERR_CUDA;
+  }
+  h->counter_turn[0] = h->counter_turn[1] = 0u;
   h->tc_state = nullptr;
   if (tc_init(&h->tc_state) != cudaSuccess || tc_fused_init() != cudaSuccess ||
       decode_mma_init(h->decode_clusters) != cudaSuccess)
@@ -564,7 +582,7 @@ restkv_status restkv_decode(restkv_handle* h, const restkv_shape* shape, const v
       RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE, launch_decode_pad(p, q, ws.q_pad, c.st), 1);
       RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE,
                     launch_tc_fused(h->tc_state, pd, ws, ws.q_pad, Kc, Vc, 0.f, h->sm_count, false, true, h->wait_limit,
-                                    nullptr, nullptr, h->dev_status + kDevStatusWords, h->dev_status, false, c.st), 1);
+                                    nullptr, nullptr, c.counters(), h->dev_status, false, c.st), 1);
       RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE, launch_decode_extract(p, ws.O_f32, ws.row_M2, out, lse, c.st), 1);
       return RESTKV_OK;
     }

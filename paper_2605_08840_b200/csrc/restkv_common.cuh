@@ -63,8 +63,12 @@ struct Workspace {
 
 constexpr int kDecodeMaxSplits = 64;
 
-// Words of the handle's device block: status, and the barrier counters of the persistent score kernel (zero between launches).
-constexpr int kDevStatusWords = 64, kDevCounterWords = 256;
+// Words of the handle's device block: status, then sets of barrier counters of the persistent score kernel (zero between
+// launches).  Every launch takes the next set in turn, so that launches which overlap against the rules (two streams without
+// ordering) count apart and end with right results or a timeout, never with barriers that open early; launches recorded into a
+// graph take theirs from sets of their own, since a graph keeps its set and may run beside later calls.
+constexpr int kDevStatusWords = 64, kDevCounterWords = 256, kCounterSets = 64;
+constexpr int kDevWords = kDevStatusWords + 2 * kCounterSets * kDevCounterWords;
 
 int pass1_splits(const Problem& p, int sm_count);
 size_t plan_workspace(const Problem& p, int budget, int sm_count, bool adaptive, void* base, Workspace* ws);

@@ -1482,6 +1482,62 @@ def test_wait_limit_runs_out_and_the_handle_recovers(handle):
     full_check(handle, inp)
 
 
+def test_overlapping_calls_count_their_blocks_apart(handle):
+    """Two evictions on two streams without ordering, each with its own workspace: against the rules, but each launch counts its
+    blocks in a set of its own, so that the outcome is right results or the timeout status, never a barrier opened by the other
+    call's blocks."""
+    import torch
+    inps = [make_inputs(Case("overlap", 1, 32, 8, 128, n, 32, 200, 7, 0, 0.9, "bf16", 0, "normal", n)) for n in (9000, 11000)]
+    runs = [DeviceRun(handle, inp) for inp in inps]
+    want = [[x.copy() for x in run.evict()] for run in runs]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    handle.set_wait_limit(400_000_000)
+    try:
+        for _ in range(5):
+            for run in runs:
+                run.scores.zero_()
+            torch.cuda.synchronize()
+            for run, stream in zip(runs, streams):
+                handle.evict(run.shape, run.Q, run.K, run.V, run.case.ema_decay, run.pool(), run.budget, run.indices, run.K_out,
+                             run.V_out, run.ws, scores_out=run.scores, stream=stream)
+            torch.cuda.synchronize()
+            status = handle.poll_status()
+            assert status in (rk.RESTKV_OK, rk.ERR_TIMEOUT)
+            if status == rk.RESTKV_OK:
+                for run, ref in zip(runs, want):
+                    np.testing.assert_array_equal(run.scores.cpu().numpy(), ref[0])
+                    np.testing.assert_array_equal(run.indices.cpu().numpy(), ref[1])
+    finally:
+        handle.set_wait_limit(2_000_000_000)
+
+
+def test_calls_and_graph_replays_in_a_row(handle):
+    """More calls than there are sets of barrier counters, and replays of a recorded call between them, all alike."""
+    import torch
+    inp = make_inputs(Case("sets", 1, 32, 8, 128, 2000, 32, 200, 7, 0, 0.9, "bf16", 32, "normal", 8))
+    run = DeviceRun(handle, inp)
+    want = [x.copy() for x in run.evict()]
+
+    def call(stream=None):
+        handle.evict(run.shape, run.Q, run.K, run.V, inp.case.ema_decay, run.pool(), run.budget, run.indices, run.K_out, run.V_out,
+                     run.ws, scores_out=run.scores, stream=stream)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call()
+    for i in range(150):
+        run.scores.zero_()
+        if i % 3 == 0:
+            graph.replay()
+        else:
+            call()
+        if i % 10 == 9:
+            torch.cuda.synchronize()
+            np.testing.assert_array_equal(run.scores.cpu().numpy(), want[0])
+            np.testing.assert_array_equal(run.indices.cpu().numpy(), want[1])
+    assert handle.poll_status() == rk.RESTKV_OK
+
+
 # ------------------------------------------------------------------ API misuse: error codes, never a fault
 def test_api_rejects_bad_arguments(handle):
     import torch
