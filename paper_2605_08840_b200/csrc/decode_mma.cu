@@ -175,8 +175,9 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
         l[r] *= f[r];
         grown = true;
       }
-      const float e0 = ex2_approx(fmaf(sc[0][2 * r], c2, -m[r])), e1 = ex2_approx(fmaf(sc[0][2 * r + 1], c2, -m[r]));
-      const float e2 = ex2_approx(fmaf(sc[1][2 * r], c2, -m[r])), e3 = ex2_approx(fmaf(sc[1][2 * r + 1], c2, -m[r]));
+      const float m_use = m[r] == -INFINITY ? 0.f : m[r];   // only logits of -inf so far: they weigh nothing
+      const float e0 = ex2_approx(fmaf(sc[0][2 * r], c2, -m_use)), e1 = ex2_approx(fmaf(sc[0][2 * r + 1], c2, -m_use));
+      const float e2 = ex2_approx(fmaf(sc[1][2 * r], c2, -m_use)), e3 = ex2_approx(fmaf(sc[1][2 * r + 1], c2, -m_use));
       l[r] += (e0 + e1) + (e2 + e3);
       p[r] = pack_bf16x2(e0, e1);
       p[2 + r] = pack_bf16x2(e2, e3);

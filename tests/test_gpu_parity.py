@@ -621,6 +621,36 @@ def test_decode_cluster_kernel(handle, spec):
     np.testing.assert_allclose(lse.cpu().numpy(), ref_lse, rtol=1e-5, atol=1e-5)
 
 
+@pytest.mark.parametrize("spec", [(1, 32, 8, 700, 130), (1, 9, 1, 3000, 2990), (4, 4, 1, 100, 33), (1, 17, 1, 400, 200)])
+def test_decode_with_logits_of_minus_infinity(handle, spec):
+    """Rows whose logits are -inf for every query (a key channel of -inf that all queries meet with a positive value) weigh
+    nothing, wherever they lie: whole tiles at the front, scattered ones behind."""
+    import torch
+    b, Hq, Hkv, rows, masked = spec
+    rng = np.random.default_rng(rows)
+
+    def draw(shape):
+        bits = round_to_bf16_bits(rng.standard_normal(shape).astype(np.float32))
+        return (bits.astype(np.uint32) << 16).view(np.float32)
+
+    q, K, V = draw((b, Hq, 128)), draw((b, Hkv, rows, 128)), draw((b, Hkv, rows, 128))
+    q[..., 5] = 1.0
+    gone = np.zeros(rows, bool)
+    gone[:masked - masked // 4] = True
+    gone[masked - masked // 4 + rng.permutation(rows - masked + masked // 4)[:masked // 4]] = True
+    ref, ref_lse = oracle.decode(q, np.ascontiguousarray(K[:, :, ~gone]), np.ascontiguousarray(V[:, :, ~gone]))
+    dev = [torch_dev((x.view(np.uint32) >> 16).astype(np.uint16).view(np.int16), "bf16") for x in (q, K, V)]
+    dev[1][:, :, torch.from_numpy(gone).cuda(), 5] = float("-inf")
+    shape = shape_of(Case("dec", b, Hq, Hkv, 128, rows, 1, dtype="bf16"))
+    out = torch.full((b, Hq, 128), float("nan"), device="cuda")
+    lse = torch.full((b, Hq), float("nan"), device="cuda")
+    ws = torch.empty(handle.workspace_bytes(shape, 0), dtype=torch.uint8, device="cuda")
+    handle.decode(shape, *dev, rows, out, ws, lse=lse)
+    torch.cuda.synchronize()
+    assert_decode_close(out.cpu().numpy(), ref, q, K[:, :, ~gone], V[:, :, ~gone], "bf16")
+    np.testing.assert_allclose(lse.cpu().numpy(), ref_lse, rtol=1e-5, atol=1e-5)
+
+
 def test_decode_over_compacted_cache_of_config2(handle):
     import torch
     inp = make_inputs(CONFIGS["cfg2"])
