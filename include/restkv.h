@@ -193,10 +193,10 @@ restkv_status restkv_evict_host(restkv_handle* h, const restkv_shape* shape, con
  *   out      device float [batch, n_q_heads, head_dim]
  *   lse      optional device float [batch, n_q_heads] (natural-log sum of exp of the scaled logits)
  * shape->n_kv, w, causal_tail and the strides are ignored.
- * RESTKV_BF16 with head_dim 128 and up to 16 query heads per KV head runs on a cluster kernel of its own, up to 128 as
- * plain attention on the tensor-core kernel when the workspace has the ~10 MB it needs, which every
- * restkv_workspace_bytes() result has (the softmax weights are rounded to bf16 before they meet V in both);
- * everything else runs on fp32 SIMT kernels, which need
+ * RESTKV_BF16 with head_dim 128 runs, when the workspace has about 10 MB, which every restkv_workspace_bytes() result has, on
+ * a cluster kernel of its own with up to 16 query heads per KV head and as plain attention on the tensor-core kernel with
+ * up to 128 (the softmax weights are rounded to bf16 before they meet V in both);
+ * everything else, and a smaller workspace, runs on fp32 SIMT kernels (fp32 weights), which need
  * batch * n_kv_heads * 64 * group * (head_dim + 2) floats and take 1, 2, 4 or 8 query heads per KV head and rows of
  * 32, 64, ..., 1024 bytes (head_dim * element size a power of two); other shapes return RESTKV_ERR_UNSUPPORTED.
  */

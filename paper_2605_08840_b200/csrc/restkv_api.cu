@@ -555,9 +555,14 @@ restkv_status restkv_decode(restkv_handle* h, const restkv_shape* shape, const v
   if (s != RESTKV_OK) return s;
   if (!workspace || ((uintptr_t)workspace & 255u) != 0) return RESTKV_ERR_WORKSPACE;
   Call c{h, (cudaStream_t)stream};
-  // bf16, head_dim 128, up to 16 query heads per KV head: a kernel of its own, one cluster of CTAs per KV head, which
-  // needs scratch only where several clusters share one
-  if (h->tc_state && h->kernel_path != 1 && p.dtype == RESTKV_BF16 && p.d == 128 && p.G <= kDecodeMmaMaxG) {
+  // bf16, head_dim 128: kernels that round the softmax weights to bf16 before they meet V.  They run when the workspace has the
+  // ~10 MB that the padded one needs (any restkv_workspace_bytes result has that); a caller who gives less gets the SIMT kernels
+  // with their fp32 weights.
+  const bool bf16_128 = h->tc_state && h->kernel_path != 1 && p.dtype == RESTKV_BF16 && p.d == 128;
+  const bool roomy = plan_decode_tc(p.BH, h->sm_count, nullptr, nullptr) <= workspace_bytes;
+  // up to 16 query heads per KV head: a kernel of its own, one cluster of CTAs per KV head, which needs scratch only where
+  // several clusters share one
+  if (bf16_128 && roomy && p.G <= kDecodeMmaMaxG) {
     int cluster, splits;
     decode_mma_plan(h->decode_clusters, p.BH, p.G, n_rows, workspace_bytes, &cluster, &splits);
     RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE,
@@ -568,17 +573,17 @@ restkv_status restkv_decode(restkv_handle* h, const restkv_shape* shape, const v
     return RESTKV_OK;
   }
   // more query heads per KV head: the decode step is plain attention of up to 128 query rows per KV head, i.e. phases A and B
-  // of the tensor-core score kernel with the group's queries padded to its 128 rows.  It needs about 10 MB of
-  // workspace (any restkv_workspace_bytes result has that); with less, or for other shapes, the SIMT kernels run.
+  // of the tensor-core score kernel with the group's queries padded to its 128 rows
   bool tc_ws_too_small = false;
-  if (h->tc_state && h->kernel_path != 1 && p.dtype == RESTKV_BF16 && p.d == 128 && p.G <= 128 && n_rows > 1) {
+  if (bf16_128 && p.G <= 128 && n_rows > 1) {
     Problem pd = p;
     pd.G = 128; pd.Hq = p.Hkv * 128; pd.w = 1; pd.R = 128; pd.tail = 0; pd.n = pd.n_kv = n_rows;
     pd.ksn = pd.vsn = p.d;
     pd.ksh = pd.vsh = (long long)n_rows * p.d;
     pd.ksb = pd.vsb = (long long)p.Hkv * n_rows * p.d;
-    Workspace ws;
-    if (plan_decode_tc(pd.BH, h->sm_count, workspace, &ws) <= workspace_bytes) {
+    if (roomy) {
+      Workspace ws;
+      plan_decode_tc(pd.BH, h->sm_count, workspace, &ws);
       RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE, launch_decode_pad(p, q, ws.q_pad, c.st), 1);
       RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE,
                     launch_tc_fused(h->tc_state, pd, ws, ws.q_pad, Kc, Vc, 0.f, h->sm_count, false, true, h->wait_limit,

@@ -8,7 +8,7 @@ import oracle
 from paper_2605_08840_b200 import binding as rk
 from paper_2605_08840_b200.inputs import CONFIGS, Case, make_inputs, make_decode_query, round_to_bf16_bits
 
-from helpers import (TOL, DeviceRun, assert_compaction_exact, assert_decode_close, assert_scores_close, assert_selection_valid,
+from helpers import (DECODE_TOL, TOL, DeviceRun, assert_compaction_exact, assert_decode_close, assert_scores_close, assert_selection_valid,
                      shape_of, torch_dev)
 
 pytestmark = pytest.mark.gpu
@@ -649,6 +649,39 @@ def test_decode_with_logits_of_minus_infinity(handle, spec):
     torch.cuda.synchronize()
     assert_decode_close(out.cpu().numpy(), ref, q, K[:, :, ~gone], V[:, :, ~gone], "bf16")
     np.testing.assert_allclose(lse.cpu().numpy(), ref_lse, rtol=1e-5, atol=1e-5)
+
+
+@pytest.mark.parametrize("spec", [(1, 32, 8, 2085), (2, 8, 4, 300), (1, 8, 8, 20000), (1, 12, 4, 500)])
+def test_decode_with_a_small_workspace(handle, spec):
+    """bf16, head_dim 128 with less workspace than restkv_workspace_bytes: the SIMT kernels with their fp32 softmax weights where
+    those have enough, a refusal where they have not or do not take the shape."""
+    import torch
+    b, Hq, Hkv, rows = spec
+    rng = np.random.default_rng(rows)
+
+    def draw(shape):
+        bits = round_to_bf16_bits(rng.standard_normal(shape).astype(np.float32))
+        return (bits.astype(np.uint32) << 16).view(np.float32), torch_dev(bits.view(np.int16), "bf16")
+
+    q, qd = draw((b, Hq, 128))
+    K, Kd = draw((b, Hkv, rows, 128))
+    V, Vd = draw((b, Hkv, rows, 128))
+    ref, _ = oracle.decode(q, K, V)
+    shape = shape_of(Case("dec", b, Hq, Hkv, 128, rows, 1, dtype="bf16"))
+    need = b * Hkv * 64 * (Hq // Hkv) * 130 * 4
+    out = torch.full((b, Hq, 128), float("nan"), device="cuda")
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+    with pytest.raises(rk.RestKVError) as e:
+        handle.decode(shape, qd, Kd, Vd, rows, out, ws[:need - 256])
+    assert e.value.status == rk.ERR_WORKSPACE
+    if Hq // Hkv == 3:
+        with pytest.raises(rk.RestKVError) as e:
+            handle.decode(shape, qd, Kd, Vd, rows, out, ws)
+        assert e.value.status == rk.ERR_WORKSPACE
+        return
+    handle.decode(shape, qd, Kd, Vd, rows, out, ws)
+    torch.cuda.synchronize()
+    assert np.max(np.abs(out.cpu().numpy() - ref) / np.abs(ref).max(axis=-1, keepdims=True)) < DECODE_TOL["f32"]
 
 
 def test_decode_over_compacted_cache_of_config2(handle):
