@@ -25,7 +25,7 @@ __device__ __forceinline__ float box_mean(const float* __restrict__ src, int n, 
     return s;
   }
   for (int t = lo; t <= hi; ++t) s += src[t];
-  return s * (1.f / (float)W);
+  return s / (float)W;
 }
 
 // grid (ceil(n_kv/256), BH).  The window (W, gamma) comes from `pool` (per head, device) when it is non-null.
@@ -96,7 +96,7 @@ __device__ __forceinline__ void wait_copy(uint64_t* bar, uint32_t parity, unsign
 // there to cnt; f(jj, score) for each.  kW = 0: the width is known only at run time, pool_max: the maximum instead.
 template <int kThreads, int kW, typename F>
 __device__ __forceinline__ void pool_slice(const float* taps, int W, bool pool_max, int scored, int cnt, F&& f) {
-  const float inv = 1.f / (float)(kW ? kW : W);
+  const float width = (float)(kW ? kW : W);   // divided by: a product with the reciprocal would round twice
 #pragma unroll 2
   for (int jj = threadIdx.x; jj < cnt; jj += kThreads) {
     float acc = 0.f;
@@ -109,7 +109,7 @@ __device__ __forceinline__ void pool_slice(const float* taps, int W, bool pool_m
 #pragma unroll 4
       for (int t = 0; t < W; ++t) acc += taps[jj + t];
     }
-    f(jj, jj < scored ? ((!kW && pool_max) ? acc : acc * inv) : INFINITY);
+    f(jj, jj < scored ? ((!kW && pool_max) ? acc : acc / width) : INFINITY);
   }
 }
 

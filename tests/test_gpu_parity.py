@@ -348,6 +348,24 @@ def test_ema_extremes(handle, decay):
     full_check(handle, make_inputs(case))
 
 
+@pytest.mark.parametrize("spec", [("f32", 64, 1000, 0), ("f32", 64, 9000, 32), ("bf16", 128, 3000, 32), ("bf16", 128, 20000, 0)])
+@pytest.mark.parametrize("width", [5, 7, 21])
+def test_box_mean_is_rounded_once(handle, spec, width):
+    """Eq. 13 in fp32, bit for bit: the taps added in ascending order, then one division by the width; from restkv_score and from
+    the selection kernel behind restkv_evict."""
+    dtype, d, n, tail = spec
+    Hq = 8 if d == 64 else 32
+    inp = make_inputs(Case("box", 1, Hq, Hq // 4, d, n, 32, 100, width, 0, 0.9, dtype, tail, "normal", n))
+    run = DeviceRun(handle, inp)
+    I_hat = run.score(pool=run.pool(width=1))[..., :n].copy()
+    padded = np.pad(I_hat, ((0, 0), (0, 0), (width // 2, width // 2)))
+    total = np.zeros_like(I_hat)
+    for k in range(width):
+        total = total + padded[..., k:k + n]
+    np.testing.assert_array_equal(run.score()[..., :n], total / np.float32(width))
+    np.testing.assert_array_equal(run.evict()[0][..., :n], total / np.float32(width))
+
+
 def test_pool_shift(handle):
     case = Case("shift", 1, 8, 2, 64, 400, 32, 50, 5, 0, 0.9, "f32", 0, "normal", 6)
     inp = make_inputs(case)
