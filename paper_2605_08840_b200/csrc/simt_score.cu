@@ -286,7 +286,9 @@ __global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T
   const T* Qh = Q + ((long long)b * p.Hq + (long long)h * p.G) * p.w * d;
   const float* Oh = O_f32 + (long long)bh * R * d;
   const bool gmax = p.group == RESTKV_GROUP_MAX;
-  for (int i = tid; i < p.w; i += kThreads) wt[i] = temporal_weight(p.temporal, ema_decay, p.w, i);
+  // (negative: the row does not count at all; 0 times the NaN of an older query would be a NaN)
+  for (int i = tid; i < p.w; i += kThreads)
+    wt[i] = p.temporal == RESTKV_TEMPORAL_NONE && i != p.w - 1 ? -1.f : temporal_weight(p.temporal, ema_decay, p.w, i);
   // The kernel before this one (the combine, or what takes its place) lets it start only after its own wait, so that Q, K and V,
   // which lie further back in the stream, may be read at once; O, m and l may not.
   load_rows<T>(Ks, K + (long long)b * p.ksb + (long long)h * p.ksh + (long long)j0 * p.ksn, p.ksn, kTB, valid, d);
@@ -361,13 +363,13 @@ __global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const int r = rl + 32 * i, row = row0 + r;
-      const float weight = r < rows ? wt[row % p.w] : 0.f;
+      const float weight = r < rows ? wt[row % p.w] : -1.f;
 #pragma unroll
       for (int t = 0; t < kTok; ++t) {
         const int tok = tl + 8 * t;
         const float I = indicator_of(p.indicator, expf(s[i][t] * p.scale - fm[i]), fl[i], ss[i][t], vlen_s[tok]);
         if (I_raw && r < rows && tok < valid) I_raw[((long long)bh * R + row) * p.n + j0 + tok] = I;
-        const float wI = r < rows ? weight * I : 0.f;
+        const float wI = weight >= 0.f ? weight * I : 0.f;
         if (gmax) Iw[r * (kTB + 1) + tok] = wI;
         else acc[t] += wI;
       }

@@ -1016,6 +1016,24 @@ def test_variant_at_full_size(handle):
     variant_check(handle, inp, VARIANTS[5], fused=True)
 
 
+@pytest.mark.parametrize("group", [rk.GROUP_MEAN, rk.GROUP_MAX])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_without_smoothing_only_the_newest_query_counts(handle, dtype, group):
+    """TEMPORAL_NONE on the SIMT kernels: whatever the older window queries are, also NaN, the scores are those of the newest."""
+    inp = make_inputs(CONFIGS["cfg1b"].with_(dtype=dtype))
+    handle.set_variant(temporal=rk.TEMPORAL_NONE, group=group)
+    try:
+        run = DeviceRun(handle, inp)
+        clean = run.score().copy()
+        run.Q[:, 1, :10] = float("nan")
+        run.Q[:, 6, 30] = float("nan")
+        np.testing.assert_array_equal(run.score(), clean)
+    finally:
+        handle.set_variant()
+    ref = oracle_scores(inp, temporal_mode=3, group_mode=group)
+    assert_scores_close(clean, ref.scores, TOL[dtype])
+
+
 def test_set_variant_validates_its_fields(handle):
     for bad in ((3, 0, 0, 0), (0, 4, 0, 0), (0, 0, 2, 0), (0, 0, 0, 2), (-1, 0, 0, 0)):
         with pytest.raises(rk.RestKVError) as e:
