@@ -11,6 +11,8 @@
 // reuse_l2 only as many heads are in flight as fit in L2, so that phase C re-reads K and V from there.
 // Every wait on data is bounded: a wait that runs out sets the sticky timeout bit, and the CTA skips the rest of
 // its work and still releases its tensor memory.
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace restkv {
@@ -28,8 +30,11 @@ static_assert(kFFirstWorker * kFRegsControl + kFWorkerWarps * kFRegsWorker <= (k
               "the register split must fit the pool the CTA is launched with");
 constexpr int kFRing = 4;                         // 32 KB tile slots after Q | O' | aug | ones
 constexpr size_t kFSmem = 2 * kTileBytes + kAugBytes + kOnesBytes + kFRing * kTileBytes + 1024;
-// A row's weights add up to 1, so that at most 8 tokens of a head (7 but for rounding) exceed kHeavyA = 1/8 in it.
-constexpr int kMaxHeavy = 8 * kRows;
+// A row's weights add up to 1, so that at most 8 tokens of a head (7 but for rounding) exceed kHeavyA = 1/8 in it: the list of
+// (token, column group) units with such a weight.  With it go four sums and four links of each unit, those of the first kNear
+// units in shared memory, the others' in the CTA's slot of part_O (64 KB, idle in phase C), where the 32 logits of up to
+// kHeavyDumps units lie, too.
+constexpr int kMaxHeavy = 8 * kRows, kNear = 32, kHeavyDumps = (kRows * 128 - 8 * kMaxHeavy) / 32;
 constexpr int kFVSlots = 3;                       // phase A: V slots = ring 2, ring 3 and the (then unused) O' tile
 
 struct FusedArgs {
@@ -158,9 +163,11 @@ struct Ctx {
   FusedBars* B;
   int* abort_flag;
   float* sm_stats;         // [6][128] floats: row maxima of the column halves [slot][half], then (m, l) hand-over
+  const float* row_weight; // [128] temporal weight of each window row but for t_scale
   volatile int* look;      // [2] whether a weight of the tile in accumulator set s may exceed kHeavyA
   float* vn_s;             // [4][128] ||v||^2 of the last four tiles of phase C (from_lse only)
-  int* heavy;              // (over sm_stats, which phase A no longer needs) [0]: count, then the tokens of this CTA's share that have a weight above kHeavyA in some row
+  int* heavy;              // (over sm_stats, which phase A no longer needs) [0]: count, then the units of this CTA's share that
+                           //  have a weight above kHeavyA: token * 4 + column group, the sign set for a token's first unit
   int warp, lane;
 };
 
@@ -751,12 +758,25 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
   }
 }
 
-// Eight values per lane -> sums over the warp: lane L returns the sum of value L / 4 (three exchanges halve the values,
-// two finish).
-__device__ __forceinline__ float reduce8_warp(float* v, int lane) {
+__device__ __forceinline__ float* heavy_scratch(const FusedArgs& a) { return a.part_O + (long long)blockIdx.x * kRows * kHeadDim; }
+__device__ __forceinline__ float* heavy_logits(const FusedArgs& a, int unit) { return heavy_scratch(a) + 8 * kMaxHeavy + unit * 32; }
+__device__ __forceinline__ float* heavy_sums(const Ctx& cx, const FusedArgs& a, int unit) {
+  return (unit < kNear ? cx.sm_stats + 1 + kMaxHeavy : heavy_scratch(a)) + 4 * unit;
+}
+__device__ __forceinline__ int4* heavy_links(const Ctx& cx, const FusedArgs& a, int unit) {
+  return reinterpret_cast<int4*>(unit < kNear ? cx.sm_stats + 1 + kMaxHeavy + 4 * kNear : heavy_scratch(a) + 4 * kMaxHeavy) + unit;
+}
+// The second of two heads' sums of each token of a head group (w = 64, maximum over the heads), where tile_max has been used up.
+__device__ __forceinline__ float* second_head(const FusedArgs& a, int bh) {
+  return a.tile_max + (long long)bh * ((a.n_kv + kTile - 1) / kTile) * kTile;
+}
+
+// N values per lane (8 or 16) -> sums over the warp: lane L returns the sum of value L * N / 32.  Each exchange halves the
+// values that a lane still holds.
+template <int N>
+__device__ __forceinline__ float reduce_warp(float* v, int lane) {
 #pragma unroll
-  for (int half = 4; half > 0; half >>= 1) {
-    const int bit = half * 4;
+  for (int half = N / 2, bit = 16; half > 0; half >>= 1, bit >>= 1) {
     const bool up = (lane & bit) != 0;
 #pragma unroll
     for (int i = 0; i < half; ++i) {
@@ -765,118 +785,196 @@ __device__ __forceinline__ float reduce8_warp(float* v, int lane) {
     }
   }
   float r = v[0];
-  r += __shfl_xor_sync(0xffffffffu, r, 2);
-  return r + __shfl_xor_sync(0xffffffffu, r, 1);
+#pragma unroll
+  for (int bit = 16 / N; bit > 0; bit >>= 1) r += __shfl_xor_sync(0xffffffffu, r, bit);
+  return r;
 }
 
-// The tokens that phase C has noted (a weight above kHeavyA in some window row: an attention sink has one in nearly every
-// row) are scored again from K, V, Q and O themselves: the expansion ||o||^2 + ||v||^2 - 2 o.v cancels when o approaches v,
-// and 1 / (1 - A) amplifies what is left.  All sixteen worker warps take one token together, eight rows each with their
-// loads side by side, so that a token costs about two L2 round trips; done inside the tile's epilogue, a row after the
-// other, a sink took the CTA that owned it 17 us.  After the loop over the tiles, so that none of it takes registers there.
-// Under the output projection the expansion (o - 2 v) . (Mt o) + v^T Mt v from exact dot products serves up to A = 0.9,
+// Phase C notes a (token, column group) that holds a weight above kHeavyA and leaves its share out of the token's score; here
+// the 32 rows of each such unit are scored with exact distances: the expansion ||o||^2 + ||v||^2 - 2 o.v cancels when o
+// approaches v, and 1 / (1 - A) amplifies what is left.  An attention sink is one token with four units, a head that copies a
+// passage has a hundred tokens with one unit each.  Four warps share the units of a column group, eight rows each, whose O is
+// loaded once; the next unit's V is on its way while one is worked on, and no barrier is met until all units are done.  After
+// the loop over the tiles, so that none of it takes registers there.  Measured, 8 heads, 3000 / 16384 rows: one sink in every
+// row 40 / 63 us (without one 36 / 60); 128 tokens in two tiles, one heavy row each, 51 / 78 us (185 / 327 when every token took
+// all sixteen warps and a barrier, 58 / 84 when each pair was done within its tile, one after the other, which a sink paid for).
+// The weights come from the same logits as the normalisers, so that the truncation of the tensor core's sums (2.5e-6 of a sink's
+// weight) cancels: phase C's own, which it has written to the CTA's idle partial, or, against a given log-sum-exp (and where there
+// are more units than kHeavyDumps), exact dot products.
+// Under the output projection the expansion o^T Mt o - 2 v . (Mt o) + v^T Mt v from exact dot products serves up to A = 0.9,
 // the full form (o - v) . (Mt o - Mt v) beyond.
-template <int kW, bool kProj>
+template <int kW, bool kLse, bool kProj>
 __device__ void heavy_pass(const Ctx& cx, const FusedArgs& a, int bh) {
   constexpr int kG = kRows / kW;
-  const int lane = cx.lane, wq = cx.warp - kFFirstWorker;
-  named_barrier_sync(1, kFWorkerWarps * 32);   // every warp has noted its tokens, and I_hat of the share is written
+  int lane = cx.lane, wq = cx.warp - kFFirstWorker;
+  asm volatile("" : "+r"(lane), "+r"(wq), "+r"(bh));   // nothing derived from them for this pass occupies registers in the loop before
+  named_barrier_sync(1, kFWorkerWarps * 32);   // every warp has noted its units, and I_hat of the share is written
   const int count = min(cx.heavy[0], kMaxHeavy);
-  if (count > 0) {
-    const int b = bh / a.Hkv, h = bh % a.Hkv;
-    const float c2 = a.scale * kLog2e;
-    const bool group_max = a.group_max != 0;
-    const __nv_bfloat16* Kh = a.K + (long long)b * a.ksb + (long long)h * a.ksh + lane * 4;
-    const __nv_bfloat16* Vh = a.V + (long long)b * a.vsb + (long long)h * a.vsh + lane * 4;
-    const int row0 = wq * 8, g = row0 / kW;
-    const long long off0 = ((long long)bh * kRows + row0) * kHeadDim + lane * 4;
-    const float M2 = a.row_M2[(long long)bh * kRows + row0 + (lane >> 2)];
-    int done = 0;
-    for (int e = 0; e < count; ++e) {
-      const int j = cx.heavy[1 + e];
-      bool seen = false;   // several warpgroups note the same token
-      for (int k = lane; k < e; k += 32) seen |= cx.heavy[1 + k] == j;
-      if (__any_sync(0xffffffffu, seen)) continue;
-      auto unpack = [](uint2 u) {
-        return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
-                           __uint_as_float(u.y & 0xFFFF0000u));
-      };
-      const float4 kj = unpack(*reinterpret_cast<const uint2*>(Kh + (long long)j * a.ksn));
-      const float4 vj = unpack(*reinterpret_cast<const uint2*>(Vh + (long long)j * a.vsn));
-      float part[8];
-      float4 o[8];
+  if (count == 0) return;
+  const int b = bh / a.Hkv, h = bh % a.Hkv;
+  const float c2 = a.scale * kLog2e;
+  const bool group_max = a.group_max != 0;
+  const __nv_bfloat16* Kh = a.K + (long long)b * a.ksb + (long long)h * a.ksh + lane * 4;
+  const __nv_bfloat16* Vh = a.V + (long long)b * a.vsb + (long long)h * a.vsh + lane * 4;
+  float* const I_head = a.I_hat + (long long)bh * a.n;
+  const int row0 = wq * 8, cgp = wq >> 2, g = row0 / kW;   // this warp's rows and their column group
+  const long long off0 = ((long long)bh * kRows + row0) * kHeadDim + lane * 4;
+  auto unpack = [](uint2 u) {
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                       __uint_as_float(u.y & 0xFFFF0000u));
+  };
+  float4 rows[8];   // O, under the projection Mt o
 #pragma unroll
-      for (int i = 0; i < 8; ++i) o[i] = *reinterpret_cast<const float4*>(a.O_f32 + off0 + i * kHeadDim);
+  for (int r = 0; r < 8; ++r) rows[r] = *reinterpret_cast<const float4*>((kProj ? a.O_proj : a.O_f32) + off0 + r * kHeadDim);
+  const int own = wq * 32 + lane;   // the unit whose token this thread may add up in the end
+  const float own_before = own < count ? I_head[(cx.heavy[1 + own] & 0x7fffffff) >> 2] : 0.f;
+
+  // The units of this warp's column group.  The eight rows' sums of two units (or, with kDot, the logits' and the distances'
+  // sums of one) are reduced together: sixteen values, of which lanes 2i and 2i + 1 end up with value i.
+  auto units = [&](auto dot_tag) {
+    constexpr bool kDot = decltype(dot_tag)::value;
+    constexpr int kU = kDot ? 1 : 2;
+    const int my_u = kDot ? 0 : lane >> 4, row = row0 + ((lane >> 1) & 7);
+    const float weight = cx.row_weight[row];
+    const float M2 = kDot ? a.row_M2[(long long)bh * kRows + row] : 0.f;
+    uint2 q[8];
+    if (kLse && !kProj) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float4 q = unpack(*reinterpret_cast<const uint2*>(a.Q + off0 + i * kHeadDim));
-        part[i] = (q.x * kj.x + q.y * kj.y) + (q.z * kj.z + q.w * kj.w);
-      }
-      const float u = ex2_approx(M2 - c2 * reduce8_warp(part, lane));   // 1 / A of row row0 + lane / 4
-      float x;
-      if (!kProj) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float d0 = o[i].x - vj.x, d1 = o[i].y - vj.y, d2 = o[i].z - vj.z, d3 = o[i].w - vj.w;
-          part[i] = (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
-        }
-        x = reduce8_warp(part, lane);
-      } else {
-        const bool extreme = __any_sync(0xffffffffu, u < 1.f / 0.9f);
-        float4 mv = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (extreme) {
-          const float* Mt = a.proj_Mt + (long long)(h * kG + g) * kHeadDim * kHeadDim + lane * 4;
-#pragma unroll 4
-          for (int k = 0; k < kHeadDim; ++k) {
-            const float own = (k & 3) == 0 ? vj.x : (k & 3) == 1 ? vj.y : (k & 3) == 2 ? vj.z : vj.w;
-            const float vk = __shfl_sync(0xffffffffu, own, k >> 2);
-            const float4 m = __ldg(reinterpret_cast<const float4*>(Mt + k * kHeadDim));
-            mv.x = fmaf(m.x, vk, mv.x); mv.y = fmaf(m.y, vk, mv.y); mv.z = fmaf(m.z, vk, mv.z); mv.w = fmaf(m.w, vk, mv.w);
-          }
-        }
-        const float vs = extreme ? 1.f : 2.f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float4 op = *reinterpret_cast<const float4*>(a.O_proj + off0 + i * kHeadDim);
-          part[i] = (fmaf(-vs, vj.x, o[i].x) * (op.x - mv.x) + fmaf(-vs, vj.y, o[i].y) * (op.y - mv.y)) +
-                    (fmaf(-vs, vj.z, o[i].z) * (op.z - mv.z) + fmaf(-vs, vj.w, o[i].w) * (op.w - mv.w));
-        }
-        x = reduce8_warp(part, lane);
-        if (!extreme) x += a.vmv[((long long)bh * kG + g) * a.n_kv + j];
-        x = fmaxf(x, 0.f);
-      }
-      const float um = u - 1.f;
-      const float I = x * rsqrt_approx(fmaf(x * um, um, 1e-36f));
-      float* buf = cx.sm_stats + 1 + kMaxHeavy + (done & 1) * kRows;
-      if ((lane & 3) == 0) {
-        buf[row0 + (lane >> 2)] = I;
-        if (a.I_raw) a.I_raw[((long long)bh * kRows + row0 + (lane >> 2)) * a.n + j] = I;
-      }
-      named_barrier_sync(1, kFWorkerWarps * 32);
-      if (wq == (done & (kFWorkerWarps - 1))) {   // one warp adds the token up; the others go on to the next one
-        float r[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int row = k * 32 + lane, i = row % kW;
-          r[k] = buf[row] * powf(a.t_decay, (float)(kW - 1 - i)) * (i == 0 ? a.t_seed_first : 1.f) *
-                 (i == kW - 1 ? a.t_seed_last : 1.f);
-#pragma unroll
-          for (int off = 1; off < 32; off <<= 1) {
-            const float other = __shfl_xor_sync(0xffffffffu, r[k], off);
-            r[k] = (off >= kW && group_max) ? fmaxf(r[k], other) : r[k] + other;   // over a query head's window, then over heads
-          }
-        }
-        float tot;
-        if (!group_max || kW == 128) tot = (r[0] + r[1]) + (r[2] + r[3]);
-        else if (kW == 64) tot = fmaxf(r[0] + r[1], r[2] + r[3]);
-        else tot = fmaxf(fmaxf(r[0], r[1]), fmaxf(r[2], r[3]));
-        if (lane == 0) a.I_hat[(long long)bh * a.n + j] = tot * a.t_scale / (group_max ? 1.f : (float)kG);
-      }
-      ++done;
+      for (int r = 0; r < 8; ++r) q[r] = *reinterpret_cast<const uint2*>(a.Q + off0 + r * kHeadDim);
     }
-    named_barrier_sync(1, kFWorkerWarps * 32);
-    if (wq == 0 && lane == 0) cx.heavy[0] = 0;
+    float on = 0.f;   // o^T Mt o of the lane's row
+    if (kProj) {
+      float part[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const float4 o = *reinterpret_cast<const float4*>(a.O_f32 + off0 + r * kHeadDim);
+        part[r] = (o.x * rows[r].x + o.y * rows[r].y) + (o.z * rows[r].z + o.w * rows[r].w);
+      }
+      on = __shfl_sync(0xffffffffu, reduce_warp<8>(part, lane), ((lane >> 1) & 7) * 4);
+    }
+#pragma unroll 1
+    for (int e0 = 0; e0 < count; e0 += 32) {
+      const int key = e0 + lane < count ? cx.heavy[1 + e0 + lane] & 0x7fffffff : ~cgp;
+      unsigned int todo = __ballot_sync(0xffffffffu, (key & 3) == cgp);
+      uint2 v_next[kU], k_next = make_uint2(0u, 0u);   // the next units' rows of V (and K) ...
+      int e_next = -1, j_next = 0;                     // ... and this lane's unit among them (-1: none)
+      float s_next = 0.f;
+      auto request = [&]() {
+        e_next = -1;
+#pragma unroll
+        for (int i = 0; i < kU; ++i) {
+          const int src = (__ffs((int)todo) - 1) & 31, j = __shfl_sync(0xffffffffu, key, src) >> 2;
+          v_next[i] = make_uint2(0u, 0u);
+          if (todo) {
+            v_next[i] = *reinterpret_cast<const uint2*>(Vh + (long long)j * a.vsn);
+            if (kDot) k_next = *reinterpret_cast<const uint2*>(Kh + (long long)j * a.ksn);
+            if (my_u == i) { e_next = e0 + src; j_next = j; }
+          }
+          todo &= todo - 1;
+        }
+        if (!kDot && e_next >= 0) s_next = heavy_logits(a, e_next)[row & 31];
+      };
+      request();
+#pragma unroll 1
+      while (__any_sync(0xffffffffu, e_next >= 0)) {
+        float4 v[kU];
+#pragma unroll
+        for (int i = 0; i < kU; ++i) {
+          v[i] = unpack(v_next[i]);
+          if (!kProj) v[i] = make_float4(-v[i].x, -v[i].y, -v[i].z, -v[i].w);
+        }
+        const float4 k = unpack(k_next);
+        const int e = e_next, j = j_next;
+        const float logit = s_next;
+        request();
+        float part[16];
+        if (kDot) {
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            const float4 qr = unpack(kLse && !kProj ? q[r] : *reinterpret_cast<const uint2*>(a.Q + off0 + r * kHeadDim));
+            const f32x2 p2 = f2_fma(f2_make(qr.z, qr.w), f2_make(k.z, k.w), f2_mul(f2_make(qr.x, qr.y), f2_make(k.x, k.y)));
+            part[r] = f2_lo(p2) + f2_hi(p2);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < kU; ++i)
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            f32x2 x01 = f2_make(rows[r].x, rows[r].y), x23 = f2_make(rows[r].z, rows[r].w);
+            f32x2 y01 = f2_make(v[i].x, v[i].y), y23 = f2_make(v[i].z, v[i].w);   // (-v without the projection)
+            if (!kProj) {
+              x01 = y01 = f2_add(x01, y01);
+              x23 = y23 = f2_add(x23, y23);
+            }
+            const f32x2 p2 = f2_fma(x23, y23, f2_mul(x01, y01));
+            part[(kDot ? 8 : 8 * i) + r] = f2_lo(p2) + f2_hi(p2);
+          }
+        float x = reduce_warp<16>(part, lane), u;   // ||o - v||^2 and 1 / A of this lane's pair
+        if (kDot) {
+          const float other = __shfl_xor_sync(0xffffffffu, x, 16);
+          u = ex2_approx(M2 - c2 * (lane < 16 ? x : other));
+          x = lane < 16 ? other : x;
+        } else {
+          u = ex2_approx(-c2 * logit);
+        }
+        if (kProj) {
+          x = fmaxf(on - 2.f * x + (e >= 0 ? a.vmv[((long long)bh * kG + g) * a.n_kv + j] : 0.f), 0.f);
+          for (int i = 0; i < kU; ++i) {
+            if (!__any_sync(0xffffffffu, e >= 0 && my_u == i && u < 1.f / 0.9f)) continue;
+            float4 mv = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float* Mt = a.proj_Mt + (long long)(h * kG + g) * kHeadDim * kHeadDim + lane * 4;
+            const float4 vi = i == 0 ? v[0] : v[kU - 1];
+#pragma unroll 4
+            for (int d = 0; d < kHeadDim; ++d) {
+              const float own_v = (d & 3) == 0 ? vi.x : (d & 3) == 1 ? vi.y : (d & 3) == 2 ? vi.z : vi.w;
+              const float vd = __shfl_sync(0xffffffffu, own_v, d >> 2);
+              const float4 m = __ldg(reinterpret_cast<const float4*>(Mt + d * kHeadDim));
+              mv.x = fmaf(m.x, vd, mv.x); mv.y = fmaf(m.y, vd, mv.y); mv.z = fmaf(m.z, vd, mv.z); mv.w = fmaf(m.w, vd, mv.w);
+            }
+            float full[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+              const float4 o = *reinterpret_cast<const float4*>(a.O_f32 + off0 + r * kHeadDim);
+              full[r] = ((o.x - vi.x) * (rows[r].x - mv.x) + (o.y - vi.y) * (rows[r].y - mv.y)) +
+                        ((o.z - vi.z) * (rows[r].z - mv.z) + (o.w - vi.w) * (rows[r].w - mv.w));
+            }
+            const float xf = __shfl_sync(0xffffffffu, reduce_warp<8>(full, lane), ((lane >> 1) & 7) * 4);
+            if (my_u == i) x = fmaxf(xf, 0.f);
+          }
+        }
+        const float um = u - 1.f;
+        const float I = x * rsqrt_approx(fmaf(x * um, um, 1e-36f));
+        if (a.I_raw && e >= 0 && (lane & 1) == 0 && (!kDot || lane < 16)) a.I_raw[((long long)bh * kRows + row) * a.n + j] = I;
+        float sum = weight * I;
+#pragma unroll
+        for (int off = 2; off < 16; off <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+        if (e >= 0 && (kDot ? lane == 0 : (lane & 15) == 0)) heavy_sums(cx, a, e)[wq & 3] = sum;
+      }
+    }
+  };
+  // (all of them one way or the other: which unit comes first differs from run to run)
+  if (!kLse && count <= kHeavyDumps) units(std::false_type());
+  if (kLse || count > kHeavyDumps) units(std::true_type());
+  named_barrier_sync(1, kFWorkerWarps * 32);
+  // the shares of a token's units join its score in the order of the column groups, by the thread of its first one
+  const float scale = a.t_scale / (group_max ? 1.f : (float)kG);
+  for (int e = own; e < count; e += kFWorkerWarps * 32) {
+    if (cx.heavy[1 + e] >= 0) continue;
+    const int j = (cx.heavy[1 + e] & 0x7fffffff) >> 2;
+    const int4 link = *heavy_links(cx, a, e);
+    auto share = [&](int unit) {
+      if (unit == 0) return 0.f;
+      const float4 p = *reinterpret_cast<const float4*>(heavy_sums(cx, a, unit - 1));
+      return (kW == 16 && group_max ? fmaxf(p.x + p.y, p.z + p.w) : (p.x + p.y) + (p.z + p.w)) * scale;
+    };
+    const float s0 = share(link.x), s1 = share(link.y), s2 = share(link.z), s3 = share(link.w);
+    const float before = e == own ? own_before : I_head[j];
+    if (!group_max || kW == 128) I_head[j] = before + ((s0 + s1) + (s2 + s3));
+    else if (kW == 64)   // the two heads' sums without the units, as the join of the shares has left them
+      I_head[j] = fmaxf(a.vnorm[(long long)bh * a.n_kv + j] + (s0 + s1), second_head(a, bh)[j] + (s2 + s3));
+    else I_head[j] = fmaxf(before, fmaxf(fmaxf(s0, s1), fmaxf(s2, s3)));
   }
+  if (wq == 0 && lane == 0) cx.heavy[0] = 0;   // (the CTA meets once more before anything is noted again)
 }
 
 // kInd: 0 = Eq. 7; 1 = the attention weight alone; 2 = attention weight times ||v|| (Appendix G.1); 3 = Eq. 7 with
@@ -927,6 +1025,25 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
   const int g_cols = (cgp * 32) / kW;
   const float* vn_head = kProj ? a.vmv + ((long long)bh * kG + g_cols) * a.n_kv : a.vnorm + (long long)bh * a.n_kv;
   float* I_head = a.I_hat + (long long)bh * n;
+  // A share of -(u + 1): unit u is left out; the links between a token's units go to its first one.
+  auto store_score = [&](int j, const float (*r)[kTile]) {
+    float r0 = r[0][t], r1 = r[1][t], r2 = r[2][t], r3 = r[3][t];
+    if (kEq7 && fminf(fminf(r0, r1), fminf(r2, r3)) < 0.f) {
+      const int4 link = make_int4(r0 < 0.f ? (int)-r0 : 0, r1 < 0.f ? (int)-r1 : 0, r2 < 0.f ? (int)-r2 : 0, r3 < 0.f ? (int)-r3 : 0);
+      const int first = link.x ? link.x : link.y ? link.y : link.z ? link.z : link.w;
+      *heavy_links(cx, a, first - 1) = link;
+      cx.heavy[first] |= (int)0x80000000;
+      r0 = r0 < 0.f ? 0.f : r0;
+      r1 = r1 < 0.f ? 0.f : r1;
+      r2 = r2 < 0.f ? 0.f : r2;
+      r3 = r3 < 0.f ? 0.f : r3;
+    }
+    I_head[j] = join_shares(r0, r1, r2, r3);
+    if (kEq7 && kW == 64 && group_max) {   // both heads' sums, should units be left out of them (the places are used up)
+      a.vnorm[(long long)bh * a.n_kv + j] = r0 + r1;
+      second_head(a, bh)[j] = r2 + r3;
+    }
+  };
   float* raw_head = (a.I_raw && !kLse) ? a.I_raw + (long long)bh * kRows * n : nullptr;
   bool ok = true;
   float vn_next = 0.f;
@@ -960,10 +1077,11 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
       const int rs = (it - 1) & 3;
       ok = ok && mbar_wait(&B->red_full[rs], (uint32_t)((it - 1) >> 2) & 1u, abort_flag, dev_status, kDevTimeout, a.wait_limit);
       const int jp = (tile0 + T - it) * kTile + t;
-      if (ok && jp < n) I_head[jp] = join_shares(red[rs][0][t], red[rs][1][t], red[rs][2][t], red[rs][3][t]);
+      if (ok && jp < n) store_score(jp, red[rs]);
     }
     ok = ok && mbar_wait(&B->acc_full[s], par, abort_flag, dev_status, kDevTimeout, a.wait_limit);
     float tot = 0.f;
+    int unit = kMaxHeavy;   // this lane's place in the list of heavy units
     if (ok) {
       tc_fence_after();
       const int j = (tile0 + T - 1 - it) * kTile + t;
@@ -1074,21 +1192,33 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
             for (int u = 0; u < 8; ++u) mx = fmaxf(mx, sv[u]);
           }
         }
+        if (kEq7 && look && __any_sync(0xffffffffu, mx > heavy_thr && j < n)) {
+          if (mx > heavy_thr && j < n) unit = atomicAdd(cx.heavy, 1);
+          float* logits = heavy_logits(a, unit);
+#pragma unroll 1
+          for (int c = 0; c < 4; ++c) {
+            float sv[8];
+            tmem_ld8(tS + c * 8, sv);
+            tmem_wait_ld();
+            if (unit < kHeavyDumps) {
+              *reinterpret_cast<float4*>(logits + c * 8) = make_float4(sv[0], sv[1], sv[2], sv[3]);
+              *reinterpret_cast<float4*>(logits + c * 8 + 4) = make_float4(sv[4], sv[5], sv[6], sv[7]);
+            }
+          }
+        }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&B->acc_empty[s]);
       }
-      // only Eq. 7 has the factor 1 / (1 - A) and the distance that need the exact form near A = 1: those tokens are noted
-      // and done again after the last tile (S' above heavy_thr <=> A > kHeavyA)
-      if (look && mx > heavy_thr && j < n) {
-        const int e = atomicAdd(cx.heavy, 1);
-        if (e < kMaxHeavy) cx.heavy[1 + e] = j;
-      }
+      // only Eq. 7 has the factor 1 / (1 - A) and the distance that need the exact form near A = 1: those units are noted
+      // and done after the last tile (S' above heavy_thr <=> A > kHeavyA)
+      if (from_lse && look && mx > heavy_thr && j < n) unit = atomicAdd(cx.heavy, 1);
+      if (unit < kMaxHeavy) cx.heavy[1 + unit] = j * 4 + cgp;
     } else {
       __syncwarp();
       if (lane == 0) mbar_arrive(&B->acc_empty[s]);
     }
-    red[it & 3][cgp][t] = tot * fin_scale;
+    red[it & 3][cgp][t] = kEq7 && unit < kMaxHeavy ? (float)(-1 - unit) : tot * fin_scale;
     __syncwarp();
     if (lane == 0) mbar_arrive(&B->red_full[it & 3]);
   }
@@ -1096,9 +1226,9 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
     const int rs = (T - 1) & 3;
     ok = ok && mbar_wait(&B->red_full[rs], (uint32_t)((T - 1) >> 2) & 1u, abort_flag, dev_status, kDevTimeout, a.wait_limit);
     const int jl = tile0 * kTile + t;   // the last tile processed is the first of the share
-    if (ok && jl < n) I_head[jl] = join_shares(red[rs][0][t], red[rs][1][t], red[rs][2][t], red[rs][3][t]);
+    if (ok && jl < n) store_score(jl, red[rs]);
   }
-  if (kEq7) heavy_pass<kW, kProj>(cx, a, bh);
+  if (kEq7) heavy_pass<kW, kLse, kProj>(cx, a, bh);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1206,7 +1336,9 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   __shared__ __align__(8) FusedBars bars;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag, go_flag, look_flag[2];
-  __shared__ float sm_stats[1 + kMaxHeavy + 2 * kRows];   // phase A's exchange (6 x 128), then the list of heavy tokens
+  __shared__ __align__(16) float sm_heavy[4 + kMaxHeavy + 8 * kNear];   // phase A's exchange (6 x 128), then the heavy units
+  __shared__ float row_weight[kRows];
+  float* const sm_stats = sm_heavy + 3;   // (the units' sums on a 16-byte boundary)
   __shared__ float vn_ring[4 * kTile];
   __shared__ float red[4][4][kTile];   // [tile & 3][warpgroup][token]: each warpgroup's share of the score
 
@@ -1220,6 +1352,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   cx.sm_stats = sm_stats;
   cx.vn_s = vn_ring;
   cx.look = look_flag;
+  cx.row_weight = row_weight;
   cx.heavy = reinterpret_cast<int*>(sm_stats);
   cx.warp = threadIdx.x >> 5;
   cx.lane = threadIdx.x & 31;
@@ -1240,6 +1373,10 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   }
   if (threadIdx.x >= 128 && threadIdx.x < 128 + (int)(kOnesBytes / 4))   // the block of ones (bf16 1.0 = 0x3F80)
     reinterpret_cast<uint32_t*>(cx.gen_base + kOffOnes)[threadIdx.x - 128] = 0x3F803F80u;
+  if (threadIdx.x >= kFThreads - kRows) {
+    const int row = threadIdx.x - (kFThreads - kRows), i = row % kW;
+    row_weight[row] = powf(a.t_decay, (float)(kW - 1 - i)) * (i == 0 ? a.t_seed_first : 1.f) * (i == kW - 1 ? a.t_seed_last : 1.f);
+  }
   fence_proxy_async_smem();
   tc_fence_before();
   __syncthreads();

@@ -802,6 +802,57 @@ def test_large_attention_weights(handle, spec, group):
         handle.set_variant()
 
 
+def _with_copied_passage(case, tokens, stride, first, rows_each):
+    """A head that copies a passage: token first + i * stride draws about a fifth of the attention of `rows_each` window rows (or
+    as much as they have), which are different from token to token."""
+    inp = make_inputs(case)
+    R = case.w * case.group
+    share = min(0.3, 0.8 * R / (tokens * rows_each))
+    logit = np.log(share / (1.0 - share * max(1.0, tokens * rows_each / R)) * 1.65 * case.n) * np.sqrt(case.head_dim)
+    for b in range(case.batch):
+        for h in range(case.n_kv_heads):
+            q = inp.Q[b, h * case.group:(h + 1) * case.group].reshape(R, case.head_dim)
+            for i in range(tokens):
+                some = q[[(i + k * (R // rows_each)) % R for k in range(rows_each)]]
+                inp.K[b, h, first + i * stride] = np.linalg.lstsq(some, np.full(rows_each, logit), rcond=None)[0]
+    inp.K = (round_to_bf16_bits(inp.K).astype(np.uint32) << 16).view(np.float32)
+    return inp
+
+
+@pytest.mark.parametrize("spec", [(32, 8, 2, 0, 128, 1, 200, 1), (32, 32, 8, 32, 200, 1, 256, 2), (32, 8, 2, 0, 100, 19, 3, 1),
+                                  (64, 4, 2, 0, 90, 1, 250, 2), (16, 16, 2, 0, 128, 2, 130, 2), (128, 2, 2, 0, 60, 3, 0, 2)])
+@pytest.mark.parametrize("group", [rk.GROUP_MEAN, rk.GROUP_MAX])
+def test_many_tokens_with_large_weights(handle, spec, group):
+    """Many tokens with a weight above 1/8 in a row or two each: side by side in one thread block, more than it keeps close by and
+    more than it keeps the logits of, and spread over all blocks; from Q, K, V, from given statistics and with the per-query
+    indicators of the adaptive window."""
+    import torch
+    w, Hq, Hkv, tail, tokens, stride, first, rows_each = spec
+    inp = _with_copied_passage(Case("copy", 1, Hq, Hkv, 128, 3000, w, 200, 5, 0, 0.9, "bf16", tail, "normal", 78), tokens, stride, first,
+                               rows_each)
+    c = inp.case
+    A = oracle_scores(inp, want_A=True).A[..., :c.n]
+    units = (A.reshape(Hkv, 4, 32, c.n) > 0.125).any(axis=2).sum(axis=(1, 2))     # (token, 32 rows) of each head
+    assert units.min() > (300 if rows_each * tokens == 400 else 50)
+    _, O, lse = _window_stats(inp, with_A_check=False)
+    handle.set_variant(group=group)
+    try:
+        ref = oracle_scores(inp, group_mode=group)
+        run = DeviceRun(handle, inp)
+        first_time = run.evict()[0].copy()
+        assert_scores_close(first_time, ref.scores, TOL["bf16"])
+        np.testing.assert_array_equal(run.evict()[0], first_time)
+        handle.score_from_lse(run.shape, run.Q, run.K, run.V, torch.from_numpy(O).cuda(), torch.from_numpy(lse).cuda(),
+                              c.ema_decay, run.pool(), run.scores, run.ws)
+        torch.cuda.synchronize()
+        assert_scores_close(run.scores.cpu().numpy(), ref.scores, TOL["bf16"])
+        run = DeviceRun(handle, inp, adaptive_budget=c.budget)
+        scores = run.score(pool=rk.adaptive_pool(1e9, c.width, c.budget))
+        assert_scores_close(scores, ref.scores, TOL["bf16"])
+    finally:
+        handle.set_variant()
+
+
 @pytest.mark.parametrize("spec", [("cfg2", 0), ("cfg2", 32), ("cfg1b", 0)])
 def test_evict_from_lse_matches_oracle(handle, spec):
     """restkv_evict_from_lse: score, select and compact from given window statistics, all three acceptance rules."""
