@@ -186,9 +186,9 @@ def test_config2_is_deterministic(handle):
 
 @pytest.mark.parametrize("spec", [("cfg2", 0, 1024, 7, 0), ("cfg2", 32, 1024, 21, 0), ("cfg2", 0, 37, 1, 0), ("cfg2", 0, 1024, 5, -9),
                                   ("cfg3", 0, 2048, 7, 0), ("cfg3", 0, 16000, 31, 4)])
-def test_selection_inside_the_score_kernel_equals_the_separate_kernel(handle, spec):
-    """restkv_evict on the tensor-core path pools, selects and gathers inside the score kernel by default; with that
-    switched off the separate kernel does: scores, indices and gathered rows must be identical bit for bit."""
+def test_selection_chained_to_the_score_kernel(handle, spec):
+    """The launch of restkv_evict that pools, selects and gathers, chained to the score kernel and in plain stream order: the same
+    bit for bit; the indices are those of a stable sort of the scores, the gathered rows exact copies."""
     name, tail, budget, width, shift = spec
     inp = make_inputs(CONFIGS[name].with_(causal_tail=tail))
     run = DeviceRun(handle, inp, budget=budget)
@@ -201,15 +201,18 @@ def test_selection_inside_the_score_kernel_equals_the_separate_kernel(handle, sp
         handle.set_fused_select(True)
     for x, y in zip(fused, separate):
         np.testing.assert_array_equal(x, y)
+    np.testing.assert_array_equal(fused[1], np.sort(np.argsort(-fused[0], axis=-1, kind="stable")[..., :budget], axis=-1))
+    _, kbits, vbits = inp.device_arrays()
+    assert_compaction_exact(fused[1], kbits, fused[2])
+    assert_compaction_exact(fused[1], vbits, fused[3])
     ref = oracle_scores(inp, width=width, shift=shift)
     assert_scores_close(fused[0], ref.scores, TOL["bf16"])
     assert_selection_valid(fused[1], ref.scores, budget, TOL["bf16"])
 
 
-def test_selection_inside_the_score_kernel_with_ties(handle):
-    """Identical keys (uniform attention) and only two distinct value rows, alternating: the scores of a head fall
-    into two classes of exact ties, so the lower index must win ties exactly as in the separate kernel, also across
-    the boundaries between the head's thread blocks."""
+def test_selection_chained_to_the_score_kernel_with_ties(handle):
+    """Identical keys (uniform attention) and only two distinct value rows, alternating: the scores of a head fall into two classes
+    of exact ties, of which the lower index must win, chained or not, as in a stable sort."""
     case = Case("ties", 1, 4, 1, 128, 5000, 32, 777, 1, 0, 0.9, "bf16", 0, "normal", 3)
     inp = make_inputs(case)
     inp.K[...] = inp.K[:, :, :1]
@@ -225,6 +228,7 @@ def test_selection_inside_the_score_kernel_with_ties(handle):
         handle.set_fused_select(True)
     for x, y in zip(fused, separate):
         np.testing.assert_array_equal(x, y)
+    np.testing.assert_array_equal(fused[1], np.sort(np.argsort(-fused[0], axis=-1, kind="stable")[..., :case.budget], axis=-1))
     ref = oracle_scores(inp)
     assert_selection_valid(fused[1], ref.scores, case.budget, TOL["bf16"])
 
@@ -443,51 +447,56 @@ def test_selection_kernel_edges(handle, spec):
 
 
 @pytest.mark.parametrize("spec", [(3, 2), (7, 3), (1023, 40), (4099, 4098), (25001, 900), (26000, 900), (51300, 2000)])
-@pytest.mark.parametrize("ties", [False, True])
-def test_adaptive_window_row_lengths(handle, spec, ties):
+def test_adaptive_window_row_lengths(handle, spec):
     """The index sums behind the adaptive window: rows that begin anywhere within 16 bytes, of a few keys, with two, one and
-    no buffers in shared memory; with all keys of a row equal (the first B_p of them count)."""
+    no buffers in shared memory."""
     n, budget = spec
-    inp = make_inputs(Case("adapt", 1, 4, 2, 16, n, 6, budget, 1, 0, 0.5, "f32", 0, "normal", n))
-    if ties:
-        inp.K[...] = inp.K[:, :, :1]
-        inp.V[...] = inp.V[:, :, :1] * np.where(np.arange(n) % 2, 1.0, -1.0).astype(np.float32)[:, None]
-    probe = oracle_scores(inp, pool_mode=1, beta=1e9, base_width=1, budget=budget)
-    delta = np.abs(probe.D[..., 0] - probe.D[..., 1])
-    if not ties and n > 4100:
-        assert delta.min() > 0
-    beta = float(delta.max() / 20.5) if delta.max() > 0 else 1.0     # the mean indices enter with a twentieth of their difference
+    for seed in range(n, n + 20):   # (of a few keys, front and rear may keep the same ones)
+        inp = make_inputs(Case("adapt", 1, 4, 2, 16, n, 6, budget, 1, 0, 0.5, "f32", 0, "normal", seed))
+        probe = oracle_scores(inp, pool_mode=1, beta=1e9, base_width=1, budget=budget)
+        delta = np.abs(probe.D[..., 0] - probe.D[..., 1])
+        if delta.max() > 0:
+            break
+    beta = float(delta.max() / 20.5)                                  # the mean indices enter with a twentieth of their difference
     ref = oracle_scores(inp, pool_mode=1, beta=beta, base_width=1, budget=budget)
     x = (probe.D[..., 0] - probe.D[..., 1]) / beta
     settled = np.abs(x - np.round(x)) > 0.02
+    assert settled.any()
     run = DeviceRun(handle, inp, adaptive_budget=budget)
     run.score(pool=rk.adaptive_pool(beta, 1, budget))
     assert handle.poll_status() == rk.RESTKV_OK
-    if not ties:                                                      # (equal in exact arithmetic only: the order is open)
-        assert np.array_equal(run.pool_used.cpu().numpy()[settled], ref.pool[settled])
+    assert np.array_equal(run.pool_used.cpu().numpy()[settled], ref.pool[settled])
 
 
-def test_select_matches_stable_sort_with_ties_and_inf(handle):
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("spec", [(3, 2), (7, 3), (1023, 40), (2049, 1500), (4099, 4098), (25001, 900), (26000, 14000), (51300, 2000)])
+def test_adaptive_window_with_exact_ties(handle, spec, dtype):
+    """Rows of two values only (attention weights over two distinct keys): of equal ones the first count, so that the index sums are
+    known exactly.  The front queries lean on the second part of the cache, the rear ones on the first; the scaling is set so that
+    a mean index that is off by 1e-5 of the difference, to either side, gives another window."""
     import torch
-    rng = np.random.default_rng(3)
-    n_kv = 5000
-    s = rng.standard_normal((2, 3, n_kv)).astype(np.float32)
-    s[0, 0, ::7] = 0.25                       # many ties
-    s[0, 1] = 1.0                             # all equal
-    s[1, 0, -40:] = np.inf
-    s[1, 1] = np.abs(s[1, 1]) * 1e-30         # tiny positives
-    s[1, 2, 100:200] = -s[1, 2, 100:200] - 5  # negatives
-    case = Case("sel", 2, 3, 3, 64, n_kv, 32)
-    shape = shape_of(case)
-    d_s = torch.from_numpy(s).cuda()
-    for B in (1, 2, 31, 32, 33, 1000, 4999, 5000, 9000):
-        keep = min(B, n_kv)
-        idx = torch.empty((2, 3, keep), dtype=torch.int32, device="cuda")
-        ws = torch.empty(handle.workspace_bytes(shape, B), dtype=torch.uint8, device="cuda")
-        handle.select(shape, d_s, B, idx, ws)
-        torch.cuda.synchronize()
-        got = idx.cpu().numpy()
-        np.testing.assert_array_equal(got, oracle.select(s.astype(np.float64), B))
+    n, budget = spec
+    d, w, Hq, Hkv = (16, 6, 4, 2) if dtype == "f32" else (128, 32, 8, 2)
+    inp = make_inputs(Case("ties", 1, Hq, Hkv, d, n, w, budget, 1, 0, 0.5, dtype, 0, "normal", n))
+    a = n // 2
+    inp.K[...] = 0.0
+    inp.K[:, :, :a, 0] = 2.0
+    inp.K[:, :, a:, 1] = 2.0
+    inp.Q[...] = 0.0
+    inp.Q[:, :, :w // 2, 1] = 2.0
+    inp.Q[:, :, w // 2:, 0] = 2.0
+    second_first = np.concatenate([np.arange(a, n), np.arange(a)])[:budget]
+    diff = second_first.sum() / budget - (budget - 1) / 2.0
+    assert diff > 0
+    handle.set_variant(indicator=rk.INDICATOR_ATTENTION)
+    try:
+        run = DeviceRun(handle, inp, adaptive_budget=budget)
+        for steps in (20 + 1e-4, 21 - 1e-4):
+            run.score(pool=rk.adaptive_pool(float(diff / steps), 1, budget))
+            assert handle.poll_status() == rk.RESTKV_OK
+            np.testing.assert_array_equal(run.pool_used.cpu().numpy()[0], [[41, 20]] * Hkv)
+    finally:
+        handle.set_variant()
 
 
 def _key_order(bits):
@@ -975,7 +984,8 @@ def test_variants_from_given_window_statistics(handle, variant):
 
 
 @pytest.mark.parametrize("variant", [VARIANTS[0], VARIANTS[4], VARIANTS[5]])
-def test_variants_with_the_selection_as_its_own_kernel(handle, variant):
+def test_variants_with_the_selection_in_stream_order(handle, variant):
+    """The selection's launch not chained to the score kernel."""
     handle.set_fused_select(False)
     try:
         variant_check(handle, make_inputs(CONFIGS["cfg2"]), variant, path=rk.PATH_TENSOR_CORE, fused=False)
