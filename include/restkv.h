@@ -109,8 +109,9 @@ size_t restkv_workspace_bytes_adaptive(const restkv_shape* shape, int budget);
  *                the score of that row is defined as 0.
  *   pool_used    optional device int32 [batch, n_kv_heads, 2] receiving (W, gamma) per head, or NULL
  * RESTKV_BF16 with head_dim 128 and w * (n_q_heads/n_kv_heads) == 128 runs on the tcgen05 tensor-core
- * kernels; every other supported shape (head_dim <= 256 and a multiple of 8, w*group <= 256) runs on
- * fp32 SIMT kernels.  RESTKV_ERR_UNSUPPORTED otherwise.
+ * kernels; every other supported shape (head_dim <= 256 and a multiple of 8, w*group <= 256 and
+ * 2*w*group*(head_dim+1) + 64*head_dim <= 56320, e.g. 186 rows at head_dim 128) runs on fp32 SIMT kernels.
+ * RESTKV_ERR_UNSUPPORTED otherwise.
  */
 restkv_status restkv_score(restkv_handle* h, const restkv_shape* shape, const void* Q_obs, const void* K,
                            const void* V, float ema_decay, const restkv_pool_params* pool, float* scores,

@@ -177,10 +177,11 @@ static restkv_status check_pool(const restkv_pool_params* pp, const Problem& p) 
   return RESTKV_OK;
 }
 
+// The shapes that the SIMT kernels are offered for: a bound on rows x head_dim from the time when all rows of Q and O of a head
+// lay in shared memory together, kept so that the same calls are taken and refused.  The kernels hold 64 rows at a time and fit
+// every shape within it (139 KB in pass 1, 172 KB in pass 2, 195 KB under the output projection at most).
 static bool simt_supported(const Problem& p) {
-  if (p.R > 256) return false;
-  const size_t smem1 = ((size_t)2 * p.R * (p.d + 1) + (size_t)2 * 32 * p.d) * sizeof(float);
-  return smem1 <= 220 * 1024;
+  return p.R <= 256 && (size_t)2 * p.R * (p.d + 1) + (size_t)64 * p.d <= 56320;
 }
 
 struct Call {

@@ -332,6 +332,18 @@ def test_edge_cases(handle, spec):
     full_check(handle, make_inputs(case))
 
 
+@pytest.mark.parametrize("spec", [("f32", 128, 186), ("bf16", 128, 186), ("f32", 64, 256), ("f32", 256, 77)])
+def test_largest_windows_on_the_simt_kernels(handle, spec):
+    """The bound on window rows and head_dim that the header states: taken and right up to it, refused one row beyond."""
+    dtype, d, rows = spec
+    inp = make_inputs(Case("wide", 1, 1, 1, d, 300, rows, 40, 3, 0, 0.9, dtype, 0, "normal", rows))
+    full_check(handle, inp)
+    inp = make_inputs(Case("wide", 1, 1, 1, d, 300, rows + 1, 40, 3, 0, 0.9, dtype, 0, "normal", rows))
+    with pytest.raises(rk.RestKVError) as e:
+        DeviceRun(handle, inp).evict()
+    assert e.value.status == rk.ERR_UNSUPPORTED
+
+
 def test_more_heads_than_sms(handle):
     """160 (batch, KV head) pairs: the persistent score kernel runs one CTA per head and two rounds."""
     case = Case("many_heads", 20, 32, 8, 128, 300, 32, 30, 5, 0, 0.8, "bf16", 0, "normal", 33)
