@@ -11,8 +11,8 @@
 //     accumulator layout of Q K^T is the operand layout of P V, so the weights never leave the registers.  (tcgen05
 //     would pad the G queries to 128 rows and bring tensor-memory round trips into every tile's chain.)
 // Measured, 8 KV heads of 4 queries, back to back, against the score kernel's attention phases between a padding and an
-// extraction kernel that ran this step before: 2085 rows 30.7 -> 8.2 us (host-bound), 8 x 2176 rows 52 -> 18.4 us
-// (3.9 TB/s), 131072 rows 129 -> 88.6 us (6.1 TB/s).
+// extraction kernel that ran this step before: 2085 rows 30.7 -> 6.4 us (host-bound), 8 x 2176 rows 52 -> 15.7 us
+// (4.5 TB/s), 131072 rows 130 -> 85 us (6.3 TB/s).
 #include <math.h>
 
 #include <cooperative_groups.h>

@@ -130,8 +130,8 @@ __device__ __forceinline__ void pool_slice(const float* taps, int W, bool pool_m
 //     as the rest of that bin is kept as a whole, usually after the second digit;
 //   - what the CTAs of a cluster tell one another (extremes, counts, positions of the kept rows) is put straight into the
 //     shared memory of whoever needs it, with one cluster barrier per exchange.
-// Measured (8 rows, gather included, timed alone): 131072 rows / 2048 kept 51 -> 31 us, 16384 / 1024 29 -> 14 us, 3032 / 1056
-// 10 us; 64 rows of 32768 / 2048 kept 73 (two kernels) -> 38 us.
+// Measured (8 rows, gather included, under ncu: cold and by itself): 131072 rows / 2048 kept 51 -> 22 us, 16384 / 1024 29 -> 15 us,
+// 3032 / 1056 11 us; 64 rows of 32768 / 2048 kept 73 (two kernels) -> 35 us.
 template <int kThreads>
 __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kernel(const __grid_constant__ SelectArgs a) {
   cg::cluster_group cluster = cg::this_cluster();

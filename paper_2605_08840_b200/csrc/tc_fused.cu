@@ -1125,7 +1125,7 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
             f32x2 Iq;
             if (kEq7) {
               // 1/A; one pair in four on the FMA pipe (1/A beyond 2^126 squares to infinity below either way): batch of 8
-              // x 32768 539 -> 522 us, 131072 258 -> 256 us; with every other pair no better, and from given statistics
+              // x 32768 544 -> 531 us, 131072 266 -> 263 us (power-limited clock); with every other pair no better, and from given statistics
               // (no pass 1, so less to wait for) slower
               const f32x2 u2 = (!from_lse && (q & 3) == 3) ? exp2_fma(f2_make(fminf(f2_lo(nt), 126.f), fminf(f2_hi(nt), 126.f)))
                                        : f2_make(ex2_approx(f2_lo(nt)), ex2_approx(f2_hi(nt)));
