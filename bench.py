@@ -72,7 +72,7 @@ def whole_job_value(tokens_per_rank_step, world, steps, total_ms):
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the dominant kernel, from an ncu capture
 # of this workload, together with the digest of the kernel sources the capture was taken on: the figure is reported
 # only while those sources are unchanged, otherwise `traffic` is null.
-KERNEL_TRAFFIC = {"cfg4": {"bytes": 1010462208 + 26525696, "sources_sha256": "f82a3d728a374223d1e35b2382da8b536c90c14671523515fafe765a679176a1"}}
+KERNEL_TRAFFIC = {"cfg4": {"bytes": 1009442304 + 26861824, "sources_sha256": "fc11fed61af69b298b2db263f61ee9bdd4d252aedba8d7e33e926c8ed45e5483"}}
 KERNEL_SOURCES = ("tc_fused.cu", "tc_common.cuh", "sm100_ptx.cuh")
 
 
