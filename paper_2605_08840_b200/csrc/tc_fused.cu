@@ -176,20 +176,42 @@ constexpr uint32_t kOffQ = 0, kOffO = kTileBytes, kOffAug = 2 * kTileBytes, kOff
 __device__ __forceinline__ uint32_t k_slot_off(int i) { return kOffRing + (uint32_t)i * kTileBytes; }
 __device__ __forceinline__ uint32_t v_slot_off(int i) { return i < 2 ? kOffRing + (uint32_t)(2 + i) * kTileBytes : kOffO; }
 
+// K and V leave L2 first: they stream through it (and lines of one priority keep their order among themselves, so that phase C
+// still finds the tiles that phase A read last), while what else the call touches again is small: the partials, the scores, the
+// tensor maps - and the code, whose first run after each synchronisation would otherwise be fetched from HBM, 4 k cycles for
+// each of the merge, its sums and the first tile of phase C.  16384 rows 71 -> 62 us, 32768 projected 137 -> 131 us; phase C's
+// loads alone 66 and 136 us, phase A's alone nothing.
+// One K tile and one V tile of phase C into stage s (ring slots 2s and 2s + 1).
+__device__ __forceinline__ void load_stage_c(const Ctx& cx, const CUtensorMap* tmK, const CUtensorMap* tmV, int b, int h,
+                                             int j0, int s, uint64_t policy) {
+  uint8_t* dK = cx.gen_base + k_slot_off(2 * s);
+  uint8_t* dV = dK + kTileBytes;
+  uint64_t* bar = &cx.B->kv_full[s];
+  mbar_arrive_expect_tx(bar, kStageBytes);
+  tma_load_4d(dK, tmK, bar, 0, j0, h, b, policy);
+  tma_load_4d(dK + kBoxBytes, tmK, bar, 64, j0, h, b, policy);
+  tma_load_4d(dV, tmV, bar, 0, j0, h, b, policy);
+  tma_load_4d(dV + kBoxBytes, tmV, bar, 64, j0, h, b, policy);
+}
+
 // ------------------------------------------------------------------------------------------------
 // Phase A: this CTA's share [tile0, tile0 + T) of one head.
 // Control warps: warp 0 loads (K ring of 2 slots, V ring of 3), warp 1 issues the MMAs (S(it), then O += P V of tile
 // it - 1), warps 2 and 3 reduce ||v_j||^2 of the tokens from the V tiles (even / odd tiles).
 // Tensor memory: tile slot g = it & 1 holds S_g at g*128 (the bf16 P_g overwrites columns [0,32) and [64,96) of
 // it) and O_g at 256 + g*128.
-__device__ void phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtensorMap* tmQ, const CUtensorMap* tmK,
-                        const CUtensorMap* tmV, int bh, int rank, int tile0, int T) {
+// Behind the share's last tiles the loader requests the first two stages of phase C (T2 tiles, walked from the last one), each
+// as its slots fall free: they arrive while the partials are merged and the memory would be idle otherwise, and are out of the
+// way of the merge's own reads.  Returns their number (the loading thread only).
+__device__ int phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtensorMap* tmQ, const CUtensorMap* tmK,
+                       const CUtensorMap* tmV, int bh, int tile0, int T, int T2) {
   FusedBars* B = cx.B;
   int* abort_flag = cx.abort_flag;
   unsigned int* dev_status = a.dev_status;
   const int b = bh / a.Hkv, h = bh % a.Hkv;
   const int warp = cx.warp, lane = cx.lane;
   const uint32_t tmem = cx.tmem;
+  int pre = 0;
 
   if (warp == 0) {
     if (lane == 0 && T > 0) {
@@ -197,23 +219,37 @@ __device__ void phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtenso
       tma_load_3d(cx.gen_base + kOffQ, tmQ, &B->q_full, 0, 0, bh);
       tma_load_3d(cx.gen_base + kOffQ + kBoxBytes, tmQ, &B->q_full, 64, 0, bh);
       int nK = 0, nV = 0;   // K and V tiles requested so far
+      // (not where the per-query indicators are written, as many bytes again: they would push the tiles out at once)
+      const uint64_t policy = a.I_raw ? policy_evict_normal() : policy_evict_first();
       for (int it = 0; it < T; ++it) {
         const int ks = it & 1, vs = it % kFVSlots;
         const int j0 = (tile0 + it) * kTile;
         if (it >= 2 && !mbar_wait(&B->k_empty[ks], ((it >> 1) - 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit)) break;
         uint8_t* dK = cx.gen_base + k_slot_off(ks);
         mbar_arrive_expect_tx(&B->k_full[ks], kTileBytes);
-        tma_load_4d(dK, tmK, &B->k_full[ks], 0, j0, h, b);
-        tma_load_4d(dK + kBoxBytes, tmK, &B->k_full[ks], 64, j0, h, b);
+        tma_load_4d(dK, tmK, &B->k_full[ks], 0, j0, h, b, policy);
+        tma_load_4d(dK + kBoxBytes, tmK, &B->k_full[ks], 64, j0, h, b, policy);
         ++nK;
         if (it >= kFVSlots &&
             !mbar_wait(&B->v_empty[vs], (it / kFVSlots - 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit))
           break;
         uint8_t* dV = cx.gen_base + v_slot_off(vs);
         mbar_arrive_expect_tx(&B->v_full[vs], kTileBytes);
-        tma_load_4d(dV, tmV, &B->v_full[vs], 0, j0, h, b);
-        tma_load_4d(dV + kBoxBytes, tmV, &B->v_full[vs], 64, j0, h, b);
+        tma_load_4d(dV, tmV, &B->v_full[vs], 0, j0, h, b, policy);
+        tma_load_4d(dV + kBoxBytes, tmV, &B->v_full[vs], 64, j0, h, b, policy);
         ++nV;
+      }
+      // ring slots 2s and 2s + 1 make up stage s: the K slots of this phase, then its first two V slots
+      for (int s = 0; s < 2 && s < T2; ++s) {
+        bool free = true;
+        for (int i = 0; i < 2 && free; ++i) {
+          const int step = s == 0 ? 2 : kFVSlots, uses = (T - i + step - 1) / step;
+          uint64_t* bar = s == 0 ? &B->k_empty[i] : &B->v_empty[i];
+          if (uses > 0) free = mbar_wait(bar, (uint32_t)(uses - 1) & 1u, abort_flag, dev_status, kDevTimeout, a.wait_limit);
+        }
+        if (!free) break;
+        load_stage_c(cx, tmK, tmV, b, h, (tile0 + T2 - 1 - s) * kTile, s, policy_evict_first());
+        ++pre;
       }
       if (*(volatile int*)abort_flag) {
         // a wait of this CTA has failed: the tiles requested last may still be on their way into shared memory
@@ -301,13 +337,13 @@ __device__ void phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtenso
       }
     }
   }
+  return pre;
 }
 
 // Worker warps in phase A: four softmax warpgroups, thread = query row; warpgroups g and g + 2 share tile slot g
 // (tokens 0-63 and 64-127 of the tile).  At the end the two slots' (m, l, O) are merged and written as the CTA's
 // partial.
-__device__ void phase_a_worker(const Ctx& cx, const FusedArgs& a, const CUtensorMap* tmQ, const CUtensorMap* tmK,
-                        const CUtensorMap* tmV, int bh, int rank, int tile0, int T) {
+__device__ void phase_a_worker(const Ctx& cx, const FusedArgs& a, int bh, int tile0, int T) {
   FusedBars* B = cx.B;
   int* abort_flag = cx.abort_flag;
   unsigned int* dev_status = a.dev_status;
@@ -420,68 +456,44 @@ __device__ void phase_a_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
     tc_fence_before();
     mbar_arrive(&B->p_full[g]);
   }
+  // ---- merge of the two slots: every thread may read its row of either accumulator, so that warpgroup wgi takes columns
+  //      [32 wgi, 32 wgi + 32) of both and only (m, l) pass through shared memory ----
+  float* st_m = cx.sm_stats;                 // [slot][row]
+  float* st_l = cx.sm_stats + 2 * kRows;     // [slot][half][row]
+  named_barrier_sync(1, kFWorkerWarps * 32); // the exchange of the row maxima is over in both slots
+  if (hf == 0) st_m[g * kRows + row] = ok ? m_ref : -INFINITY;
+  st_l[(g * 2 + hf) * kRows + row] = ok ? l2.x + l2.y : 0.f;
+  // each slot's warps wait for its last O += P V; past the barrier both accumulators are complete
   if (uses > 0 && ok) ok = mbar_wait(&B->pv_done[g], (uint32_t)(uses - 1) & 1u, abort_flag, dev_status, kDevTimeout, a.wait_limit);
-  if (ok && uses > 0) tc_fence_after();
-  const bool have = ok && uses > 0;
-  const float m_mine = have ? m_ref : -INFINITY, l_mine = have ? l2.x + l2.y : 0.f;
-
-  // ---- merge: the halves add their l, then slot 1 hands (m, l, O) to slot 0 through shared memory (the K
-  //      slots are idle: every MMA of this phase has completed once all warpgroups have seen their last
-  //      O += P V).  Each thread moves the 64 columns of O of its half. ----
-  float* xO = reinterpret_cast<float*>(cx.gen_base + k_slot_off(0));   // [128 cols][128 rows] floats, 64 KB
-  float* st_l = cx.sm_stats + 4 * kRows;   // [slot][row]: l of the second half
-  float* st_m1 = cx.sm_stats;              // slot 1's m     (the row-maxima exchange is over)
-  float* st_l1 = cx.sm_stats + kRows;      // slot 1's l
+  tc_fence_before();
   named_barrier_sync(1, kFWorkerWarps * 32);
-  if (hf == 1) st_l[g * kRows + row] = l_mine;
-  named_barrier_sync(1, kFWorkerWarps * 32);
-  const float l_slot = l_mine + (hf == 0 ? st_l[g * kRows + row] : 0.f);   // meaningful in the first half only
-  if (g == 1) {
-    if (hf == 0) { st_m1[row] = m_mine; st_l1[row] = l_slot; }
+  tc_fence_after();
+  const bool have0 = ok && T > 0, have1 = ok && T > 1;
+  const float m0 = st_m[row], m1 = st_m[kRows + row], m = fmaxf(m0, m1);
+  const float a0 = (m0 == -INFINITY) ? 0.f : ex2_approx(m0 - m);
+  const float a1 = (m1 == -INFINITY) ? 0.f : ex2_approx(m1 - m);
+  // The partial lies in pieces of four columns, [32][128 rows][4]: a warp's 32 rows of a piece are 512 bytes in a row for the
+  // stores here, and eight rows of it 128 bytes for the merge.  (As [row][128] every store touched 32 lines; with the second
+  // slot handed over through shared memory the merge of the slots took 8 k cycles, so 2.6 k.)
+  float* Op = a.part_O + (long long)blockIdx.x * kRows * kHeadDim + (wgi * 8 * kRows + row) * 4;
+  const uint32_t tO0 = tmem + 256u + lane_base + (uint32_t)wgi * 32u;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float o[16];
-      if (have) {
-        tmem_ld16(tO + c * 16, o);
-        tmem_wait_ld();
-      } else {
+  for (int c = 0; c < 2; ++c) {
+    float o[16], x[16];
+    tmem_ld16(tO0 + c * 16, o);           // (whatever lies there without tiles)
+    tmem_ld16(tO0 + 128u + c * 16, x);
+    tmem_wait_ld();
 #pragma unroll
-        for (int u = 0; u < 16; ++u) o[u] = 0.f;
-      }
+    for (int u = 0; u < 16; ++u) o[u] = (have0 ? o[u] * a0 : 0.f) + (have1 ? x[u] * a1 : 0.f);
 #pragma unroll
-      for (int u = 0; u < 16; ++u) xO[(hf * 64 + c * 16 + u) * 128 + row] = o[u];
-    }
+    for (int u = 0; u < 16; u += 4)
+      *reinterpret_cast<float4*>(Op + (c * 4 + u / 4) * kRows * 4) = make_float4(o[u], o[u + 1], o[u + 2], o[u + 3]);
   }
-  named_barrier_sync(1, kFWorkerWarps * 32);
-  if (g == 0) {
-    const float m1 = st_m1[row], l1 = st_l1[row];
-    const float m = fmaxf(m_mine, m1);
-    const float a0 = (m_mine == -INFINITY) ? 0.f : ex2_approx(m_mine - m);
-    const float a1 = (m1 == -INFINITY) ? 0.f : ex2_approx(m1 - m);
-    const long long o_idx = (long long)blockIdx.x * kRows + row;
-    float* Op = a.part_O + o_idx * kHeadDim + hf * 64;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float o[16];
-      if (have) {
-        tmem_ld16(tO + c * 16, o);
-        tmem_wait_ld();
-      } else {
-#pragma unroll
-        for (int u = 0; u < 16; ++u) o[u] = 0.f;
-      }
-#pragma unroll
-      for (int u = 0; u < 16; ++u) o[u] = o[u] * a0 + xO[(hf * 64 + c * 16 + u) * 128 + row] * a1;
-#pragma unroll
-      for (int u = 0; u < 16; u += 4)
-        *reinterpret_cast<float4*>(Op + c * 16 + u) = make_float4(o[u], o[u + 1], o[u + 2], o[u + 3]);
-    }
-    if (hf == 0) {
-      a.part_m[o_idx] = m;
-      a.part_l[o_idx] = l_slot * a0 + l1 * a1;
-    }
+  if (wgi == 0) {
+    a.part_m[(long long)blockIdx.x * kRows + row] = m;
+    a.part_l[(long long)blockIdx.x * kRows + row] =
+        (st_l[row] + st_l[kRows + row]) * a0 + (st_l[2 * kRows + row] + st_l[3 * kRows + row]) * a1;
   }
-  fence_proxy_async_smem();   // the hand-over buffer lies in the tile ring, which TMA loads refill next
   tc_fence_before();
 }
 
@@ -498,133 +510,199 @@ __device__ __forceinline__ float4 project_row_warp(const float* __restrict__ Mt,
   return acc;
 }
 
-// x = hi + mid + lo with three bf16 pieces (24 significant bits).
-__device__ __forceinline__ void split3(float x, __nv_bfloat16* out) {
+// x = hi + mid + lo with three bf16 pieces (24 significant bits): their bits.
+__device__ __forceinline__ uint3 split3(float x) {
   const __nv_bfloat16 hi = __float2bfloat16_rn(x);
   const float r1 = x - __bfloat162float(hi);
   const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-  out[0] = hi;
-  out[1] = mid;
-  out[2] = __float2bfloat16_rn(r1 - __bfloat162float(mid));
+  const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
+  return make_uint3(__bfloat16_as_ushort(hi), __bfloat16_as_ushort(mid), __bfloat16_as_ushort(lo));
+}
+__device__ __forceinline__ void split3(float x, __nv_bfloat16* out) {
+  const uint3 p = split3(x);
+  out[0] = __ushort_as_bfloat16((unsigned short)p.x);
+  out[1] = __ushort_as_bfloat16((unsigned short)p.y);
+  out[2] = __ushort_as_bfloat16((unsigned short)p.z);
 }
 
 // ------------------------------------------------------------------------------------------------
-// Phase B: the group's `cpg` partials of one query row are merged by `wpr` warps (lane = four output dims; warp
-// `sub` of the row takes partials sub, sub + wpr, ...), whose sums meet in shared memory and are added in a fixed
-// order: the result does not depend on timing.  Written for phase C: O (fp32), -2 bf16(O), and the row's strip
-// of bf16 constant pieces.  Called by all sixteen worker warps; r < 0 means this warp has no row.
+// Phase B: the group's `cpg` partials are merged.  A CTA takes a run of rows (a power of two, two at least, so that the pieces of
+// four columns that it reads are whole sectors): eight of them where 18 CTAs share a head, 16 KB of each partial.  Thread =
+// (row, four columns), several threads to one where there are few rows, each with every `splits`-th partial; their sums meet
+// in shared memory.  Every order is fixed: the result does not depend on timing.  Written for phase C: O (fp32), -2 bf16(O),
+// and the rows' strips of bf16 constant pieces.  Called by all sixteen worker warps.
+// What bounds it: one trip to L2 for the partials (requested before the weights, which take a trip and two synchronisations
+// of their own), one to write, and the first fetch of its instructions (run twice, the second time takes half).  8 heads of 16384
+// rows: 11.7 k cycles with two warps to a row, 8.1 k so; under the output projection, whose Mt every row's warp read for itself,
+// 27 k and 13 k.
 template <bool kProj>
-__device__ void combine_rows(const FusedArgs& a, int bh, int group, int r, int sub, int wpr, int wq, int lane,
-                             float (*xch)[kHeadDim + 4]) {
+__device__ void combine_rows(const Ctx& cx, const FusedArgs& a, int bh, int group, int rank) {
+  int wt = threadIdx.x - kFFirstWorker * 32, cpg = a.cpg;
+  asm volatile("" : "+r"(wt), "+r"(cpg));   // nothing derived from them here occupies registers in the loops over the tiles
+  const int wq = wt >> 5, lane = wt & 31;
+  int lrb = 1;
+  while ((cpg << lrb) < kRows) ++lrb;
+  const int rb = 1 << lrb, r0 = rank << lrb;
+  if (r0 >= kRows) return;
+  constexpr int kThreads = kFWorkerWarps * 32, kBatch = 9;   // partials in flight per thread
+  const int items = rb * (kHeadDim / 4), per_pass = min(items, kThreads), splits = kThreads / per_pass, split = wt / per_pass;
+  const long long slot0 = (long long)group * cpg;
+  float4 v[kBatch];
+  auto request = [&](int item, int p0) {
+    const float* src = a.part_O + slot0 * kRows * kHeadDim + ((item >> lrb) * kRows + r0 + (item & (rb - 1))) * 4;
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) {
+      const int p = p0 + k * splits;
+      v[k] = *reinterpret_cast<const float4*>(src + (long long)min(p, cpg - 1) * kRows * kHeadDim);
+    }
+  };
+  request(wt % per_pass, split);
+  // ---- weights of the partials, [p][row], and per row 1 / l and the log2 normaliser ----
+  const int pairs = cpg << lrb;   // 512 at most (cpg < 128: below 256)
+  float* sm_w = cx.sm_stats;
+  float* sm_l = sm_w + 512;
+  float* sm_inv = sm_l + 512;
+  float* sm_M2 = sm_inv + kRows;
+  for (int e = wt; e < pairs; e += kThreads) {
+    const long long at = (slot0 + (e >> lrb)) * kRows + r0 + (e & (rb - 1));
+    sm_w[e] = a.part_m[at];
+    sm_l[e] = a.part_l[at];
+  }
+  named_barrier_sync(2, kThreads);
+  // four lanes to a row, or a warp where there are many partials: all rows at once (rb is 4 at most in the second case)
+  const int team = cpg > 32 ? 32 : 4, tl = wt & (team - 1), tr = wt / team;
   float m = -INFINITY, l = 0.f;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (r >= 0) {
-    const long long base = (long long)group * a.cpg * kRows + r;   // + p * kRows
-    // running merge of this warp's partials (all loads of a batch are issued before any is used)
-    constexpr int kBatch = 10;   // loads in flight per lane
+  if (tr < rb)
+    for (int p = tl; p < cpg; p += team) m = fmaxf(m, sm_w[(p << lrb) + tr]);
 #pragma unroll 1
-    for (int p0 = sub; p0 < a.cpg; p0 += kBatch * wpr) {
-      float mp[kBatch], lp[kBatch];
-      float4 v[kBatch];
+  for (int off = team >> 1; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+  if (tr < rb)
+    for (int p = tl; p < cpg; p += team) {
+      const float mp = sm_w[(p << lrb) + tr], w = (mp == -INFINITY) ? 0.f : ex2_approx(mp - m);   // an empty partial weighs 0
+      sm_w[(p << lrb) + tr] = w;
+      l = fmaf(sm_l[(p << lrb) + tr], w, l);
+    }
+#pragma unroll 1
+  for (int off = team >> 1; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+  if (tl == 0 && tr < rb) {
+    sm_inv[tr] = 1.f / l;
+    sm_M2[tr] = m + log2f(l);        // A = exp2(s * c2 - M2)
+  }
+  named_barrier_sync(2, kThreads);
+  // ---- O ----
+  float* on_part = reinterpret_cast<float*>(cx.gen_base + kOffAug);                        // [32 pieces or fewer][rb]
+  float4* split_sum = reinterpret_cast<float4*>(cx.gen_base + kOffAug + kAugBytes / 2);    // [splits - 1][items], rb <= 8
+  for (int item = wt % per_pass; item < items; item += kThreads) {
+    const int r = item & (rb - 1), piece = item >> lrb;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int p0 = split;;) {
 #pragma unroll
       for (int k = 0; k < kBatch; ++k) {
-        const int p = p0 + k * wpr;
-        const bool in = p < a.cpg;
-        const long long pi = base + (long long)(in ? p : p0) * kRows;
-        mp[k] = in ? a.part_m[pi] : -INFINITY;
-        lp[k] = a.part_l[pi];
-        v[k] = *reinterpret_cast<const float4*>(a.part_O + pi * kHeadDim + lane * 4);
+        const int p = p0 + k * splits;
+        if (p < cpg) {
+          const float w = sm_w[(p << lrb) + r];
+          acc.x = fmaf(v[k].x, w, acc.x); acc.y = fmaf(v[k].y, w, acc.y); acc.z = fmaf(v[k].z, w, acc.z); acc.w = fmaf(v[k].w, w, acc.w);
+        }
       }
-#pragma unroll
-      for (int k = 0; k < kBatch; ++k) {
-        const float m_new = fmaxf(m, mp[k]);
-        const float s_old = (m == -INFINITY) ? 0.f : ex2_approx(m - m_new);
-        const float s_p = (mp[k] == -INFINITY) ? 0.f : ex2_approx(mp[k] - m_new);   // an empty partial weighs 0
-        l = l * s_old + lp[k] * s_p;
-        acc.x = acc.x * s_old + v[k].x * s_p;
-        acc.y = acc.y * s_old + v[k].y * s_p;
-        acc.z = acc.z * s_old + v[k].z * s_p;
-        acc.w = acc.w * s_old + v[k].w * s_p;
-        m = m_new;
+      p0 += kBatch * splits;
+      const bool more = p0 < cpg;
+      if (more || item + kThreads < items) request(more ? item : item + kThreads, more ? p0 : split);   // the next ones
+      if (!more) break;
+    }
+    if (splits > 1) {   // (a single pass then: uniform)
+      if (split > 0) split_sum[(split - 1) * items + item] = acc;
+      named_barrier_sync(2, kThreads);
+      if (split > 0) break;
+      for (int k = 0; k < splits - 1; ++k) {
+        const float4 u = split_sum[k * items + item];
+        acc.x += u.x; acc.y += u.y; acc.z += u.z; acc.w += u.w;
       }
     }
-    *reinterpret_cast<float4*>(&xch[wq][lane * 4]) = acc;
-    if (lane == 0) { xch[wq][kHeadDim] = l; xch[wq][kHeadDim + 1] = m; }
-  }
-  named_barrier_sync(2, kFWorkerWarps * 32);
-  if (r < 0 || sub != 0) return;
-  {
-    // the row's wpr warp results, merged in a fixed order
-    float mm = m;
-    for (int k = 1; k < wpr; ++k) mm = fmaxf(mm, xch[wq + k][kHeadDim + 1]);
-    const float s0 = (m == -INFINITY) ? 0.f : ex2_approx(m - mm);
-    acc.x *= s0; acc.y *= s0; acc.z *= s0; acc.w *= s0;
-    l *= s0;
-    for (int k = 1; k < wpr; ++k) {
-      const float mk = xch[wq + k][kHeadDim + 1];
-      const float sk = (mk == -INFINITY) ? 0.f : ex2_approx(mk - mm);
-      const float4 v = *reinterpret_cast<const float4*>(&xch[wq + k][lane * 4]);
-      acc.x = fmaf(v.x, sk, acc.x); acc.y = fmaf(v.y, sk, acc.y); acc.z = fmaf(v.z, sk, acc.z); acc.w = fmaf(v.w, sk, acc.w);
-      l = fmaf(xch[wq + k][kHeadDim], sk, l);
+    const float inv_l = sm_inv[r];
+    const float4 o = make_float4(acc.x * inv_l, acc.y * inv_l, acc.z * inv_l, acc.w * inv_l);
+    const long long at = ((long long)bh * kRows + r0 + r) * kHeadDim + piece * 4;
+    *reinterpret_cast<float4*>(a.O_f32 + at) = o;
+    if (!kProj) {
+      const uint32_t b01 = pack_bf16x2(o.x, o.y), b23 = pack_bf16x2(o.z, o.w);
+      const float f0 = __uint_as_float(b01 << 16), f1 = __uint_as_float(b01 & 0xFFFF0000u), f2 = __uint_as_float(b23 << 16),
+                  f3 = __uint_as_float(b23 & 0xFFFF0000u);
+      *reinterpret_cast<uint2*>(a.O_m2 + at) = make_uint2(pack_bf16x2(-2.f * f0, -2.f * f1), pack_bf16x2(-2.f * f2, -2.f * f3));   // exact
+      on_part[item] = (f0 * f0 + f1 * f1) + (f2 * f2 + f3 * f3);
     }
-    m = mm;
   }
-  const float inv_l = 1.f / l;
-  const float4 o = make_float4(acc.x * inv_l, acc.y * inv_l, acc.z * inv_l, acc.w * inv_l);
-  const long long ri = (long long)bh * kRows + r;
-  *reinterpret_cast<float4*>(a.O_f32 + ri * kHeadDim + lane * 4) = o;
-  __nv_bfloat16* om = a.O_m2 + ri * kHeadDim + lane * 4;
-  float on;
+  named_barrier_sync(2, kThreads);
+  // With the output projection: the row of the third contraction is -2 bf16(Mt o), its constant o^T Mt o.  Eight rows at a time,
+  // which belong to one query head: thread = (column, quarter of the sum), so that Mt comes once for all eight.
   if (kProj) {
-    // with the output projection: the row of the third contraction is -2 bf16(Mt o), its constant o^T Mt o
-    __syncwarp();
-    *reinterpret_cast<float4*>(&xch[wq][lane * 4]) = o;   // the warp's own slot: its partials were merged above
-    __syncwarp();
-    const float4 mo = project_row_warp(a.proj_Mt + (long long)((bh % a.Hkv) * (kRows / a.w) + r / a.w) * kHeadDim * kHeadDim,
-                                       xch[wq], lane);
-    *reinterpret_cast<float4*>(a.O_proj + ri * kHeadDim + lane * 4) = mo;
-    om[0] = __float2bfloat16_rn(-2.f * mo.x);
-    om[1] = __float2bfloat16_rn(-2.f * mo.y);
-    om[2] = __float2bfloat16_rn(-2.f * mo.z);
-    om[3] = __float2bfloat16_rn(-2.f * mo.w);
-    on = (o.x * mo.x + o.y * mo.y) + (o.z * mo.z + o.w * mo.w);
-  } else {
-    const __nv_bfloat16 b0 = __float2bfloat16_rn(o.x), b1 = __float2bfloat16_rn(o.y), b2 = __float2bfloat16_rn(o.z),
-                        b3 = __float2bfloat16_rn(o.w);
-    const float f0 = __bfloat162float(b0), f1 = __bfloat162float(b1), f2 = __bfloat162float(b2),
-                f3 = __bfloat162float(b3);
-    om[0] = __float2bfloat16_rn(-2.f * f0);   // -2 x is exact for a bf16 x
-    om[1] = __float2bfloat16_rn(-2.f * f1);
-    om[2] = __float2bfloat16_rn(-2.f * f2);
-    om[3] = __float2bfloat16_rn(-2.f * f3);
-    on = (f0 * f0 + f1 * f1) + (f2 * f2 + f3 * f3);
-  }
+    float* rows = reinterpret_cast<float*>(cx.gen_base + kOffO);              // [8][128]
+    float* quarters = rows + 8 * kHeadDim;                                    // [4][8][128]
+    const int c = wt & (kHeadDim - 1), q = wt >> 7;
+    for (int g0 = 0; g0 < rb; g0 += 8) {
+      const int nr = min(8, rb);
+      const long long ri = (long long)bh * kRows + r0 + g0;
+      if (wt < 8 * (kHeadDim / 4))
+        reinterpret_cast<float4*>(rows)[wt] = wt < nr * (kHeadDim / 4) ? reinterpret_cast<const float4*>(a.O_f32 + ri * kHeadDim)[wt]
+                                                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float* Mt = a.proj_Mt + (long long)((bh % a.Hkv) * (kRows / a.w) + (r0 + g0) / a.w) * kHeadDim * kHeadDim +
+                        q * 32 * kHeadDim + c;
+      float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      named_barrier_sync(2, kThreads);
+#pragma unroll 2
+      for (int k = 0; k < 32; k += 4) {
+        float m4[4];
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) on += __shfl_xor_sync(0xffffffffu, on, off);
-  __nv_bfloat16* arow = a.aug + ri * 64;
-  arow[2 * lane] = __float2bfloat16_rn(0.f);
-  arow[2 * lane + 1] = __float2bfloat16_rn(0.f);
-  __syncwarp();
-  if (lane == 0) {
-    const float c2 = a.scale * kLog2e;
-    const float M2 = m + log2f(l);        // A = exp2(s * c2 - M2)
-    a.row_M2[ri] = M2;
-    split3(-M2 / c2, arow);
-    split3(on, arow + 16);
+        for (int i = 0; i < 4; ++i) m4[i] = __ldg(Mt + (k + i) * kHeadDim);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const float4 o = *reinterpret_cast<const float4*>(rows + r * kHeadDim + q * 32 + k);
+          sum[r] = fmaf(m4[3], o.w, fmaf(m4[2], o.z, fmaf(m4[1], o.y, fmaf(m4[0], o.x, sum[r]))));
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r) quarters[(q * 8 + r) * kHeadDim + c] = sum[r];
+      named_barrier_sync(2, kThreads);
+      const int r = wq >> 1, c2 = (wq & 1) * 64 + lane * 2;   // two warps to a row
+      float2 mo = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float2 u = *reinterpret_cast<const float2*>(quarters + (k * 8 + r) * kHeadDim + c2);
+        mo.x += u.x; mo.y += u.y;
+      }
+      const float2 o = *reinterpret_cast<const float2*>(rows + r * kHeadDim + c2);
+      float on = fmaf(o.x, mo.x, o.y * mo.y);
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) on += __shfl_xor_sync(0xffffffffu, on, off);
+      if (r < nr) {
+        *reinterpret_cast<float2*>(a.O_proj + (ri + r) * kHeadDim + c2) = mo;
+        *reinterpret_cast<uint32_t*>(a.O_m2 + (ri + r) * kHeadDim + c2) = pack_bf16x2(-2.f * mo.x, -2.f * mo.y);
+        if (lane == 0) on_part[(wq & 1) * rb + g0 + r] = on;
+      }
+      named_barrier_sync(2, kThreads);   // the rows are overwritten by the next eight
+    }
   }
-}
-
-// One K tile and one V tile of phase C into stage s (ring slots 2s and 2s + 1).
-__device__ __forceinline__ void load_stage_c(const Ctx& cx, const CUtensorMap* tmK, const CUtensorMap* tmV, int b, int h,
-                                             int j0, int s) {
-  uint8_t* dK = cx.gen_base + k_slot_off(2 * s);
-  uint8_t* dV = dK + kTileBytes;
-  uint64_t* bar = &cx.B->kv_full[s];
-  mbar_arrive_expect_tx(bar, kStageBytes);
-  tma_load_4d(dK, tmK, bar, 0, j0, h, b);
-  tma_load_4d(dK + kBoxBytes, tmK, bar, 64, j0, h, b);
-  tma_load_4d(dV, tmV, bar, 0, j0, h, b);
-  tma_load_4d(dV + kBoxBytes, tmV, bar, 64, j0, h, b);
+  // ---- the strips: 64 bf16 a row, zero but for the pieces of -M2 / c2 and of ||o||^2 ----
+  for (int e = wt; e < rb * 8; e += kThreads) {
+    const int r = e >> 3, part = e & 7;
+    const long long ri = (long long)bh * kRows + r0 + r;
+    uint4 u = make_uint4(0u, 0u, 0u, 0u);
+    if ((part & ~2) == 0) {
+      float x;
+      if (part == 0) {
+        x = -sm_M2[r] / (a.scale * kLog2e);
+        a.row_M2[ri] = sm_M2[r];
+      } else {
+        x = 0.f;
+        constexpr int kParts = kProj ? 2 : kHeadDim / 4;
+#pragma unroll
+        for (int k = 0; k < kParts; ++k) x += on_part[k * rb + r];
+      }
+      const uint3 p3 = split3(x);
+      u.x = p3.x | (p3.y << 16);
+      u.y = p3.z;
+    }
+    *reinterpret_cast<uint4*>(a.aug + ri * 64 + part * 8) = u;
+  }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -637,7 +715,7 @@ __device__ __forceinline__ void load_stage_c(const Ctx& cx, const CUtensorMap* t
 template <int kW, bool kLse>
 __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtensorMap* tmQ, const CUtensorMap* tmO,
                                 const CUtensorMap* tmAug, const CUtensorMap* tmK, const CUtensorMap* tmV, int bh,
-                                int tile0, int T, int pre) {
+                                int tile0, int T, int pre, int started) {
   constexpr int kG = kRows / kW;
   FusedBars* B = cx.B;
   int* abort_flag = cx.abort_flag;
@@ -659,10 +737,11 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
       tma_load_3d(cx.gen_base + kOffO + kBoxBytes, tmO, &B->const_full, 64, 0, bh);
       tma_load_3d(cx.gen_base + kOffAug, tmAug, &B->const_full, 0, 0, bh);
       int nS = pre;   // stages requested so far
+      const uint64_t policy = policy_evict_first();
       for (int it = pre; it < T; ++it) {   // the first `pre` tiles were requested before the group barriers
         const int s = it & 1;
         if (it >= 2 && !mbar_wait(&B->kv_empty[s], ((it >> 1) - 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit)) break;
-        load_stage_c(cx, tmK, tmV, b, h, (tile0 + T - 1 - it) * kTile, s);
+        load_stage_c(cx, tmK, tmV, b, h, (tile0 + T - 1 - it) * kTile, s, policy);
         ++nS;
       }
       if (*(volatile int*)abort_flag) {
@@ -683,7 +762,7 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
         tc_fence_after();
         const uint32_t sK = cx.smem_base + k_slot_off(2 * s), sV = sK + kTileBytes;
         const uint32_t tS = tmem + (uint32_t)s * 256u, tC = tS + 128u;
-        mma_tile_kk(tS, sK, sQ, false);                       // S^T = K Q^T
+        if (it >= started) mma_tile_kk(tS, sK, sQ, false);    // S^T = K Q^T
         umma_ss(tS, ones_desc, aug_s, kIdescKK, true);        //   + row constant
         mma_tile_kk(tC, sV, sO, false);                       // C^T = V (-2 O)^T
         umma_ss(tC, ones_desc, aug_c, kIdescKK, true);        //   + ||o||^2
@@ -1254,31 +1333,37 @@ __device__ void control_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, 
     }
     if (kLse) {
       // O and the rows' normalisers are given: phase C only, and no CTA waits for another
-      phase_c_control<kW, kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, 0);
+      phase_c_control<kW, kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, 0, 0);
       tc_fence_before();
       __syncthreads();
       tc_fence_after();
       continue;
     }
-    phase_a_control(cx, a, tmQ, tmK, tmV, bh, pl.rank, pl.tile0, pl.T1);
-    // Phase A no longer needs the tile ring: request phase C's first two K/V stages now, so that they arrive
-    // while the group merges its partials (K and V are inputs; only O' depends on the merge).
-    __syncthreads();
-    const int pre = pl.T2 < 2 ? pl.T2 : 2;
-    if (threadIdx.x == 0)
-      for (int it = 0; it < pre; ++it)
-        load_stage_c(cx, tmK, tmV, bh / a.Hkv, bh % a.Hkv, (pl.tile0 + pl.T2 - 1 - it) * kTile, it);
+    const int pre = phase_a_control(cx, a, tmQ, tmK, tmV, bh, pl.tile0, pl.T1, pl.T2);
     bool through = group_barrier(counter, (++epoch) * (unsigned int)a.cpg, abort_flag, go, a.dev_status, a.wait_limit);
-    // phase B belongs to the worker warps
+    // Phase B belongs to the worker warps.  Meanwhile S^T = K Q^T of the first two tiles of phase C, which do not need its results
+    // (the accumulators of phase A have been read, and Q is still there).
+    int started = 0;
+    if (through && cx.warp == 1 && cx.lane == 0) {
+      tc_fence_after();
+      for (; started < 2 && started < pl.T2; ++started) {
+        if (!mbar_wait(&bars->kv_full[started], 0, abort_flag, a.dev_status, kDevTimeout, a.wait_limit)) break;
+        mma_tile_kk(cx.tmem + (uint32_t)started * 256u, cx.smem_base + k_slot_off(2 * started), cx.smem_base + kOffQ, false);
+      }
+    }
     through = through && group_barrier(counter, (++epoch) * (unsigned int)a.cpg, abort_flag, go, a.dev_status, a.wait_limit);
     if (!through) {
-      // a barrier gave up: the stages requested above must have landed before this CTA may return
+      // a barrier gave up: the stages requested above must have landed, and the products been formed, before this CTA may return
       if (threadIdx.x == 0)
         for (int it = 0; it < pre; ++it) wait_issued(&bars->kv_full[it], 0);
+      if (started > 0) {
+        umma_commit(&bars->drain);
+        wait_issued(&bars->drain, 0);
+      }
       break;
     }
     tc_fence_after();
-    phase_c_control<kW, kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, pre);
+    phase_c_control<kW, kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, pre, started);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1299,24 +1384,12 @@ __device__ void worker_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, c
       tc_fence_after();
       continue;
     }
-    phase_a_worker(cx, a, tmQ, tmK, tmV, bh, pl.rank, pl.tile0, pl.T1);
-    __syncthreads();
+    phase_a_worker(cx, a, bh, pl.tile0, pl.T1);
     if (!group_barrier_follow(go)) break;
-    {
-      const int wq = cx.warp - kFFirstWorker;
-      const int rows_max = (kRows + a.cpg - 1) / a.cpg;          // rows of the busiest CTA of the group
-      int wpr = kFWorkerWarps;                                    // warps per row: 16, 8, 4, 2 or 1
-      while (wpr > 1 && kFWorkerWarps / wpr < rows_max) wpr >>= 1;
-      const int rows_at_once = kFWorkerWarps / wpr;
-      float (*xch)[kHeadDim + 4] = reinterpret_cast<float (*)[kHeadDim + 4]>(cx.gen_base + kOffAug);
-      for (int k0 = 0; k0 < rows_max; k0 += rows_at_once) {
-        const int r = pl.rank + (k0 + wq / wpr) * a.cpg;
-        combine_rows<kInd == 3>(a, bh, pl.group, r < kRows ? r : -1, wq % wpr, wpr, wq, cx.lane, xch);
-        named_barrier_sync(2, kFWorkerWarps * 32);   // the exchange buffer is reused by the next batch of rows
-      }
-      fence_proxy_async_smem();   // the exchange buffer is overwritten by a TMA load in phase C
-      if (threadIdx.x == kFFirstWorker * 32) cx.heavy[0] = 0;
-    }
+    combine_rows<kInd == 3>(cx, a, bh, pl.group, pl.rank);
+    fence_proxy_async_smem();   // the exchange buffers are overwritten by TMA loads in phase C
+    named_barrier_sync(2, kFWorkerWarps * 32);   // (the strips' weights lie where the heavy units are noted)
+    if (threadIdx.x == kFFirstWorker * 32) cx.heavy[0] = 0;
     if (!group_barrier_follow(go)) break;
     tc_fence_after();
     phase_c_worker<kW, kLse, kInd>(cx, a, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, 0, red);
