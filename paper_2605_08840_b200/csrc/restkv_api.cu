@@ -242,14 +242,15 @@ static restkv_status run_score(Call& c, const Problem& p, const Workspace& ws, c
     if (e != cudaSuccess) return c.fail(e);
   } else if (O_given) {
     // the window rows' outputs and log-sum-exps come from the caller: pass 1 and the merge are not needed
-    RESTKV_LAUNCH(c, RESTKV_KERNEL_COMBINE, launch_from_lse_prep(p, ws, O_given, LSE_given, use_tc, c.st), 1);
+    // (the score kernel reads them itself where no projection has to be applied to O first)
+    if (!use_tc || p.proj.M) RESTKV_LAUNCH(c, RESTKV_KERNEL_COMBINE, launch_from_lse_prep(p, ws, O_given, LSE_given, use_tc, c.st), 1);
     if (use_tc && p.proj.M)
       RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS1,
                     launch_tc_vmv(c.h->tc_state, p, V, ws.vmv, c.h->sm_count, c.h->wait_limit, c.h->dev_status, c.st), 1);
     if (use_tc) {
       RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS2,
                     launch_tc_fused(c.h->tc_state, p, ws, Q, K, V, ema_decay, c.h->sm_count, false, false, c.h->wait_limit,
-                                    O_given, nullptr, nullptr, c.h->dev_status, true, c.st), 1);
+                                    O_given, LSE_given, nullptr, nullptr, c.h->dev_status, true, c.st), 1);
     } else {
       Workspace wsl = ws;
       wsl.O_f32 = const_cast<float*>(O_given);
@@ -266,7 +267,7 @@ static restkv_status run_score(Call& c, const Problem& p, const Workspace& ws, c
                     launch_tc_vmv(c.h->tc_state, p, V, ws.vmv, c.h->sm_count, c.h->wait_limit, c.h->dev_status, c.st), 1);
     RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS2,
                   launch_tc_fused(c.h->tc_state, p, ws, Q, K, V, ema_decay, c.h->sm_count, reuse_l2, false, c.h->wait_limit,
-                                  nullptr, adaptive ? ws.I_raw : nullptr, c.counters(), c.h->dev_status, true, c.st), 1);
+                                  nullptr, nullptr, adaptive ? ws.I_raw : nullptr, c.counters(), c.h->dev_status, true, c.st), 1);
   } else {
     RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS1, launch_simt_pass1(p, ws, Q, K, V, c.st), 1);
     RESTKV_LAUNCH(c, RESTKV_KERNEL_COMBINE, launch_combine(p, ws, c.st), 1);
@@ -588,7 +589,7 @@ restkv_status restkv_decode(restkv_handle* h, const restkv_shape* shape, const v
       RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE, launch_decode_pad(p, q, ws.q_pad, c.st), 1);
       RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE,
                     launch_tc_fused(h->tc_state, pd, ws, ws.q_pad, Kc, Vc, 0.f, h->sm_count, false, true, h->wait_limit,
-                                    nullptr, nullptr, c.counters(), h->dev_status, false, c.st), 1);
+                                    nullptr, nullptr, nullptr, c.counters(), h->dev_status, false, c.st), 1);
       RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE, launch_decode_extract(p, ws.O_f32, ws.row_M2, out, lse, c.st), 1);
       return RESTKV_OK;
     }

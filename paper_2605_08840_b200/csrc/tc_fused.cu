@@ -57,6 +57,7 @@ struct FusedArgs {
   float* vnorm;                      // [BH, n_kv]
   float* tile_max;                   // [BH, tiles, 128] largest scaled logit (log2 units) of each query row in each tile
   float* row_M2;                     // [BH, 128] m*log2e + log2 l of each query row (written by the merge)
+  const float* lse;                  // from_lse without a projection: the rows' given log-sum-exp (natural), else null
   float* I_hat;                      // [BH, n]
   float* I_raw;                      // [BH, 128, n] or null: the per-query indicators, for the adaptive window of
                                      //  Eq. 10-12; every tile then takes the slower epilogue that holds them
@@ -99,7 +100,7 @@ __device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
 }
 
 // (Re)initialises every mbarrier of the CTA for one phase.  Called by one thread between two __syncthreads.
-__device__ void init_bars(FusedBars* B, bool first, bool from_lse) {
+__device__ void init_bars(FusedBars* B, bool first, bool from_lse, bool own_rows) {
   uint64_t* all = reinterpret_cast<uint64_t*>(B);
   constexpr int kCount = sizeof(FusedBars) / sizeof(uint64_t);
   if (!first)
@@ -120,7 +121,7 @@ __device__ void init_bars(FusedBars* B, bool first, bool from_lse) {
     mbar_init(&B->v_full[i], 1);
     mbar_init(&B->v_empty[i], 1 + 1);   // MMA commit + the warp that reduces ||v||^2
   }
-  mbar_init(&B->const_full, 1);
+  mbar_init(&B->const_full, own_rows ? 1 + kFWorkerWarps : 1);   // (+ the warps that form the row operands themselves)
   mbar_init(&B->drain, 1);
   for (int i = 0; i < 4; ++i) mbar_init(&B->red_full[i], kFWorkerWarps);
   for (int i = 0; i < 4; ++i) mbar_init(&B->vn_full[i], 2);
@@ -728,14 +729,17 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
   if (warp == 0) {
     if (lane == 0 && T > 0) {
       fence_proxy_async_all();   // O' and the constant strip were written with ordinary stores by other CTAs
-      mbar_arrive_expect_tx(&B->const_full, kTileBytes + kAugBytes + (kLse ? kTileBytes : 0u));
+      const bool own_rows = kLse && a.lse;   // O' and the strip are formed by the worker warps
+      mbar_arrive_expect_tx(&B->const_full, (own_rows ? 0u : kTileBytes + kAugBytes) + (kLse ? kTileBytes : 0u));
       if (kLse) {   // no phase A has brought Q in
         tma_load_3d(cx.gen_base + kOffQ, tmQ, &B->const_full, 0, 0, bh);
         tma_load_3d(cx.gen_base + kOffQ + kBoxBytes, tmQ, &B->const_full, 64, 0, bh);
       }
-      tma_load_3d(cx.gen_base + kOffO, tmO, &B->const_full, 0, 0, bh);
-      tma_load_3d(cx.gen_base + kOffO + kBoxBytes, tmO, &B->const_full, 64, 0, bh);
-      tma_load_3d(cx.gen_base + kOffAug, tmAug, &B->const_full, 0, 0, bh);
+      if (!own_rows) {
+        tma_load_3d(cx.gen_base + kOffO, tmO, &B->const_full, 0, 0, bh);
+        tma_load_3d(cx.gen_base + kOffO + kBoxBytes, tmO, &B->const_full, 64, 0, bh);
+        tma_load_3d(cx.gen_base + kOffAug, tmAug, &B->const_full, 0, 0, bh);
+      }
       int nS = pre;   // stages requested so far
       const uint64_t policy = policy_evict_first();
       for (int it = pre; it < T; ++it) {   // the first `pre` tiles were requested before the group barriers
@@ -915,7 +919,7 @@ __device__ void heavy_pass(const Ctx& cx, const FusedArgs& a, int bh) {
     constexpr int kU = kDot ? 1 : 2;
     const int my_u = kDot ? 0 : lane >> 4, row = row0 + ((lane >> 1) & 7);
     const float weight = cx.row_weight[row];
-    const float M2 = kDot ? a.row_M2[(long long)bh * kRows + row] : 0.f;
+    const float M2 = !kDot ? 0.f : kLse && !kProj ? a.lse[(long long)bh * kRows + row] * kLog2e : a.row_M2[(long long)bh * kRows + row];
     uint2 q[8];
     if (kLse && !kProj) {
 #pragma unroll
@@ -1056,6 +1060,43 @@ __device__ void heavy_pass(const Ctx& cx, const FusedArgs& a, int bh) {
   if (wq == 0 && lane == 0) cx.heavy[0] = 0;   // (the CTA meets once more before anything is noted again)
 }
 
+// The row operands of phase C from given window statistics: -2 bf16(O) as the 128-byte-swizzled tile that the products read, and
+// of the rows' strips the four 16-byte pieces that they reach.  Every CTA forms them for itself (64 KB of O from L2, while the
+// first K and V tiles are on their way); a kernel of its own before this one took 2 us and the boundary behind it.
+// A warp takes eight rows, a lane four columns.
+__device__ void stage_given_rows(const Ctx& cx, const FusedArgs& a, int bh) {
+  const int lane = cx.lane, row0 = (cx.warp - kFFirstWorker) * 8;
+  const long long r0 = (long long)bh * kRows + row0;
+  float4 o[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) o[r] = __ldg(reinterpret_cast<const float4*>(a.O_f32 + (r0 + r) * kHeadDim + lane * 4));
+  const float lse = __ldg(a.lse + r0 + (lane >> 2));
+  float on[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const uint32_t b01 = pack_bf16x2(o[r].x, o[r].y), b23 = pack_bf16x2(o[r].z, o[r].w);
+    const float f0 = __uint_as_float(b01 << 16), f1 = __uint_as_float(b01 & 0xFFFF0000u), f2 = __uint_as_float(b23 << 16),
+                f3 = __uint_as_float(b23 & 0xFFFF0000u);
+    on[r] = (f0 * f0 + f1 * f1) + (f2 * f2 + f3 * f3);
+    // (row0 is a multiple of 8: chunk c of row r of a box sits at chunk c ^ r)
+    *reinterpret_cast<uint2*>(cx.gen_base + kOffO + (lane >> 4) * kBoxBytes + row0 * 128 + r * 128 +
+                              ((((lane & 15) >> 1) ^ r) << 4) + (lane & 1) * 8) =
+        make_uint2(pack_bf16x2(-2.f * f0, -2.f * f1), pack_bf16x2(-2.f * f2, -2.f * f3));   // exact
+  }
+  const float sum = reduce_warp<8>(on, lane);   // of row lane / 4
+  const int r = lane >> 2, part = lane & 3;
+  uint4 u = make_uint4(0u, 0u, 0u, 0u);
+  if ((part & 1) == 0) {
+    const uint3 p3 = split3(part == 0 ? -(lse * kLog2e) / (a.scale * kLog2e) : sum);   // A = exp2(s * c2 - M2), M2 = lse * log2e
+    u.x = p3.x | (p3.y << 16);
+    u.y = p3.z;
+  }
+  *reinterpret_cast<uint4*>(cx.gen_base + kOffAug + row0 * 128 + r * 128 + ((part ^ r) << 4)) = u;
+  fence_proxy_async_smem();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(&cx.B->const_full);
+}
+
 // kInd: 0 = Eq. 7; 1 = the attention weight alone; 2 = attention weight times ||v|| (Appendix G.1); 3 = Eq. 7 with
 // the output projection of Eq. 4 inside its norm.
 template <int kW, bool kLse, int kInd>
@@ -1125,6 +1166,7 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
   };
   float* raw_head = (a.I_raw && !kLse) ? a.I_raw + (long long)bh * kRows * n : nullptr;
   bool ok = true;
+  if (kLse && !kProj && T > 0) stage_given_rows(cx, a, bh);
   float vn_next = 0.f;
   // from_lse: no phase A has left ||v||^2 and the tiles' row maxima behind; ||v||^2 comes from the control warps
   // through shared memory and a warp finds out from the logits themselves whether its part of a tile is heavy
@@ -1328,7 +1370,7 @@ __device__ void control_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, 
   unsigned int epoch = 0;
   for (int bh = pl.group; bh < a.BH; bh += a.groups) {
     if (bh != pl.group) {   // fresh barriers for every head: nothing is in flight between two __syncthreads
-      if (threadIdx.x == 0) init_bars(bars, false, kLse);
+      if (threadIdx.x == 0) init_bars(bars, false, kLse, a.lse != nullptr);
       __syncthreads();
     }
     if (kLse) {
@@ -1433,7 +1475,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   if (threadIdx.x == 0) {
     abort_flag = 0;
     cx.heavy[0] = 0;
-    init_bars(&bars, true, kLse);
+    init_bars(&bars, true, kLse, a.lse != nullptr);
     prefetch_tensormap(&tmQ);
     prefetch_tensormap(&tmK);
     prefetch_tensormap(&tmV);
@@ -1493,10 +1535,9 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 }
 
 // ------------------------------------------------------------------------------------------------
-// The window rows' outputs O and log-sum-exps given by the caller (the prefill attention has them): what phase B
-// would have written for phase C.  One warp per query row, lane = four output dims.
-// With the output projection (proj_Mt non-null): the row becomes -2 bf16(Mt o), the constant o^T Mt o, and Mt o is
-// kept in O_proj.
+// The window rows' outputs O and log-sum-exps given by the caller (the prefill attention has them), under the output
+// projection: what phase B would have written for phase C, the row -2 bf16(Mt o), the constant o^T Mt o, and Mt o itself.
+// One warp per query row, lane = four output dims.
 __global__ void from_lse_prep_kernel(int rows, float scale, const float* __restrict__ O, const float* __restrict__ LSE,
                                      __nv_bfloat16* __restrict__ O_m2, __nv_bfloat16* __restrict__ aug,
                                      float* __restrict__ row_M2, const float* __restrict__ proj_Mt,
@@ -1509,28 +1550,17 @@ __global__ void from_lse_prep_kernel(int rows, float scale, const float* __restr
   if (ri >= rows) return;
   const float4 o = *reinterpret_cast<const float4*>(O + (long long)ri * kHeadDim + lane * 4);
   __nv_bfloat16* om = O_m2 + (long long)ri * kHeadDim + lane * 4;
-  float on;
-  if (proj_Mt) {
-    *reinterpret_cast<float4*>(&xs[wi][lane * 4]) = o;
-    __syncwarp();
-    const int bh = ri / kRows, r = ri % kRows;
-    const float4 mo = project_row_warp(proj_Mt + (long long)((bh % Hkv) * (kRows / w) + r / w) * kHeadDim * kHeadDim,
-                                       xs[wi], lane);
-    *reinterpret_cast<float4*>(O_proj + (long long)ri * kHeadDim + lane * 4) = mo;
-    om[0] = __float2bfloat16_rn(-2.f * mo.x);
-    om[1] = __float2bfloat16_rn(-2.f * mo.y);
-    om[2] = __float2bfloat16_rn(-2.f * mo.z);
-    om[3] = __float2bfloat16_rn(-2.f * mo.w);
-    on = (o.x * mo.x + o.y * mo.y) + (o.z * mo.z + o.w * mo.w);
-  } else {
-    const float f0 = __bfloat162float(__float2bfloat16_rn(o.x)), f1 = __bfloat162float(__float2bfloat16_rn(o.y));
-    const float f2 = __bfloat162float(__float2bfloat16_rn(o.z)), f3 = __bfloat162float(__float2bfloat16_rn(o.w));
-    om[0] = __float2bfloat16_rn(-2.f * f0);   // -2 x is exact for a bf16 x
-    om[1] = __float2bfloat16_rn(-2.f * f1);
-    om[2] = __float2bfloat16_rn(-2.f * f2);
-    om[3] = __float2bfloat16_rn(-2.f * f3);
-    on = (f0 * f0 + f1 * f1) + (f2 * f2 + f3 * f3);
-  }
+  *reinterpret_cast<float4*>(&xs[wi][lane * 4]) = o;
+  __syncwarp();
+  const int bh = ri / kRows, r = ri % kRows;
+  const float4 mo = project_row_warp(proj_Mt + (long long)((bh % Hkv) * (kRows / w) + r / w) * kHeadDim * kHeadDim,
+                                     xs[wi], lane);
+  *reinterpret_cast<float4*>(O_proj + (long long)ri * kHeadDim + lane * 4) = mo;
+  om[0] = __float2bfloat16_rn(-2.f * mo.x);
+  om[1] = __float2bfloat16_rn(-2.f * mo.y);
+  om[2] = __float2bfloat16_rn(-2.f * mo.z);
+  om[3] = __float2bfloat16_rn(-2.f * mo.w);
+  float on = (o.x * mo.x + o.y * mo.y) + (o.z * mo.z + o.w * mo.w);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) on += __shfl_xor_sync(0xffffffffu, on, off);
   __nv_bfloat16* arow = aug + (long long)ri * 64;
@@ -1694,7 +1724,7 @@ bool tc_variant_supported(const Problem& p, float ema_decay) {
 // with the timeout status instead of hanging.  (A cooperative launch would guarantee residency but costs ~25 us.)
 cudaError_t launch_tc_fused(void* state, const Problem& p, const Workspace& ws, const void* Q, const void* K,
                             const void* V, float ema_decay, int sm_count, bool reuse_l2, bool attention_only,
-                            long long wait_limit, const float* O_given, float* I_raw, unsigned int* counters,
+                            long long wait_limit, const float* O_given, const float* LSE_given, float* I_raw, unsigned int* counters,
                             unsigned int* dev_status, bool chained, cudaStream_t st) {
   TcState* ts = (TcState*)state;
   CUtensorMap tmQ, tmK, tmV, tmO, tmAug;
@@ -1725,6 +1755,7 @@ cudaError_t launch_tc_fused(void* state, const Problem& p, const Workspace& ws, 
   a.wait_limit = wait_limit;
   a.I_raw = O_given ? nullptr : I_raw;
   if (O_given) a.O_f32 = const_cast<float*>(O_given);   // read only in this mode
+  a.lse = O_given && !a.proj_Mt ? LSE_given : nullptr;
   const dim3 grid(a.groups * a.cpg);
   FusedKernel kernel = attention_only ? pick_fused(32, false, 0) : pick_fused(p.w, a.from_lse != 0, a.proj_Mt ? 3 : p.indicator);
   if (!kernel) return cudaErrorInvalidValue;
