@@ -119,7 +119,7 @@ __device__ void init_bars(FusedBars* B, bool first, bool from_lse, bool own_rows
   }
   for (int i = 0; i < kFVSlots; ++i) {
     mbar_init(&B->v_full[i], 1);
-    mbar_init(&B->v_empty[i], 1 + 1);   // MMA commit + the warp that reduces ||v||^2
+    mbar_init(&B->v_empty[i], 1 + 2);   // MMA commit + the two ||v||^2 warps
   }
   mbar_init(&B->const_full, own_rows ? 1 + kFWorkerWarps : 1);   // (+ the warps that form the row operands themselves)
   mbar_init(&B->drain, 1);
@@ -303,8 +303,11 @@ __device__ int phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtensor
     bool ok = true;
     for (int it = 0; it < T && ok; ++it) {
       const int vs = it % kFVSlots;
-      // both warps wait for every tile so that neither falls a whole phase behind a slot's barrier
-      ok = mbar_wait(&B->v_full[vs], (it / kFVSlots) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit);
+      // Both warps wait for every tile, and the slot is refilled only once both have: otherwise one that is held up between its
+      // own tile and this wait (its instructions on their way from memory again) could find the slot's barrier two phases on, which
+      // looks like none, and wait for ever.
+      ok = __all_sync(0xffffffffu, mbar_wait(&B->v_full[vs], (it / kFVSlots) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit));
+      if (ok && (it & 1) != vg && lane == 0) mbar_arrive(&B->v_empty[vs]);
       if (!ok || (it & 1) != vg) continue;
       const uint8_t* vt = cx.gen_base + v_slot_off(vs);
       float vn[4];

@@ -1710,6 +1710,28 @@ def test_calls_and_graph_replays_in_a_row(handle):
     assert handle.poll_status() == rk.RESTKV_OK
 
 
+def test_many_calls_of_several_handles_end_in_time():
+    """Calls of four handles in turn over more K and V than L2 holds, so that code and data come from memory again and again and
+    the warps of the score kernel drift apart: no wait may miss its phase.  (One of the ||v||^2 warps could, and the call then
+    ended with the timeout status.)"""
+    import torch
+    case = Case("many", 1, 32, 8, 128, 16384, 32, 256, 7, 0, 0.9, "bf16", 0, "normal", 3)
+    runs = []
+    for _ in range(4):
+        h = rk.Handle()
+        runs.append(DeviceRun(h, make_inputs(case)))
+    want = [x.copy() for x in runs[0].evict()]
+    for _ in range(300):
+        for run in runs:
+            run.h.evict(run.shape, run.Q, run.K, run.V, case.ema_decay, run.pool(), run.budget, run.indices, run.K_out, run.V_out,
+                        run.ws, scores_out=run.scores)
+    torch.cuda.synchronize()
+    for run in runs:
+        assert run.h.poll_status() == rk.RESTKV_OK
+        np.testing.assert_array_equal(run.scores.cpu().numpy(), want[0])
+        run.h.close()
+
+
 # ------------------------------------------------------------------ API misuse: error codes, never a fault
 def test_api_rejects_bad_arguments(handle):
     import torch
