@@ -35,6 +35,7 @@ constexpr size_t kFSmem = 2 * kTileBytes + kAugBytes + kOnesBytes + kFRing * kTi
 // units in shared memory, the others' in the CTA's slot of part_O (64 KB, idle in phase C), where the 32 logits of up to
 // kHeavyDumps units lie, too.
 constexpr int kMaxHeavy = 8 * kRows, kNear = 32, kHeavyDumps = (kRows * 128 - 8 * kMaxHeavy) / 32;
+constexpr int kFStay = 5;                         // tiles of a CTA's share that phase A leaves in L2 at normal priority
 constexpr int kFVSlots = 3;                       // phase A: V slots = ring 2, ring 3 and the (then unused) O' tile
 
 struct FusedArgs {
@@ -177,8 +178,7 @@ constexpr uint32_t kOffQ = 0, kOffO = kTileBytes, kOffAug = 2 * kTileBytes, kOff
 __device__ __forceinline__ uint32_t k_slot_off(int i) { return kOffRing + (uint32_t)i * kTileBytes; }
 __device__ __forceinline__ uint32_t v_slot_off(int i) { return i < 2 ? kOffRing + (uint32_t)(2 + i) * kTileBytes : kOffO; }
 
-// K and V leave L2 first: they stream through it (and lines of one priority keep their order among themselves, so that phase C
-// still finds the tiles that phase A read last), while what else the call touches again is small: the partials, the scores, the
+// K and V leave L2 first: they stream through it, while what else the call touches again is small: the partials, the scores, the
 // tensor maps - and the code, whose first run after each synchronisation would otherwise be fetched from HBM, 4 k cycles for
 // each of the merge, its sums and the first tile of phase C.  16384 rows 71 -> 62 us, 32768 projected 137 -> 131 us; phase C's
 // loads alone 66 and 136 us, phase A's alone nothing.
@@ -220,11 +220,12 @@ __device__ int phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtensor
       tma_load_3d(cx.gen_base + kOffQ, tmQ, &B->q_full, 0, 0, bh);
       tma_load_3d(cx.gen_base + kOffQ + kBoxBytes, tmQ, &B->q_full, 64, 0, bh);
       int nK = 0, nV = 0;   // K and V tiles requested so far
-      // (not where the per-query indicators are written, as many bytes again: they would push the tiles out at once)
-      const uint64_t policy = a.I_raw ? policy_evict_normal() : policy_evict_first();
       for (int it = 0; it < T; ++it) {
         const int ks = it & 1, vs = it % kFVSlots;
         const int j0 = (tile0 + it) * kTile;
+        // The share's last tiles, which phase C reads first, stay (five per CTA are 47 MB).  All of them do where the per-query
+        // indicators are written, as many bytes again: those would push them out at once.
+        const uint64_t policy = a.I_raw || it + kFStay >= T ? policy_evict_normal() : policy_evict_first();
         if (it >= 2 && !mbar_wait(&B->k_empty[ks], ((it >> 1) - 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit)) break;
         uint8_t* dK = cx.gen_base + k_slot_off(ks);
         mbar_arrive_expect_tx(&B->k_full[ks], kTileBytes);
@@ -1507,10 +1508,14 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   pl.group = group;
   pl.rank = rank;
   const int nt1 = (a.n_kv + kTile - 1) / kTile, nt2 = (a.n + kTile - 1) / kTile;
-  const int per = (nt1 + a.cpg - 1) / a.cpg;
-  pl.tile0 = rank * per;
-  pl.T1 = max(0, min(nt1, pl.tile0 + per) - pl.tile0);
-  pl.T2 = a.attention_only ? 0 : max(0, min(nt2, pl.tile0 + per) - pl.tile0);
+  // The first CTA gets what the others leave: a prompt's first tokens are where nearly every head has its sink, whose exact scores
+  // (4.5 k cycles after the last tile, as long as a tile and a half) then hide behind the others' tiles instead of ending the
+  // kernel.
+  const int most = (nt1 + a.cpg - 1) / a.cpg, head = min(most, max(1, nt1 - most * (a.cpg - 1)));
+  const int per = a.cpg > 1 ? (nt1 - head + a.cpg - 2) / (a.cpg - 1) : 0;
+  pl.tile0 = rank == 0 ? 0 : min(nt1, head + (rank - 1) * per);
+  pl.T1 = rank == 0 ? head : min(nt1, pl.tile0 + per) - pl.tile0;
+  pl.T2 = a.attention_only ? 0 : max(0, min(nt2, pl.tile0 + pl.T1) - pl.tile0);
 
   // Each role's code sits behind its own register-budget change, so that the sixteen worker warps can be
   // compiled for more registers than the launch gives every thread.
