@@ -8,26 +8,29 @@ namespace restkv {
 
 namespace {
 
-constexpr int kRsThreads = 1024;
 constexpr int kRsBins = 2048;        // 11-bit digits
 constexpr int kRsList = 1024;        // keys of the last digit that are ranked one by one
 constexpr int kRsMaxSmem = 200 * 1024;
+constexpr int kRsHalfSmem = 92 * 1024;   // dynamic shared memory of a block when two lie on an SM
 
 // Sum of the indices of the Bp largest of each row's n values (ties to the lower index), all rows of the raw indicator.
 // What bounds it: the rows come once from HBM or L2; against that stand three walks over a row's keys in shared memory.
-// So one persistent block per SM, the next row on its way by bulk copy while this one is worked on (two buffers; one for
-// rows past 100 KB; longer rows are read again on every walk), and no more than the walks that are needed: the extremes,
+// So two persistent blocks of 512 threads per SM, each a row at a time (one's synchronisations and its next row's way in are
+// covered by the other's walks), rows past 92 KB in one block of 1024 (past 200 KB they are read again on every walk), and no
+// more than the walks that are needed: the extremes,
 // a histogram of 11-bit digits of the offsets from the smallest (about a thousand bins in use, so one histogram serves all
 // warps without contention), then the sum above the digit that holds the Bp-th largest while that digit's few keys are
-// listed and ranked, a key per warp.  1024 rows of 20011: 62 us as selections in two blocks of 512 threads per SM, 43 us so
-// (10 k cycles per row: 0.8 k extremes, 3 k histogram, 2.6 k the last walk, the rest synchronisation).
-template <bool kHeld>   // false: no buffers, the keys are read from global memory on every walk
-__global__ void __launch_bounds__(kRsThreads, 1)
+// listed and ranked, a key per warp.  1024 rows of 20011: 43 us with one block of 1024 threads and two rows in flight per SM
+// (10 k cycles per row, 3.6 k of them synchronisation); the whole call 134.0 us with that, 129.7-131 us so and with the windows
+// worked out by the selection.
+template <int kRsThreads, bool kHeld>   // kHeld false: no buffers, the keys are read from global memory on every walk
+__global__ void __launch_bounds__(kRsThreads, kRsThreads <= 512 ? 2 : 1)
 row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buffers, unsigned long long* __restrict__ sums,
                 unsigned int* dev_status) {
   extern __shared__ __align__(16) uint4 rs_buf[];   // `buffers` rows of quads + 1
   __shared__ __align__(16) unsigned int hist[kRsBins];
   __shared__ unsigned int list_v[kRsList], list_i[kRsList];
+  constexpr int kWarps = kRsThreads / 32, kBpt = kRsBins / kRsThreads;
   __shared__ unsigned int warp_a[32], warp_b[32];
   __shared__ unsigned long long warp_s[32];
   __shared__ unsigned int s_digit, s_rest, s_count, s_listed;
@@ -100,8 +103,8 @@ row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buff
     if (lane == 0) { warp_a[wid] = kmin; warp_b[wid] = kmax; }
     if (tid == 0) s_listed = 0u;
     __syncthreads();
-    kmin = __reduce_min_sync(0xffffffffu, warp_a[lane]);
-    kmax = __reduce_max_sync(0xffffffffu, warp_b[lane]);
+    kmin = __reduce_min_sync(0xffffffffu, lane < kWarps ? warp_a[lane] : 0xFFFFFFFFu);
+    kmax = __reduce_max_sync(0xffffffffu, lane < kWarps ? warp_b[lane] : 0u);
     // ---- digits from the top, until the digit's keys fit the list ----
     int hi = 32 - __clz((int)(kmax - kmin)), lo = hi;   // bits [hi - 1 .. 0] of the offsets vary
     unsigned int prefix = 0u, rest = (unsigned int)Bp, listed = (unsigned int)n;
@@ -115,9 +118,13 @@ row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buff
         if ((v >> top) == (prefix >> top)) atomicAdd(&hist[(v >> lo) & (kRsBins - 1)], 1u);
       });
       __syncthreads();
-      const int first = kRsBins - 2 * (tid + 1);   // this thread's two bins, walked from the top
-      const uint2 own = *reinterpret_cast<const uint2*>(&hist[first]);
-      const unsigned int sum = own.x + own.y;
+      const int first = kRsBins - kBpt * (tid + 1);   // this thread's bins, walked from the top
+      unsigned int own[kBpt], sum = 0u;
+#pragma unroll
+      for (int i = 0; i < kBpt; ++i) {
+        own[i] = hist[first + i];
+        sum += own[i];
+      }
       unsigned int incl = sum;
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
@@ -125,14 +132,20 @@ row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buff
         if (lane >= off) incl += t;
       }
       if (lane == 31) warp_a[wid] = incl;
-      *reinterpret_cast<uint2*>(&hist[first]) = make_uint2(0u, 0u);   // ready for the next time
+#pragma unroll
+      for (int i = 0; i < kBpt; ++i) hist[first + i] = 0u;   // ready for the next time
       __syncthreads();
-      const unsigned int acc = __reduce_add_sync(0xffffffffu, lane < wid ? warp_a[lane] : 0u) + incl - sum;
+      unsigned int acc = __reduce_add_sync(0xffffffffu, lane < wid ? warp_a[lane] : 0u) + incl - sum;
       if (acc < rest && rest <= acc + sum) {   // exactly one thread
-        const bool upper = rest <= acc + own.y;
-        s_digit = (unsigned int)(first + (upper ? 1 : 0));
-        s_rest = rest - acc - (upper ? 0u : own.y);
-        s_count = upper ? own.y : own.x;
+#pragma unroll
+        for (int i = kBpt - 1; i >= 0; --i) {
+          if (acc < rest && rest <= acc + own[i]) {
+            s_digit = (unsigned int)(first + i);
+            s_rest = rest - acc;
+            s_count = own[i];
+          }
+          acc += own[i];
+        }
       }
       __syncthreads();
       prefix |= s_digit << lo;
@@ -156,7 +169,7 @@ row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buff
     if (!ties) {
       if (kHeld && tid == kRsThreads - 1 && row + (long long)buffers * gridDim.x < rows) request(row + buffers * gridDim.x, it + buffers);
       // a listed key per warp: the lanes count the keys that come before it
-      for (unsigned int t = wid; t < listed; t += kRsThreads / 32) {
+      for (unsigned int t = wid; t < listed; t += kWarps) {
         const unsigned int v = list_v[t], i = list_i[t];
         unsigned int before = 0u;
         for (unsigned int u0 = 0; u0 < listed; u0 += 32) {
@@ -168,7 +181,7 @@ row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buff
       }
     } else {
       // more equal keys than the list takes: the first `rest` of them, counted in order (a warp owns a run of the row)
-      const int cw = ((quads * 4 + 31) / 32 + 31) & ~31, wbeg = wid * cw;
+      const int cw = ((quads * 4 + kWarps - 1) / kWarps + 31) & ~31, wbeg = wid * cw;
       const unsigned int* keys = reinterpret_cast<const unsigned int*>(quad) + mis;
       unsigned int eq = 0u;
       for (int i = wbeg + lane; i < min(n, wbeg + cw); i += 32) eq += keys[i] == k0;
@@ -191,7 +204,7 @@ row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buff
     if (lane == 0) warp_s[wid] = isum;
     __syncthreads();
     if (wid == 0) {
-      isum = warp_s[lane];
+      isum = lane < kWarps ? warp_s[lane] : 0ull;
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) isum += __shfl_xor_sync(0xffffffffu, isum, off);
       if (lane == 0) sums[row] = isum;
@@ -199,59 +212,52 @@ row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buff
   }
 }
 
-// grid BH, block 128: the index sums of the head's w * G rows (front and rear half of the window apart) and from them the
-// head's window.
-__global__ void window_params_kernel(int G, int w, int Bp, double beta, int base_width, const unsigned long long* __restrict__ sums,
-                                     int* __restrict__ pool) {
+// grid BH, one warp: the head's window from its rows' index sums.
+__global__ void window_params_kernel(const WindowArgs w, int* __restrict__ pool) {
   ptx::grid_dependency_wait();
   ptx::grid_dependency_launch();
-  const int bh = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  unsigned long long front = 0, rear = 0;
-  for (int e = threadIdx.x; e < G * w; e += blockDim.x) {
-    const unsigned long long s = sums[(long long)bh * G * w + e];
-    if (e % w < w / 2) front += s;
-    else rear += s;
+  int W, gamma;
+  head_window(w, blockIdx.x, &W, &gamma);
+  if (threadIdx.x == 0) {
+    pool[2 * blockIdx.x] = W;
+    pool[2 * blockIdx.x + 1] = gamma;
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    front += __shfl_xor_sync(0xffffffffu, front, off);
-    rear += __shfl_xor_sync(0xffffffffu, rear, off);
-  }
-  __shared__ unsigned long long red[4][2];
-  if (lane == 0) { red[wid][0] = front; red[wid][1] = rear; }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  for (int k = 1; k < 4; ++k) { front += red[k][0]; rear += red[k][1]; }
-  const long long cnt_front = (long long)G * (w / 2) * Bp;
-  const long long cnt_rear = (long long)G * (w - w / 2) * Bp;
-  const double D_rear = (double)rear / (double)cnt_rear;
-  const double D_front = cnt_front ? (double)front / (double)cnt_front : D_rear;
-  const double x = (D_front - D_rear) / beta;
-  const int Ws = 2 * (int)floor(fabs(x)) + 1;   // Eq. 11
-  const int gamma = (int)trunc(x);              // Eq. 12, truncating toward zero
-  pool[2 * bh] = Ws + base_width - 1;
-  pool[2 * bh + 1] = gamma;
 }
 
 }  // namespace
 
 cudaError_t adaptive_init() {
-  return cudaFuncSetAttribute(row_sums_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsMaxSmem);
+  cudaError_t e = cudaFuncSetAttribute(row_sums_kernel<1024, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsMaxSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(row_sums_kernel<512, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsHalfSmem);
+  return e;
 }
 
-cudaError_t launch_adaptive_params(const Problem& p, const Workspace& ws, int budget, float beta, int base_width, int sm_count,
-                                   unsigned int* dev_status, cudaStream_t st, int* n_launches) {
-  int Bp = budget - p.tail;
-  if (Bp > p.n) Bp = p.n;
-  const int rows = p.batch * p.Hq * p.w;
+static int rows_counted(const Problem& p, int budget) {   // of each query, Eq. 10
+  const int Bp = budget - p.tail;
+  return Bp > p.n ? p.n : Bp;
+}
+
+WindowArgs window_args(const Problem& p, const Workspace& ws, int budget, float beta, int base_width) {
+  return WindowArgs{ws.adaptive_sums, (double)beta, p.G, p.w, rows_counted(p, budget), base_width};
+}
+
+// The index sums of every query's top rows.
+cudaError_t launch_row_sums(const Problem& p, const Workspace& ws, int budget, int sm_count, unsigned int* dev_status, cudaStream_t st) {
+  const int rows = p.batch * p.Hq * p.w, Bp = rows_counted(p, budget);
   const size_t room = ((size_t)(p.n + 3) / 4 + 1) * 16;
-  const int buffers = 2 * room <= (size_t)kRsMaxSmem ? 2 : room <= (size_t)kRsMaxSmem ? 1 : 0;
-  *n_launches = 2;
-  const cudaError_t e = launch_chained(buffers ? row_sums_kernel<true> : row_sums_kernel<false>, dim3((unsigned int)(rows < sm_count ? rows : sm_count)), kRsThreads,
-                                       buffers * room, st, rows, p.n, Bp, ws.I_raw, buffers, ws.adaptive_sums, dev_status);
-  if (e != cudaSuccess) return e;
-  return launch_chained(window_params_kernel, dim3((unsigned int)p.BH), 128, 0, st, p.G, p.w, Bp, (double)beta, base_width,
-                        ws.adaptive_sums, ws.pool);
+  if (room <= (size_t)kRsHalfSmem) {
+    const int buffers = 2 * room <= (size_t)kRsHalfSmem ? 2 : 1;
+    return launch_chained(row_sums_kernel<512, true>, dim3((unsigned int)(rows < 2 * sm_count ? rows : 2 * sm_count)), 512, buffers * room, st,
+                          rows, p.n, Bp, ws.I_raw, buffers, ws.adaptive_sums, dev_status);
+  }
+  const bool held = room <= (size_t)kRsMaxSmem;
+  const int buffers = 2 * room <= (size_t)kRsMaxSmem ? 2 : held ? 1 : 0;
+  return launch_chained(held ? row_sums_kernel<1024, true> : row_sums_kernel<1024, false>, dim3((unsigned int)(rows < sm_count ? rows : sm_count)), 1024,
+                        buffers * room, st, rows, p.n, Bp, ws.I_raw, buffers, ws.adaptive_sums, dev_status);
+}
+
+cudaError_t launch_window_params(const Problem& p, const Workspace& ws, int budget, float beta, int base_width, cudaStream_t st) {
+  return launch_chained(window_params_kernel, dim3((unsigned int)p.BH), 32, 0, st, window_args(p, ws, budget, beta, base_width), ws.pool);
 }
 
 }  // namespace restkv

@@ -59,16 +59,16 @@ struct SelectArgs {
   int n, n_kv, keep;            // keep: entries per row, also the row stride of the outputs
   const int* keep_rows;         // non-null: row r keeps min(max(keep_rows[r], 1), keep), the rest of its indices is -1
   const float* I_hat;           // non-null: pool first (Eq. 13) and write the pooled scores; null: read `scores`
-  const int* pool;              // per row (W, gamma) on the device, or null: W, gamma below
+  WindowArgs window;            // with sums: the row's window is worked out from them; else W, gamma below
   int W, gamma, pool_max;
   float* scores;
   int32_t* indices;
   int parts;                    // blocks per row: the cluster's, or (no cluster) blocks that each select from the whole row
   int per;                      // keys of one block's slice
   int held;                     // 1: the slice's keys stay in shared memory; 0: they are formed again from the scores
-  int room;                     // floats of shared memory behind the keys: the taps, later the indices this block gathers and
-                                //  the rows on their way
-  int copy_rows;                // rows that a warp copies at a time
+  int room;                     // floats of shared memory behind the keys: the taps, later the indices this block gathers and,
+                                //  where they go by bulk copies, the rows on their way
+  int copy_rows;                // rows that a warp copies at a time by bulk copies; 0: a warp per row by loads and stores
   int own_idx;                  // 1: the indices fit there
   unsigned int* dev_status;
   GatherArgs ga;
@@ -81,6 +81,13 @@ constexpr unsigned int kInfKey = 0xFF800000u;
 // (a NaN in a head's V makes all its scores NaN; after a wait that ran out they are anything).  NaNs rank above +inf; the
 // highest key is kept free, as a bound that no row reaches.
 __device__ __forceinline__ unsigned int select_key(float x) { return min(float_key(x), 0xFFFFFFFEu); }
+
+// (Out of line: the selection's instructions come from L2 when they first run, and these lie in the middle of them.)
+__device__ __noinline__ int2 adaptive_window(const WindowArgs& a, int row) {
+  int2 w;
+  head_window(a, row, &w.x, &w.y);
+  return w;
+}
 
 // Bounded wait for a bulk copy.
 __device__ __forceinline__ void wait_copy(uint64_t* bar, uint32_t parity, unsigned int* dev_status) {
@@ -132,8 +139,9 @@ __device__ __forceinline__ void pool_slice(const float* taps, int W, bool pool_m
 //     shared memory of whoever needs it, with one cluster barrier per exchange.
 // Measured (8 rows, gather included, under ncu: cold and by itself): 131072 rows / 2048 kept 51 -> 22 us, 16384 / 1024 29 -> 15 us,
 // 3032 / 1056 11 us; 64 rows of 32768 / 2048 kept 73 (two kernels) -> 35 us.
-template <int kThreads>
-__global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kernel(const __grid_constant__ SelectArgs a) {
+// (Two blocks of 512 threads share an SM, or three, where a row has a block of its own and there are more rows than SMs.)
+template <int kThreads, int kBlocks>
+__global__ void __launch_bounds__(kThreads, kBlocks) select_kernel(const __grid_constant__ SelectArgs a) {
   cg::cluster_group cluster = cg::this_cluster();
   const int CS = (int)cluster.num_blocks();
   const int row = (int)blockIdx.x / a.parts, part = (int)blockIdx.x % a.parts;
@@ -160,22 +168,44 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
     ptx::fence_mbar_init();
   }
   csync();
-  ptx::grid_dependency_wait();
+  // ---- all that does not depend on the kernel before comes before the wait for it ----
   const int n = a.n, n_kv = a.n_kv;
   const int rank = CS > 1 ? part : 0;
   const long long j0 = (long long)rank * a.per;
   const int cnt = (int)max(0ll, min((long long)n_kv, j0 + a.per) - j0);
   float* srow = a.scores + (long long)row * n_kv + j0;
   int32_t* dst = a.indices + (long long)row * a.keep;
+  // this warp's run of the slice
+  const int cw = (((a.per + kWarps - 1) / kWarps) + 31) & ~31;
+  const int wbeg = min(cnt, wid * cw), wlen = min(cnt, wbeg + cw) - wbeg;
+  // blocks that all select from the whole row write a share of its pooled scores each
+  const int w_per = CS > 1 ? cnt : (cnt + a.parts - 1) / a.parts, w0 = CS > 1 ? 0 : part * w_per, w1 = min(cnt, w0 + w_per);
+  int W = a.W, gamma = a.gamma;
+  if (a.window.sums) {   // worked out by every block for itself: a kernel of its own cost 2 us and the boundary behind it
+    ptx::grid_dependency_wait();
+    if (wid == 0) {
+      const int2 w = adaptive_window(a.window, row);
+      if (lane == 0) { warp_a[0] = (unsigned int)w.x; warp_b[0] = (unsigned int)w.y; }
+    }
+    __syncthreads();
+    W = (int)warp_a[0];
+    gamma = (int)warp_b[0];
+    __syncthreads();
+  }
+  // the slice's taps [lo, hi) and where they are put
+  const float* const src = a.I_hat + (long long)row * n;
+  const long long lo = j0 - W / 2 + gamma, hi = lo + cnt + W - 1;
+  const long long g0 = lo < 0 ? 0 : (lo < n ? lo : n), g1 = hi > n ? n : (hi > 0 ? hi : 0);
+  const int mis = (int)((reinterpret_cast<uintptr_t>(src + g0) >> 2) & 3);   // floats between the boundary and tap g0
+  const int shift = 4 - (int)((g0 - lo + 4 - mis) & 3);                      // so that the boundary is one in here, too
+  float* const taps = room + (shift & 3);                                    // taps[t - lo]
+  ptx::grid_dependency_wait();
   int keep = a.keep;
   if (a.keep_rows) {
     keep = min(max(a.keep_rows[row], 1), a.keep);
     if (part == 0)
       for (int pos = keep + tid; pos < a.keep; pos += kThreads) dst[pos] = -1;
   }
-  // this warp's run of the slice
-  const int cw = (((a.per + kWarps - 1) / kWarps) + 31) & ~31;
-  const int wbeg = min(cnt, wid * cw), wlen = min(cnt, wbeg + cw) - wbeg;
   auto key_at = [&](int i) { return a.held ? skeys[wbeg + i] : select_key(srow[wbeg + i]); };   // i: position in the run
 
   // ---- keys of the slice, the smallest and the largest but +inf ----
@@ -187,11 +217,6 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
     if (a.held) skeys[jj] = key;
   };
   if (a.I_hat) {
-    int W = a.W, gamma = a.gamma;
-    if (a.pool) { W = a.pool[2 * row]; gamma = a.pool[2 * row + 1]; }
-    const float* src = a.I_hat + (long long)row * n;
-    // blocks that all select from the whole row write a share of its pooled scores each
-    const int w_per = CS > 1 ? cnt : (cnt + a.parts - 1) / a.parts, w0 = CS > 1 ? 0 : part * w_per, w1 = min(cnt, w0 + w_per);
     auto put = [&](int jj, float score) {
       if (!a.held || (jj >= w0 && jj < w1)) srow[jj] = score;
       take(jj, score);
@@ -200,11 +225,6 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
       // The slice's taps, zeros outside the scored rows: every row then takes the same W taps without a bounds check
       // (adding 0 changes nothing), in the order of box_mean.  One bulk copy brings them in, from the 16-byte boundary
       // before the first one to the boundary behind the last one (both inside the workspace that I_hat lies in).
-      const long long lo = j0 - W / 2 + gamma, hi = lo + cnt + W - 1;   // taps [lo, hi)
-      const long long g0 = lo < 0 ? 0 : (lo < n ? lo : n), g1 = hi > n ? n : (hi > 0 ? hi : 0);
-      const int mis = (int)((reinterpret_cast<uintptr_t>(src + g0) >> 2) & 3);   // floats between the boundary and tap g0
-      const int shift = 4 - (int)((g0 - lo + 4 - mis) & 3);                      // so that the boundary is one in here, too
-      float* const taps = room + (shift & 3);                                    // taps[t - lo]
       if (g1 > g0) {
         if (tid == 0) {
           const uint32_t bytes = (uint32_t)(((g1 - g0 + mis) * 4 + 15) & ~15ll);
@@ -395,50 +415,79 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_kern
     if (CS > 1) cluster.sync();   // shared memory stays alive until every peer has done with it
     return;
   }
-  ptx::fence_proxy_async_smem();   // rows are about to land where keys and taps were
+  ptx::fence_proxy_async_smem();   // rows may be about to land where keys and taps were
   csync();   // all positions of this block's share have arrived
 
-  // ---- gather: every warp copies batches of copy_rows rows through its own two buffers, row by row in and as one piece
-  //      out, by bulk copies (with loads and stores the same work took twice as long: 14 k cycles for 256 rows a CTA) ----
+  // ---- gather.  Many rows a block: every warp copies batches of copy_rows rows through its own two buffers, row by row in and as
+  //      one piece out, by bulk copies, of which one starts every 23 cycles.  Few: a warp per row, its lanes over the 16-byte pieces
+  //      of the row of K and the row of V, four rows in flight, where the bulk copies' start and end cost more (the launch says
+  //      where the line lies) ----
   const int rows = (int)(last - first);
   if (own_idx)
     for (int i = tid; i < rows; i += kThreads) dst[first + i] = s_idx[i];
-  const int b = row / a.ga.Hkv, h = row % a.ga.Hkv, es = a.ga.esize, rb = a.ga.row_chunks * 16, R = a.copy_rows;
-  const unsigned char* Kh = a.ga.K + ((long long)b * a.ga.ksb + (long long)h * a.ga.ksh) * es;
-  const unsigned char* Vh = a.ga.V + ((long long)b * a.ga.vsb + (long long)h * a.ga.vsh) * es;
-  const long long out0 = (long long)row * a.keep + first;
-  uint8_t* const stage = reinterpret_cast<uint8_t*>(s_idx) + (own_idx ? ((int)share * 4 + 15) & ~15 : 0) + wid * 4 * R * rb;
-  const int batches = (rows + R - 1) / R, mine = batches > wid ? (batches - wid + kWarps - 1) / kWarps : 0;
-  auto rows_of = [&](int it) { return min(R, rows - (wid + it * kWarps) * R); };
-  for (int it = 0; it <= mine; ++it) {
-    if (it < mine) {
-      const int r0 = (wid + it * kWarps) * R, cr = rows_of(it);
-      uint8_t* buf = stage + (it & 1) * 2 * R * rb;
-      if (lane == 0) {
-        if (it >= 2) ptx::bulk_store_wait_read<0>();   // the buffer's last batch has left
-        ptx::mbar_arrive_expect_tx(&copy_bar[wid][it & 1], (uint32_t)(2 * cr * rb));
+  const int b = row / a.ga.Hkv, h = row - b * a.ga.Hkv, es = a.ga.esize, chunks = a.ga.row_chunks;
+  if (a.copy_rows > 0) {
+    const int rb = chunks * 16, R = a.copy_rows;
+    const unsigned char* Kh = a.ga.K + ((long long)b * a.ga.ksb + (long long)h * a.ga.ksh) * es;
+    const unsigned char* Vh = a.ga.V + ((long long)b * a.ga.vsb + (long long)h * a.ga.vsh) * es;
+    const long long out0 = (long long)row * a.keep + first;
+    uint8_t* const stage = reinterpret_cast<uint8_t*>(s_idx) + (own_idx ? ((int)share * 4 + 15) & ~15 : 0) + wid * 4 * R * rb;
+    const int batches = (rows + R - 1) / R, mine = batches > wid ? (batches - wid + kWarps - 1) / kWarps : 0;
+    auto rows_of = [&](int it) { return min(R, rows - (wid + it * kWarps) * R); };
+    for (int it = 0; it <= mine; ++it) {
+      if (it < mine) {
+        const int r0 = (wid + it * kWarps) * R, cr = rows_of(it);
+        uint8_t* buf = stage + (it & 1) * 2 * R * rb;
+        if (lane == 0) {
+          if (it >= 2) ptx::bulk_store_wait_read<0>();   // the buffer's last batch has left
+          ptx::mbar_arrive_expect_tx(&copy_bar[wid][it & 1], (uint32_t)(2 * cr * rb));
+        }
+        __syncwarp();
+        if (lane < 2 * cr) {
+          const bool isV = lane >= cr;
+          const int r = isV ? lane - cr : lane;
+          // (bounded, should the taps' copy that was given up on have landed over the indices after all)
+          const long long j = min((unsigned int)(own_idx ? s_idx[r0 + r] : dst[first + r0 + r]), (unsigned int)n_kv - 1u);
+          const unsigned char* src = isV ? Vh + j * a.ga.vsn * es : Kh + j * a.ga.ksn * es;
+          ptx::bulk_load(buf + (isV ? R * rb : 0) + r * rb, src, (uint32_t)rb, &copy_bar[wid][it & 1]);
+        }
       }
-      __syncwarp();
-      if (lane < 2 * cr) {
-        const bool isV = lane >= cr;
-        const int r = isV ? lane - cr : lane;
-        // (bounded, should the taps' copy that was given up on have landed over the indices after all)
-        const long long j = min((unsigned int)(own_idx ? s_idx[r0 + r] : dst[first + r0 + r]), (unsigned int)n_kv - 1u);
-        const unsigned char* src = isV ? Vh + j * a.ga.vsn * es : Kh + j * a.ga.ksn * es;
-        ptx::bulk_load(buf + (isV ? R * rb : 0) + r * rb, src, (uint32_t)rb, &copy_bar[wid][it & 1]);
+      if (it > 0 && lane == 0) {
+        const int p = it - 1, cr = rows_of(p);
+        const long long at = (out0 + (long long)(wid + p * kWarps) * R) * rb;
+        uint8_t* buf = stage + (p & 1) * 2 * R * rb;
+        wait_copy(&copy_bar[wid][p & 1], (uint32_t)(p >> 1) & 1u, a.dev_status);
+        ptx::bulk_store(a.ga.K_out + at, ptx::smem_u32(buf), (uint32_t)(cr * rb));
+        ptx::bulk_store(a.ga.V_out + at, ptx::smem_u32(buf + R * rb), (uint32_t)(cr * rb));
+        ptx::bulk_store_commit();
       }
     }
-    if (it > 0 && lane == 0) {
-      const int p = it - 1, cr = rows_of(p);
-      const long long at = (out0 + (long long)(wid + p * kWarps) * R) * rb;
-      uint8_t* buf = stage + (p & 1) * 2 * R * rb;
-      wait_copy(&copy_bar[wid][p & 1], (uint32_t)(p >> 1) & 1u, a.dev_status);
-      ptx::bulk_store(a.ga.K_out + at, ptx::smem_u32(buf), (uint32_t)(cr * rb));
-      ptx::bulk_store(a.ga.V_out + at, ptx::smem_u32(buf + R * rb), (uint32_t)(cr * rb));
-      ptx::bulk_store_commit();
+    if (lane == 0) ptx::bulk_store_wait();
+    return;
+  }
+#pragma unroll 1
+  for (int c = lane; c < 2 * chunks; c += 32) {
+    const bool isV = c >= chunks;
+    const int at = (isV ? c - chunks : c) * 16;
+    const unsigned char* from = (isV ? a.ga.V + ((long long)b * a.ga.vsb + (long long)h * a.ga.vsh) * es
+                                     : a.ga.K + ((long long)b * a.ga.ksb + (long long)h * a.ga.ksh) * es) + at;
+    const long long step = (isV ? a.ga.vsn : a.ga.ksn) * es;
+    unsigned char* to = (isV ? a.ga.V_out : a.ga.K_out) + ((long long)row * a.keep + first) * (chunks * 16) + at;
+#pragma unroll 1
+    for (int r0 = wid; r0 < rows; r0 += 4 * kWarps) {
+      uint4 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = min(r0 + u * kWarps, rows - 1);   // (past the end: the last row again, not stored)
+        // (bounded, should the taps' copy that was given up on have landed over the indices after all)
+        const unsigned int j = min((unsigned int)(own_idx ? s_idx[r] : dst[first + r]), (unsigned int)n_kv - 1u);
+        v[u] = __ldg(reinterpret_cast<const uint4*>(from + (long long)j * step));
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (r0 + u * kWarps < rows) *reinterpret_cast<uint4*>(to + (long long)(r0 + u * kWarps) * (chunks * 16)) = v[u];
     }
   }
-  if (lane == 0) ptx::bulk_store_wait();
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -488,7 +537,7 @@ constexpr size_t kSelMaxSmem = 200 * 1024;
 // clusters_of: how many clusters of 1, 2, 4 and 8 CTAs of the large kind the device holds at once.
 cudaError_t select_init(int* clusters_of) {
   cudaError_t e = cudaSuccess;
-  for (SelectKernel kernel : {select_kernel<512>, select_kernel<1024>})
+  for (SelectKernel kernel : {select_kernel<512, 3>, select_kernel<512, 2>, select_kernel<1024, 1>})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelMaxSmem);
   for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
     cudaLaunchConfig_t cfg = {};
@@ -501,7 +550,7 @@ cudaError_t select_init(int* clusters_of) {
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaOccupancyMaxActiveClusters(&clusters_of[i], select_kernel<1024>, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&clusters_of[i], select_kernel<1024, 1>, &cfg);
   }
   return e;
 }
@@ -520,11 +569,15 @@ static int select_cluster(int rows, int n_kv, const int* clusters_of) {
 // Rows up to this length are selected from by every block of the row for itself when the blocks only share the gather: a
 // block of 1024 threads forms 8 keys per thread in about the time that the cluster's four barriers take.
 constexpr int kSelLocalRows = 8192;
+constexpr int kSelShortRows = 1536;
+// Rows per block from which bulk copies gather them.  59 rows: 5.3 k cycles by bulk copies, 4.9 k by loads and stores; 128 rows: 8.0
+// and 6.0 k; 256 rows: 11.8 k either way; 1024 rows in 128 blocks, which HBM bounds: 34 and 45 k.
+constexpr int kSelFewRows = 192;
 
 // rows x n_kv scores -> rows x min(budget, n_kv) indices.  I_hat non-null: pool first (n scored rows per row of I_hat, window
-// from pool_dev or (W, gamma)) and write the pooled scores.  chained: the launch may overlap the end of the kernel
+// from the index sums in `window` or (W, gamma)) and write the pooled scores.  chained: the launch may overlap the end of the kernel
 // before it in the stream (it waits for that kernel's results itself).
-cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep_rows, const float* I_hat, const int* pool_dev,
+cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep_rows, const float* I_hat, const WindowArgs* window,
                           int W, int gamma, bool pool_max, float* scores, int32_t* indices, const Problem* gather, const void* K, const void* V, void* K_out, void* V_out,
                           const int* clusters_of, unsigned int* dev_status, bool chained, cudaStream_t st) {
   SelectArgs a{};
@@ -537,8 +590,9 @@ cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep
     a.ga.Hkv = gather->Hkv; a.ga.esize = gather->dtype == RESTKV_BF16 ? 2 : 4; a.ga.row_chunks = gather->d * a.ga.esize / 16;
   }
   a.n = n; a.n_kv = n_kv; a.keep = budget < n_kv ? budget : n_kv; a.keep_rows = keep_rows;
-  a.I_hat = I_hat; a.pool = pool_dev; a.W = W; a.gamma = gamma; a.pool_max = pool_max ? 1 : 0;
+  a.I_hat = I_hat; a.W = W; a.gamma = gamma; a.pool_max = pool_max ? 1 : 0;
   a.scores = scores; a.indices = indices;
+  if (window) a.window = *window;
   int CS = select_cluster(rows, n_kv, clusters_of);
   a.parts = CS;
   if (I_hat && gather && n_kv <= kSelLocalRows && rows <= clusters_of[0]) {
@@ -547,23 +601,26 @@ cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep
     if (a.parts > (a.keep + 31) / 32) a.parts = (a.keep + 31) / 32;   // at least a row per warp to copy
   }
   a.per = (n_kv + CS - 1) / CS;
-  const bool small_blocks = rows > clusters_of[0];
+  // 512 threads: several blocks to an SM; and for the shortest rows, where a thread of 1024 has little more than a key to itself
+  // and each instruction's issue for 32 warps costs more than it saves (1024 rows 28.7 -> 27.5 us, but 2176 rows 21.2 -> 22.4)
+  const bool many = rows > clusters_of[0], small_blocks = many || (CS == 1 && n_kv <= kSelShortRows);
   const int threads = small_blocks ? 512 : 1024;
   // the taps of a slice (with some margin for a window known on the device only), later the indices the block gathers
   const long long cap = kSelMaxSmem / 4, per4 = (a.per + 3) & ~3;
-  long long room = I_hat ? (long long)a.per + 7 + (pool_dev ? 256 : W) : 0;
+  long long room = I_hat ? (long long)a.per + 7 + (window ? 256 : W) : 0;
   long long need = I_hat ? a.per / 2 : 0;   // held keys leave at least this (longer windows then read their taps from memory)
-  if (gather) {   // the indices, and behind them two buffers of copy_rows rows of K and V for every warp
-    const long long buf = (long long)(threads / 32) * a.ga.row_chunks * 16, idx = (((a.keep + a.parts - 1) / a.parts) + 3) & ~3;
-    a.held = per4 + (need > buf ? need : buf) <= cap ? 1 : 0;
-    const long long most = cap - (a.held ? per4 : 0);
-    a.own_idx = idx + buf <= most ? 1 : 0;
-    a.copy_rows = 4;
-    while (a.copy_rows > 1 && (a.own_idx ? idx : 0) + a.copy_rows * buf > most) a.copy_rows >>= 1;
+  a.held = per4 + need <= cap ? 1 : 0;
+  if (gather) {   // the indices, and behind them, for bulk copies, two buffers of copy_rows rows of K and V for every warp
+    const long long share = (a.keep + a.parts - 1) / a.parts, idx = (share + 3) & ~3;
+    const long long buf = share > kSelFewRows ? (long long)(threads / 32) * a.ga.row_chunks * 16 : 0;
+    if (need < buf) need = buf;
+    a.held = per4 + need <= cap ? 1 : 0;
+    const long long free = cap - (a.held ? per4 : 0);
+    a.own_idx = idx + buf <= free ? 1 : 0;
+    a.copy_rows = buf ? 4 : 0;
+    while (a.copy_rows > 1 && (a.own_idx ? idx : 0) + a.copy_rows * buf > free) a.copy_rows >>= 1;
     const long long copies = (a.own_idx ? idx : 0) + a.copy_rows * buf;
     if (room < copies) room = copies;
-  } else {
-    a.held = per4 + need <= cap ? 1 : 0;
   }
   const long long most = cap - (a.held ? per4 : 0);
   a.room = (int)(room < most ? room : most);
@@ -581,7 +638,7 @@ cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chained ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, small_blocks ? select_kernel<512> : select_kernel<1024>, a);
+  return cudaLaunchKernelEx(&cfg, many ? select_kernel<512, 3> : small_blocks ? select_kernel<512, 2> : select_kernel<1024, 1>, a);
 }
 
 cudaError_t launch_compact(const Problem& p, const void* K, const void* V, const int32_t* indices, int n_sel,

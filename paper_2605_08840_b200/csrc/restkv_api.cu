@@ -275,10 +275,9 @@ static restkv_status run_score(Call& c, const Problem& p, const Workspace& ws, c
     RESTKV_LAUNCH(c, RESTKV_KERNEL_PASS2, launch_simt_pass2(p, ws, Q, K, V, ema_decay, adaptive ? ws.I_raw : nullptr, c.st), 1);
   }
   if (adaptive) {
-    int nl = 0;
-    cudaError_t e = launch_adaptive_params(p, ws, pool->budget, pool->beta, pool->base_width, c.h->sm_count, c.h->dev_status, c.st, &nl);
-    if (e != cudaSuccess) return c.fail(e);
-    c.h->launches += nl;
+    RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE, launch_row_sums(p, ws, pool->budget, c.h->sm_count, c.h->dev_status, c.st), 1);
+    if (scores)   // (the selection works the windows out for itself)
+      RESTKV_LAUNCH(c, RESTKV_KERNEL_NONE, launch_window_params(p, ws, pool->budget, pool->beta, pool->base_width, c.st), 1);
   }
   if (scores)
     RESTKV_LAUNCH(c, RESTKV_KERNEL_POOL,
@@ -465,8 +464,10 @@ static restkv_status evict_impl(restkv_handle* h, const restkv_shape* shape, con
   // this itself for long: six group barriers and four digit passes by 144 CTAs of which each had little to do, half of a
   // short context's time; a 3000-row prompt went from 54.8 to 40.9 us.)
   h->last_evict_fused = on_tc && !adaptive && !budgets && h->fused_select;
+  WindowArgs window{};
+  if (adaptive) window = window_args(p, ws, pool->budget, pool->beta, pool->base_width);
   RESTKV_LAUNCH(c, RESTKV_KERNEL_SELECT,
-                launch_select(p.BH, p.n, p.n_kv, budget, budgets, ws.I_hat, adaptive ? ws.pool : nullptr, pool->width,
+                launch_select(p.BH, p.n, p.n_kv, budget, budgets, ws.I_hat, adaptive ? &window : nullptr, pool->width,
                               pool->shift, p.spatial == RESTKV_SPATIAL_MAX, scores, indices, &p, K, V, K_out, V_out,
                               h->select_clusters, h->dev_status, h->fused_select, c.st), 1);
   return RESTKV_OK;

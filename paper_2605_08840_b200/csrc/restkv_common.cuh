@@ -73,6 +73,14 @@ constexpr int kDevWords = kDevStatusWords + 2 * kCounterSets * kDevCounterWords;
 int pass1_splits(const Problem& p, int sm_count);
 size_t plan_workspace(const Problem& p, int budget, int sm_count, bool adaptive, void* base, Workspace* ws);
 
+// The adaptive window: the per-query index sums, and a head's window from them, either by whoever needs it (head_window) or by a
+// kernel of its own into ws.pool.
+struct WindowArgs {
+  const unsigned long long* sums;   // [BH * G * w], null: no adaptive window
+  double beta;
+  int G, w, Bp, base_width;
+};
+
 // ---- launches (each returns the cudaError_t of the launch) -------------------------------------
 cudaError_t launch_simt_pass1(const Problem& p, const Workspace& ws, const void* Q, const void* K, const void* V,
                               cudaStream_t st);
@@ -82,7 +90,7 @@ cudaError_t launch_simt_pass2(const Problem& p, const Workspace& ws, const void*
 cudaError_t launch_pool(const Problem& p, const Workspace& ws, const int* pool_dev, int W, int gamma, float* scores,
                         int32_t* pool_used, cudaStream_t st);
 cudaError_t select_init(int* clusters_of);   // [4]
-cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep_rows, const float* I_hat, const int* pool_dev,
+cudaError_t launch_select(int rows, int n, int n_kv, int budget, const int* keep_rows, const float* I_hat, const WindowArgs* window,
                           int W, int gamma, bool pool_max, float* scores, int32_t* indices, const Problem* gather, const void* K, const void* V, void* K_out, void* V_out,
                           const int* clusters_of, unsigned int* dev_status, bool chained, cudaStream_t st);
 cudaError_t launch_compact(const Problem& p, const void* K, const void* V, const int32_t* indices, int n_sel,
@@ -97,8 +105,9 @@ void decode_mma_plan(const int* clusters_of, int BH, int G, int n_rows, size_t s
 cudaError_t launch_decode_mma(void* state, const Problem& p, const void* q, const void* Kc, const void* Vc, int n_rows,
                               float* out, float* lse, float* part, int cluster, int splits, long long wait_limit,
                               unsigned int* dev_status, cudaStream_t st);
-cudaError_t launch_adaptive_params(const Problem& p, const Workspace& ws, int budget, float beta, int base_width,
-                                   int sm_count, unsigned int* dev_status, cudaStream_t st, int* n_launches);
+WindowArgs window_args(const Problem& p, const Workspace& ws, int budget, float beta, int base_width);
+cudaError_t launch_row_sums(const Problem& p, const Workspace& ws, int budget, int sm_count, unsigned int* dev_status, cudaStream_t st);
+cudaError_t launch_window_params(const Problem& p, const Workspace& ws, int budget, float beta, int base_width, cudaStream_t st);
 cudaError_t adaptive_init();
 
 // Output projection (Eq. 4): the caller-owned factor buffer and the per-call projected rows.
@@ -146,6 +155,29 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, int threa
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// Eq. 10-12 for one head from the index sums of its rows (front and rear half of the window apart).  Called by a whole warp, every
+// lane of which gets the result.
+__device__ __forceinline__ void head_window(const WindowArgs& a, int bh, int* W, int* gamma) {
+  unsigned long long front = 0, rear = 0;
+  for (int e = threadIdx.x & 31; e < a.G * a.w; e += 32) {
+    const unsigned long long s = a.sums[(long long)bh * a.G * a.w + e];
+    if (e % a.w < a.w / 2) front += s;
+    else rear += s;
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    front += __shfl_xor_sync(0xffffffffu, front, off);
+    rear += __shfl_xor_sync(0xffffffffu, rear, off);
+  }
+  const long long cnt_front = (long long)a.G * (a.w / 2) * a.Bp;
+  const long long cnt_rear = (long long)a.G * (a.w - a.w / 2) * a.Bp;
+  const double D_rear = (double)rear / (double)cnt_rear;
+  const double D_front = cnt_front ? (double)front / (double)cnt_front : D_rear;
+  const double x = (D_front - D_rear) / a.beta;
+  *W = 2 * (int)floor(fabs(x)) + a.base_width;   // Eq. 11, and the base width around it
+  *gamma = (int)trunc(x);                        // Eq. 12, truncating toward zero
 }
 
 // Scores map to unsigned keys whose order matches the float order.
