@@ -20,9 +20,8 @@ constexpr int kRsHalfSmem = 92 * 1024;   // dynamic shared memory of a block whe
 // more than the walks that are needed: the extremes,
 // a histogram of 11-bit digits of the offsets from the smallest (about a thousand bins in use, so one histogram serves all
 // warps without contention), then the sum above the digit that holds the Bp-th largest while that digit's few keys are
-// listed and ranked, a key per warp.  1024 rows of 20011: 43 us with one block of 1024 threads and two rows in flight per SM
-// (10 k cycles per row, 3.6 k of them synchronisation); the whole call 134.0 us with that, 129.7-131 us so and with the windows
-// worked out by the selection.
+// listed and ranked, a key per warp.  1024 rows of 20011: 43.5 us with one block of 1024 threads and two rows in flight per SM
+// (10 k cycles per row, 3.6 k of them synchronisation), 39 us so.
 template <int kRsThreads, bool kHeld>   // kHeld false: no buffers, the keys are read from global memory on every walk
 __global__ void __launch_bounds__(kRsThreads, kRsThreads <= 512 ? 2 : 1)
 row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buffers, unsigned long long* __restrict__ sums,
