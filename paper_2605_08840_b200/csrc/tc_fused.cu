@@ -515,6 +515,11 @@ __device__ __forceinline__ float4 project_row_warp(const float* __restrict__ Mt,
   return acc;
 }
 
+// One element's share of the constant o^T Mt o that goes with a row rounded to -2 y, y = bf16(Mt o): o (2 y - Mt o).  Of the
+// rounding error eps = y - Mt o it leaves 2 eps . (o - v) in the squared distance; with o . Mt o it left 2 eps . v, which does not
+// shrink as o approaches v: values within 5 % of each other were off by 7 %, within 2 % by half, and came out negative.
+__device__ __forceinline__ float projected_constant(float o, float mo, float minus_2y) { return o * (-minus_2y - mo); }
+
 // x = hi + mid + lo with three bf16 pieces (24 significant bits): their bits.
 __device__ __forceinline__ uint3 split3(float x) {
   const __nv_bfloat16 hi = __float2bfloat16_rn(x);
@@ -637,8 +642,8 @@ __device__ void combine_rows(const Ctx& cx, const FusedArgs& a, int bh, int grou
     }
   }
   named_barrier_sync(2, kThreads);
-  // With the output projection: the row of the third contraction is -2 bf16(Mt o), its constant o^T Mt o.  Eight rows at a time,
-  // which belong to one query head: thread = (column, quarter of the sum), so that Mt comes once for all eight.
+  // With the output projection: the row of the third contraction is -2 bf16(Mt o), its constant (projected_constant) o^T Mt o.
+  // Eight rows at a time, which belong to one query head: thread = (column, quarter of the sum), so that Mt comes once for all eight.
   if (kProj) {
     float* rows = reinterpret_cast<float*>(cx.gen_base + kOffO);              // [8][128]
     float* quarters = rows + 8 * kHeadDim;                                    // [4][8][128]
@@ -675,12 +680,13 @@ __device__ void combine_rows(const Ctx& cx, const FusedArgs& a, int bh, int grou
         mo.x += u.x; mo.y += u.y;
       }
       const float2 o = *reinterpret_cast<const float2*>(rows + r * kHeadDim + c2);
-      float on = fmaf(o.x, mo.x, o.y * mo.y);
+      const uint32_t m2 = pack_bf16x2(-2.f * mo.x, -2.f * mo.y);
+      float on = projected_constant(o.x, mo.x, __uint_as_float(m2 << 16)) + projected_constant(o.y, mo.y, __uint_as_float(m2 & 0xFFFF0000u));
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) on += __shfl_xor_sync(0xffffffffu, on, off);
       if (r < nr) {
         *reinterpret_cast<float2*>(a.O_proj + (ri + r) * kHeadDim + c2) = mo;
-        *reinterpret_cast<uint32_t*>(a.O_m2 + (ri + r) * kHeadDim + c2) = pack_bf16x2(-2.f * mo.x, -2.f * mo.y);
+        *reinterpret_cast<uint32_t*>(a.O_m2 + (ri + r) * kHeadDim + c2) = m2;
         if (lane == 0) on_part[(wq & 1) * rb + g0 + r] = on;
       }
       named_barrier_sync(2, kThreads);   // the rows are overwritten by the next eight
@@ -1212,7 +1218,8 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
       const int j = (tile0 + T - 1 - it) * kTile + t;
       const uint32_t tS = tmem + (uint32_t)s * 256u + lane_base + (uint32_t)cgp * 32u, tC = tS + 128u;
       // ||o - v||^2 = C' + ||v||^2 is formed with ||v||^2 raised by 2^-16 of itself: a bias of ~1e-5 that keeps
-      // the sum positive when the expansion cancels, so that no clamp is needed.
+      // the sum positive when the expansion cancels: C' is that of the rounded o exactly, so that no clamp is needed.  Under the
+      // projection no vector need belong to the rounded Mt o (Mt may be nearly singular): there a negative sum counts as 0.
       const float vnb = vn * 1.0000152587890625f;
       const f32x2 vn2 = f2_make(vnb, vnb);
       const float vlen = kInd == 2 ? sqrtf(vn) : 1.f;          // ||v_j||
@@ -1255,7 +1262,8 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
               const f32x2 u2 = (!from_lse && (q & 3) == 3) ? exp2_fma(f2_make(fminf(f2_lo(nt), 126.f), fminf(f2_hi(nt), 126.f)))
                                        : f2_make(ex2_approx(f2_lo(nt)), ex2_approx(f2_hi(nt)));
               const f32x2 um = f2_add(u2, m1);                                                       // 1/A - 1
-              const f32x2 x = f2_add(f2_make(cv[2 * q], cv[2 * q + 1]), vn2);                       // ||o - v||^2
+              f32x2 x = f2_add(f2_make(cv[2 * q], cv[2 * q + 1]), vn2);                             // ||o - v||^2
+              if (kProj) x = f2_make(fmaxf(f2_lo(x), 0.f), fmaxf(f2_hi(x), 0.f));
               const f32x2 bq = f2_fma(f2_mul(x, um), um, tiny2);                                    // x (1/A - 1)^2
               Iq = f2_mul(x, f2_make(rsqrt_approx(f2_lo(bq)), rsqrt_approx(f2_hi(bq))));
             } else {
@@ -1285,7 +1293,7 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
             mx = fmaxf(mx, sv[u]);
             if (kEq7) {
               const float um = ex2_approx(sv[u] * neg_c2) - 1.f;
-              const float x = cv[u] + vnb;
+              const float x = kProj ? fmaxf(cv[u] + vnb, 0.f) : cv[u] + vnb;
               I[u] = x * rsqrt_approx(fmaf(x * um, um, 1e-36f));
             } else {
               I[u] = ex2_approx(-sv[u] * neg_c2) * vlen;
@@ -1544,7 +1552,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
 // ------------------------------------------------------------------------------------------------
 // The window rows' outputs O and log-sum-exps given by the caller (the prefill attention has them), under the output
-// projection: what phase B would have written for phase C, the row -2 bf16(Mt o), the constant o^T Mt o, and Mt o itself.
+// projection: what phase B would have written for phase C, the row -2 bf16(Mt o), its constant o^T Mt o, and Mt o itself.
 // One warp per query row, lane = four output dims.
 __global__ void from_lse_prep_kernel(int rows, float scale, const float* __restrict__ O, const float* __restrict__ LSE,
                                      __nv_bfloat16* __restrict__ O_m2, __nv_bfloat16* __restrict__ aug,
@@ -1564,11 +1572,13 @@ __global__ void from_lse_prep_kernel(int rows, float scale, const float* __restr
   const float4 mo = project_row_warp(proj_Mt + (long long)((bh % Hkv) * (kRows / w) + r / w) * kHeadDim * kHeadDim,
                                      xs[wi], lane);
   *reinterpret_cast<float4*>(O_proj + (long long)ri * kHeadDim + lane * 4) = mo;
-  om[0] = __float2bfloat16_rn(-2.f * mo.x);
-  om[1] = __float2bfloat16_rn(-2.f * mo.y);
-  om[2] = __float2bfloat16_rn(-2.f * mo.z);
-  om[3] = __float2bfloat16_rn(-2.f * mo.w);
-  float on = (o.x * mo.x + o.y * mo.y) + (o.z * mo.z + o.w * mo.w);
+  const float ov[4] = {o.x, o.y, o.z, o.w}, mv[4] = {mo.x, mo.y, mo.z, mo.w};
+  float on = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    om[i] = __float2bfloat16_rn(-2.f * mv[i]);
+    on += projected_constant(ov[i], mv[i], __bfloat162float(om[i]));
+  }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) on += __shfl_xor_sync(0xffffffffu, on, off);
   __nv_bfloat16* arow = aug + (long long)ri * 64;

@@ -6,7 +6,7 @@ import pytest
 
 import oracle
 from paper_2605_08840_b200 import binding as rk
-from paper_2605_08840_b200.inputs import CONFIGS, Case, make_inputs, make_decode_query, round_to_bf16_bits
+from paper_2605_08840_b200.inputs import CONFIGS, Case, bf16_bits_to_f32, make_inputs, make_decode_query, round_to_bf16_bits
 
 from helpers import (DECODE_TOL, TOL, DeviceRun, assert_compaction_exact, assert_decode_close, assert_scores_close, assert_selection_valid,
                      shape_of, torch_dev)
@@ -1378,6 +1378,62 @@ def test_projection_at_other_window_lengths(handle, spec):
 def test_projection_with_a_variant(handle):
     inp = make_inputs(CONFIGS["cfg2"])
     projection_check(handle, inp, 48, path=rk.PATH_TENSOR_CORE, variant=(REC, INV, rk.SPATIAL_MAX, rk.GROUP_MAX))
+
+
+@pytest.mark.parametrize("call", ["evict", "from_lse", "adaptive"])
+@pytest.mark.parametrize("d_model", [96, 300])
+@pytest.mark.parametrize("spread", [0.05, 0.02, 0.01])
+def test_projection_with_values_close_together(handle, spread, d_model, call):
+    """Rows of V that differ by a few percent from one vector: o comes close to every v, and the three terms of
+    (o - v)^T M (o - v) cancel to spread^2 of themselves.  The constant and the cross term must then belong to the same rounded row,
+    as without a projection, and no squared distance may come out negative (its root would be a NaN, which is kept first).
+
+    The tolerance follows from the formats, per (window row, token): Mt o meets v in bf16, an error of at most 2^-8 of each element,
+    2^-8 / sqrt(3) rms, of which the consistent constant leaves 2 eps . (o - v), taken at six times its rms; ||v||^2 in the norm
+    of M is raised by 2^-16; the tensor core's sums are truncated (2^-18 of the terms).  Half of that against the squared distance
+    is the norm's error, and a score is a weighted mean of such norms."""
+    import torch
+    case = Case("close", 1, 8, 2, 128, 1100, 32, 200, 1, 0, 0.9, "bf16", 0, "normal", 77)
+    inp = make_inputs(case)
+    rng = np.random.default_rng(5)
+    common = rng.standard_normal((1, 2, 1, 128))
+    inp.V = bf16_bits_to_f32(round_to_bf16_bits((common + spread * inp.V).astype(np.float32)))
+    W, factor = _make_projection(handle, case, d_model, seed=6)
+    run = DeviceRun(handle, inp, adaptive_budget=case.budget if call == "adaptive" else 0)
+    handle.set_kernel_path(rk.PATH_TENSOR_CORE)
+    handle.set_output_projection(factor, case.n_q_heads, case.head_dim)
+    try:
+        if call == "from_lse":
+            _, O, lse = _window_stats(inp, with_A_check=False)
+            handle.evict_from_lse(run.shape, run.Q, run.K, run.V, torch.from_numpy(O).cuda(), torch.from_numpy(lse).cuda(),
+                                  case.ema_decay, run.pool(), run.budget, run.indices, run.K_out, run.V_out, run.ws,
+                                  scores_out=run.scores)
+            torch.cuda.synchronize()
+            scores, idx = run.scores.cpu().numpy(), run.indices.cpu().numpy()
+        else:   # (a window of one row either way)
+            scores, idx, _, _ = run.evict(pool=rk.adaptive_pool(1e9, 1, run.budget) if call == "adaptive" else None)
+        assert handle.poll_status() == rk.RESTKV_OK
+    finally:
+        handle.set_kernel_path(rk.PATH_AUTO)
+        handle.set_output_projection(None)
+    ref = oracle_scores(inp, W_O=W, want_O=True)
+    tol = np.zeros(ref.scores.shape)
+    for hq in range(case.n_q_heads):
+        h = hq // case.group
+        M = W[hq].astype(np.float64) @ W[hq].astype(np.float64).T
+        v = inp.V[0, h].astype(np.float64)
+        vMv = np.einsum("ni,ni->n", v @ M, v)
+        for o in ref.O[0, hq]:
+            diff, Mo = o - v, M @ o
+            x = np.einsum("ni,ni->n", diff @ M, diff)
+            err = 6 * 2 * 2.0 ** -8 / np.sqrt(3) * np.sqrt((diff ** 2) @ (Mo ** 2)) + 2.0 ** -16 * vMv + 2.0 ** -18 * (o @ Mo + vMv)
+            tol[0, h] = np.maximum(tol[0, h], 0.5 * err / x)
+    assert np.all(np.isfinite(scores))
+    off = np.abs(scores - ref.scores) / ref.scores
+    worst = np.unravel_index(np.argmax(off / (tol + TOL["bf16"])), off.shape)
+    assert np.all(off <= tol + TOL["bf16"]), "score off by %.2e where %.2e is allowed" % (off[worst], tol[worst] + TOL["bf16"])
+    want = np.sort(np.argsort(-scores, axis=-1, kind="stable")[..., :run.keep], axis=-1)
+    np.testing.assert_array_equal(idx, want)
 
 
 def test_projection_is_ignored_by_the_attention_weight_indicators(handle):
