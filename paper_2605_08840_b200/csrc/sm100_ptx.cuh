@@ -42,7 +42,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 }
 
 // Bounded wait: gives up after `max_cycles` SM clocks or as soon as *abort_flag is set, records the
-// failure in *abort_flag and the device status word, and returns false.  Never spins for ever.
+// failure in *abort_flag and the device status word, and returns false.  Never spins for ever.  Every lane has a verdict of its own:
+// what takes the whole warp (tensor-memory loads, votes, __syncwarp) must not depend on it.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                           unsigned int* dev_status, unsigned int status_bit,
                                           long long max_cycles = 2000000000ll) {

@@ -158,6 +158,11 @@ __device__ bool group_barrier_follow(volatile int* go) {
   return *go != 0;
 }
 
+// Tiles that the loading thread has requested for the present head: K and V of phase A, stages of phase C.
+struct Loads {
+  int k, v, c;
+};
+
 struct Ctx {
   uint32_t smem_base;      // shared-window address of the 1024-aligned dynamic region
   uint8_t* gen_base;       // the same location as a generic pointer
@@ -195,6 +200,9 @@ __device__ __forceinline__ void load_stage_c(const Ctx& cx, const CUtensorMap* t
   tma_load_4d(dV + kBoxBytes, tmV, bar, 64, j0, h, b, policy);
 }
 
+// Where a wait of a warp has run out, the loops over the tiles run on without waiting, on whatever lies there: each lane has given up
+// for itself, and what the warp does together must not depend on that.  (The call ends with the timeout status.)
+
 // ------------------------------------------------------------------------------------------------
 // Phase A: this CTA's share [tile0, tile0 + T) of one head.
 // Control warps: warp 0 loads (K ring of 2 slots, V ring of 3), warp 1 issues the MMAs (S(it), then O += P V of tile
@@ -203,23 +211,21 @@ __device__ __forceinline__ void load_stage_c(const Ctx& cx, const CUtensorMap* t
 // it) and O_g at 256 + g*128.
 // Behind the share's last tiles the loader requests the first two stages of phase C (T2 tiles, walked from the last one), each
 // as its slots fall free: they arrive while the partials are merged and the memory would be idle otherwise, and are out of the
-// way of the merge's own reads.  Returns their number (the loading thread only).
-__device__ int phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtensorMap* tmQ, const CUtensorMap* tmK,
-                       const CUtensorMap* tmV, int bh, int tile0, int T, int T2) {
+// way of the merge's own reads.
+__device__ void phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtensorMap* tmQ, const CUtensorMap* tmK,
+                        const CUtensorMap* tmV, int bh, int tile0, int T, int T2, Loads* ld) {
   FusedBars* B = cx.B;
   int* abort_flag = cx.abort_flag;
   unsigned int* dev_status = a.dev_status;
   const int b = bh / a.Hkv, h = bh % a.Hkv;
   const int warp = cx.warp, lane = cx.lane;
   const uint32_t tmem = cx.tmem;
-  int pre = 0;
 
   if (warp == 0) {
     if (lane == 0 && T > 0) {
       mbar_arrive_expect_tx(&B->q_full, kTileBytes);
       tma_load_3d(cx.gen_base + kOffQ, tmQ, &B->q_full, 0, 0, bh);
       tma_load_3d(cx.gen_base + kOffQ + kBoxBytes, tmQ, &B->q_full, 64, 0, bh);
-      int nK = 0, nV = 0;   // K and V tiles requested so far
       for (int it = 0; it < T; ++it) {
         const int ks = it & 1, vs = it % kFVSlots;
         const int j0 = (tile0 + it) * kTile;
@@ -231,7 +237,7 @@ __device__ int phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtensor
         mbar_arrive_expect_tx(&B->k_full[ks], kTileBytes);
         tma_load_4d(dK, tmK, &B->k_full[ks], 0, j0, h, b, policy);
         tma_load_4d(dK + kBoxBytes, tmK, &B->k_full[ks], 64, j0, h, b, policy);
-        ++nK;
+        ++ld->k;
         if (it >= kFVSlots &&
             !mbar_wait(&B->v_empty[vs], (it / kFVSlots - 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit))
           break;
@@ -239,7 +245,7 @@ __device__ int phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtensor
         mbar_arrive_expect_tx(&B->v_full[vs], kTileBytes);
         tma_load_4d(dV, tmV, &B->v_full[vs], 0, j0, h, b, policy);
         tma_load_4d(dV + kBoxBytes, tmV, &B->v_full[vs], 64, j0, h, b, policy);
-        ++nV;
+        ++ld->v;
       }
       // ring slots 2s and 2s + 1 make up stage s: the K slots of this phase, then its first two V slots
       for (int s = 0; s < 2 && s < T2; ++s) {
@@ -251,13 +257,7 @@ __device__ int phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtensor
         }
         if (!free) break;
         load_stage_c(cx, tmK, tmV, b, h, (tile0 + T2 - 1 - s) * kTile, s, policy_evict_first());
-        ++pre;
-      }
-      if (*(volatile int*)abort_flag) {
-        // a wait of this CTA has failed: the tiles requested last may still be on their way into shared memory
-        wait_issued(&B->q_full, 0);
-        for (int i = max(0, nK - 2); i < nK; ++i) wait_issued(&B->k_full[i & 1], (uint32_t)(i >> 1));
-        for (int i = max(0, nV - kFVSlots); i < nV; ++i) wait_issued(&B->v_full[i % kFVSlots], (uint32_t)(i / kFVSlots));
+        ++ld->c;
       }
     }
   } else if (warp == 1) {
@@ -293,23 +293,22 @@ __device__ int phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtensor
           umma_commit(&B->v_empty[vs]);
         }
       }
-      if (*(volatile int*)abort_flag) {   // let the MMAs already issued finish before the CTA goes on to return
-        umma_commit(&B->drain);
-        wait_issued(&B->drain, 0);
-      }
     }
   } else if (warp < kFFirstWorker) {
     // ---------------- ||v||^2: one warp takes the even tiles, the other the odd ones; lane = 4 tokens ----------------
     const int vg = warp - 2;
     bool ok = true;
-    for (int it = 0; it < T && ok; ++it) {
+    for (int it = 0; it < T; ++it) {
       const int vs = it % kFVSlots;
       // Both warps wait for every tile, and the slot is refilled only once both have: otherwise one that is held up between its
       // own tile and this wait (its instructions on their way from memory again) could find the slot's barrier two phases on, which
       // looks like none, and wait for ever.
-      ok = __all_sync(0xffffffffu, mbar_wait(&B->v_full[vs], (it / kFVSlots) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit));
-      if (ok && (it & 1) != vg && lane == 0) mbar_arrive(&B->v_empty[vs]);
-      if (!ok || (it & 1) != vg) continue;
+      ok = ok && mbar_wait(&B->v_full[vs], (it / kFVSlots) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit);
+      if ((it & 1) != vg) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&B->v_empty[vs]);
+        continue;
+      }
       const uint8_t* vt = cx.gen_base + v_slot_off(vs);
       float vn[4];
 #pragma unroll
@@ -342,7 +341,6 @@ __device__ int phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtensor
       }
     }
   }
-  return pre;
 }
 
 // Worker warps in phase A: four softmax warpgroups, thread = query row; warpgroups g and g + 2 share tile slot g
@@ -378,7 +376,7 @@ __device__ void phase_a_worker(const Ctx& cx, const FusedArgs& a, int bh, int ti
   int uses = 0;                             // tiles this warpgroup has processed
   for (int it = g; it < T; it += 2, ++uses) {
     ok = ok && mbar_wait(&B->s_full[g], (uint32_t)uses & 1u, abort_flag, dev_status, kDevTimeout, a.wait_limit);
-    if (ok) tc_fence_after();
+    tc_fence_after();
     const int j0 = (tile0 + it) * kTile + hf * 64;
     const bool ragged = j0 + 64 > n;   // rows past the scored prefix: window rows (causal) or padding
     auto mask = [&](float* s, int c) {
@@ -392,24 +390,21 @@ __device__ void phase_a_worker(const Ctx& cx, const FusedArgs& a, int bh, int ti
     float sa[16], sb[16];
     // ---- sweep 1: row maximum of this half of the tile; the next 16 columns travel while 16 are reduced ----
     float tmax = -INFINITY;
-    if (ok) {
-      tmem_ld16(tS, sa);
+    tmem_ld16(tS, sa);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        float* cur = (c & 1) ? sb : sa;
-        float* nxt = (c & 1) ? sa : sb;
-        tmem_wait_ld();
-        tmem_ld16(tS + ((c + 1) & 3) * 16, nxt);   // after the last chunk: chunk 0 again, for sweep 2
-        if (ragged) mask(cur, c);
+    for (int c = 0; c < 4; ++c) {
+      float* cur = (c & 1) ? sb : sa;
+      float* nxt = (c & 1) ? sa : sb;
+      tmem_wait_ld();
+      tmem_ld16(tS + ((c + 1) & 3) * 16, nxt);   // after the last chunk: chunk 0 again, for sweep 2
+      if (ragged) mask(cur, c);
 #pragma unroll
-        for (int u = 0; u < 16; ++u) tmax = fmaxf(tmax, cur[u]);
-      }
+      for (int u = 0; u < 16; ++u) tmax = fmaxf(tmax, cur[u]);
     }
     my_max[row] = tmax;
     named_barrier_sync(3 + g, 256);            // the two halves of the slot exchange their row maxima
     tmax = fmaxf(tmax, other_max[row]);
     named_barrier_sync(3 + g, 256);            // both have read before the next tile overwrites
-    if (!ok) continue;
     const float m_tile = tmax * c2;
     // phase C takes the exact distance only in tiles where some weight can exceed kHeavyA: it compares this
     // maximum with the row's final normaliser
@@ -726,7 +721,7 @@ __device__ void combine_rows(const Ctx& cx, const FusedArgs& a, int bh, int grou
 template <int kW, bool kLse>
 __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtensorMap* tmQ, const CUtensorMap* tmO,
                                 const CUtensorMap* tmAug, const CUtensorMap* tmK, const CUtensorMap* tmV, int bh,
-                                int tile0, int T, int pre, int started) {
+                                int tile0, int T, int started, Loads* ld) {
   constexpr int kG = kRows / kW;
   FusedBars* B = cx.B;
   int* abort_flag = cx.abort_flag;
@@ -750,17 +745,12 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
         tma_load_3d(cx.gen_base + kOffO + kBoxBytes, tmO, &B->const_full, 64, 0, bh);
         tma_load_3d(cx.gen_base + kOffAug, tmAug, &B->const_full, 0, 0, bh);
       }
-      int nS = pre;   // stages requested so far
       const uint64_t policy = policy_evict_first();
-      for (int it = pre; it < T; ++it) {   // the first `pre` tiles were requested before the group barriers
+      for (int it = ld->c; it < T; ++it) {   // the first tiles were requested before the group barriers
         const int s = it & 1;
         if (it >= 2 && !mbar_wait(&B->kv_empty[s], ((it >> 1) - 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit)) break;
         load_stage_c(cx, tmK, tmV, b, h, (tile0 + T - 1 - it) * kTile, s, policy);
-        ++nS;
-      }
-      if (*(volatile int*)abort_flag) {
-        wait_issued(&B->const_full, 0);
-        for (int i = max(0, nS - 2); i < nS; ++i) wait_issued(&B->kv_full[i & 1], (uint32_t)(i >> 1));
+        ++ld->c;
       }
     }
   } else if (warp == 1) {
@@ -783,10 +773,6 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
         umma_commit(&B->acc_full[s]);
         umma_commit(&B->kv_empty[s]);
       }
-      if (*(volatile int*)abort_flag) {
-        umma_commit(&B->drain);
-        wait_issued(&B->drain, 0);
-      }
     }
   } else if (!kLse && warp == 2) {
     // ---- which tiles need their logits looked at: some row's largest logit reaches that row's M2 - log2(1 / kHeavyA).
@@ -799,6 +785,7 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
       m2r[k] = a.row_M2[(long long)bh * kRows + k * 32 + lane] - log2f(1.f / kHeavyA);
       next[k] = T > 0 ? tm[(long long)(T - 1) * kRows + k * 32] : -INFINITY;
     }
+    bool ok = true;
     for (int it = 0; it < T; ++it) {
       const int s = it & 1;
       const bool any = __any_sync(0xffffffffu, next[0] > m2r[0] || next[1] > m2r[1] || next[2] > m2r[2] || next[3] > m2r[3]);
@@ -806,7 +793,7 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
 #pragma unroll
         for (int k = 0; k < 4; ++k) next[k] = tm[(long long)(T - 2 - it) * kRows + k * 32];
       }
-      if (it >= 2 && !mbar_wait(&B->acc_empty[s], ((it >> 1) - 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit)) break;
+      ok = ok && (it < 2 || mbar_wait(&B->acc_empty[s], ((it >> 1) - 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit));
       if (lane == 0) {
         cx.look[s] = any;
         mbar_arrive(&B->acc_full[s]);
@@ -816,10 +803,9 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
     // ---- ||v||^2 of the tile's tokens from the V tile in shared memory (phase A, which computes it otherwise, does
     //      not run): warp 2 takes tokens 0-63, warp 3 tokens 64-127, a lane two rows; ring of four tiles ----
     bool ok = true;
-    for (int it = 0; it < T && ok; ++it) {
+    for (int it = 0; it < T; ++it) {
       const int s = it & 1;
-      ok = mbar_wait(&B->kv_full[s], (it >> 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit);
-      if (!ok) break;
+      ok = ok && mbar_wait(&B->kv_full[s], (it >> 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit);
       const uint8_t* vt = cx.gen_base + k_slot_off(2 * s) + kTileBytes;
 #pragma unroll
       for (int rr = 0; rr < 2; ++rr) {
@@ -1213,145 +1199,141 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensor
     ok = ok && mbar_wait(&B->acc_full[s], par, abort_flag, dev_status, kDevTimeout, a.wait_limit);
     float tot = 0.f;
     int unit = kMaxHeavy;   // this lane's place in the list of heavy units
-    if (ok) {
-      tc_fence_after();
-      const int j = (tile0 + T - 1 - it) * kTile + t;
-      const uint32_t tS = tmem + (uint32_t)s * 256u + lane_base + (uint32_t)cgp * 32u, tC = tS + 128u;
-      // ||o - v||^2 = C' + ||v||^2 is formed with ||v||^2 raised by 2^-16 of itself: a bias of ~1e-5 that keeps
-      // the sum positive when the expansion cancels: C' is that of the rounded o exactly, so that no clamp is needed.  Under the
-      // projection no vector need belong to the rounded Mt o (Mt may be nearly singular): there a negative sum counts as 0.
-      const float vnb = vn * 1.0000152587890625f;
-      const f32x2 vn2 = f2_make(vnb, vnb);
-      const float vlen = kInd == 2 ? sqrtf(vn) : 1.f;          // ||v_j||
-      const f32x2 vlen2 = f2_make(vlen, vlen);
-      f32x2 h2 = f2_make(0.f, 0.f);
-      float sv0[16], cv0[16], sv1[16], cv1[16];
-      const bool look = kEq7 && (from_lse || cx.look[s] != 0);
-      float mx = -INFINITY;   // where a weight may exceed kHeavyA: this lane's largest logit
-      if (raw_head == nullptr) {
-        tmem_ld16(tS, sv0);
-        if (kEq7) tmem_ld16(tC, cv0);
+    tc_fence_after();
+    const int j = (tile0 + T - 1 - it) * kTile + t;
+    const uint32_t tS = tmem + (uint32_t)s * 256u + lane_base + (uint32_t)cgp * 32u, tC = tS + 128u;
+    // ||o - v||^2 = C' + ||v||^2 is formed with ||v||^2 raised by 2^-16 of itself: a bias of ~1e-5 that keeps
+    // the sum positive when the expansion cancels: C' is that of the rounded o exactly, so that no clamp is needed.  Under the
+    // projection no vector need belong to the rounded Mt o (Mt may be nearly singular): there a negative sum counts as 0.
+    const float vnb = vn * 1.0000152587890625f;
+    const f32x2 vn2 = f2_make(vnb, vnb);
+    const float vlen = kInd == 2 ? sqrtf(vn) : 1.f;          // ||v_j||
+    const f32x2 vlen2 = f2_make(vlen, vlen);
+    f32x2 h2 = f2_make(0.f, 0.f);
+    float sv0[16], cv0[16], sv1[16], cv1[16];
+    const bool look = kEq7 && (from_lse || cx.look[s] != 0);
+    float mx = -INFINITY;   // where a weight may exceed kHeavyA: this lane's largest logit
+    if (raw_head == nullptr) {
+      tmem_ld16(tS, sv0);
+      if (kEq7) tmem_ld16(tC, cv0);
+      tmem_wait_ld();
+      tmem_ld16(tS + 16, sv1);   // the second half of the columns travels while the first is worked on
+      if (kEq7) tmem_ld16(tC + 16, cv1);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const float* sv = c == 0 ? sv0 : sv1;
+        const float* cv = c == 0 ? cv0 : cv1;
+        if (c == 1) {
+          tmem_wait_ld();
+          // every tensor-memory read of this tile is done: the MMA warp may refill the accumulators (the logits of a
+          // tile that may hold a large weight are read once more below; the check between the two halves instead
+          // kept their instructions from mixing, 2 % of the whole call)
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0 && (from_lse || !look)) mbar_arrive(&B->acc_empty[s]);
+        }
+        if (from_lse && kEq7) {
+#pragma unroll
+          for (int u = 0; u < 16; ++u) mx = fmaxf(mx, sv[u]);
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const f32x2 nt = f2_mul(f2_make(sv[2 * q], sv[2 * q + 1]), nc2);
+          f32x2 Iq;
+          if (kEq7) {
+            // 1/A; one pair in four on the FMA pipe (1/A beyond 2^126 squares to infinity below either way): batch of 8
+            // x 32768 544 -> 531 us, 131072 266 -> 263 us (power-limited clock); with every other pair no better, and from given statistics
+            // (no pass 1, so less to wait for) slower
+            const f32x2 u2 = (!from_lse && (q & 3) == 3) ? exp2_fma(f2_make(fminf(f2_lo(nt), 126.f), fminf(f2_hi(nt), 126.f)))
+                                     : f2_make(ex2_approx(f2_lo(nt)), ex2_approx(f2_hi(nt)));
+            const f32x2 um = f2_add(u2, m1);                                                       // 1/A - 1
+            f32x2 x = f2_add(f2_make(cv[2 * q], cv[2 * q + 1]), vn2);                             // ||o - v||^2
+            if (kProj) x = f2_make(fmaxf(f2_lo(x), 0.f), fmaxf(f2_hi(x), 0.f));
+            const f32x2 bq = f2_fma(f2_mul(x, um), um, tiny2);                                    // x (1/A - 1)^2
+            Iq = f2_mul(x, f2_make(rsqrt_approx(f2_lo(bq)), rsqrt_approx(f2_hi(bq))));
+          } else {
+            Iq = f2_make(ex2_approx(-f2_lo(nt)), ex2_approx(-f2_hi(nt)));                         // A
+            if (kInd == 2) Iq = f2_mul(Iq, vlen2);
+          }
+          if (q == 0 && (c * 16) % kRun == 0) Iq = f2_mul(Iq, seed2);
+          if (q == 7 && (c * 16 + 16) % kRun == 0) Iq = f2_mul(Iq, last2);
+          h2 = f2_fma(h2, d2, Iq);
+        }
+        if ((c * 16 + 16) % kRun == 0) {   // end of a run
+          const float run = fmaf(f2_lo(h2), ema_decay, f2_hi(h2));
+          tot = group_max ? fmaxf(tot, run) : tot + run;
+          h2 = f2_make(0.f, 0.f);
+        }
+      }
+    } else {
+      // the epilogue of every tile when the per-query indicators are wanted
+#pragma unroll 1
+      for (int c = 0; c < 4; ++c) {
+        float sv[8], cv[8], I[8];
+        tmem_ld8(tS + c * 8, sv);
+        tmem_ld8(tC + c * 8, cv);
         tmem_wait_ld();
-        tmem_ld16(tS + 16, sv1);   // the second half of the columns travels while the first is worked on
-        if (kEq7) tmem_ld16(tC + 16, cv1);
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const float* sv = c == 0 ? sv0 : sv1;
-          const float* cv = c == 0 ? cv0 : cv1;
-          if (c == 1) {
-            tmem_wait_ld();
-            // every tensor-memory read of this tile is done: the MMA warp may refill the accumulators (the logits of a
-            // tile that may hold a large weight are read once more below; the check between the two halves instead
-            // kept their instructions from mixing, 2 % of the whole call)
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0 && (from_lse || !look)) mbar_arrive(&B->acc_empty[s]);
-          }
-          if (from_lse && kEq7) {
-#pragma unroll
-            for (int u = 0; u < 16; ++u) mx = fmaxf(mx, sv[u]);
-          }
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const f32x2 nt = f2_mul(f2_make(sv[2 * q], sv[2 * q + 1]), nc2);
-            f32x2 Iq;
-            if (kEq7) {
-              // 1/A; one pair in four on the FMA pipe (1/A beyond 2^126 squares to infinity below either way): batch of 8
-              // x 32768 544 -> 531 us, 131072 266 -> 263 us (power-limited clock); with every other pair no better, and from given statistics
-              // (no pass 1, so less to wait for) slower
-              const f32x2 u2 = (!from_lse && (q & 3) == 3) ? exp2_fma(f2_make(fminf(f2_lo(nt), 126.f), fminf(f2_hi(nt), 126.f)))
-                                       : f2_make(ex2_approx(f2_lo(nt)), ex2_approx(f2_hi(nt)));
-              const f32x2 um = f2_add(u2, m1);                                                       // 1/A - 1
-              f32x2 x = f2_add(f2_make(cv[2 * q], cv[2 * q + 1]), vn2);                             // ||o - v||^2
-              if (kProj) x = f2_make(fmaxf(f2_lo(x), 0.f), fmaxf(f2_hi(x), 0.f));
-              const f32x2 bq = f2_fma(f2_mul(x, um), um, tiny2);                                    // x (1/A - 1)^2
-              Iq = f2_mul(x, f2_make(rsqrt_approx(f2_lo(bq)), rsqrt_approx(f2_hi(bq))));
-            } else {
-              Iq = f2_make(ex2_approx(-f2_lo(nt)), ex2_approx(-f2_hi(nt)));                         // A
-              if (kInd == 2) Iq = f2_mul(Iq, vlen2);
-            }
-            if (q == 0 && (c * 16) % kRun == 0) Iq = f2_mul(Iq, seed2);
-            if (q == 7 && (c * 16 + 16) % kRun == 0) Iq = f2_mul(Iq, last2);
-            h2 = f2_fma(h2, d2, Iq);
-          }
-          if ((c * 16 + 16) % kRun == 0) {   // end of a run
-            const float run = fmaf(f2_lo(h2), ema_decay, f2_hi(h2));
-            tot = group_max ? fmaxf(tot, run) : tot + run;
-            h2 = f2_make(0.f, 0.f);
+        for (int u = 0; u < 8; ++u) {
+          mx = fmaxf(mx, sv[u]);
+          if (kEq7) {
+            const float um = ex2_approx(sv[u] * neg_c2) - 1.f;
+            const float x = kProj ? fmaxf(cv[u] + vnb, 0.f) : cv[u] + vnb;
+            I[u] = x * rsqrt_approx(fmaf(x * um, um, 1e-36f));
+          } else {
+            I[u] = ex2_approx(-sv[u] * neg_c2) * vlen;
           }
         }
-      } else {
-        // the epilogue of every tile when the per-query indicators are wanted
+        if (j < n) {
+#pragma unroll
+          for (int u = 0; u < 8; ++u) raw_head[(long long)(cgp * 32 + c * 8 + u) * n + j] = I[u];
+        }
+        if ((c * 8) % kRun == 0) I[0] *= seed_coef;
+        if ((c * 8 + 8) % kRun == 0) I[7] *= last_coef;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) h2 = f2_fma(h2, d2, f2_make(I[2 * q], I[2 * q + 1]));
+        if ((c * 8 + 8) % kRun == 0) {   // end of a run
+          const float run = fmaf(f2_lo(h2), ema_decay, f2_hi(h2));
+          tot = group_max ? fmaxf(tot, run) : tot + run;
+          h2 = f2_make(0.f, 0.f);
+        }
+      }
+    }
+    if (raw_head != nullptr || (!from_lse && look)) {
+      if (kEq7 && raw_head == nullptr) {
 #pragma unroll 1
         for (int c = 0; c < 4; ++c) {
-          float sv[8], cv[8], I[8];
+          float sv[8];
           tmem_ld8(tS + c * 8, sv);
-          tmem_ld8(tC + c * 8, cv);
           tmem_wait_ld();
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            mx = fmaxf(mx, sv[u]);
-            if (kEq7) {
-              const float um = ex2_approx(sv[u] * neg_c2) - 1.f;
-              const float x = kProj ? fmaxf(cv[u] + vnb, 0.f) : cv[u] + vnb;
-              I[u] = x * rsqrt_approx(fmaf(x * um, um, 1e-36f));
-            } else {
-              I[u] = ex2_approx(-sv[u] * neg_c2) * vlen;
-            }
-          }
-          if (j < n) {
-#pragma unroll
-            for (int u = 0; u < 8; ++u) raw_head[(long long)(cgp * 32 + c * 8 + u) * n + j] = I[u];
-          }
-          if ((c * 8) % kRun == 0) I[0] *= seed_coef;
-          if ((c * 8 + 8) % kRun == 0) I[7] *= last_coef;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) h2 = f2_fma(h2, d2, f2_make(I[2 * q], I[2 * q + 1]));
-          if ((c * 8 + 8) % kRun == 0) {   // end of a run
-            const float run = fmaf(f2_lo(h2), ema_decay, f2_hi(h2));
-            tot = group_max ? fmaxf(tot, run) : tot + run;
-            h2 = f2_make(0.f, 0.f);
+          for (int u = 0; u < 8; ++u) mx = fmaxf(mx, sv[u]);
+        }
+      }
+      if (kEq7 && look && __any_sync(0xffffffffu, mx > heavy_thr && j < n)) {
+        if (mx > heavy_thr && j < n) unit = atomicAdd(cx.heavy, 1);
+        float* logits = heavy_logits(a, unit);
+#pragma unroll 1
+        for (int c = 0; c < 4; ++c) {
+          float sv[8];
+          tmem_ld8(tS + c * 8, sv);
+          tmem_wait_ld();
+          if (unit < kHeavyDumps) {
+            *reinterpret_cast<float4*>(logits + c * 8) = make_float4(sv[0], sv[1], sv[2], sv[3]);
+            *reinterpret_cast<float4*>(logits + c * 8 + 4) = make_float4(sv[4], sv[5], sv[6], sv[7]);
           }
         }
       }
-      if (raw_head != nullptr || (!from_lse && look)) {
-        if (kEq7 && raw_head == nullptr) {
-#pragma unroll 1
-          for (int c = 0; c < 4; ++c) {
-            float sv[8];
-            tmem_ld8(tS + c * 8, sv);
-            tmem_wait_ld();
-#pragma unroll
-            for (int u = 0; u < 8; ++u) mx = fmaxf(mx, sv[u]);
-          }
-        }
-        if (kEq7 && look && __any_sync(0xffffffffu, mx > heavy_thr && j < n)) {
-          if (mx > heavy_thr && j < n) unit = atomicAdd(cx.heavy, 1);
-          float* logits = heavy_logits(a, unit);
-#pragma unroll 1
-          for (int c = 0; c < 4; ++c) {
-            float sv[8];
-            tmem_ld8(tS + c * 8, sv);
-            tmem_wait_ld();
-            if (unit < kHeavyDumps) {
-              *reinterpret_cast<float4*>(logits + c * 8) = make_float4(sv[0], sv[1], sv[2], sv[3]);
-              *reinterpret_cast<float4*>(logits + c * 8 + 4) = make_float4(sv[4], sv[5], sv[6], sv[7]);
-            }
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&B->acc_empty[s]);
-      }
-      // only Eq. 7 has the factor 1 / (1 - A) and the distance that need the exact form near A = 1: those units are noted
-      // and done after the last tile (S' above heavy_thr <=> A > kHeavyA)
-      if (from_lse && look && mx > heavy_thr && j < n) unit = atomicAdd(cx.heavy, 1);
-      if (unit < kMaxHeavy) cx.heavy[1 + unit] = j * 4 + cgp;
-    } else {
+      tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&B->acc_empty[s]);
     }
-    red[it & 3][cgp][t] = kEq7 && unit < kMaxHeavy ? (float)(-1 - unit) : tot * fin_scale;
+    // only Eq. 7 has the factor 1 / (1 - A) and the distance that need the exact form near A = 1: those units are noted
+    // and done after the last tile (S' above heavy_thr <=> A > kHeavyA)
+    if (from_lse && look && mx > heavy_thr && j < n) unit = atomicAdd(cx.heavy, 1);
+    if (unit < kMaxHeavy) cx.heavy[1 + unit] = j * 4 + cgp;
+    // (nothing that only looks like a unit: without the accumulators the sum is anything)
+    red[it & 3][cgp][t] = kEq7 && unit < kMaxHeavy ? (float)(-1 - unit) : ok ? tot * fin_scale : 0.f;
     __syncwarp();
     if (lane == 0) mbar_arrive(&B->red_full[it & 3]);
   }
@@ -1369,6 +1351,23 @@ struct Plan {
   int group, rank, tile0, T1, T2;
 };
 
+// After a wait that ran out: what this CTA has set in motion must have landed before it gives its memory back.  Called once all
+// threads have met behind their last wait (one that had gone ahead could not know that another would still give up).  The
+// constants and Q are waited for where the phase asked for them: a barrier without a request behind it has its first phase open.
+__device__ void drain_issued(const Ctx& cx, const Loads& ld, bool consts) {
+  FusedBars* B = cx.B;
+  if (threadIdx.x == 0) {
+    if (ld.k > 0) wait_issued(&B->q_full, 0);
+    for (int i = max(0, ld.k - 2); i < ld.k; ++i) wait_issued(&B->k_full[i & 1], (uint32_t)(i >> 1));
+    for (int i = max(0, ld.v - kFVSlots); i < ld.v; ++i) wait_issued(&B->v_full[i % kFVSlots], (uint32_t)(i / kFVSlots));
+    if (consts) wait_issued(&B->const_full, 0);
+    for (int i = max(0, ld.c - 2); i < ld.c; ++i) wait_issued(&B->kv_full[i & 1], (uint32_t)(i >> 1));
+  } else if (cx.warp == 1 && cx.lane == 0) {
+    umma_commit(&B->drain);
+    wait_issued(&B->drain, 0);
+  }
+}
+
 // The two role loops below run through the same sequence of CTA-wide synchronisations: per head a barrier
 // re-initialisation (from the second head on), phase A, the prefetch point, group barrier, phase B, group
 // barrier, phase C, and a closing __syncthreads.
@@ -1385,42 +1384,37 @@ __device__ void control_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, 
       if (threadIdx.x == 0) init_bars(bars, false, kLse, a.lse != nullptr);
       __syncthreads();
     }
-    if (kLse) {
-      // O and the rows' normalisers are given: phase C only, and no CTA waits for another
-      phase_c_control<kW, kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, 0, 0);
-      tc_fence_before();
-      __syncthreads();
-      tc_fence_after();
-      continue;
-    }
-    const int pre = phase_a_control(cx, a, tmQ, tmK, tmV, bh, pl.tile0, pl.T1, pl.T2);
-    bool through = group_barrier(counter, (++epoch) * (unsigned int)a.cpg, abort_flag, go, a.dev_status, a.wait_limit);
-    // Phase B belongs to the worker warps.  Meanwhile S^T = K Q^T of the first two tiles of phase C, which do not need its results
-    // (the accumulators of phase A have been read, and Q is still there).
-    int started = 0;
-    if (through && cx.warp == 1 && cx.lane == 0) {
-      tc_fence_after();
-      for (; started < 2 && started < pl.T2; ++started) {
-        if (!mbar_wait(&bars->kv_full[started], 0, abort_flag, a.dev_status, kDevTimeout, a.wait_limit)) break;
-        mma_tile_kk(cx.tmem + (uint32_t)started * 256u, cx.smem_base + k_slot_off(2 * started), cx.smem_base + kOffQ, false);
+    Loads ld = {0, 0, 0};
+    if (!kLse) {   // (given O and the rows' normalisers: phase C only, and no CTA waits for another)
+      phase_a_control(cx, a, tmQ, tmK, tmV, bh, pl.tile0, pl.T1, pl.T2, &ld);
+      bool through = group_barrier(counter, (++epoch) * (unsigned int)a.cpg, abort_flag, go, a.dev_status, a.wait_limit);
+      // Phase B belongs to the worker warps.  Meanwhile S^T = K Q^T of the first two tiles of phase C, which do not need its results
+      // (the accumulators of phase A have been read, and Q is still there).
+      int started = 0;
+      if (through && cx.warp == 1 && cx.lane == 0) {
+        tc_fence_after();
+        for (; started < 2 && started < pl.T2; ++started) {
+          if (!mbar_wait(&bars->kv_full[started], 0, abort_flag, a.dev_status, kDevTimeout, a.wait_limit)) break;
+          mma_tile_kk(cx.tmem + (uint32_t)started * 256u, cx.smem_base + k_slot_off(2 * started), cx.smem_base + kOffQ, false);
+        }
       }
-    }
-    through = through && group_barrier(counter, (++epoch) * (unsigned int)a.cpg, abort_flag, go, a.dev_status, a.wait_limit);
-    if (!through) {
-      // a barrier gave up: the stages requested above must have landed, and the products been formed, before this CTA may return
-      if (threadIdx.x == 0)
-        for (int it = 0; it < pre; ++it) wait_issued(&bars->kv_full[it], 0);
-      if (started > 0) {
-        umma_commit(&bars->drain);
-        wait_issued(&bars->drain, 0);
+      through = through && group_barrier(counter, (++epoch) * (unsigned int)a.cpg, abort_flag, go, a.dev_status, a.wait_limit);
+      if (!through) {
+        drain_issued(cx, ld, false);
+        break;
       }
-      break;
+      tc_fence_after();
+      phase_c_control<kW, kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, started, &ld);
+    } else {
+      phase_c_control<kW, kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, 0, &ld);
     }
-    tc_fence_after();
-    phase_c_control<kW, kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, pre, started);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (*(volatile int*)abort_flag) {   // nobody waits any more: the same for every thread
+      drain_issued(cx, ld, pl.T2 > 0);
+      break;
+    }
   }
 }
 
@@ -1431,25 +1425,21 @@ __device__ void worker_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, c
                             const CUtensorMap* tmAug, int* go, float (*red)[4][kTile]) {
   for (int bh = pl.group; bh < a.BH; bh += a.groups) {
     if (bh != pl.group) __syncthreads();
-    if (kLse) {
-      phase_c_worker<kW, kLse, kInd>(cx, a, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, 0, red);
-      tc_fence_before();
-      __syncthreads();
+    if (!kLse) {
+      phase_a_worker(cx, a, bh, pl.tile0, pl.T1);
+      if (!group_barrier_follow(go)) break;
+      combine_rows<kInd == 3>(cx, a, bh, pl.group, pl.rank);
+      fence_proxy_async_smem();   // the exchange buffers are overwritten by TMA loads in phase C
+      named_barrier_sync(2, kFWorkerWarps * 32);   // (the strips' weights lie where the heavy units are noted)
+      if (threadIdx.x == kFFirstWorker * 32) cx.heavy[0] = 0;
+      if (!group_barrier_follow(go)) break;
       tc_fence_after();
-      continue;
     }
-    phase_a_worker(cx, a, bh, pl.tile0, pl.T1);
-    if (!group_barrier_follow(go)) break;
-    combine_rows<kInd == 3>(cx, a, bh, pl.group, pl.rank);
-    fence_proxy_async_smem();   // the exchange buffers are overwritten by TMA loads in phase C
-    named_barrier_sync(2, kFWorkerWarps * 32);   // (the strips' weights lie where the heavy units are noted)
-    if (threadIdx.x == kFFirstWorker * 32) cx.heavy[0] = 0;
-    if (!group_barrier_follow(go)) break;
-    tc_fence_after();
     phase_c_worker<kW, kLse, kInd>(cx, a, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, 0, red);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (*(volatile int*)cx.abort_flag) break;
   }
 }
 

@@ -92,9 +92,10 @@ vmv_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUte
   grid_dependency_wait();
   grid_dependency_launch();
 
+  int heads_seen = 0, issued = 0;   // factor tiles of heads and tiles of V that the loading thread has requested
   if (warp == 0) {
     if (lane == 0) {
-      int prev_bh = -1, heads_seen = 0, issued = 0;
+      int prev_bh = -1;
       bool ok = true;
       for (int it = 0; it < cnt && ok; ++it) {
         const long long idx = first + it;
@@ -128,15 +129,10 @@ vmv_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUte
         tma_load_4d(dv + kBoxBytes, &tmV, &B->v_full[s], 64, tile * kTile, bh % a.Hkv, bh / a.Hkv);
         issued = it + 1;
       }
-      if (*(volatile int*)&abort_flag) {
-        // the tiles requested last may still be on their way into shared memory
-        if (heads_seen > 0) wait_issued(&B->lt_full, (uint32_t)(heads_seen - 1));
-        for (int i = max(0, issued - kVRing); i < issued; ++i) wait_issued(&B->v_full[i % kVRing], (uint32_t)(i / kVRing));
-      }
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      int prev_bh = -1, heads_seen = 0;
+      int prev_bh = -1;
       bool ok = true;
       for (int it = 0; it < cnt && ok; ++it) {
         const long long idx = first + it;
@@ -168,10 +164,6 @@ vmv_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUte
         }
         if (ok) umma_commit(&B->v_empty[s]);   // the tile's slot is free once its last product has read it
       }
-      if (*(volatile int*)&abort_flag) {   // let the products already issued finish before the CTA returns
-        umma_commit(&B->drain);
-        wait_issued(&B->drain, 0);
-      }
     }
   } else {
     const int quad = warp & 3;   // the tensor-memory lane quarter this warp may touch
@@ -179,43 +171,54 @@ vmv_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUte
     const int t = quad * 32 + lane;
     const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
     bool ok = true;
-    for (int it = 0; it < cnt && ok; ++it) {
+    // (a warp whose wait has run out runs on without waiting: each lane has given up for itself, and the loads take the warp together)
+    for (int it = 0; it < cnt; ++it) {
       const long long idx = first + it;
       const int bh = (int)(idx / a.tiles), tile = (int)(idx % a.tiles);
       const int j = tile * kTile + t;
-      for (int g = g_first; g < a.G && ok; g += 4) {
-        ok = mbar_wait(&B->acc_full[g >> 1], (uint32_t)it & 1u, &abort_flag, dev_status, kDevTimeout, a.wait_limit);
+      for (int g = g_first; g < a.G; g += 4) {
+        ok = ok && mbar_wait(&B->acc_full[g >> 1], (uint32_t)it & 1u, &abort_flag, dev_status, kDevTimeout, a.wait_limit);
         float sum = 0.f;
-        if (ok) {
-          tc_fence_after();
-          const uint32_t tY = tmem + lane_base + (uint32_t)g * 128u;
+        tc_fence_after();
+        const uint32_t tY = tmem + lane_base + (uint32_t)g * 128u;
 #pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            float y0[32], y1[32];
-            tmem_ld32(tY + (uint32_t)c * 64u, y0);
-            tmem_ld32(tY + (uint32_t)c * 64u + 32u, y1);
-            tmem_wait_ld();
-            float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+        for (int c = 0; c < 2; ++c) {
+          float y0[32], y1[32];
+          tmem_ld32(tY + (uint32_t)c * 64u, y0);
+          tmem_ld32(tY + (uint32_t)c * 64u + 32u, y1);
+          tmem_wait_ld();
+          float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
 #pragma unroll
-            for (int u = 0; u < 32; u += 2) {
-              s0 = fmaf(y0[u], y0[u], s0); s1 = fmaf(y0[u + 1], y0[u + 1], s1);
-              s2 = fmaf(y1[u], y1[u], s2); s3 = fmaf(y1[u + 1], y1[u + 1], s3);
-            }
-            sum += (s0 + s1) + (s2 + s3);
+          for (int u = 0; u < 32; u += 2) {
+            s0 = fmaf(y0[u], y0[u], s0); s1 = fmaf(y0[u + 1], y0[u + 1], s1);
+            s2 = fmaf(y1[u], y1[u], s2); s3 = fmaf(y1[u + 1], y1[u + 1], s3);
           }
-          tc_fence_before();
+          sum += (s0 + s1) + (s2 + s3);
         }
+        tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&B->acc_empty[g >> 1]);
-        if (ok && j < a.n_kv) a.out[((long long)bh * a.G + g) * a.n_kv + j] = sum;
+        if (j < a.n_kv) a.out[((long long)bh * a.G + g) * a.n_kv + j] = sum;
       }
     }
   }
 
   tc_fence_before();
   __syncthreads();
+  tc_fence_after();
+  if (*(volatile int*)&abort_flag) {
+    // a wait has run out: what is under way lands before the CTA gives its memory back (all threads have met behind their
+    // last wait, so that the flag is the same for all)
+    if (threadIdx.x == 0) {
+      if (heads_seen > 0) wait_issued(&B->lt_full, (uint32_t)(heads_seen - 1));
+      for (int i = max(0, issued - kVRing); i < issued; ++i) wait_issued(&B->v_full[i % kVRing], (uint32_t)(i / kVRing));
+    } else if (warp == 1 && lane == 0) {
+      umma_commit(&B->drain);
+      wait_issued(&B->drain, 0);
+    }
+    __syncthreads();
+  }
   if (warp == 1) {
-    tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
 }

@@ -1710,6 +1710,51 @@ def test_wait_limit_runs_out_and_the_handle_recovers(handle):
     full_check(handle, inp)
 
 
+@pytest.mark.parametrize("form", ["from_lse", "projected", "projected_from_lse", "adaptive"])
+def test_waits_that_run_out_end_alike_for_a_whole_warp(handle, form):
+    """The other forms of the score kernel under a wait limit of one SM clock: whichever waits run out, and for whichever of a warp's
+    lanes first, each call returns by itself, with the timeout status or with all its results, and the handle then gives the oracle's."""
+    import torch
+    case = Case("timeout2", 1, 16, 4, 128, 9000, 32, 100, 5, 0, 0.9, "bf16", 0, "normal", 124)
+    inp = make_inputs(case)
+    given, projected = "lse" in form, "projected" in form
+    run = DeviceRun(handle, inp, adaptive_budget=case.budget if form == "adaptive" else 0)
+    pool = rk.adaptive_pool(1e9, 5, case.budget) if form == "adaptive" else run.pool()
+    W = None
+    if projected:
+        W, factor = _make_projection(handle, case, 40, seed=3)
+    ref = oracle_scores(inp, W_O=W, want_O=True)
+    if given:
+        _, O, lse = _window_stats(inp, with_A_check=False)
+        O, lse = torch.from_numpy(O).cuda(), torch.from_numpy(lse).cuda()
+
+    def call():
+        args = (run.shape, run.Q, run.K, run.V) + ((O, lse) if given else ())
+        (handle.evict_from_lse if given else handle.evict)(*args, case.ema_decay, pool, run.budget, run.indices, run.K_out, run.V_out,
+                                                           run.ws, scores_out=run.scores)
+        torch.cuda.synchronize()
+        return handle.poll_status()
+
+    handle.set_kernel_path(rk.PATH_TENSOR_CORE)
+    if projected:
+        handle.set_output_projection(factor, case.n_q_heads, case.head_dim)
+    try:
+        handle.set_wait_limit(1)
+        for _ in range(20):
+            status = call()
+            assert status in (rk.RESTKV_OK, rk.ERR_TIMEOUT)
+            if status == rk.RESTKV_OK:
+                assert_scores_close(run.scores.cpu().numpy(), ref.scores, TOL["bf16"])
+        handle.set_wait_limit(2_000_000_000)
+        assert call() == rk.RESTKV_OK
+        assert_scores_close(run.scores.cpu().numpy(), ref.scores, TOL["bf16"])
+        assert_selection_valid(run.indices.cpu().numpy(), ref.scores, case.budget, TOL["bf16"])
+    finally:
+        handle.set_wait_limit(2_000_000_000)
+        handle.set_kernel_path(rk.PATH_AUTO)
+        handle.set_output_projection(None)
+
+
 def test_overlapping_calls_count_their_blocks_apart(handle):
     """Two evictions on two streams without ordering, each with its own workspace: against the rules, but each launch counts its
     blocks in a set of its own, so that the outcome is right results or the timeout status, never a barrier opened by the other
