@@ -358,6 +358,31 @@ def test_more_heads_than_sms(handle):
     assert_compaction_exact(idx, vbits, V_out)
 
 
+@pytest.mark.parametrize("tail", [0, 32])
+def test_more_heads_than_sms_from_given_window_statistics(handle, tail):
+    """160 heads with their statistics given: a CTA forms the row operands of a second head after those of the first."""
+    import torch
+    case = Case("many_heads_lse", 20, 32, 8, 128, 300, 32, 60, 5, 0, 0.8, "bf16", tail, "normal", 34)
+    inp = make_inputs(case)
+    ref, O, lse = _window_stats(inp, with_A_check=False)
+    run = DeviceRun(handle, inp)
+    dO, dL = torch.from_numpy(O).cuda(), torch.from_numpy(lse).cuda()
+    handle.evict_from_lse(run.shape, run.Q, run.K, run.V, dO, dL, case.ema_decay, run.pool(), run.budget, run.indices, run.K_out,
+                          run.V_out, run.ws, scores_out=run.scores)
+    torch.cuda.synchronize()
+    assert handle.poll_status() == rk.RESTKV_OK
+    idx = run.indices.cpu().numpy()
+    assert_scores_close(run.scores.cpu().numpy(), ref.scores, TOL["bf16"])
+    assert_selection_valid(idx, ref.scores, case.budget, TOL["bf16"])
+    _, kbits, vbits = inp.device_arrays()
+    assert_compaction_exact(idx, kbits, run._bits(run.K_out))
+    assert_compaction_exact(idx, vbits, run._bits(run.V_out))
+    run.scores.zero_()
+    handle.score_from_lse(run.shape, run.Q, run.K, run.V, dO, dL, case.ema_decay, run.pool(), run.scores, run.ws)
+    torch.cuda.synchronize()
+    assert_scores_close(run.scores.cpu().numpy(), ref.scores, TOL["bf16"])
+
+
 @pytest.mark.parametrize("decay", [0.0, 1.0])
 def test_ema_extremes(handle, decay):
     case = Case("ema", 1, 8, 2, 128, 600, 16, 50, 1, 0, decay, "bf16", 0, "normal", 5)
@@ -458,13 +483,17 @@ def test_selection_kernel_edges(handle, spec):
     full_check(handle, inp)
 
 
-@pytest.mark.parametrize("spec", [(3, 2), (7, 3), (1023, 40), (4099, 4098), (25001, 900), (26000, 900), (51300, 2000)])
+@pytest.mark.parametrize("spec", [(3, 2), (7, 3), (1023, 40), (4099, 4098), (25001, 900), (26000, 900), (51300, 2000),
+                                  (1023, 40, 30), (11772, 900), (11773, 900, 25), (23548, 900, 25), (23549, 900), (25001, 900, 13),
+                                  (51300, 2000, 7)])
 def test_adaptive_window_row_lengths(handle, spec):
-    """The index sums behind the adaptive window: rows that begin anywhere within 16 bytes, of a few keys, with two, one and
-    no buffers in shared memory."""
-    n, budget = spec
+    """The index sums behind the adaptive window: rows that begin anywhere within 16 bytes, of a few keys, with two buffers and
+    one in small blocks (to 11772 and 23548 keys), two, one and none in large ones (to 25596 and 51196 keys and beyond), and more
+    rows than there are blocks, so that a block's buffers are filled again."""
+    n, budget = spec[:2]
+    batch = spec[2] if len(spec) > 2 else 1
     for seed in range(n, n + 20):   # (of a few keys, front and rear may keep the same ones)
-        inp = make_inputs(Case("adapt", 1, 4, 2, 16, n, 6, budget, 1, 0, 0.5, "f32", 0, "normal", seed))
+        inp = make_inputs(Case("adapt", batch, 4, 2, 16, n, 6, budget, 1, 0, 0.5, "f32", 0, "normal", seed))
         probe = oracle_scores(inp, pool_mode=1, beta=1e9, base_width=1, budget=budget)
         delta = np.abs(probe.D[..., 0] - probe.D[..., 1])
         if delta.max() > 0:
@@ -481,15 +510,19 @@ def test_adaptive_window_row_lengths(handle, spec):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
-@pytest.mark.parametrize("spec", [(3, 2), (7, 3), (1023, 40), (2049, 1500), (4099, 4098), (25001, 900), (26000, 14000), (51300, 2000)])
+@pytest.mark.parametrize("spec", [(3, 2), (7, 3), (1023, 40), (2049, 1500), (4099, 4098), (25001, 900), (26000, 14000), (51300, 2000),
+                                  (11773, 1500, 3), (20011, 11000, 26)])
 def test_adaptive_window_with_exact_ties(handle, spec, dtype):
     """Rows of two values only (attention weights over two distinct keys): of equal ones the first count, so that the index sums are
     known exactly.  The front queries lean on the second part of the cache, the rear ones on the first; the scaling is set so that
     a mean index that is off by 1e-5 of the difference, to either side, gives another window."""
     import torch
-    n, budget = spec
+    n, budget = spec[:2]
+    batch = spec[2] if len(spec) > 2 else 1
+    if dtype == "bf16":   # (256 rows a sequence there, 24 here)
+        batch = min(batch, 3)
     d, w, Hq, Hkv = (16, 6, 4, 2) if dtype == "f32" else (128, 32, 8, 2)
-    inp = make_inputs(Case("ties", 1, Hq, Hkv, d, n, w, budget, 1, 0, 0.5, dtype, 0, "normal", n))
+    inp = make_inputs(Case("ties", batch, Hq, Hkv, d, n, w, budget, 1, 0, 0.5, dtype, 0, "normal", n))
     a = n // 2
     inp.K[...] = 0.0
     inp.K[:, :, :a, 0] = 2.0
@@ -506,7 +539,7 @@ def test_adaptive_window_with_exact_ties(handle, spec, dtype):
         for steps in (20 + 1e-4, 21 - 1e-4):
             run.score(pool=rk.adaptive_pool(float(diff / steps), 1, budget))
             assert handle.poll_status() == rk.RESTKV_OK
-            np.testing.assert_array_equal(run.pool_used.cpu().numpy()[0], [[41, 20]] * Hkv)
+            np.testing.assert_array_equal(run.pool_used.cpu().numpy(), [[[41, 20]] * Hkv] * batch)
     finally:
         handle.set_variant()
 
@@ -1375,6 +1408,14 @@ def test_projection_at_other_window_lengths(handle, spec):
     projection_check(handle, make_inputs(case), 160, path=rk.PATH_TENSOR_CORE if w >= 32 else rk.PATH_AUTO)
 
 
+@pytest.mark.parametrize("spec", [(4, 32, 8, 32, 200, 24), (5, 8, 8, 128, 150, 24), (8, 32, 8, 32, 140, 24)])
+def test_projection_with_many_heads(handle, spec):
+    """Few CTAs share a head (four, three and two), so that each merges 32 or 64 of its rows, eight at a time."""
+    batch, Hq, Hkv, w, n, d_model = spec
+    case = Case("proj_many", batch, Hq, Hkv, 128, n, w, 40, 5, 0, 0.9, "bf16", 0, "normal", 57)
+    projection_check(handle, make_inputs(case), d_model, path=rk.PATH_TENSOR_CORE)
+
+
 def test_projection_with_a_variant(handle):
     inp = make_inputs(CONFIGS["cfg2"])
     projection_check(handle, inp, 48, path=rk.PATH_TENSOR_CORE, variant=(REC, INV, rk.SPATIAL_MAX, rk.GROUP_MAX))
@@ -1830,6 +1871,9 @@ def test_many_calls_of_several_handles_end_in_time():
     for run in runs:
         assert run.h.poll_status() == rk.RESTKV_OK
         np.testing.assert_array_equal(run.scores.cpu().numpy(), want[0])
+        np.testing.assert_array_equal(run.indices.cpu().numpy(), want[1])
+        np.testing.assert_array_equal(run._bits(run.K_out), want[2])
+        np.testing.assert_array_equal(run._bits(run.V_out), want[3])
         run.h.close()
 
 
