@@ -350,7 +350,6 @@ __device__ void phase_a_worker(const Ctx& cx, const FusedArgs& a, int bh, int ti
   FusedBars* B = cx.B;
   int* abort_flag = cx.abort_flag;
   unsigned int* dev_status = a.dev_status;
-  const int b = bh / a.Hkv, h = bh % a.Hkv;
   const int warp = cx.warp, lane = cx.lane;
   const uint32_t tmem = cx.tmem;
 
@@ -718,18 +717,16 @@ __device__ void combine_rows(const Ctx& cx, const FusedArgs& a, int bh, int grou
 // [32c, 32c + 32)).  Q is still in shared memory from phase A.  The per-query-row constants ride through the
 // tensor core (one extra K = 16 step against a block of ones), so with u = exp2(-scale*log2e * S') = 1/A and
 // x = C' + ||v||^2 = ||o - v||^2 the indicator is x * rsqrt(x * (u - 1)^2).
-template <int kW, bool kLse>
+template <bool kLse>
 __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtensorMap* tmQ, const CUtensorMap* tmO,
                                 const CUtensorMap* tmAug, const CUtensorMap* tmK, const CUtensorMap* tmV, int bh,
                                 int tile0, int T, int started, Loads* ld) {
-  constexpr int kG = kRows / kW;
   FusedBars* B = cx.B;
   int* abort_flag = cx.abort_flag;
   unsigned int* dev_status = a.dev_status;
   const int b = bh / a.Hkv, h = bh % a.Hkv;
   const int warp = cx.warp, lane = cx.lane;
   const uint32_t tmem = cx.tmem;   // buffer s: S' at s*256, C' at s*256 + 128
-  const int n = a.n;
 
   if (warp == 0) {
     if (lane == 0 && T > 0) {
@@ -1096,15 +1093,12 @@ __device__ void stage_given_rows(const Ctx& cx, const FusedArgs& a, int bh) {
 // kInd: 0 = Eq. 7; 1 = the attention weight alone; 2 = attention weight times ||v|| (Appendix G.1); 3 = Eq. 7 with
 // the output projection of Eq. 4 inside its norm.
 template <int kW, bool kLse, int kInd>
-__device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, const CUtensorMap* tmO, const CUtensorMap* tmAug,
-                        const CUtensorMap* tmK, const CUtensorMap* tmV, int bh, int tile0, int T, int pre,
-                        float (*red)[4][kTile]) {
+__device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, int bh, int tile0, int T, float (*red)[4][kTile]) {
   constexpr int kG = kRows / kW;
   constexpr bool kEq7 = kInd == 0 || kInd == 3, kProj = kInd == 3;
   FusedBars* B = cx.B;
   int* abort_flag = cx.abort_flag;
   unsigned int* dev_status = a.dev_status;
-  const int b = bh / a.Hkv, h = bh % a.Hkv;
   const int warp = cx.warp, lane = cx.lane;
   const uint32_t tmem = cx.tmem;   // buffer s: S' at s*256, C' at s*256 + 128
   const int n = a.n;
@@ -1373,7 +1367,7 @@ __device__ void drain_issued(const Ctx& cx, const Loads& ld, bool consts) {
 // barrier, phase C, and a closing __syncthreads.
 
 // Warps 0-3: TMA producer, MMA issuer, the two ||v||^2 warps; thread 0 also runs the group barriers.
-template <int kW, bool kLse>
+template <bool kLse>
 __device__ void control_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, const CUtensorMap* tmQ,
                              const CUtensorMap* tmK, const CUtensorMap* tmV, const CUtensorMap* tmO,
                              const CUtensorMap* tmAug, FusedBars* bars, int* abort_flag, int* go) {
@@ -1404,9 +1398,9 @@ __device__ void control_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, 
         break;
       }
       tc_fence_after();
-      phase_c_control<kW, kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, started, &ld);
+      phase_c_control<kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, started, &ld);
     } else {
-      phase_c_control<kW, kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, 0, &ld);
+      phase_c_control<kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, 0, &ld);
     }
     tc_fence_before();
     __syncthreads();
@@ -1420,9 +1414,7 @@ __device__ void control_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, 
 
 // Warps 4-19: softmax in phase A, the merge of the partials in phase B, the indicator epilogue in phase C.
 template <int kW, bool kLse, int kInd>
-__device__ void worker_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, const CUtensorMap* tmQ,
-                            const CUtensorMap* tmK, const CUtensorMap* tmV, const CUtensorMap* tmO,
-                            const CUtensorMap* tmAug, int* go, float (*red)[4][kTile]) {
+__device__ void worker_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, int* go, float (*red)[4][kTile]) {
   for (int bh = pl.group; bh < a.BH; bh += a.groups) {
     if (bh != pl.group) __syncthreads();
     if (!kLse) {
@@ -1435,7 +1427,7 @@ __device__ void worker_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, c
       if (!group_barrier_follow(go)) break;
       tc_fence_after();
     }
-    phase_c_worker<kW, kLse, kInd>(cx, a, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, 0, red);
+    phase_c_worker<kW, kLse, kInd>(cx, a, bh, pl.tile0, pl.T2, red);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1519,10 +1511,10 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   // compiled for more registers than the launch gives every thread.
   if (cx.warp < kFFirstWorker) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFRegsControl));
-    control_main<kW, kLse>(cx, a, pl, &tmQ, &tmK, &tmV, &tmO, &tmAug, &bars, &abort_flag, &go_flag);
+    control_main<kLse>(cx, a, pl, &tmQ, &tmK, &tmV, &tmO, &tmAug, &bars, &abort_flag, &go_flag);
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kFRegsWorker));
-    worker_main<kW, kLse, kInd>(cx, a, pl, &tmQ, &tmK, &tmV, &tmO, &tmAug, &go_flag, red);
+    worker_main<kW, kLse, kInd>(cx, a, pl, &go_flag, red);
   }
 
   tc_fence_before();
