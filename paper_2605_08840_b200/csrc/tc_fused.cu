@@ -58,6 +58,8 @@ struct FusedArgs {
   float* vnorm;                      // [BH, n_kv]
   float* tile_max;                   // [BH, tiles, 128] largest scaled logit (log2 units) of each query row in each tile
   float* row_M2;                     // [BH, 128] m*log2e + log2 l of each query row (written by the merge)
+  int raw_fits, raw_streams;         // the indicators of a call that writes them leave room in L2 for K and V, or do not (both 0
+                                     //  without them)
   const float* lse;                  // from_lse without a projection: the rows' given log-sum-exp (natural), else null
   float* I_hat;                      // [BH, n]
   float* I_raw;                      // [BH, 128, n] or null: the per-query indicators, for the adaptive window of
@@ -186,7 +188,13 @@ __device__ __forceinline__ uint32_t v_slot_off(int i) { return i < 2 ? kOffRing 
 // K and V leave L2 first: they stream through it, while what else the call touches again is small: the partials, the scores, the
 // tensor maps - and the code, whose first run after each synchronisation would otherwise be fetched from HBM, 4 k cycles for
 // each of the merge, its sums and the first tile of phase C.  16384 rows 71 -> 62 us, 32768 projected 137 -> 131 us; phase C's
-// loads alone 66 and 136 us, phase A's alone nothing.
+// loads alone 66 and 136 us, phase A's alone nothing.  (A little of it is that part of the K and V of an earlier call survives a
+// stream that leaves first: 16384 rows, 67 MB, over two, four and sixteen sets of inputs in turn 64.9 -> 58.1, 65.2 -> 59.0,
+// 64.8 -> 59.4 us.)  With reuse_l2 it makes no difference to speak of whether phase A's loads leave first or not: 8 heads of 131072
+// rows 397 and 399 us, 64 of 32768 687 and 689.
+// Where phase C writes the per-query indicators and these are more than half of L2, its K and V go through at normal priority: "evict
+// first" would only make room for indicators that the next kernel finds gone anyway (131072 rows, 537 MB of them, 584 -> 568 us,
+// 40000 rows 205 -> 202; 20011 rows, 82 MB, 130.2 -> 129.6; 8192 rows, 34 MB, 80 -> 83.5, hence the line).
 // One K tile and one V tile of phase C into stage s (ring slots 2s and 2s + 1).
 __device__ __forceinline__ void load_stage_c(const Ctx& cx, const CUtensorMap* tmK, const CUtensorMap* tmV, int b, int h,
                                              int j0, int s, uint64_t policy) {
@@ -229,9 +237,8 @@ __device__ void phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtenso
       for (int it = 0; it < T; ++it) {
         const int ks = it & 1, vs = it % kFVSlots;
         const int j0 = (tile0 + it) * kTile;
-        // The share's last tiles, which phase C reads first, stay (five per CTA are 47 MB).  All of them do where the per-query
-        // indicators are written, as many bytes again: those would push them out at once.
-        const uint64_t policy = a.I_raw || it + kFStay >= T ? policy_evict_normal() : policy_evict_first();
+        // The share's last tiles, which phase C reads first, stay (five per CTA are 47 MB); all of them do beside a few indicators.
+        const uint64_t policy = a.raw_fits || it + kFStay >= T ? policy_evict_normal() : policy_evict_first();
         if (it >= 2 && !mbar_wait(&B->k_empty[ks], ((it >> 1) - 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit)) break;
         uint8_t* dK = cx.gen_base + k_slot_off(ks);
         mbar_arrive_expect_tx(&B->k_full[ks], kTileBytes);
@@ -256,7 +263,7 @@ __device__ void phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtenso
           if (uses > 0) free = mbar_wait(bar, (uint32_t)(uses - 1) & 1u, abort_flag, dev_status, kDevTimeout, a.wait_limit);
         }
         if (!free) break;
-        load_stage_c(cx, tmK, tmV, b, h, (tile0 + T2 - 1 - s) * kTile, s, policy_evict_first());
+        load_stage_c(cx, tmK, tmV, b, h, (tile0 + T2 - 1 - s) * kTile, s, a.raw_streams ? policy_evict_normal() : policy_evict_first());
         ++ld->c;
       }
     }
@@ -552,6 +559,8 @@ __device__ void combine_rows(const Ctx& cx, const FusedArgs& a, int bh, int grou
   const int items = rb * (kHeadDim / 4), per_pass = min(items, kThreads), splits = kThreads / per_pass, split = wt / per_pass;
   const long long slot0 = (long long)group * cpg;
   float4 v[kBatch];
+  // (Past the last partial it is that one again, not used.  Loads left out by a predicate cost the whole kernel its order of
+  // instructions: 8 x 32768 rows, where two CTAs share a head and seven of nine are not needed, 499 -> 531 us.)
   auto request = [&](int item, int p0) {
     const float* src = a.part_O + slot0 * kRows * kHeadDim + ((item >> lrb) * kRows + r0 + (item & (rb - 1))) * 4;
 #pragma unroll
@@ -742,7 +751,7 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
         tma_load_3d(cx.gen_base + kOffO + kBoxBytes, tmO, &B->const_full, 64, 0, bh);
         tma_load_3d(cx.gen_base + kOffAug, tmAug, &B->const_full, 0, 0, bh);
       }
-      const uint64_t policy = policy_evict_first();
+      const uint64_t policy = a.raw_streams ? policy_evict_normal() : policy_evict_first();
       for (int it = ld->c; it < T; ++it) {   // the first tiles were requested before the group barriers
         const int s = it & 1;
         if (it >= 2 && !mbar_wait(&B->kv_empty[s], ((it >> 1) - 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit)) break;
@@ -1756,6 +1765,10 @@ cudaError_t launch_tc_fused(void* state, const Problem& p, const Workspace& ws, 
   a.I_raw = O_given ? nullptr : I_raw;
   if (O_given) a.O_f32 = const_cast<float*>(O_given);   // read only in this mode
   a.lse = O_given && !a.proj_Mt ? LSE_given : nullptr;
+  if (a.I_raw) {
+    a.raw_streams = (long long)p.BH * kRows * p.n * 4 > (64ll << 20) ? 1 : 0;
+    a.raw_fits = !a.raw_streams;
+  }
   const dim3 grid(a.groups * a.cpg);
   FusedKernel kernel = attention_only ? pick_fused(32, false, 0) : pick_fused(p.w, a.from_lse != 0, a.proj_Mt ? 3 : p.indicator);
   if (!kernel) return cudaErrorInvalidValue;
