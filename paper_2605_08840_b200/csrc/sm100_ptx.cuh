@@ -16,6 +16,16 @@ __device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddep
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// One thread of a converged warp, the same one each time.  What issues tcgen05.mma stands behind this and not behind lane == 0: the
+// compiler then knows that a single thread runs and keeps descriptors and addresses in uniform registers.  The eight K = 16 steps
+// of a 128 x 128 x 128 product take the issuing thread 137 cycles so, 420 to 490 behind lane == 0 (operands in tensor memory: 55
+// and 400); the tensor pipe needs 512.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 // ---- mbarrier --------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");

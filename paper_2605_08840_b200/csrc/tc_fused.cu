@@ -230,7 +230,7 @@ __device__ void phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtenso
   const uint32_t tmem = cx.tmem;
 
   if (warp == 0) {
-    if (lane == 0 && T > 0) {
+    if (T > 0 && elect_one()) {
       mbar_arrive_expect_tx(&B->q_full, kTileBytes);
       tma_load_3d(cx.gen_base + kOffQ, tmQ, &B->q_full, 0, 0, bh);
       tma_load_3d(cx.gen_base + kOffQ + kBoxBytes, tmQ, &B->q_full, 64, 0, bh);
@@ -269,7 +269,7 @@ __device__ void phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtenso
     }
   } else if (warp == 1) {
     // S(it), then O += P V of tile it - 1
-    if (lane == 0 && T > 0) {
+    if (T > 0 && elect_one()) {
       bool ok = mbar_wait(&B->q_full, 0, abort_flag, dev_status, kDevTimeout, a.wait_limit);
       for (int it = 0; ok && it <= T; ++it) {
         if (it < T) {
@@ -738,7 +738,7 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
   const uint32_t tmem = cx.tmem;   // buffer s: S' at s*256, C' at s*256 + 128
 
   if (warp == 0) {
-    if (lane == 0 && T > 0) {
+    if (T > 0 && elect_one()) {
       fence_proxy_async_all();   // O' and the constant strip were written with ordinary stores by other CTAs
       const bool own_rows = kLse && a.lse;   // O' and the strip are formed by the worker warps
       mbar_arrive_expect_tx(&B->const_full, (own_rows ? 0u : kTileBytes + kAugBytes) + (kLse ? kTileBytes : 0u));
@@ -760,7 +760,7 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && T > 0) {
+    if (T > 0 && elect_one()) {
       bool ok = mbar_wait(&B->const_full, 0, abort_flag, dev_status, kDevTimeout, a.wait_limit);
       const uint32_t sQ = cx.smem_base + kOffQ, sO = cx.smem_base + kOffO, sAug = cx.smem_base + kOffAug;
       const uint64_t ones_desc = make_smem_desc(cx.smem_base + kOffOnes, 16, 0);   // every 8-row group reads the same block
@@ -1359,13 +1359,13 @@ struct Plan {
 // constants and Q are waited for where the phase asked for them: a barrier without a request behind it has its first phase open.
 __device__ void drain_issued(const Ctx& cx, const Loads& ld, bool consts) {
   FusedBars* B = cx.B;
-  if (threadIdx.x == 0) {
+  if (cx.warp == 0 && elect_one()) {
     if (ld.k > 0) wait_issued(&B->q_full, 0);
     for (int i = max(0, ld.k - 2); i < ld.k; ++i) wait_issued(&B->k_full[i & 1], (uint32_t)(i >> 1));
     for (int i = max(0, ld.v - kFVSlots); i < ld.v; ++i) wait_issued(&B->v_full[i % kFVSlots], (uint32_t)(i / kFVSlots));
     if (consts) wait_issued(&B->const_full, 0);
     for (int i = max(0, ld.c - 2); i < ld.c; ++i) wait_issued(&B->kv_full[i & 1], (uint32_t)(i >> 1));
-  } else if (cx.warp == 1 && cx.lane == 0) {
+  } else if (cx.warp == 1 && elect_one()) {
     umma_commit(&B->drain);
     wait_issued(&B->drain, 0);
   }
@@ -1394,7 +1394,7 @@ __device__ void control_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, 
       // Phase B belongs to the worker warps.  Meanwhile S^T = K Q^T of the first two tiles of phase C, which do not need its results
       // (the accumulators of phase A have been read, and Q is still there).
       int started = 0;
-      if (through && cx.warp == 1 && cx.lane == 0) {
+      if (through && cx.warp == 1 && elect_one()) {
         tc_fence_after();
         for (; started < 2 && started < pl.T2; ++started) {
           if (!mbar_wait(&bars->kv_full[started], 0, abort_flag, a.dev_status, kDevTimeout, a.wait_limit)) break;

@@ -94,7 +94,7 @@ vmv_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUte
 
   int heads_seen = 0, issued = 0;   // factor tiles of heads and tiles of V that the loading thread has requested
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       int prev_bh = -1;
       bool ok = true;
       for (int it = 0; it < cnt && ok; ++it) {
@@ -131,7 +131,7 @@ vmv_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUte
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       int prev_bh = -1;
       bool ok = true;
       for (int it = 0; it < cnt && ok; ++it) {
@@ -209,10 +209,10 @@ vmv_kernel(const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUte
   if (*(volatile int*)&abort_flag) {
     // a wait has run out: what is under way lands before the CTA gives its memory back (all threads have met behind their
     // last wait, so that the flag is the same for all)
-    if (threadIdx.x == 0) {
+    if (warp == 0 && elect_one()) {
       if (heads_seen > 0) wait_issued(&B->lt_full, (uint32_t)(heads_seen - 1));
       for (int i = max(0, issued - kVRing); i < issued; ++i) wait_issued(&B->v_full[i % kVRing], (uint32_t)(i / kVRing));
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && elect_one()) {
       umma_commit(&B->drain);
       wait_issued(&B->drain, 0);
     }
