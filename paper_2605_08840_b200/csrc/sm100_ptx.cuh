@@ -309,6 +309,18 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
   return make_float2(f2_lo(d), f2_hi(d));
 }
 
+// lo^2 and hi^2 of a bf16 pair added to two sums: the squares are exact, the sums fp32.
+__device__ __forceinline__ void square_add(float& sum_lo, float& sum_hi, uint32_t pair) {
+  asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tfma.rn.f32.bf16 %0, l, l, %0;\n\tfma.rn.f32.bf16 %1, h, h, %1;\n\t}"
+      : "+f"(sum_lo), "+f"(sum_hi)
+      : "r"(pair));
+}
+// 16 bytes of shared memory by their shared-window address; the loads stay in program order among themselves.
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   uint32_t r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));

@@ -211,6 +211,31 @@ __device__ __forceinline__ void load_stage_c(const Ctx& cx, const CUtensorMap* t
 // Where a wait of a warp has run out, the loops over the tiles run on without waiting, on whatever lies there: each lane has given up
 // for itself, and what the warp does together must not depend on that.  (The call ends with the timeout status.)
 
+// ||v||^2 of row `row` of a [128 x 128] bf16 tile (two 128-byte-swizzled boxes, in which 16-byte chunk c of row r sits at chunk
+// c ^ (r & 7)).  Every instruction counts twice here: one warp does it for a tile while sixteen others use the issue slots.  One fma
+// per element that takes the bf16 as it is (its square is exact), four sums, and three loads in flight, which is what 32 registers
+// hold: 1.8 k cycles a tile beside busy workers, 2.6 k with two loads and 2.3 k with four in flight, 5.6 k with a shift, a mask and
+// a packed fma per pair, which had become what phase A waited for (and 0.6 k of each tile from given statistics).
+__device__ __forceinline__ float row_square_sum(uint32_t tile, int row) {
+  const uint32_t at = tile + (uint32_t)(row >> 3) * 1024u + (uint32_t)(row & 7) * (128u + 16u);
+  constexpr int kDepth = 3;
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+  uint4 u[kDepth];
+  auto request = [&](int c) { return lds128((at ^ (uint32_t)((c & 7) << 4)) + (uint32_t)(c >> 3) * kBoxBytes); };
+#pragma unroll
+  for (int c = 0; c < kDepth; ++c) u[c] = request(c);
+#pragma unroll
+  for (int c = 0; c < 16; ++c) {
+    const uint4 v = u[c % kDepth];
+    square_add(s[0], s[1], v.x);
+    square_add(s[2], s[3], v.y);
+    square_add(s[0], s[1], v.z);
+    square_add(s[2], s[3], v.w);
+    if (c + kDepth < 16) u[c % kDepth] = request(c + kDepth);
+  }
+  return (s[0] + s[1]) + (s[2] + s[3]);
+}
+
 // ------------------------------------------------------------------------------------------------
 // Phase A: this CTA's share [tile0, tile0 + T) of one head.
 // Control warps: warp 0 loads (K ring of 2 slots, V ring of 3), warp 1 issues the MMAs (S(it), then O += P V of tile
@@ -316,36 +341,14 @@ __device__ void phase_a_control(const Ctx& cx, const FusedArgs& a, const CUtenso
         if (lane == 0) mbar_arrive(&B->v_empty[vs]);
         continue;
       }
-      const uint8_t* vt = cx.gen_base + v_slot_off(vs);
-      float vn[4];
-#pragma unroll
+#pragma unroll 1
       for (int rr = 0; rr < 4; ++rr) {
-        const int row = rr * 32 + lane;
-        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          // 16-byte chunk c of row r of a 128-byte-swizzled box sits at chunk c ^ (r & 7)
-          const uint8_t* rowp = vt + half * kBoxBytes + (row >> 3) * 1024 + (row & 7) * 128;
-#pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            const uint4 u = *reinterpret_cast<const uint4*>(rowp + ((c ^ (row & 7)) << 4));
-            const unsigned int wv[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const float2 e = make_float2(__uint_as_float(wv[q] << 16), __uint_as_float(wv[q] & 0xFFFF0000u));
-              acc = ffma2(e, e, acc);
-            }
-          }
-        }
-        vn[rr] = acc.x + acc.y;
+        const float vn = row_square_sum(cx.smem_base + v_slot_off(vs), rr * 32 + lane);
+        const int j = (tile0 + it) * kTile + rr * 32 + lane;
+        if (j < a.n_kv && !a.attention_only) a.vnorm[(long long)bh * a.n_kv + j] = vn;
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&B->v_empty[vs]);
-#pragma unroll
-      for (int rr = 0; rr < 4; ++rr) {
-        const int j = (tile0 + it) * kTile + rr * 32 + lane;
-        if (j < a.n_kv && !a.attention_only) a.vnorm[(long long)bh * a.n_kv + j] = vn[rr];
-      }
     }
   }
 }
@@ -812,27 +815,10 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
     for (int it = 0; it < T; ++it) {
       const int s = it & 1;
       ok = ok && mbar_wait(&B->kv_full[s], (it >> 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit);
-      const uint8_t* vt = cx.gen_base + k_slot_off(2 * s) + kTileBytes;
-#pragma unroll
+#pragma unroll 1
       for (int rr = 0; rr < 2; ++rr) {
         const int row = (warp - 2) * 64 + rr * 32 + lane;
-        f32x2 acc[4] = {f2_make(0.f, 0.f), f2_make(0.f, 0.f), f2_make(0.f, 0.f), f2_make(0.f, 0.f)};
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          const uint8_t* rowp = vt + half * kBoxBytes + (row >> 3) * 1024 + (row & 7) * 128;
-#pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            const uint4 u = *reinterpret_cast<const uint4*>(rowp + ((c ^ (row & 7)) << 4));
-            const unsigned int wv[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const f32x2 e = f2_make(__uint_as_float(wv[q] << 16), __uint_as_float(wv[q] & 0xFFFF0000u));
-              acc[q] = f2_fma(e, e, acc[q]);
-            }
-          }
-        }
-        const f32x2 t2 = f2_add(f2_add(acc[0], acc[1]), f2_add(acc[2], acc[3]));
-        cx.vn_s[(it & 3) * kTile + row] = f2_lo(t2) + f2_hi(t2);
+        cx.vn_s[(it & 3) * kTile + row] = row_square_sum(cx.smem_base + k_slot_off(2 * s) + kTileBytes, row);
       }
       __syncwarp();
       if (lane == 0) {
