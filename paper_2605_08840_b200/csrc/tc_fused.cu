@@ -1151,6 +1151,15 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, int bh, int ti
   };
   float* raw_head = (a.I_raw && !kLse) ? a.I_raw + (long long)bh * kRows * n : nullptr;
   bool ok = true;
+  // The shares of a tile are summed in a fixed order by one warpgroup, another one for each tile, two tiles later: by then all
+  // sixteen warps have stored theirs and nobody waits.  (One tile later the warpgroup that did it waited for the slowest of the
+  // others in every tile, came 0.6 k cycles late to the next and held up its accumulators.)  A slot of `red` is rewritten four tiles
+  // later, which the two accumulator buffers only allow after every warp has moved past this point.
+  auto join_tile = [&](int u) {
+    ok = ok && mbar_wait(&B->red_full[u & 3], (uint32_t)(u >> 2) & 1u, abort_flag, dev_status, kDevTimeout, a.wait_limit);
+    const int ju = (tile0 + T - 1 - u) * kTile + t;
+    if (ok && ju < n) store_score(ju, red[u & 3]);
+  };
   if (kLse && !kProj && T > 0) stage_given_rows(cx, a, bh);
   float vn_next = 0.f;
   // from_lse: no phase A has left ||v||^2 and the tiles' row maxima behind; ||v||^2 comes from the control warps
@@ -1176,15 +1185,7 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, int bh, int ti
       const int jn = (tile0 + T - 2 - it) * kTile + t;
       vn_next = (jn < n) ? vn_head[jn] : 1.f;
     }
-    // The shares of the previous tile are summed in a fixed order by warpgroup 0 once all sixteen warps have
-    // stored theirs.  A slot of `red` is rewritten four tiles later, which the two accumulator buffers only
-    // allow after every warp has moved past this point.
-    if (it > 0 && cgp == 0) {
-      const int rs = (it - 1) & 3;
-      ok = ok && mbar_wait(&B->red_full[rs], (uint32_t)((it - 1) >> 2) & 1u, abort_flag, dev_status, kDevTimeout, a.wait_limit);
-      const int jp = (tile0 + T - it) * kTile + t;
-      if (ok && jp < n) store_score(jp, red[rs]);
-    }
+    if (it >= 2 && cgp == (it & 3)) join_tile(it - 2);
     ok = ok && mbar_wait(&B->acc_full[s], par, abort_flag, dev_status, kDevTimeout, a.wait_limit);
     float tot = 0.f;
     int unit = kMaxHeavy;   // this lane's place in the list of heavy units
@@ -1326,12 +1327,9 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, int bh, int ti
     __syncwarp();
     if (lane == 0) mbar_arrive(&B->red_full[it & 3]);
   }
-  if (T > 0 && cgp == 0) {
-    const int rs = (T - 1) & 3;
-    ok = ok && mbar_wait(&B->red_full[rs], (uint32_t)((T - 1) >> 2) & 1u, abort_flag, dev_status, kDevTimeout, a.wait_limit);
-    const int jl = tile0 * kTile + t;   // the last tile processed is the first of the share
-    if (ok && jl < n) store_score(jl, red[rs]);
-  }
+#pragma unroll 1
+  for (int u = max(T - 2, 0); u < T; ++u)
+    if (cgp == ((u + 2) & 3)) join_tile(u);
   if (kEq7) heavy_pass<kW, kLse, kProj>(cx, a, bh);
 }
 
