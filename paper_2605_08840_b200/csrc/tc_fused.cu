@@ -1200,34 +1200,41 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, int bh, int ti
     const float vlen = kInd == 2 ? sqrtf(vn) : 1.f;          // ||v_j||
     const f32x2 vlen2 = f2_make(vlen, vlen);
     f32x2 h2 = f2_make(0.f, 0.f);
-    float sv0[16], cv0[16], sv1[16], cv1[16];
     const bool look = kEq7 && (from_lse || cx.look[s] != 0);
     float mx = -INFINITY;   // where a weight may exceed kHeavyA: this lane's largest logit
     if (raw_head == nullptr) {
-      tmem_ld16(tS, sv0);
-      if (kEq7) tmem_ld16(tC, cv0);
-      tmem_wait_ld();
-      tmem_ld16(tS + 16, sv1);   // the second half of the columns travels while the first is worked on
-      if (kEq7) tmem_ld16(tC + 16, cv1);
+      // The next columns travel while some are worked on: eight at a time, so that the compiler can mix the instructions of a whole
+      // chunk (with sixteen 131072 rows 226 us, with eight 222; 20011 rows adaptive 122.3 and 120.8), but sixteen from given
+      // statistics, where there is more to do per column and HBM to keep up with (50021 rows 63.6, with eight 64.1).
+      constexpr int kCols = kLse ? 16 : 8, kChunks = 32 / kCols;
+      auto request = [](uint32_t at, float* v) {
+        if constexpr (kCols == 16) tmem_ld16(at, v);
+        else tmem_ld8(at, v);
+      };
+      float sv0[kCols], cv0[kCols], sv1[kCols], cv1[kCols];
+      request(tS, sv0);
+      if (kEq7) request(tC, cv0);
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const float* sv = c == 0 ? sv0 : sv1;
-        const float* cv = c == 0 ? cv0 : cv1;
-        if (c == 1) {
-          tmem_wait_ld();
-          // every tensor-memory read of this tile is done: the MMA warp may refill the accumulators (the logits of a
-          // tile that may hold a large weight are read once more below; the check between the two halves instead
-          // kept their instructions from mixing, 2 % of the whole call)
+      for (int c = 0; c < kChunks; ++c) {
+        const float* sv = (c & 1) ? sv1 : sv0;
+        const float* cv = (c & 1) ? cv1 : cv0;
+        tmem_wait_ld();
+        if (c + 1 < kChunks) {
+          request(tS + (c + 1) * kCols, (c & 1) ? sv0 : sv1);
+          if (kEq7) request(tC + (c + 1) * kCols, (c & 1) ? cv0 : cv1);
+        } else {
+          // Every tensor-memory read of this tile is done: the MMA warp may refill the accumulators (the logits of a tile that may
+          // hold a large weight are read once more below).
           tc_fence_before();
           __syncwarp();
           if (lane == 0 && (from_lse || !look)) mbar_arrive(&B->acc_empty[s]);
         }
         if (from_lse && kEq7) {
 #pragma unroll
-          for (int u = 0; u < 16; ++u) mx = fmaxf(mx, sv[u]);
+          for (int u = 0; u < kCols; u += 2) mx = fmax3(mx, sv[u], sv[u + 1]);
         }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < kCols / 2; ++q) {
           const f32x2 nt = f2_mul(f2_make(sv[2 * q], sv[2 * q + 1]), nc2);
           f32x2 Iq;
           if (kEq7) {
@@ -1245,11 +1252,11 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, int bh, int ti
             Iq = f2_make(ex2_approx(-f2_lo(nt)), ex2_approx(-f2_hi(nt)));                         // A
             if (kInd == 2) Iq = f2_mul(Iq, vlen2);
           }
-          if (q == 0 && (c * 16) % kRun == 0) Iq = f2_mul(Iq, seed2);
-          if (q == 7 && (c * 16 + 16) % kRun == 0) Iq = f2_mul(Iq, last2);
+          if (q == 0 && (c * kCols) % kRun == 0) Iq = f2_mul(Iq, seed2);
+          if (q == kCols / 2 - 1 && (c * kCols + kCols) % kRun == 0) Iq = f2_mul(Iq, last2);
           h2 = f2_fma(h2, d2, Iq);
         }
-        if ((c * 16 + 16) % kRun == 0) {   // end of a run
+        if ((c * kCols + kCols) % kRun == 0) {   // end of a run
           const float run = fmaf(f2_lo(h2), ema_decay, f2_hi(h2));
           tot = group_max ? fmaxf(tot, run) : tot + run;
           h2 = f2_make(0.f, 0.f);
