@@ -86,7 +86,6 @@ struct FusedBars {
   // phase C
   uint64_t const_full, kv_full[2], kv_empty[2], acc_full[2], acc_empty[2], red_full[4];
   uint64_t drain;   // only after a failed wait: completion of the MMAs issued so far
-  uint64_t vn_full[4];   // from_lse: ||v||^2 of a tile is in shared memory (ring of four tiles)
 };
 
 __device__ __forceinline__ void mbar_inval(uint64_t* bar) {
@@ -103,7 +102,7 @@ __device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
 }
 
 // (Re)initialises every mbarrier of the CTA for one phase.  Called by one thread between two __syncthreads.
-__device__ void init_bars(FusedBars* B, bool first, bool from_lse, bool own_rows) {
+__device__ void init_bars(FusedBars* B, bool first, bool own_rows) {
   uint64_t* all = reinterpret_cast<uint64_t*>(B);
   constexpr int kCount = sizeof(FusedBars) / sizeof(uint64_t);
   if (!first)
@@ -116,8 +115,8 @@ __device__ void init_bars(FusedBars* B, bool first, bool from_lse, bool own_rows
     mbar_init(&B->p_full[i], 256);
     mbar_init(&B->pv_done[i], 1);
     mbar_init(&B->kv_full[i], 1);
-    mbar_init(&B->kv_empty[i], from_lse ? 3 : 1);   // MMA commit (+ the two ||v||^2 warps, which read the V tile)
-    mbar_init(&B->acc_full[i], from_lse ? 1 : 2);   // MMA commit (+ the warp that tells which tiles may hold a large weight)
+    mbar_init(&B->kv_empty[i], own_rows ? 3 : 1);   // MMA commit (+ warps 2 and 3, which read the V tile for ||v||^2)
+    mbar_init(&B->acc_full[i], 3);                  // MMA commit + warps 2 and 3
     mbar_init(&B->acc_empty[i], kFWorkerWarps);
   }
   for (int i = 0; i < kFVSlots; ++i) {
@@ -127,7 +126,6 @@ __device__ void init_bars(FusedBars* B, bool first, bool from_lse, bool own_rows
   mbar_init(&B->const_full, own_rows ? 1 + kFWorkerWarps : 1);   // (+ the warps that form the row operands themselves)
   mbar_init(&B->drain, 1);
   for (int i = 0; i < 4; ++i) mbar_init(&B->red_full[i], kFWorkerWarps);
-  for (int i = 0; i < 4; ++i) mbar_init(&B->vn_full[i], 2);
   fence_mbar_init();
 }
 
@@ -174,7 +172,9 @@ struct Ctx {
   float* sm_stats;         // [6][128] floats: row maxima of the column halves [slot][half], then (m, l) hand-over
   const float* row_weight; // [128] temporal weight of each window row but for t_scale
   volatile int* look;      // [2] whether a weight of the tile in accumulator set s may exceed kHeavyA
-  float* vn_s;             // [4][128] ||v||^2 of the last four tiles of phase C (from_lse only)
+  float* vn_s;             // the tokens' own terms (||v||^2, under the projection v^T Mt v of each query head) of phase C's tiles: a
+                           //  ring of two tiles, from given statistics of four
+  float (*red)[4][kTile];  // [tile & 1][warpgroup][token]: each warpgroup's share of the score (from given statistics [tile & 3])
   int* heavy;              // (over sm_stats, which phase A no longer needs) [0]: count, then the units of this CTA's share that
                            //  have a weight above kHeavyA: token * 4 + column group, the sign set for a token's first unit
   int warp, lane;
@@ -722,14 +722,173 @@ __device__ void combine_rows(const Ctx& cx, const FusedArgs& a, int bh, int grou
   }
 }
 
+__device__ __forceinline__ float* heavy_scratch(const FusedArgs& a) { return a.part_O + (long long)blockIdx.x * kRows * kHeadDim; }
+__device__ __forceinline__ float* heavy_logits(const FusedArgs& a, int unit) { return heavy_scratch(a) + 8 * kMaxHeavy + unit * 32; }
+__device__ __forceinline__ float* heavy_sums(const Ctx& cx, const FusedArgs& a, int unit) {
+  return (unit < kNear ? cx.sm_stats + 1 + kMaxHeavy : heavy_scratch(a)) + 4 * unit;
+}
+__device__ __forceinline__ int4* heavy_links(const Ctx& cx, const FusedArgs& a, int unit) {
+  return reinterpret_cast<int4*>(unit < kNear ? cx.sm_stats + 1 + kMaxHeavy + 4 * kNear : heavy_scratch(a) + 4 * kMaxHeavy) + unit;
+}
+// The second of two heads' sums of each token of a head group (w = 64, maximum over the heads), where tile_max has been used up.
+__device__ __forceinline__ float* second_head(const FusedArgs& a, int bh) {
+  return a.tile_max + (long long)bh * ((a.n_kv + kTile - 1) / kTile) * kTile;
+}
+
+// ||v||^2 of rows [row0, row0 + 64) of the V tile of phase C's tile `it`, by one warp.
+__device__ __forceinline__ void half_terms(const Ctx& cx, int it, int row0) {
+#pragma unroll 1
+  for (int rr = 0; rr < 2; ++rr) {
+    const int row = row0 + rr * 32 + cx.lane;
+    cx.vn_s[(it & 3) * kTile + row] = row_square_sum(cx.smem_base + k_slot_off(2 * (it & 1)) + kTileBytes, row);
+  }
+  __syncwarp();
+  if (cx.lane == 0) {
+    mbar_arrive(&cx.B->kv_empty[it & 1]);
+    mbar_arrive(&cx.B->acc_full[it & 1]);
+  }
+}
+
+// Terms per token under the projection: one of each query head (which has no instantiation in use with w below 32).
+template <int kW> constexpr int kTerms = kRows / (kW < 32 ? 32 : kW);
+
+// Warp 2 in phase C: what the epilogue needs to know of a tile beside the accumulators, told with their barrier, so that the
+// sixteen epilogue warps spend neither loads nor registers nor the wait for them on it.
+//   - the tokens' own terms: ||v||^2 as phase A has left it (under the projection v^T Mt v of each query head); from given statistics
+//     from the V tile in shared memory, of which warp 3 takes the second half;
+//   - whether the logits need to be looked at: some row's largest logit reaches that row's M2 - log2(1 / kHeavyA).
+template <int kW, bool kLse, int kInd>
+__device__ void stage_terms(const Ctx& cx, const FusedArgs& a, int bh, int tile0, int T) {
+  constexpr bool kProj = kInd == 3;
+  constexpr int kG = kProj ? kTerms<kW> : 1;   // terms per token
+  FusedBars* B = cx.B;
+  const int lane = cx.lane;
+  bool ok = true;
+  if (kLse && !kProj) {
+    for (int it = 0; it < T; ++it) {
+      ok = ok && mbar_wait(&B->kv_full[it & 1], (uint32_t)(it >> 1) & 1u, cx.abort_flag, a.dev_status, kDevTimeout, a.wait_limit);
+      half_terms(cx, it, 0);
+    }
+    return;
+  }
+  const int nt_all = (a.n_kv + kTile - 1) / kTile;
+  const float* tm = a.tile_max + ((long long)bh * nt_all + tile0) * kRows + lane;
+  const float* terms = (kProj ? a.vmv : a.vnorm) + (long long)bh * kG * a.n_kv + tile0 * kTile + lane;
+  float m2r[4], top[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    m2r[k] = kLse ? 0.f : a.row_M2[(long long)bh * kRows + k * 32 + lane] - log2f(1.f / kHeavyA);
+    top[k] = -INFINITY;
+  }
+#pragma unroll 1
+  for (int it = 0; it < T; ++it) {
+    const int s = it & 1, tile = T - 1 - it;
+    // requested before the wait: the accumulators' set comes free a tile's time before its products are complete
+    float v[kG][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const bool in = (tile0 + tile) * kTile + k * 32 + lane < a.n;
+#pragma unroll
+      for (int g = 0; g < kG; ++g) v[g][k] = in ? terms[(long long)g * a.n_kv + tile * kTile + k * 32] : 1.f;
+      if (!kLse) top[k] = tm[(long long)tile * kRows + k * 32];
+    }
+    ok = ok && (it < 2 || mbar_wait(&B->acc_empty[s], ((it >> 1) - 1) & 1, cx.abort_flag, a.dev_status, kDevTimeout, a.wait_limit));
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int g = 0; g < kG; ++g) cx.vn_s[(s * kG + g) * kTile + k * 32 + lane] = v[g][k];
+    const bool any = __any_sync(0xffffffffu, top[0] > m2r[0] || top[1] > m2r[1] || top[2] > m2r[2] || top[3] > m2r[3]);
+    if (lane == 0) cx.look[s] = any;
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&B->acc_full[s]);
+  }
+}
+
+// A token's score from the four warpgroups' shares, summed in a fixed order, to its place j in the head.
+template <int kW, int kInd>
+__device__ __forceinline__ void join_values(const Ctx& cx, const FusedArgs& a, int bh, bool group_max, int j, float r0, float r1, float r2, float r3) {
+  constexpr bool kEq7 = kInd == 0 || kInd == 3;
+  // A share of -(u + 1): unit u is left out; the links between a token's units go to its first one.
+  if (kEq7 && fminf(fminf(r0, r1), fminf(r2, r3)) < 0.f) {
+    const int4 link = make_int4(r0 < 0.f ? (int)-r0 : 0, r1 < 0.f ? (int)-r1 : 0, r2 < 0.f ? (int)-r2 : 0, r3 < 0.f ? (int)-r3 : 0);
+    const int first = link.x ? link.x : link.y ? link.y : link.z ? link.z : link.w;
+    *heavy_links(cx, a, first - 1) = link;
+    cx.heavy[first] |= (int)0x80000000;
+    r0 = r0 < 0.f ? 0.f : r0;
+    r1 = r1 < 0.f ? 0.f : r1;
+    r2 = r2 < 0.f ? 0.f : r2;
+    r3 = r3 < 0.f ? 0.f : r3;
+  }
+  // every 32 columns are one query head's window when w = 32, several whole windows when w < 32, half a window when
+  // w = 64 and a quarter when w = 128
+  const float r01 = r0 + r1, r23 = r2 + r3;
+  a.I_hat[(long long)bh * a.n + j] = !group_max || kW == 128 ? r01 + r23
+                                     : kW == 64              ? fmaxf(r01, r23)
+                                                             : fmaxf(fmaxf(r0, r1), fmaxf(r2, r3));
+  if (kEq7 && kW == 64 && group_max) {   // both heads' sums, should units be left out of them (the places are used up)
+    a.vnorm[(long long)bh * a.n_kv + j] = r01;
+    second_head(a, bh)[j] = r23;
+  }
+}
+
+// From given statistics: the shares of a tile are joined by one warpgroup, another one for each tile, two tiles later, when
+// nobody waits.  A slot of `red` is rewritten four tiles later, which the two accumulator buffers only allow after every warp has
+// moved past this point.
+template <int kW, int kInd>
+__device__ __forceinline__ bool join_own(const Ctx& cx, const FusedArgs& a, int bh, int tile0, int T, int u, int t, bool ok) {
+  ok = ok && mbar_wait(&cx.B->red_full[u & 3], (uint32_t)(u >> 2) & 1u, cx.abort_flag, a.dev_status, kDevTimeout, a.wait_limit);
+  const int ju = (tile0 + T - 1 - u) * kTile + t;
+  const float (*r)[kTile] = cx.red[u & 3];
+  if (ok && ju < a.n) join_values<kW, kInd>(cx, a, bh, a.group_max != 0, ju, r[0][t], r[1][t], r[2][t], r[3][t]);
+  return ok;
+}
+
+// Warp 3 in phase C: joins the shares of each tile once all sixteen warps have stored theirs.  It lets tile `it` begin only behind the
+// join of tile it - 2, whose slot of `red` it takes.  (Done by warpgroup 0 for the tile before, it cost 0.6 k cycles a tile, by the
+// warpgroups in turn two tiles later 0.8 k of every fourth of a warp's.)  From given statistics warp 3 has half of the tile's ||v||^2
+// to compute, and the warpgroups join in turn after all: with both on this warp 50021 rows took 67.3 us instead of 63.6.
+template <int kW, bool kLse, int kInd>
+__device__ void join_tiles(const Ctx& cx, const FusedArgs& a, int bh, int tile0, int T) {
+  FusedBars* B = cx.B;
+  const int lane = cx.lane;
+  const bool group_max = a.group_max != 0;
+  bool ok = true;
+  if (kLse && kInd != 3) {
+    for (int it = 0; it < T; ++it) {
+      ok = ok && mbar_wait(&B->kv_full[it & 1], (uint32_t)(it >> 1) & 1u, cx.abort_flag, a.dev_status, kDevTimeout, a.wait_limit);
+      half_terms(cx, it, 64);
+    }
+    return;
+  }
+#pragma unroll 1
+  for (int it = 0; it < T + 2; ++it) {
+    const int s = it & 1;
+    if (it >= 2) {
+      ok = ok && mbar_wait(&B->red_full[s], (uint32_t)((it >> 1) - 1) & 1u, cx.abort_flag, a.dev_status, kDevTimeout, a.wait_limit);
+#pragma unroll 1
+      for (int k = 0; k < 4; ++k) {
+        const int t = k * 32 + lane, j = (tile0 + T + 1 - it) * kTile + t;
+        const float r0 = cx.red[s][0][t], r1 = cx.red[s][1][t], r2 = cx.red[s][2][t], r3 = cx.red[s][3][t];
+        if (!ok || j >= a.n) continue;
+        join_values<kW, kInd>(cx, a, bh, group_max, j, r0, r1, r2, r3);
+      }
+    }
+    if (it < T) {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&B->acc_full[s]);
+    }
+  }
+  if (kInd == 0 || kInd == 3) named_barrier_sync(1, kFWorkerWarps * 32 + 32);   // (the large weights' pass begins)
+}
+
 // ------------------------------------------------------------------------------------------------
 // Phase C: this CTA's share [tile0, tile0 + T) of the scored rows of one head, walked from the last tile to the
 // first (the tiles phase A read last are the likeliest to still be in L2).  Warp 0 loads, warp 1 issues the
-// MMAs, the sixteen worker warps are four epilogue warpgroups (thread = token, warpgroup c = accumulator columns
+// MMAs, warps 2 and 3 do what the epilogue shares (above), the sixteen worker warps are four epilogue warpgroups (thread = token, warpgroup c = accumulator columns
 // [32c, 32c + 32)).  Q is still in shared memory from phase A.  The per-query-row constants ride through the
 // tensor core (one extra K = 16 step against a block of ones), so with u = exp2(-scale*log2e * S') = 1/A and
 // x = C' + ||v||^2 = ||o - v||^2 the indicator is x * rsqrt(x * (u - 1)^2).
-template <bool kLse>
+template <int kW, bool kLse, int kInd>
 __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtensorMap* tmQ, const CUtensorMap* tmO,
                                 const CUtensorMap* tmAug, const CUtensorMap* tmK, const CUtensorMap* tmV, int bh,
                                 int tile0, int T, int started, Loads* ld) {
@@ -783,63 +942,11 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
         umma_commit(&B->kv_empty[s]);
       }
     }
-  } else if (!kLse && warp == 2) {
-    // ---- which tiles need their logits looked at: some row's largest logit reaches that row's M2 - log2(1 / kHeavyA).
-    //      Told with the accumulators' barrier, so that the epilogue warps spend neither loads nor registers on it. ----
-    const int nt_all = (a.n_kv + kTile - 1) / kTile;
-    const float* tm = a.tile_max + ((long long)bh * nt_all + tile0) * kRows + lane;
-    float m2r[4], next[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      m2r[k] = a.row_M2[(long long)bh * kRows + k * 32 + lane] - log2f(1.f / kHeavyA);
-      next[k] = T > 0 ? tm[(long long)(T - 1) * kRows + k * 32] : -INFINITY;
-    }
-    bool ok = true;
-    for (int it = 0; it < T; ++it) {
-      const int s = it & 1;
-      const bool any = __any_sync(0xffffffffu, next[0] > m2r[0] || next[1] > m2r[1] || next[2] > m2r[2] || next[3] > m2r[3]);
-      if (it + 1 < T) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) next[k] = tm[(long long)(T - 2 - it) * kRows + k * 32];
-      }
-      ok = ok && (it < 2 || mbar_wait(&B->acc_empty[s], ((it >> 1) - 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit));
-      if (lane == 0) {
-        cx.look[s] = any;
-        mbar_arrive(&B->acc_full[s]);
-      }
-    }
-  } else if (kLse) {
-    // ---- ||v||^2 of the tile's tokens from the V tile in shared memory (phase A, which computes it otherwise, does
-    //      not run): warp 2 takes tokens 0-63, warp 3 tokens 64-127, a lane two rows; ring of four tiles ----
-    bool ok = true;
-    for (int it = 0; it < T; ++it) {
-      const int s = it & 1;
-      ok = ok && mbar_wait(&B->kv_full[s], (it >> 1) & 1, abort_flag, dev_status, kDevTimeout, a.wait_limit);
-#pragma unroll 1
-      for (int rr = 0; rr < 2; ++rr) {
-        const int row = (warp - 2) * 64 + rr * 32 + lane;
-        cx.vn_s[(it & 3) * kTile + row] = row_square_sum(cx.smem_base + k_slot_off(2 * s) + kTileBytes, row);
-      }
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&B->vn_full[it & 3]);
-        mbar_arrive(&B->kv_empty[s]);
-      }
-    }
+  } else if (warp == 2) {
+    stage_terms<kW, kLse, kInd>(cx, a, bh, tile0, T);
+  } else {
+    join_tiles<kW, kLse, kInd>(cx, a, bh, tile0, T);
   }
-}
-
-__device__ __forceinline__ float* heavy_scratch(const FusedArgs& a) { return a.part_O + (long long)blockIdx.x * kRows * kHeadDim; }
-__device__ __forceinline__ float* heavy_logits(const FusedArgs& a, int unit) { return heavy_scratch(a) + 8 * kMaxHeavy + unit * 32; }
-__device__ __forceinline__ float* heavy_sums(const Ctx& cx, const FusedArgs& a, int unit) {
-  return (unit < kNear ? cx.sm_stats + 1 + kMaxHeavy : heavy_scratch(a)) + 4 * unit;
-}
-__device__ __forceinline__ int4* heavy_links(const Ctx& cx, const FusedArgs& a, int unit) {
-  return reinterpret_cast<int4*>(unit < kNear ? cx.sm_stats + 1 + kMaxHeavy + 4 * kNear : heavy_scratch(a) + 4 * kMaxHeavy) + unit;
-}
-// The second of two heads' sums of each token of a head group (w = 64, maximum over the heads), where tile_max has been used up.
-__device__ __forceinline__ float* second_head(const FusedArgs& a, int bh) {
-  return a.tile_max + (long long)bh * ((a.n_kv + kTile - 1) / kTile) * kTile;
 }
 
 // N values per lane (8 or 16) -> sums over the warp: lane L returns the sum of value L * N / 32.  Each exchange halves the
@@ -879,7 +986,7 @@ __device__ void heavy_pass(const Ctx& cx, const FusedArgs& a, int bh) {
   constexpr int kG = kRows / kW;
   int lane = cx.lane, wq = cx.warp - kFFirstWorker;
   asm volatile("" : "+r"(lane), "+r"(wq), "+r"(bh));   // nothing derived from them for this pass occupies registers in the loop before
-  named_barrier_sync(1, kFWorkerWarps * 32);   // every warp has noted its units, and I_hat of the share is written
+  named_barrier_sync(1, kFWorkerWarps * 32 + (kLse && !kProj ? 0 : 32));   // every unit is noted and I_hat of the share written (by warp 3)
   const int count = min(cx.heavy[0], kMaxHeavy);
   if (count == 0) return;
   const int b = bh / a.Hkv, h = bh % a.Hkv;
@@ -1088,7 +1195,7 @@ __device__ void stage_given_rows(const Ctx& cx, const FusedArgs& a, int bh) {
 // kInd: 0 = Eq. 7; 1 = the attention weight alone; 2 = attention weight times ||v|| (Appendix G.1); 3 = Eq. 7 with
 // the output projection of Eq. 4 inside its norm.
 template <int kW, bool kLse, int kInd>
-__device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, int bh, int tile0, int T, float (*red)[4][kTile]) {
+__device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, int bh, int tile0, int T) {
   constexpr int kG = kRows / kW;
   constexpr bool kEq7 = kInd == 0 || kInd == 3, kProj = kInd == 3;
   FusedBars* B = cx.B;
@@ -1118,79 +1225,29 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, int bh, int ti
   const f32x2 d2 = f2_make(ema_decay * ema_decay, ema_decay * ema_decay);
   const f32x2 nc2 = f2_make(neg_c2, neg_c2), m1 = f2_make(-1.f, -1.f), tiny2 = f2_make(1e-36f, 1e-36f);
   const f32x2 seed2 = f2_make(seed_coef, 1.f), last2 = f2_make(1.f, last_coef);
-  // the shares of the four warpgroups: every 32 columns are one query head's window when w = 32, several whole
-  // windows when w < 32, half a window when w = 64 and a quarter when w = 128
-  auto join_shares = [group_max](float r0, float r1, float r2, float r3) {
-    if (!group_max || kW == 128) return (r0 + r1) + (r2 + r3);
-    if (kW == 64) return fmaxf(r0 + r1, r2 + r3);
-    return fmaxf(fmaxf(r0, r1), fmaxf(r2, r3));
-  };
-  // with the output projection the token's own term is v^T Mt v of the query head that this warpgroup's 32 columns
-  // belong to (w >= 32 there)
-  const int g_cols = (cgp * 32) / kW;
-  const float* vn_head = kProj ? a.vmv + ((long long)bh * kG + g_cols) * a.n_kv : a.vnorm + (long long)bh * a.n_kv;
-  float* I_head = a.I_hat + (long long)bh * n;
-  // A share of -(u + 1): unit u is left out; the links between a token's units go to its first one.
-  auto store_score = [&](int j, const float (*r)[kTile]) {
-    float r0 = r[0][t], r1 = r[1][t], r2 = r[2][t], r3 = r[3][t];
-    if (kEq7 && fminf(fminf(r0, r1), fminf(r2, r3)) < 0.f) {
-      const int4 link = make_int4(r0 < 0.f ? (int)-r0 : 0, r1 < 0.f ? (int)-r1 : 0, r2 < 0.f ? (int)-r2 : 0, r3 < 0.f ? (int)-r3 : 0);
-      const int first = link.x ? link.x : link.y ? link.y : link.z ? link.z : link.w;
-      *heavy_links(cx, a, first - 1) = link;
-      cx.heavy[first] |= (int)0x80000000;
-      r0 = r0 < 0.f ? 0.f : r0;
-      r1 = r1 < 0.f ? 0.f : r1;
-      r2 = r2 < 0.f ? 0.f : r2;
-      r3 = r3 < 0.f ? 0.f : r3;
-    }
-    I_head[j] = join_shares(r0, r1, r2, r3);
-    if (kEq7 && kW == 64 && group_max) {   // both heads' sums, should units be left out of them (the places are used up)
-      a.vnorm[(long long)bh * a.n_kv + j] = r0 + r1;
-      second_head(a, bh)[j] = r2 + r3;
-    }
-  };
   float* raw_head = (a.I_raw && !kLse) ? a.I_raw + (long long)bh * kRows * n : nullptr;
   bool ok = true;
-  // The shares of a tile are summed in a fixed order by one warpgroup, another one for each tile, two tiles later: by then all
-  // sixteen warps have stored theirs and nobody waits.  (One tile later the warpgroup that did it waited for the slowest of the
-  // others in every tile, came 0.6 k cycles late to the next and held up its accumulators.)  A slot of `red` is rewritten four tiles
-  // later, which the two accumulator buffers only allow after every warp has moved past this point.
-  auto join_tile = [&](int u) {
-    ok = ok && mbar_wait(&B->red_full[u & 3], (uint32_t)(u >> 2) & 1u, abort_flag, dev_status, kDevTimeout, a.wait_limit);
-    const int ju = (tile0 + T - 1 - u) * kTile + t;
-    if (ok && ju < n) store_score(ju, red[u & 3]);
-  };
   if (kLse && !kProj && T > 0) stage_given_rows(cx, a, bh);
-  float vn_next = 0.f;
-  // from_lse: no phase A has left ||v||^2 and the tiles' row maxima behind; ||v||^2 comes from the control warps
-  // through shared memory and a warp finds out from the logits themselves whether its part of a tile is heavy
+  // from_lse: no phase A has left the tiles' row maxima behind; a warp finds out from the logits themselves whether its part of a
+  // tile is heavy
   constexpr bool from_lse = kLse;
-  const bool vn_global = !from_lse || kProj;   // the token's own term is read from global memory
-  if (T > 0 && vn_global) {
-    const int j = (tile0 + T - 1) * kTile + t;
-    vn_next = (j < n) ? vn_head[j] : 1.f;
-  }
+  // where this token's own term is told, under the projection that of the query head that this warpgroup's 32 columns belong to
+  const float* own_term = cx.vn_s + (kProj ? (cgp * 32) / kW * kTile : 0) + t;
+
+  constexpr bool kJoin = kLse && !kProj;
 
   for (int it = 0; it < T; ++it) {
     const int s = it & 1;
     const uint32_t par = (uint32_t)(it >> 1) & 1u;
-    float vn = vn_next;
-    // only Eq. 7 has the factor 1 / (1 - A) and the distance that need the exact form near A = 1
-    if (from_lse) {
-      ok = ok && mbar_wait(&B->vn_full[it & 3], (uint32_t)(it >> 2) & 1u, abort_flag, dev_status, kDevTimeout, a.wait_limit);
-      const int jv = (tile0 + T - 1 - it) * kTile + t;
-      if (!vn_global) vn = (ok && jv < n) ? cx.vn_s[(it & 3) * kTile + t] : 1.f;
+    if constexpr (kJoin) {
+      if (it >= 2 && cgp == (it & 3)) ok = join_own<kW, kInd>(cx, a, bh, tile0, T, it - 2, t, ok);
     }
-    if (it + 1 < T && vn_global) {   // next tile's ||v||^2 (or v^T Mt v), well ahead of its use
-      const int jn = (tile0 + T - 2 - it) * kTile + t;
-      vn_next = (jn < n) ? vn_head[jn] : 1.f;
-    }
-    if (it >= 2 && cgp == (it & 3)) join_tile(it - 2);
     ok = ok && mbar_wait(&B->acc_full[s], par, abort_flag, dev_status, kDevTimeout, a.wait_limit);
     float tot = 0.f;
     int unit = kMaxHeavy;   // this lane's place in the list of heavy units
     tc_fence_after();
     const int j = (tile0 + T - 1 - it) * kTile + t;
+    const float vn = own_term[(kLse && !kProj ? it & 3 : s * (kProj ? kTerms<kW> : 1)) * kTile];
     const uint32_t tS = tmem + (uint32_t)s * 256u + lane_base + (uint32_t)cgp * 32u, tC = tS + 128u;
     // ||o - v||^2 = C' + ||v||^2 is formed with ||v||^2 raised by 2^-16 of itself: a bias of ~1e-5 that keeps
     // the sum positive when the expansion cancels: C' is that of the rounded o exactly, so that no clamp is needed.  Under the
@@ -1330,13 +1387,15 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, int bh, int ti
     if (from_lse && look && mx > heavy_thr && j < n) unit = atomicAdd(cx.heavy, 1);
     if (unit < kMaxHeavy) cx.heavy[1 + unit] = j * 4 + cgp;
     // (nothing that only looks like a unit: without the accumulators the sum is anything)
-    red[it & 3][cgp][t] = kEq7 && unit < kMaxHeavy ? (float)(-1 - unit) : ok ? tot * fin_scale : 0.f;
+    cx.red[kJoin ? it & 3 : s][cgp][t] = kEq7 && unit < kMaxHeavy ? (float)(-1 - unit) : ok ? tot * fin_scale : 0.f;
     __syncwarp();
-    if (lane == 0) mbar_arrive(&B->red_full[it & 3]);
+    if (lane == 0) mbar_arrive(&B->red_full[kJoin ? it & 3 : s]);
   }
+  if constexpr (kJoin) {
 #pragma unroll 1
-  for (int u = max(T - 2, 0); u < T; ++u)
-    if (cgp == ((u + 2) & 3)) join_tile(u);
+    for (int u = max(T - 2, 0); u < T; ++u)
+      if (cgp == ((u + 2) & 3)) ok = join_own<kW, kInd>(cx, a, bh, tile0, T, u, t, ok);
+  }
   if (kEq7) heavy_pass<kW, kLse, kProj>(cx, a, bh);
 }
 
@@ -1367,7 +1426,7 @@ __device__ void drain_issued(const Ctx& cx, const Loads& ld, bool consts) {
 // barrier, phase C, and a closing __syncthreads.
 
 // Warps 0-3: TMA producer, MMA issuer, the two ||v||^2 warps; thread 0 also runs the group barriers.
-template <bool kLse>
+template <int kW, bool kLse, int kInd>
 __device__ void control_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, const CUtensorMap* tmQ,
                              const CUtensorMap* tmK, const CUtensorMap* tmV, const CUtensorMap* tmO,
                              const CUtensorMap* tmAug, FusedBars* bars, int* abort_flag, int* go) {
@@ -1375,7 +1434,7 @@ __device__ void control_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, 
   unsigned int epoch = 0;
   for (int bh = pl.group; bh < a.BH; bh += a.groups) {
     if (bh != pl.group) {   // fresh barriers for every head: nothing is in flight between two __syncthreads
-      if (threadIdx.x == 0) init_bars(bars, false, kLse, a.lse != nullptr);
+      if (threadIdx.x == 0) init_bars(bars, false, kLse && kInd != 3);
       __syncthreads();
     }
     Loads ld = {0, 0, 0};
@@ -1398,9 +1457,9 @@ __device__ void control_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, 
         break;
       }
       tc_fence_after();
-      phase_c_control<kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, started, &ld);
+      phase_c_control<kW, kLse, kInd>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, started, &ld);
     } else {
-      phase_c_control<kLse>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, 0, &ld);
+      phase_c_control<kW, kLse, kInd>(cx, a, tmQ, tmO, tmAug, tmK, tmV, bh, pl.tile0, pl.T2, 0, &ld);
     }
     tc_fence_before();
     __syncthreads();
@@ -1414,7 +1473,7 @@ __device__ void control_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, 
 
 // Warps 4-19: softmax in phase A, the merge of the partials in phase B, the indicator epilogue in phase C.
 template <int kW, bool kLse, int kInd>
-__device__ void worker_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, int* go, float (*red)[4][kTile]) {
+__device__ void worker_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, int* go) {
   for (int bh = pl.group; bh < a.BH; bh += a.groups) {
     if (bh != pl.group) __syncthreads();
     if (!kLse) {
@@ -1427,7 +1486,7 @@ __device__ void worker_main(const Ctx& cx, const FusedArgs& a, const Plan& pl, i
       if (!group_barrier_follow(go)) break;
       tc_fence_after();
     }
-    phase_c_worker<kW, kLse, kInd>(cx, a, bh, pl.tile0, pl.T2, red);
+    phase_c_worker<kW, kLse, kInd>(cx, a, bh, pl.tile0, pl.T2);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1448,8 +1507,8 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   __shared__ __align__(16) float sm_heavy[4 + kMaxHeavy + 8 * kNear];   // phase A's exchange (6 x 128), then the heavy units
   __shared__ float row_weight[kRows];
   float* const sm_stats = sm_heavy + 3;   // (the units' sums on a 16-byte boundary)
-  __shared__ float vn_ring[4 * kTile];
-  __shared__ float red[4][4][kTile];   // [tile & 3][warpgroup][token]: each warpgroup's share of the score
+  __shared__ float vn_ring[(kInd == 3 ? 2 * kTerms<kW> : kLse ? 4 : 2) * kTile];
+  __shared__ float red[kLse && kInd != 3 ? 4 : 2][4][kTile];
 
   const int group = blockIdx.x / a.cpg, rank = blockIdx.x % a.cpg;
 
@@ -1460,6 +1519,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   cx.abort_flag = &abort_flag;
   cx.sm_stats = sm_stats;
   cx.vn_s = vn_ring;
+  cx.red = red;
   cx.look = look_flag;
   cx.row_weight = row_weight;
   cx.heavy = reinterpret_cast<int*>(sm_stats);
@@ -1469,7 +1529,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   if (threadIdx.x == 0) {
     abort_flag = 0;
     cx.heavy[0] = 0;
-    init_bars(&bars, true, kLse, a.lse != nullptr);
+    init_bars(&bars, true, kLse && kInd != 3);
     prefetch_tensormap(&tmQ);
     prefetch_tensormap(&tmK);
     prefetch_tensormap(&tmV);
@@ -1511,10 +1571,10 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   // compiled for more registers than the launch gives every thread.
   if (cx.warp < kFFirstWorker) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFRegsControl));
-    control_main<kLse>(cx, a, pl, &tmQ, &tmK, &tmV, &tmO, &tmAug, &bars, &abort_flag, &go_flag);
+    control_main<kW, kLse, kInd>(cx, a, pl, &tmQ, &tmK, &tmV, &tmO, &tmAug, &bars, &abort_flag, &go_flag);
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kFRegsWorker));
-    worker_main<kW, kLse, kInd>(cx, a, pl, &go_flag, red);
+    worker_main<kW, kLse, kInd>(cx, a, pl, &go_flag);
   }
 
   tc_fence_before();
