@@ -21,7 +21,7 @@ constexpr int kRsHalfSmem = 92 * 1024;   // dynamic shared memory of a block whe
 // a histogram of 11-bit digits of the offsets from the smallest (about a thousand bins in use, so one histogram serves all
 // warps without contention), then the sum above the digit that holds the Bp-th largest while that digit's few keys are
 // listed and ranked, a key per warp.  1024 rows of 20011: 43.5 us with one block of 1024 threads and two rows in flight per SM
-// (10 k cycles per row, 3.6 k of them synchronisation), 39 us so.
+// (10 k cycles per row, 3.6 k of them synchronisation), 39 us so, 35 with the short last walk.
 template <int kRsThreads, bool kHeld>   // kHeld false: no buffers, the keys are read from global memory on every walk
 __global__ void __launch_bounds__(kRsThreads, kRsThreads <= 512 ? 2 : 1)
 row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buffers, unsigned long long* __restrict__ sums,
@@ -154,16 +154,39 @@ row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buff
     // ---- the sum above the digit; the digit's keys [k0, k1] listed (or, more equal keys than the list takes, counted) ----
     const unsigned int k0 = kmin + prefix, k1 = k0 + ((lo < 32 ? 1u << lo : 0u) - 1u);
     const bool ties = listed > kRsList;
+    // (Two instructions a key for the sum, in 32 bits a quad at a time, and one branch a quad for the few keys of the digit: with a
+    // 64-bit sum and a branch for every key this walk took 5 to 7 k cycles of a row's 14 k, so 3 to 4 k.)
     unsigned long long isum = 0ull;
-    each([&](unsigned int i, unsigned int key) {
-      if (key > k1) {
-        isum += i;
-      } else if (key >= k0 && !ties) {
+    const unsigned int span = k1 - k0;
+    auto list_key = [&](unsigned int i, unsigned int key) {
+      if (key - k0 <= span) {
         const unsigned int slot = atomicAdd(&s_listed, 1u);
         list_v[slot] = key;
         list_i[slot] = i;
       }
-    });
+    };
+#pragma unroll 2
+    for (int q = q0 + tid; q < q1; q += kRsThreads) {
+      const uint4 k4 = quad[q];
+      const unsigned int i = (unsigned int)(4 * q - mis);
+      unsigned int part = 0u;   // (rows are shorter than 2^30)
+      if (k4.x > k1) part += i;
+      if (k4.y > k1) part += i + 1u;
+      if (k4.z > k1) part += i + 2u;
+      if (k4.w > k1) part += i + 3u;
+      isum += part;
+      if (!ties && ((k4.x - k0 <= span) | (k4.y - k0 <= span) | (k4.z - k0 <= span) | (k4.w - k0 <= span))) {
+        list_key(i, k4.x);
+        list_key(i + 1, k4.y);
+        list_key(i + 2, k4.z);
+        list_key(i + 3, k4.w);
+      }
+    }
+    if (tid < ends) {
+      const unsigned int i = (unsigned int)(tid < head || q1 < q0 ? tid : n - tail + (tid - head)), key = words[mis + i];
+      if (key > k1) isum += i;
+      else if (!ties) list_key(i, key);
+    }
     __syncthreads();   // the row has been walked for the last time (but for ties), the list is complete
     if (!ties) {
       if (kHeld && tid == kRsThreads - 1 && row + (long long)buffers * gridDim.x < rows) request(row + buffers * gridDim.x, it + buffers);
