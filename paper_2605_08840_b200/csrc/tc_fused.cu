@@ -46,6 +46,7 @@ struct FusedArgs {
   float t_decay, t_seed_first, t_seed_last, t_scale;
   int group_max;                     // 1: maximum over the query heads of a group instead of their mean
   int groups, cpg;                   // CTA groups and CTAs per group
+  int lrb;                           // log2 of the rows that a CTA merges: the smallest, 1 at least, with cpg << lrb >= 128
   int attention_only;                // 1: stop after the merge (phases A and B): plain attention of the 128 rows
   int from_lse;                      // 1: O and the rows' log-sum-exp are given: phases A and B are skipped, phase C
                                      //    computes ||v||^2 and finds the tiles with large weights by itself
@@ -546,20 +547,20 @@ __device__ __forceinline__ void split3(float x, __nv_bfloat16* out) {
 // in shared memory.  Every order is fixed: the result does not depend on timing.  Written for phase C: O (fp32), -2 bf16(O),
 // and the rows' strips of bf16 constant pieces.  Called by all sixteen worker warps.
 // What bounds it: one trip to L2 for the partials (requested before the weights, which take a trip and two synchronisations
-// of their own), one to write, and the first fetch of its instructions (run twice, the second time takes half).  8 heads of 16384
-// rows: 11.7 k cycles with two warps to a row, 8.1 k so; under the output projection, whose Mt every row's warp read for itself,
+// of their own; 73 KB per CTA arrive at 21 bytes a cycle and SM) and one to write.  8 heads of 16384 rows: 11.7 k cycles with two
+// warps to a row, 7.3 k with its divisions and the weights passed through shared memory twice, 6.3 k so; under the output projection, whose Mt every row's warp read for itself,
 // 27 k and 13 k.
 template <bool kProj>
 __device__ void combine_rows(const Ctx& cx, const FusedArgs& a, int bh, int group, int rank) {
-  int wt = threadIdx.x - kFFirstWorker * 32, cpg = a.cpg;
-  asm volatile("" : "+r"(wt), "+r"(cpg));   // nothing derived from them here occupies registers in the loops over the tiles
+  int wt = threadIdx.x - kFFirstWorker * 32, cpg = a.cpg, lrb = a.lrb;
+  asm volatile("" : "+r"(wt), "+r"(cpg), "+r"(lrb));   // nothing derived from them here occupies registers in the loops over the tiles
   const int wq = wt >> 5, lane = wt & 31;
-  int lrb = 1;
-  while ((cpg << lrb) < kRows) ++lrb;
   const int rb = 1 << lrb, r0 = rank << lrb;
   if (r0 >= kRows) return;
   constexpr int kThreads = kFWorkerWarps * 32, kBatch = 9;   // partials in flight per thread
-  const int items = rb * (kHeadDim / 4), per_pass = min(items, kThreads), splits = kThreads / per_pass, split = wt / per_pass;
+  static_assert(kThreads == 512 && kHeadDim == 128, "the shifts below");
+  // (powers of two throughout: divisions by them as such took 0.8 k cycles before the first load was on its way)
+  const int items = rb << 5, lsplits = max(0, 4 - lrb), splits = 1 << lsplits, split = wt >> (9 - lsplits), item0 = wt & (kThreads / splits - 1);
   const long long slot0 = (long long)group * cpg;
   float4 v[kBatch];
   // (Past the last partial it is that one again, not used.  Loads left out by a predicate cost the whole kernel its order of
@@ -572,32 +573,35 @@ __device__ void combine_rows(const Ctx& cx, const FusedArgs& a, int bh, int grou
       v[k] = *reinterpret_cast<const float4*>(src + (long long)min(p, cpg - 1) * kRows * kHeadDim);
     }
   };
-  request(wt % per_pass, split);
-  // ---- weights of the partials, [p][row], and per row 1 / l and the log2 normaliser ----
-  const int pairs = cpg << lrb;   // 512 at most (cpg < 128: below 256)
-  float* sm_w = cx.sm_stats;
-  float* sm_l = sm_w + 512;
-  float* sm_inv = sm_l + 512;
+  request(item0, split);
+  // ---- weights of the partials, [p][row], and per row 1 / l and the log2 normaliser: a warp to a row, a lane to a partial, or the
+  //      512 / rb lanes that there are where a CTA has more rows than warps (then there are fewer partials) ----
+  float* sm_w = cx.sm_stats;   // 512 at most (cpg < 128: below 256)
+  float* sm_inv = sm_w + 1024;
   float* sm_M2 = sm_inv + kRows;
-  for (int e = wt; e < pairs; e += kThreads) {
-    const long long at = (slot0 + (e >> lrb)) * kRows + r0 + (e & (rb - 1));
-    sm_w[e] = a.part_m[at];
-    sm_l[e] = a.part_l[at];
-  }
-  named_barrier_sync(2, kThreads);
-  // four lanes to a row, or a warp where there are many partials: all rows at once (rb is 4 at most in the second case)
-  const int team = cpg > 32 ? 32 : 4, tl = wt & (team - 1), tr = wt / team;
-  float m = -INFINITY, l = 0.f;
-  if (tr < rb)
-    for (int p = tl; p < cpg; p += team) m = fmaxf(m, sm_w[(p << lrb) + tr]);
+  const int lteam = lrb <= 4 ? 5 : 9 - lrb, team = 1 << lteam, tl = wt & (team - 1), tr = wt >> lteam;
+  const float* pm = a.part_m + slot0 * kRows + r0 + tr;
+  const float* pl = a.part_l + slot0 * kRows + r0 + tr;
+  const bool mine = tr < rb && tl < cpg;
+  const float m_own = mine ? pm[tl * kRows] : -INFINITY, l_own = mine ? pl[tl * kRows] : 0.f;
+  float m = m_own, l = 0.f;
+  if (mine)
+    for (int p = tl + team; p < cpg; p += team) m = fmaxf(m, pm[p * kRows]);
 #pragma unroll 1
   for (int off = team >> 1; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-  if (tr < rb)
-    for (int p = tl; p < cpg; p += team) {
-      const float mp = sm_w[(p << lrb) + tr], w = (mp == -INFINITY) ? 0.f : ex2_approx(mp - m);   // an empty partial weighs 0
+  if (mine) {
+    float mp = m_own, lp = l_own;
+#pragma unroll 1
+    for (int p = tl;;) {
+      const float w = (mp == -INFINITY) ? 0.f : ex2_approx(mp - m);   // an empty partial weighs 0
       sm_w[(p << lrb) + tr] = w;
-      l = fmaf(sm_l[(p << lrb) + tr], w, l);
+      l = fmaf(lp, w, l);
+      p += team;
+      if (p >= cpg) break;
+      mp = pm[p * kRows];
+      lp = pl[p * kRows];
     }
+  }
 #pragma unroll 1
   for (int off = team >> 1; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
   if (tl == 0 && tr < rb) {
@@ -608,7 +612,7 @@ __device__ void combine_rows(const Ctx& cx, const FusedArgs& a, int bh, int grou
   // ---- O ----
   float* on_part = reinterpret_cast<float*>(cx.gen_base + kOffAug);                        // [32 pieces or fewer][rb]
   float4* split_sum = reinterpret_cast<float4*>(cx.gen_base + kOffAug + kAugBytes / 2);    // [splits - 1][items], rb <= 8
-  for (int item = wt % per_pass; item < items; item += kThreads) {
+  for (int item = item0; item < items; item += kThreads) {
     const int r = item & (rb - 1), piece = item >> lrb;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
@@ -698,27 +702,26 @@ __device__ void combine_rows(const Ctx& cx, const FusedArgs& a, int bh, int grou
       named_barrier_sync(2, kThreads);   // the rows are overwritten by the next eight
     }
   }
-  // ---- the strips: 64 bf16 a row, zero but for the pieces of -M2 / c2 and of ||o||^2 ----
-  for (int e = wt; e < rb * 8; e += kThreads) {
-    const int r = e >> 3, part = e & 7;
+  // ---- the strips: 64 bf16 a row, zero but for the pieces of -M2 / c2 and of ||o||^2, which the row's eight threads add up ----
+  for (int e = wt; (e & ~31) < rb * 8; e += kThreads) {
+    const int r = min(e >> 3, rb - 1), part = e & 7;
     const long long ri = (long long)bh * kRows + r0 + r;
+    constexpr int kParts = kProj ? 2 : kHeadDim / 4;
+    float on = 0.f;
+#pragma unroll
+    for (int k = 0; k < kParts; k += 8) on += k + part < kParts ? on_part[(k + part) * rb + r] : 0.f;
+#pragma unroll
+    for (int off = 1; off < 8; off <<= 1) on += __shfl_xor_sync(0xffffffffu, on, off);
     uint4 u = make_uint4(0u, 0u, 0u, 0u);
     if ((part & ~2) == 0) {
-      float x;
-      if (part == 0) {
-        x = -sm_M2[r] / (a.scale * kLog2e);
-        a.row_M2[ri] = sm_M2[r];
-      } else {
-        x = 0.f;
-        constexpr int kParts = kProj ? 2 : kHeadDim / 4;
-#pragma unroll
-        for (int k = 0; k < kParts; ++k) x += on_part[k * rb + r];
-      }
-      const uint3 p3 = split3(x);
+      const uint3 p3 = split3(part == 0 ? -sm_M2[r] / (a.scale * kLog2e) : on);
       u.x = p3.x | (p3.y << 16);
       u.y = p3.z;
     }
-    *reinterpret_cast<uint4*>(a.aug + ri * 64 + part * 8) = u;
+    if (e < rb * 8) {
+      *reinterpret_cast<uint4*>(a.aug + ri * 64 + part * 8) = u;
+      if (part == 0) a.row_M2[ri] = sm_M2[r];
+    }
   }
 }
 
@@ -1807,6 +1810,7 @@ cudaError_t launch_tc_fused(void* state, const Problem& p, const Workspace& ws, 
   a.attention_only = attention_only ? 1 : 0;
   a.from_lse = O_given ? 1 : 0;
   fused_plan(p, sm_count, reuse_l2, &a.groups, &a.cpg);
+  for (a.lrb = 1; (a.cpg << a.lrb) < kRows;) ++a.lrb;
   a.part_m = ws.part_m; a.part_l = ws.part_l; a.part_O = ws.part_O;
   a.O_f32 = ws.O_f32; a.O_m2 = ws.O_m2; a.aug = ws.aug; a.vnorm = ws.vnorm; a.I_hat = ws.I_hat;
   a.Q = (const __nv_bfloat16*)Q; a.K = (const __nv_bfloat16*)K; a.V = (const __nv_bfloat16*)V;
