@@ -211,22 +211,43 @@ __global__ void __launch_bounds__(128) combine_kernel(int R, int d, int splits, 
   __shared__ __align__(16) float sums[4][256];
   const int r = blockIdx.x, bh = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const long long base = (long long)bh * splits * R + r;   // + s * R
-  float m = -INFINITY;
-  for (int s = lane; s < splits; s += 32) m = fmaxf(m, part_m[base + (long long)s * R]);
+  // everything that up to 32 splits need is requested at once: the weights, and the eight partial rows that a warp adds up
+  constexpr int kAhead = 8;
+  float4 ahead[kAhead];
+#pragma unroll
+  for (int k = 0; k < kAhead; ++k) {
+    const int s = wid + 4 * k;
+    ahead[k] = s < splits && lane * 4 < d ? *reinterpret_cast<const float4*>(part_O + (base + (long long)s * R) * d + lane * 4)
+                                          : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  const float m_own = lane < splits ? part_m[base + (long long)lane * R] : -INFINITY;
+  const float l_own = lane < splits ? part_l[base + (long long)lane * R] : 0.f;
+  float m = m_own;
+  for (int s = lane + 32; s < splits; s += 32) m = fmaxf(m, part_m[base + (long long)s * R]);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-  float l = 0.f;
-  for (int s = lane; s < splits; s += 32) l += part_l[base + (long long)s * R] * expf(part_m[base + (long long)s * R] - m);
+  const float w_own = lane < splits ? expf(m_own - m) : 0.f;   // an empty split weighs 0
+  float l = lane < splits ? l_own * w_own : 0.f;
+  for (int s = lane + 32; s < splits; s += 32) l += part_l[base + (long long)s * R] * expf(part_m[base + (long long)s * R] - m);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
-  for (int c = lane * 4; c < d; c += 128) {
+  for (int c0 = 0; c0 < d; c0 += 128) {
+    const int c = c0 + lane * 4;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-    for (int s = wid; s < splits; s += 4) {
-      const float w = expf(part_m[base + (long long)s * R] - m);   // an empty split weighs 0
-      const float4 v = *reinterpret_cast<const float4*>(part_O + (base + (long long)s * R) * d + c);
+    auto add = [&](float4 v, float w) {
       acc.x = fmaf(v.x, w, acc.x); acc.y = fmaf(v.y, w, acc.y); acc.z = fmaf(v.z, w, acc.z); acc.w = fmaf(v.w, w, acc.w);
+    };
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) {
+      const int s = wid + 4 * k;
+      const float w = __shfl_sync(0xffffffffu, w_own, s & 31);
+      if (s >= splits || c >= d) continue;
+      add(c0 == 0 ? ahead[k] : *reinterpret_cast<const float4*>(part_O + (base + (long long)s * R) * d + c), w);
     }
+    if (c >= d) continue;
+#pragma unroll 4
+    for (int s = wid + 4 * kAhead; s < splits; s += 4)
+      add(*reinterpret_cast<const float4*>(part_O + (base + (long long)s * R) * d + c), expf(part_m[base + (long long)s * R] - m));
     *reinterpret_cast<float4*>(&sums[wid][c]) = acc;
   }
   __syncthreads();
@@ -312,6 +333,16 @@ __global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T
   for (int t = 0; t < kTok; ++t) acc[t] = 0.f;
   ptx::grid_dependency_wait();
   ptx::grid_dependency_launch();
+  float fm_next[2], fl_next[2];
+  auto row_stats = [&](int row0) {   // m and l of this thread's rows in the step from row0 on
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int row = row0 + rl + 32 * i;
+      fm_next[i] = row < R ? fin_m[(long long)bh * R + row] : 0.f;
+      fl_next[i] = row < R ? fin_l[(long long)bh * R + row] : 1.f;
+    }
+  };
+  row_stats(0);
 
   for (int row0 = 0; row0 < R; row0 += kP2Rows) {
     const int rows = min(kP2Rows, R - row0);
@@ -327,10 +358,10 @@ __global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T
     float fm[2], fl[2];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const int r = rl + 32 * i;
-      fm[i] = r < rows ? fin_m[(long long)bh * R + row0 + r] : 0.f;
-      fl[i] = r < rows ? fin_l[(long long)bh * R + row0 + r] : 1.f;
+      fm[i] = fm_next[i];
+      fl[i] = fl_next[i];
     }
+    row_stats(row0 + kP2Rows);   // the next step's are on their way meanwhile
     if (row0 % held == 0) {
       load_wait();
       __syncthreads();
