@@ -22,7 +22,6 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kP1Tile = 32;   // tokens per tile of pass 1
 constexpr int kP1Rows = 64;   // query rows per block of pass 1
-constexpr int kP2Rows = 64;   // query rows per step of pass 2
 
 __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
   const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
@@ -280,17 +279,19 @@ __device__ __forceinline__ float temporal_weight(int mode, float decay, int w, i
 }
 
 // ------------------------------------------------------------------------------------------------
-// Pass 2 without an output projection.  grid (blocks of kTB tokens, BH), block 256: a thread owns two rows of each step of
-// 64 and kTB / 8 tokens.  Shared memory: K, V [kTB][d+4], Q, O [held][d+4] (held: a multiple of 64, all rows if they fit), the temporal weights [w], and for the maximum over
-// the query heads the weighted indicators of a step [64][kTB+1] and the heads' sums [G][kTB].
-template <typename T, int kTB>
+// Pass 2 without an output projection.  grid (blocks of kTB tokens, BH), block 256: a thread owns kRT rows of each step of
+// 32 kRT and kTB / 8 tokens.  Shared memory: K, V [kTB][d+4], Q, O [held][d+4] (held: a multiple of a step, all rows if they fit), the
+// temporal weights [w], and for the maximum over the query heads the weighted indicators of a step [32 kRT][kTB+1] and the heads' sums
+// [G][kTB].  What bounds the products is shared memory, 16 bytes per lane and load, four cycles each: a pair of a 2 x 2 block
+// takes two loads every four dims, of a 4 x 2 or 2 x 4 block one and a half.
+template <typename T, int kTB, int kRT>
 __global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T* __restrict__ Q, const T* __restrict__ K,
                                                               const T* __restrict__ V, const float* __restrict__ fin_m,
                                                               const float* __restrict__ fin_l, const float* __restrict__ O_f32,
                                                               float ema_decay, float* __restrict__ I_hat, float* __restrict__ I_raw,
                                                               int held) {
   extern __shared__ __align__(16) float smem[];
-  constexpr int kTok = kTB / 8;
+  constexpr int kTok = kTB / 8, kP2Rows = 32 * kRT;
   const int d = p.d, ld = d + 4, R = p.R;
   float* Ks = smem;
   float* Vs = Ks + kTB * ld;
@@ -333,10 +334,10 @@ __global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T
   for (int t = 0; t < kTok; ++t) acc[t] = 0.f;
   ptx::grid_dependency_wait();
   ptx::grid_dependency_launch();
-  float fm_next[2], fl_next[2];
+  float fm_next[kRT], fl_next[kRT];
   auto row_stats = [&](int row0) {   // m and l of this thread's rows in the step from row0 on
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kRT; ++i) {
       const int row = row0 + rl + 32 * i;
       fm_next[i] = row < R ? fin_m[(long long)bh * R + row] : 0.f;
       fl_next[i] = row < R ? fin_l[(long long)bh * R + row] : 1.f;
@@ -355,9 +356,9 @@ __global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T
     }
     const float* Qs = Qh_s + (row0 % held) * ld;
     const float* Os = Oh_s + (row0 % held) * ld;
-    float fm[2], fl[2];
+    float fm[kRT], fl[kRT];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kRT; ++i) {
       fm[i] = fm_next[i];
       fl[i] = fl_next[i];
     }
@@ -366,16 +367,16 @@ __global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T
       load_wait();
       __syncthreads();
     }
-    float s[2][kTok], ss[2][kTok];
+    float s[kRT][kTok], ss[kRT][kTok];
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < kRT; ++i)
 #pragma unroll
       for (int t = 0; t < kTok; ++t) s[i][t] = ss[i][t] = 0.f;
 #pragma unroll 2
     for (int k = 0; k < d; k += 4) {
-      float4 q[2], o[2];
+      float4 q[kRT], o[kRT];
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
+      for (int i = 0; i < kRT; ++i) {
         q[i] = *reinterpret_cast<const float4*>(Qs + (rl + 32 * i) * ld + k);
         o[i] = *reinterpret_cast<const float4*>(Os + (rl + 32 * i) * ld + k);
       }
@@ -384,7 +385,7 @@ __global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T
         const float4 kv = *reinterpret_cast<const float4*>(Ks + (tl + 8 * t) * ld + k);
         const float4 v = *reinterpret_cast<const float4*>(Vs + (tl + 8 * t) * ld + k);
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < kRT; ++i) {
           s[i][t] = dot4(q[i], kv, s[i][t]);
           const float4 df = make_float4(o[i].x - v.x, o[i].y - v.y, o[i].z - v.z, o[i].w - v.w);
           ss[i][t] = dot4(df, df, ss[i][t]);
@@ -392,7 +393,7 @@ __global__ void __launch_bounds__(kThreads) simt_pass2_kernel(Problem p, const T
       }
     }
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kRT; ++i) {
       const int r = rl + 32 * i, row = row0 + r;
       const float weight = r < rows ? wt[row % p.w] : -1.f;
 #pragma unroll
@@ -539,20 +540,23 @@ cudaError_t pass2(const Problem& p, const Workspace& ws, const void* Q, const vo
     return chain(simt_pass2_proj_kernel<T>, dim3((p.n + kP2Tile - 1) / kP2Tile, p.BH), kP2Tile * GP, smem, st, p, (const T*)Q,
                  (const T*)K, (const T*)V, ws.fin_m, ws.fin_l, ws.O_f32, ws.O_proj, ema_decay, ws.I_hat, I_raw, GP);
   }
-  const int all = (p.R + kP2Rows - 1) / kP2Rows * kP2Rows;
-  auto floats = [&](int tb, int held) {
-    return (size_t)2 * (tb + held) * (p.d + 4) + p.w +
-           (p.group == RESTKV_GROUP_MAX ? (size_t)kP2Rows * (tb + 1) + (size_t)p.G * tb : 0);
+  auto floats = [&](int tb, int step, int held) {
+    return (size_t)2 * (tb + held) * (p.d + 4) + p.w + (p.group == RESTKV_GROUP_MAX ? (size_t)step * (tb + 1) + (size_t)p.G * tb : 0);
   };
   // 32 tokens per block share the loads of Q and O better; 16 where that would leave SMs with a single block, or where 32
   // do not fit shared memory (8 were slower even for 1024 rows of 2 heads, one block per SM: 33.8 against 28.6 us)
-  const bool wide = (long long)(p.n + 31) / 32 * p.BH >= 296 && floats(32, kP2Rows) * sizeof(float) <= 220 * 1024;
+  const bool wide = (long long)(p.n + 31) / 32 * p.BH >= 296 && floats(32, 64, 64) * sizeof(float) <= 220 * 1024;
   const int tb = wide ? 32 : 16;
+  // four rows per thread where there are more than 64 (fewer would leave half a step to do for nothing) and two blocks of a step of
+  // 128 fit an SM: 1500 rows of 2 heads 33.4 -> 32.4 us, 1024 rows no difference; not with 32 tokens, whose 16 pairs per thread take
+  // the registers of the second block on the SM (4 sequences of 5000 rows 164 -> 191 us)
+  const bool tall = !wide && p.R > 64 && floats(tb, 128, 128) * sizeof(float) <= 110 * 1024;
+  const int step = tall ? 128 : 64, all = (p.R + step - 1) / step * step;
   // all rows of Q and O stay in shared memory where two blocks of that size fit an SM
-  const int held = floats(tb, all) * sizeof(float) <= 110 * 1024 ? all : kP2Rows;
-  return chain(wide ? simt_pass2_kernel<T, 32> : simt_pass2_kernel<T, 16>, dim3((p.n + tb - 1) / tb, p.BH), kThreads,
-               floats(tb, held) * sizeof(float), st, p, (const T*)Q, (const T*)K, (const T*)V, ws.fin_m, ws.fin_l, ws.O_f32, ema_decay,
-               ws.I_hat, I_raw, held);
+  const int held = floats(tb, step, all) * sizeof(float) <= 110 * 1024 ? all : step;
+  auto kernel = wide ? simt_pass2_kernel<T, 32, 2> : tall ? simt_pass2_kernel<T, 16, 4> : simt_pass2_kernel<T, 16, 2>;
+  return chain(kernel, dim3((p.n + tb - 1) / tb, p.BH), kThreads, floats(tb, step, held) * sizeof(float), st, p, (const T*)Q, (const T*)K,
+               (const T*)V, ws.fin_m, ws.fin_l, ws.O_f32, ema_decay, ws.I_hat, I_raw, held);
 }
 
 }  // namespace
