@@ -471,6 +471,28 @@ def test_evict_host_matches_oracle(handle):
     assert int(dQ.view(torch.int16).abs().max()) == 0
 
 
+@pytest.mark.parametrize("spec", [(1, 1, 700), (1, 2, 3000), (1, 3, 701), (1, 5, 1300), (2, 8, 900), (5, 8, 513), (9, 8, 1025), (19, 8, 129),
+                                  (19, 8, 700)])
+@pytest.mark.parametrize("given", [False, True])
+def test_ctas_per_head_and_tiles_per_cta(handle, spec, given):
+    """From 148 CTAs per head to one, with none to six tiles each: how many rows a CTA merges and how many threads share one, and the
+    shares of a tile joined two tiles later, whatever is left at the end.  Given statistics as the oracle computes them."""
+    batch, heads, n = spec
+    inp = make_inputs(Case("split", batch, 4 * heads, heads, 128, n, 32, min(n, 200), 5, 0, 0.9, "bf16", 0, "planted", 7 + n))
+    if given:
+        variant_check(handle, inp, (0, 0, 0, 0), path=rk.PATH_TENSOR_CORE, from_lse=True)
+    else:
+        full_check(handle, inp)
+
+
+@pytest.mark.parametrize("heads_w", [(1, 64), (4, 18), (4, 32), (2, 65), (17, 8)])
+@pytest.mark.parametrize("n", [15, 33, 1500])
+def test_fp32_pass2_rows_per_thread(handle, heads_w, n):
+    """Query rows on either side of the 64 and 128 of a step (two and four rows per thread), tokens around a block's 16."""
+    group, w = heads_w
+    full_check(handle, make_inputs(Case("rows", 1, 2 * group, 2, 64, n, w, min(n, 100), 5, 0, 0.9, "f32", 0, "normal", group * w + n)))
+
+
 # ------------------------------------------------------------------ unit: select, compact, decode
 @pytest.mark.parametrize("spec", [(1, 1, 1, 1), (1, 31, 7, 5), (2, 255, 254, 7), (3, 1025, 40, 33), (2, 8160, 3000, 7), (2, 8161, 3000, 5),
                                   (20, 8161, 77, 7), (40, 9000, 700, 3), (160, 1500, 64, 7), (150, 26001, 100, 5),
