@@ -35,8 +35,8 @@ __device__ __forceinline__ uint64_t kmajor_desc(uint32_t addr) { return make_sme
 
 // D[128 x 128] (+)= A[128 x 128] * B[128 x 128]^T, both operands K-major 128B-swizzled [128 x 128] bf16 tiles
 // made of two [128 x 64] boxes.  One thread issues the eight K = 16 steps.
-// (The issuing thread's own instruction stream is what bounds a run of small products: the two descriptors are built
-// once and stepped by adding to their address field, which counts 16-byte units.)
+// (The two descriptors are built once and stepped by adding to their address field, which counts 16-byte units: 17 cycles of
+// the issuing thread a step behind elect.sync, 64 of the tensor pipe.)
 __device__ __forceinline__ void mma_tile_kk(uint32_t tmem_d, uint32_t a_smem, uint32_t b_smem, bool accumulate) {
   const uint64_t a0 = kmajor_desc(a_smem), b0 = kmajor_desc(b_smem);
 #pragma unroll

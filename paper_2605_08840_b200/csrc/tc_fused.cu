@@ -19,7 +19,8 @@ namespace restkv {
 
 namespace {
 
-constexpr int kFFirstWorker = 4;                  // warp 0: TMA producer, 1: MMA issuer, 2-3: ||v||^2 during phase A
+constexpr int kFFirstWorker = 4;                  // warp 0: TMA producer, 1: MMA issuer, 2-3: ||v||^2 during phase A, what
+                                                  // the epilogue shares during phase C
 constexpr int kFWorkerWarps = 16;                 // warps 4..19
 constexpr int kFThreads = (kFFirstWorker + kFWorkerWarps) * 32;
 // Registers per thread: 96 at launch (640 threads), i.e. a pool of 20 warps x 32 x 96 = 61440 for the CTA.  The control
@@ -546,10 +547,10 @@ __device__ __forceinline__ void split3(float x, __nv_bfloat16* out) {
 // (row, four columns), several threads to one where there are few rows, each with every `splits`-th partial; their sums meet
 // in shared memory.  Every order is fixed: the result does not depend on timing.  Written for phase C: O (fp32), -2 bf16(O),
 // and the rows' strips of bf16 constant pieces.  Called by all sixteen worker warps.
-// What bounds it: one trip to L2 for the partials (requested before the weights, which take a trip and two synchronisations
+// What bounds it: one trip to L2 for the partials (requested before the weights, which take a trip and a synchronisation
 // of their own; 73 KB per CTA arrive at 21 bytes a cycle and SM) and one to write.  8 heads of 16384 rows: 11.7 k cycles with two
-// warps to a row, 7.3 k with its divisions and the weights passed through shared memory twice, 6.3 k so; under the output projection, whose Mt every row's warp read for itself,
-// 27 k and 13 k.
+// warps to a row, 7.3 k with its divisions and the weights passed through shared memory twice, 6.3 k so; under the output
+// projection, with Mt read by every row's warp for itself, 27 k and 13 k.
 template <bool kProj>
 __device__ void combine_rows(const Ctx& cx, const FusedArgs& a, int bh, int group, int rank) {
   int wt = threadIdx.x - kFFirstWorker * 32, cpg = a.cpg, lrb = a.lrb;

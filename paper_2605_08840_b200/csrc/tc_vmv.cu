@@ -9,10 +9,9 @@
 //   warp 0     TMA: the head's G factor tiles L_g^T [128 x 128] bf16 (reloaded when the share enters a new head),
 //              then the V tiles through a ring that takes the rest of shared memory (three to six tiles: the loads
 //              are latency-bound, so every tile in flight counts)
-//   warp 1     MMA issue: for each tile one product per pair of query heads (eight K = 16 steps of N = 256; N = 128
-//              with a single head), each committed to the pair's barrier.  A step costs the issuing thread and the
-//              tensor pipe about as much at N = 64 as at N = 128, so fewer, wider steps are what pays (narrowing
-//              the steps to the triangular factor's non-zero columns did not)
+//   warp 1     MMA issue: for each tile one product per pair of query heads (eight K = 16 steps of N = 256, 128 cycles of
+//              the tensor pipe each; N = 128, 64 cycles, with a single head), each committed to the pair's barrier.  Steps
+//              of N = 64 take 48 cycles, so that narrowing them to the triangular factor's non-zero columns does not pay
 //   warps 2-17 read-out: thread = token (tensor-memory lane), 128 columns squared and summed; each of the four warps
 //              of a lane quarter takes one query head
 // Every wait is bounded; after a failed wait the roles stop, wait for what they issued and the CTA returns.
