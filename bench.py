@@ -72,7 +72,7 @@ def whole_job_value(tokens_per_rank_step, world, steps, total_ms):
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the dominant kernel, from an ncu capture
 # of this workload, together with the digest of the kernel sources the capture was taken on: the figure is reported
 # only while those sources are unchanged, otherwise `traffic` is null.
-KERNEL_TRAFFIC = {"cfg4": {"bytes": 1003404288 + 5186304, "sources_sha256": "fdd6e60c71156785fbe8f6614832f5b89564dad5f6d7f9013df1ee6ab983b133"}}
+KERNEL_TRAFFIC = {"cfg4": {"bytes": 1004717312 + 6083840, "sources_sha256": "11b4a5a7776d9179f5c73cc0e4d701ce19e3257521c84568864f46954050e1ba"}}
 KERNEL_SOURCES = ("tc_fused.cu", "tc_common.cuh", "sm100_ptx.cuh")
 
 
