@@ -12,18 +12,19 @@ constexpr int kRsBins = 2048;        // 11-bit digits
 constexpr int kRsList = 1024;        // keys of the last digit that are ranked one by one
 constexpr int kRsMaxSmem = 200 * 1024;
 constexpr int kRsHalfSmem = 92 * 1024;   // dynamic shared memory of a block when two lie on an SM
+constexpr int kRsThirdSmem = 57 * 1024;  // ... and when three do
 
 // Sum of the indices of the Bp largest of each row's n values (ties to the lower index), all rows of the raw indicator.
 // What bounds it: the rows come once from HBM or L2; against that stand three walks over a row's keys in shared memory.
-// So two persistent blocks of 512 threads per SM, each a row at a time (one's synchronisations and its next row's way in are
+// So two persistent blocks of 512 threads per SM (three for rows up to 57 KB), each a row at a time (one's synchronisations and its next row's way in are
 // covered by the other's walks), rows past 92 KB in one block of 1024 (past 200 KB they are read again on every walk), and no
 // more than the walks that are needed: the extremes,
 // a histogram of 11-bit digits of the offsets from the smallest (about a thousand bins in use, so one histogram serves all
 // warps without contention), then the sum above the digit that holds the Bp-th largest while that digit's few keys are
 // listed and ranked, a key per warp.  1024 rows of 20011: 43.5 us with one block of 1024 threads and two rows in flight per SM
 // (10 k cycles per row, 3.6 k of them synchronisation), 39 us so, 35 with the short last walk.
-template <int kRsThreads, bool kHeld>   // kHeld false: no buffers, the keys are read from global memory on every walk
-__global__ void __launch_bounds__(kRsThreads, kRsThreads <= 512 ? 2 : 1)
+template <int kRsThreads, bool kHeld, int kRsBlocks>   // kHeld false: no buffers, the keys are read from global memory on every walk
+__global__ void __launch_bounds__(kRsThreads, kRsBlocks)
 row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buffers, unsigned long long* __restrict__ sums,
                 unsigned int* dev_status) {
   extern __shared__ __align__(16) uint4 rs_buf[];   // `buffers` rows of quads + 1
@@ -249,8 +250,9 @@ __global__ void window_params_kernel(const WindowArgs w, int* __restrict__ pool)
 }  // namespace
 
 cudaError_t adaptive_init() {
-  cudaError_t e = cudaFuncSetAttribute(row_sums_kernel<1024, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsMaxSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(row_sums_kernel<512, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsHalfSmem);
+  cudaError_t e = cudaFuncSetAttribute(row_sums_kernel<1024, true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsMaxSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(row_sums_kernel<512, true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsHalfSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(row_sums_kernel<512, true, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsThirdSmem);
   return e;
 }
 
@@ -267,14 +269,22 @@ WindowArgs window_args(const Problem& p, const Workspace& ws, int budget, float 
 cudaError_t launch_row_sums(const Problem& p, const Workspace& ws, int budget, int sm_count, unsigned int* dev_status, cudaStream_t st) {
   const int rows = p.batch * p.Hq * p.w, Bp = rows_counted(p, budget);
   const size_t room = ((size_t)(p.n + 3) / 4 + 1) * 16;
+  // Three blocks per SM where the rows are short enough and more than two would take at once: a row's synchronisations are then covered
+  // by two others' walks (3 sequences of 6000 rows, 3072 of indicators, 125.6 -> 118.6 us; one sequence of 8192 or 11000 75.5 -> 74.7 and
+  // 85.9 -> 84.8).
+  if (room <= (size_t)kRsThirdSmem && rows > 2 * sm_count) {
+    const int buffers = 2 * room <= (size_t)kRsThirdSmem ? 2 : 1;
+    return launch_chained(row_sums_kernel<512, true, 3>, dim3((unsigned int)(rows < 3 * sm_count ? rows : 3 * sm_count)), 512, buffers * room, st,
+                          rows, p.n, Bp, ws.I_raw, buffers, ws.adaptive_sums, dev_status);
+  }
   if (room <= (size_t)kRsHalfSmem) {
     const int buffers = 2 * room <= (size_t)kRsHalfSmem ? 2 : 1;
-    return launch_chained(row_sums_kernel<512, true>, dim3((unsigned int)(rows < 2 * sm_count ? rows : 2 * sm_count)), 512, buffers * room, st,
+    return launch_chained(row_sums_kernel<512, true, 2>, dim3((unsigned int)(rows < 2 * sm_count ? rows : 2 * sm_count)), 512, buffers * room, st,
                           rows, p.n, Bp, ws.I_raw, buffers, ws.adaptive_sums, dev_status);
   }
   const bool held = room <= (size_t)kRsMaxSmem;
   const int buffers = 2 * room <= (size_t)kRsMaxSmem ? 2 : held ? 1 : 0;
-  return launch_chained(held ? row_sums_kernel<1024, true> : row_sums_kernel<1024, false>, dim3((unsigned int)(rows < sm_count ? rows : sm_count)), 1024,
+  return launch_chained(held ? row_sums_kernel<1024, true, 1> : row_sums_kernel<1024, false, 1>, dim3((unsigned int)(rows < sm_count ? rows : sm_count)), 1024,
                         buffers * room, st, rows, p.n, Bp, ws.I_raw, buffers, ws.adaptive_sums, dev_status);
 }
 
