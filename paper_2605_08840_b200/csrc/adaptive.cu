@@ -16,8 +16,8 @@ constexpr int kRsThirdSmem = 57 * 1024;  // ... and when three do
 
 // Sum of the indices of the Bp largest of each row's n values (ties to the lower index), all rows of the raw indicator.
 // What bounds it: the rows come once from HBM or L2; against that stand three walks over a row's keys in shared memory.
-// So two persistent blocks of 512 threads per SM (three for rows up to 57 KB), each a row at a time (one's synchronisations and its next row's way in are
-// covered by the other's walks), rows past 92 KB in one block of 1024 (past 200 KB they are read again on every walk), and no
+// So two persistent blocks of 512 threads per SM (three for rows up to 57 KB), each a row at a time (one's synchronisations and its
+// next row's way in are covered by the others' walks), rows past 92 KB in one block of 1024 (past 200 KB they are read again on every walk), and no
 // more than the walks that are needed: the extremes,
 // a histogram of 11-bit digits of the offsets from the smallest (about a thousand bins in use, so one histogram serves all
 // warps without contention), then the sum above the digit that holds the Bp-th largest while that digit's few keys are

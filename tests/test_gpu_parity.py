@@ -531,6 +531,12 @@ def test_adaptive_window_row_lengths(handle, spec):
     assert np.array_equal(run.pool_used.cpu().numpy()[settled], ref.pool[settled])
 
 
+@pytest.mark.parametrize("spec", [(7292, 300, 25), (7293, 300, 13), (14588, 500, 25), (14589, 500, 13)])
+def test_adaptive_window_three_blocks(handle, spec):
+    """Rows on either side of what two buffers (7292 keys) and one (14588) of three blocks per SM take, more of them than blocks."""
+    test_adaptive_window_row_lengths(handle, spec)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("spec", [(3, 2), (7, 3), (1023, 40), (2049, 1500), (4099, 4098), (25001, 900), (26000, 14000), (51300, 2000),
                                   (11773, 1500, 3), (20011, 11000, 26)])
