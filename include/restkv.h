@@ -224,11 +224,11 @@ restkv_status restkv_decode(restkv_handle* h, const restkv_shape* shape, const v
  *    splits as fit (at most 64), so very wide batches run with fewer splits than restkv_decode would use.
  *  - Every GPU that loads the library carries the 2 MiB until the process exits.
  *  - The first call on each device looks up the array's device address (cudaGetSymbolAddress, with that
- *    device current) and remembers it; make that first call outside any stream capture.  With CUDA's lazy
- *    module loading that first call is also the moment the driver places the module, array included, in
- *    device memory: a host that hands all device memory to its own pool must make one call (any small
- *    shape) BEFORE it does so, or the first call can fail with RESTKV_ERR_CUDA (out of memory);
- *    restkv_decode_static_last_cuda_error() then returns the cudaError_t.
+ *    device current), has the driver load every kernel that a later call of any shape can launch (with CUDA's lazy
+ *    loading that, and placing the module with the array, is where device memory is taken), and remembers both; make
+ *    that first call outside any stream capture.  A host that hands all device memory to its own pool must make one
+ *    call (any small shape) BEFORE it does so, or the first call can fail with RESTKV_ERR_CUDA (out of memory);
+ *    restkv_decode_static_last_cuda_error() then returns the cudaError_t.  Later calls take no device memory.
  *  - All calls on a device share the one array.  A call overwrites every slot it later reads, so nothing from
  *    an earlier call leaks into a result; but two calls whose kernels overlap on the GPU (different streams,
  *    no ordering between them) race on it.  Order them on one stream or with events.

@@ -186,45 +186,65 @@ __global__ void decode_combine_kernel(int Hq, int G, int d, int splits, const fl
   if (lse && threadIdx.x == 0) lse[(long long)b * Hq + hq] = mm + logf(ll);
 }
 
+template <typename T>
+using PartialKernel = void (*)(int, int, int, int, float, const T*, const T*, const T*, float*, int);
+
+// The instantiation for rows of `chunks` 16-byte chunks; null if there is none (head_dim is 256 at most, so that only fp32 rows
+// have 64 chunks).  One chunk per lane where the row allows it: few registers per thread, several CTAs per SM.
 template <typename T, int G>
-cudaError_t launch_partial(const Problem& p, const void* q, const void* Kc, const void* Vc, int n_rows, float* part,
-                           int splits, cudaStream_t st) {
-  constexpr int E = Chunk<T>::kElems;
-  dim3 grid(splits, p.BH);
-  const int chunks = p.d / E;   // 16-byte chunks per row
-  const size_t smem = (size_t)(kDecThreads / 32) * G * (p.d + 2) * sizeof(float);
-#define RESTKV_DEC(LPR, CPL)                                                                                    \
-  do {                                                                                                          \
-    if (smem > 48 * 1024) {                                                                                     \
-      cudaError_t e_ = cudaFuncSetAttribute(decode_partial_kernel<T, G, LPR, CPL>,                              \
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);            \
-      if (e_ != cudaSuccess) return e_;                                                                         \
-    }                                                                                                           \
-    decode_partial_kernel<T, G, LPR, CPL><<<grid, kDecThreads, smem, st>>>(                                     \
-        p.Hq, p.Hkv, p.d, n_rows, p.scale, (const T*)q, (const T*)Kc, (const T*)Vc, part, splits);              \
-  } while (0)
-  // one 16-byte chunk per lane where the row allows it: few registers per thread, several CTAs per SM
-  if (chunks == 8) RESTKV_DEC(8, 1);
-  else if (chunks == 16) RESTKV_DEC(16, 1);
-  else if (chunks == 32) RESTKV_DEC(32, 1);
-  else if (chunks == 64) RESTKV_DEC(32, 2);
-  else if (chunks == 4) RESTKV_DEC(4, 1);
-  else if (chunks == 2) RESTKV_DEC(2, 1);
-  else return cudaErrorInvalidValue;
-#undef RESTKV_DEC
-  return cudaGetLastError();
+PartialKernel<T> pick_partial(int chunks) {
+  switch (chunks) {
+    case 2: return decode_partial_kernel<T, G, 2, 1>;
+    case 4: return decode_partial_kernel<T, G, 4, 1>;
+    case 8: return decode_partial_kernel<T, G, 8, 1>;
+    case 16: return decode_partial_kernel<T, G, 16, 1>;
+    case 32: return decode_partial_kernel<T, G, 32, 1>;
+    case 64:
+      if constexpr (sizeof(T) == 4) return decode_partial_kernel<T, G, 32, 2>;
+      return nullptr;
+    default: return nullptr;
+  }
 }
 
 template <typename T>
-cudaError_t launch_partial_g(const Problem& p, const void* q, const void* Kc, const void* Vc, int n_rows, float* part,
-                             int splits, cudaStream_t st) {
-  switch (p.G) {
-    case 1: return launch_partial<T, 1>(p, q, Kc, Vc, n_rows, part, splits, st);
-    case 2: return launch_partial<T, 2>(p, q, Kc, Vc, n_rows, part, splits, st);
-    case 4: return launch_partial<T, 4>(p, q, Kc, Vc, n_rows, part, splits, st);
-    case 8: return launch_partial<T, 8>(p, q, Kc, Vc, n_rows, part, splits, st);
-    default: return cudaErrorInvalidValue;
+PartialKernel<T> pick_partial_g(int G, int chunks) {
+  switch (G) {
+    case 1: return pick_partial<T, 1>(chunks);
+    case 2: return pick_partial<T, 2>(chunks);
+    case 4: return pick_partial<T, 4>(chunks);
+    case 8: return pick_partial<T, 8>(chunks);
+    default: return nullptr;
   }
+}
+
+template <typename T>
+cudaError_t launch_partial(const Problem& p, const void* q, const void* Kc, const void* Vc, int n_rows, float* part,
+                           int splits, cudaStream_t st) {
+  const PartialKernel<T> kernel = pick_partial_g<T>(p.G, p.d / Chunk<T>::kElems);
+  if (!kernel) return cudaErrorInvalidValue;
+  const size_t smem = (size_t)(kDecThreads / 32) * p.G * (p.d + 2) * sizeof(float);
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  kernel<<<dim3(splits, p.BH), kDecThreads, smem, st>>>(p.Hq, p.Hkv, p.d, n_rows, p.scale, (const T*)q, (const T*)Kc, (const T*)Vc,
+                                                        part, splits);
+  return cudaGetLastError();
+}
+
+// Has the driver place the code of every instantiation in the current device's memory.  CUDA loads a kernel when it is first
+// used, and takes another 2 MiB of device memory for it when the code loaded before fills what it holds.
+template <typename T>
+cudaError_t load_partial_kernels() {
+  const int heads[] = {1, 2, 4, 8}, chunks[] = {2, 4, 8, 16, 32, 64};
+  for (int G : heads)
+    for (int c : chunks)
+      if (const PartialKernel<T> kernel = pick_partial_g<T>(G, c)) {
+        cudaFuncAttributes attributes;
+        const cudaError_t e = cudaFuncGetAttributes(&attributes, kernel);
+        if (e != cudaSuccess) return e;
+      }
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -232,11 +252,19 @@ cudaError_t launch_partial_g(const Problem& p, const void* q, const void* Kc, co
 cudaError_t launch_decode(const Problem& p, const void* q, const void* Kc, const void* Vc, int n_rows, float* out,
                           float* lse, float* part, int splits, cudaStream_t st, int* n_launches) {
   cudaError_t e = (p.dtype == RESTKV_BF16)
-                      ? launch_partial_g<__nv_bfloat16>(p, q, Kc, Vc, n_rows, part, splits, st)
-                      : launch_partial_g<float>(p, q, Kc, Vc, n_rows, part, splits, st);
+                      ? launch_partial<__nv_bfloat16>(p, q, Kc, Vc, n_rows, part, splits, st)
+                      : launch_partial<float>(p, q, Kc, Vc, n_rows, part, splits, st);
   if (e != cudaSuccess) return e;
   *n_launches = 2;
   return launch_decode_combine(p, part, splits, out, lse, st);
+}
+
+static cudaError_t load_decode_kernels() {
+  cudaFuncAttributes attributes;
+  cudaError_t e = cudaFuncGetAttributes(&attributes, decode_combine_kernel);
+  if (e == cudaSuccess) e = load_partial_kernels<__nv_bfloat16>();
+  if (e == cudaSuccess) e = load_partial_kernels<float>();
+  return e;
 }
 
 cudaError_t launch_decode_combine(const Problem& p, const float* part, int splits, float* out, float* lse, cudaStream_t st) {
@@ -305,7 +333,8 @@ int g_static_sm_count[kMaxDevices];
 int g_static_last_cuda_error = 0;
 
 // In host code `g_static_decode_scratch` only names the symbol; the address a kernel can use comes from the
-// runtime, for the device that is current.
+// runtime, for the device that is current.  The first time on a device everything that later calls can launch is loaded there, too:
+// a call after that takes no device memory, whatever its shape.
 cudaError_t static_scratch_for_current_device(float** ptr, int* sm_count) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -315,6 +344,8 @@ cudaError_t static_scratch_for_current_device(float** ptr, int* sm_count) {
   if (!g_static_scratch_addr[dev]) {
     void* addr = nullptr;
     e = cudaGetSymbolAddress(&addr, g_static_decode_scratch);
+    if (e != cudaSuccess) return e;
+    e = load_decode_kernels();
     if (e != cudaSuccess) return e;
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -8,6 +8,10 @@ row with different inputs (the shared array keeps the previous call's contents, 
 that the amount of free device memory does not move across a call, and that shapes beyond the array's capacity are
 refused.  It is collected last on purpose.
 """
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -71,6 +75,67 @@ def test_static_decode_matches_oracle_and_decode_on_calls_in_a_row():
         np.testing.assert_allclose(lse.cpu().numpy(), ref_lse.cpu().numpy(), rtol=1e-5, atol=1e-5)
     assert handle.poll_status() == rk.RESTKV_OK
     handle.close()
+
+
+# Run in a process of its own, whose first call decides what is loaded.  Small modules of another origin are loaded until the driver
+# takes memory for them, twice, and then as many as lay between the two but two: what the driver holds for code is nearly full,
+# and the first kernel that still had to be loaded would make it take more.
+LATER_CALLS = r"""
+import torch
+from cuda.bindings import driver
+from paper_2605_08840_b200 import binding as rk
+
+PTX = b'''\
+.version 7.0
+.target sm_80
+.address_size 64
+.visible .entry fill(.param .u64 p) { .reg .u64 a; ld.param.u64 a, [p]; cvta.to.global.u64 a, a; st.global.u32 [a], 1; ret; }
+\0'''
+CHUNKS = {"bf16": (2, 4, 8, 16, 32), "f32": (2, 4, 8, 16, 32, 64)}   # 16-byte chunks of a row
+
+def call(G, dim, dtype):
+    t = torch.bfloat16 if dtype == "bf16" else torch.float32
+    q, K, V = (torch.zeros(s, dtype=t, device="cuda") for s in ((1, G, dim), (1, 1, 300, dim), (1, 1, 300, dim)))
+    shape = rk.make_shape(1, G, 1, dim, 300, 1, 0, rk.BF16 if dtype == "bf16" else rk.F32)
+    return shape, q, K, V, 300, torch.zeros(1, G, dim, device="cuda")
+
+def load():
+    err, module = driver.cuModuleLoadData(PTX)
+    assert int(err) == 0, err
+    err, function = driver.cuModuleGetFunction(module, b"fill")
+    assert int(err) == 0, err
+    assert int(driver.cuFuncLoad(function)[0]) == 0
+
+def free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+calls = [call(G, c * (8 if t == "bf16" else 4), t) for t in CHUNKS for G in (1, 2, 4, 8) for c in CHUNKS[t]]
+rk.decode_static(*calls[0])
+loaded, steps, last = 0, [], free()
+while len(steps) < 2:
+    load()
+    loaded += 1
+    assert loaded < 20000
+    if free() != last:
+        steps, last = steps + [loaded], free()
+for _ in range(steps[1] - steps[0] - 2):
+    load()
+assert free() == last, "the driver took memory out of step"
+for args in calls:
+    rk.decode_static(*args)
+    assert free() == last, "device memory taken by %d query heads, head_dim %d, dtype %d" % (
+        args[0].n_q_heads, args[0].head_dim, args[0].dtype)
+print("no device memory taken by %d shapes" % len(calls))
+"""
+
+
+def test_static_decode_loads_its_kernels_in_the_first_call():
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = {k: v for k, v in os.environ.items() if k != "CUDA_MODULE_LOADING"}
+    res = subprocess.run([sys.executable, "-c", LATER_CALLS], cwd=root, env=env, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0, res.stdout + res.stderr
+    assert "no device memory taken by 44 shapes" in res.stdout
 
 
 def test_static_decode_refuses_what_does_not_fit():
