@@ -748,8 +748,9 @@ __device__ __forceinline__ void half_terms(const Ctx& cx, int it, int row0) {
   }
   __syncwarp();
   if (cx.lane == 0) {
-    mbar_arrive(&cx.B->kv_empty[it & 1]);
+    // in this order: once the slot is free the other warp can be at tile it + 2, whose arrival must not count for this tile
     mbar_arrive(&cx.B->acc_full[it & 1]);
+    mbar_arrive(&cx.B->kv_empty[it & 1]);
   }
 }
 

@@ -82,3 +82,35 @@ def test_product_does_not_import_the_oracle():
         if f.endswith((".py", ".c")):
             src = open(os.path.join(ROOT, "oracle", f)).read()
             assert "paper_2605_08840_b200" not in src and "librestkv.so" not in src, f
+
+
+def test_accumulator_phases_take_arrivals_of_their_own_tile_only():
+    """Score kernel from given statistics: a stage's kv_empty and acc_full count three arrivals a tile, of the two warps that sum
+    ||v||^2 and of the products' commit.  Every order in which the roles can run, with the warps' two arrivals in the order that the
+    source has them: no arrival may count for another tile than its own."""
+    source = open(os.path.join(ROOT, "paper_2605_08840_b200", "csrc", "tc_fused.cu")).read()
+    body = source[source.index("void half_terms("):]
+    order = re.findall(r"mbar_arrive\(&cx\.B->(\w+)\[", body[:body.index("\n}\n")])
+    assert sorted(order) == ["acc_full", "kv_empty"]
+    tiles = 3                                      # of one stage
+    helper = [(t, bar) for t in range(tiles) for bar in order]
+    commit = [(t, bar) for t in range(tiles) for bar in ("acc_full", "kv_empty")]
+    seen, todo = set(), [(0, 0, 0)]                # operations that the two warps and the issuing thread have done
+    while todo:
+        state = todo.pop()
+        if state in seen:
+            continue
+        seen.add(state)
+        done = [op for ops, n in zip((helper, helper, commit), state) for op in ops[:n]]
+        phase = {bar: sum(1 for _, b in done if b == bar) // 3 for bar in ("acc_full", "kv_empty")}
+        for role, ops in enumerate((helper, helper, commit)):
+            if state[role] == len(ops):
+                continue
+            tile, bar = ops[state[role]]
+            # the stage holds the tile once kv_empty has let the loader refill it; the products also want the epilogue to have
+            # read the accumulators of the tile before
+            if phase["kv_empty"] < tile or (role == 2 and phase["acc_full"] < tile):
+                continue
+            assert phase[bar] == tile, "an arrival of tile %d counts for tile %d of %s" % (tile, phase[bar], bar)
+            todo.append(tuple(n + (r == role) for r, n in enumerate(state)))
+    assert (len(helper), len(helper), len(commit)) in seen
