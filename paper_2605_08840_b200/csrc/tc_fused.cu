@@ -754,8 +754,8 @@ __device__ __forceinline__ void half_terms(const Ctx& cx, int it, int row0) {
   }
 }
 
-// Terms per token under the projection: one of each query head (which has no instantiation in use with w below 32).
-template <int kW> constexpr int kTerms = kRows / (kW < 32 ? 32 : kW);
+// Terms per token under the projection: one of each query head.
+template <int kW> constexpr int kTerms = kRows / kW;
 
 // Warp 2 in phase C: what the epilogue needs to know of a tile beside the accumulators, told with their barrier, so that the
 // sixteen epilogue warps spend neither loads nor registers nor the wait for them on it.
@@ -1203,6 +1203,7 @@ template <int kW, bool kLse, int kInd>
 __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, int bh, int tile0, int T) {
   constexpr int kG = kRows / kW;
   constexpr bool kEq7 = kInd == 0 || kInd == 3, kProj = kInd == 3;
+  static_assert(!kProj || kW >= 32, "a warpgroup's columns belong to one query head");
   FusedBars* B = cx.B;
   int* abort_flag = cx.abort_flag;
   unsigned int* dev_status = a.dev_status;
@@ -1716,13 +1717,17 @@ using FusedKernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap,
 
 template <int kW>
 static FusedKernel pick_fused_w(bool from_lse, int indicator) {
+  if (indicator == 3) {
+    // (below 32 a warpgroup's 32 columns belong to several query heads, each with a term of its own; the kernel that computes the
+    // terms takes four heads at most)
+    if constexpr (kW >= 32) return from_lse ? tc_fused_kernel<kW, true, 3> : tc_fused_kernel<kW, false, 3>;
+    return nullptr;
+  }
   if (from_lse) {
     if (indicator == 0) return tc_fused_kernel<kW, true, 0>;
-    if (indicator == 3) return tc_fused_kernel<kW, true, 3>;
     return indicator == 1 ? tc_fused_kernel<kW, true, 1> : tc_fused_kernel<kW, true, 2>;
   }
   if (indicator == 0) return tc_fused_kernel<kW, false, 0>;
-  if (indicator == 3) return tc_fused_kernel<kW, false, 3>;
   return indicator == 1 ? tc_fused_kernel<kW, false, 1> : tc_fused_kernel<kW, false, 2>;
 }
 
@@ -1746,6 +1751,7 @@ cudaError_t tc_fused_init() {
     for (int lse = 0; lse < 2; ++lse)
       for (int ind = 0; ind < 4; ++ind) {
         FusedKernel kernel = pick_fused(w, lse != 0, ind);
+        if (!kernel) continue;
         if (e == cudaSuccess) e = check_launch_regs(kernel);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFSmem);
       }
