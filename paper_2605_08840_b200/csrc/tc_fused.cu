@@ -739,18 +739,22 @@ __device__ __forceinline__ float* second_head(const FusedArgs& a, int bh) {
   return a.tile_max + (long long)bh * ((a.n_kv + kTile - 1) / kTile) * kTile;
 }
 
-// ||v||^2 of rows [row0, row0 + 64) of the V tile of phase C's tile `it`, by one warp.
-__device__ __forceinline__ void half_terms(const Ctx& cx, int it, int row0) {
+// Warps 2 and 3 in phase C from given statistics: ||v||^2 of rows [row0, row0 + 64) of every tile's V, by one warp.
+__device__ __forceinline__ void half_terms(const Ctx& cx, const FusedArgs& a, int T, int row0) {
+  bool ok = true;
+  for (int it = 0; it < T; ++it) {
+    ok = ok && mbar_wait(&cx.B->kv_full[it & 1], (uint32_t)(it >> 1) & 1u, cx.abort_flag, a.dev_status, kDevTimeout, a.wait_limit);
 #pragma unroll 1
-  for (int rr = 0; rr < 2; ++rr) {
-    const int row = row0 + rr * 32 + cx.lane;
-    cx.vn_s[(it & 3) * kTile + row] = row_square_sum(cx.smem_base + k_slot_off(2 * (it & 1)) + kTileBytes, row);
-  }
-  __syncwarp();
-  if (cx.lane == 0) {
-    // in this order: once the slot is free the other warp can be at tile it + 2, whose arrival must not count for this tile
-    mbar_arrive(&cx.B->acc_full[it & 1]);
-    mbar_arrive(&cx.B->kv_empty[it & 1]);
+    for (int rr = 0; rr < 2; ++rr) {
+      const int row = row0 + rr * 32 + cx.lane;
+      cx.vn_s[(it & 3) * kTile + row] = row_square_sum(cx.smem_base + k_slot_off(2 * (it & 1)) + kTileBytes, row);
+    }
+    __syncwarp();
+    if (cx.lane == 0) {
+      // in this order: once the slot is free the other warp can be at tile it + 2, whose arrival must not count for this tile
+      mbar_arrive(&cx.B->acc_full[it & 1]);
+      mbar_arrive(&cx.B->kv_empty[it & 1]);
+    }
   }
 }
 
@@ -759,8 +763,7 @@ template <int kW> constexpr int kTerms = kRows / kW;
 
 // Warp 2 in phase C: what the epilogue needs to know of a tile beside the accumulators, told with their barrier, so that the
 // sixteen epilogue warps spend neither loads nor registers nor the wait for them on it.
-//   - the tokens' own terms: ||v||^2 as phase A has left it (under the projection v^T Mt v of each query head); from given statistics
-//     from the V tile in shared memory, of which warp 3 takes the second half;
+//   - the tokens' own terms: ||v||^2 as phase A has left it, under the projection v^T Mt v of each query head;
 //   - whether the logits need to be looked at: some row's largest logit reaches that row's M2 - log2(1 / kHeavyA).
 template <int kW, bool kLse, int kInd>
 __device__ void stage_terms(const Ctx& cx, const FusedArgs& a, int bh, int tile0, int T) {
@@ -769,13 +772,6 @@ __device__ void stage_terms(const Ctx& cx, const FusedArgs& a, int bh, int tile0
   FusedBars* B = cx.B;
   const int lane = cx.lane;
   bool ok = true;
-  if (kLse && !kProj) {
-    for (int it = 0; it < T; ++it) {
-      ok = ok && mbar_wait(&B->kv_full[it & 1], (uint32_t)(it >> 1) & 1u, cx.abort_flag, a.dev_status, kDevTimeout, a.wait_limit);
-      half_terms(cx, it, 0);
-    }
-    return;
-  }
   const int nt_all = (a.n_kv + kTile - 1) / kTile;
   const float* tm = a.tile_max + ((long long)bh * nt_all + tile0) * kRows + lane;
   const float* terms = (kProj ? a.vmv : a.vnorm) + (long long)bh * kG * a.n_kv + tile0 * kTile + lane;
@@ -858,13 +854,6 @@ __device__ void join_tiles(const Ctx& cx, const FusedArgs& a, int bh, int tile0,
   const int lane = cx.lane;
   const bool group_max = a.group_max != 0;
   bool ok = true;
-  if (kLse && kInd != 3) {
-    for (int it = 0; it < T; ++it) {
-      ok = ok && mbar_wait(&B->kv_full[it & 1], (uint32_t)(it >> 1) & 1u, cx.abort_flag, a.dev_status, kDevTimeout, a.wait_limit);
-      half_terms(cx, it, 64);
-    }
-    return;
-  }
 #pragma unroll 1
   for (int it = 0; it < T + 2; ++it) {
     const int s = it & 1;
@@ -901,7 +890,7 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
   int* abort_flag = cx.abort_flag;
   unsigned int* dev_status = a.dev_status;
   const int b = bh / a.Hkv, h = bh % a.Hkv;
-  const int warp = cx.warp, lane = cx.lane;
+  const int warp = cx.warp;
   const uint32_t tmem = cx.tmem;   // buffer s: S' at s*256, C' at s*256 + 128
 
   if (warp == 0) {
@@ -947,6 +936,8 @@ __device__ void phase_c_control(const Ctx& cx, const FusedArgs& a, const CUtenso
         umma_commit(&B->kv_empty[s]);
       }
     }
+  } else if constexpr (kLse && kInd != 3) {
+    half_terms(cx, a, T, (warp - 2) * 64);
   } else if (warp == 2) {
     stage_terms<kW, kLse, kInd>(cx, a, bh, tile0, T);
   } else {
