@@ -1,6 +1,7 @@
 // Adaptive window parameters (Eq. 10-12): D_front / D_rear are the mean indices of the per-query
 // top-B rows of the raw indicator over the first and second half of the window queries; the box
 // width and shift follow from their difference.
+#include "index_sum.cuh"
 #include "restkv_common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -170,12 +171,7 @@ row_sums_kernel(int rows, int n, int Bp, const float* __restrict__ src, int buff
     for (int q = q0 + tid; q < q1; q += kRsThreads) {
       const uint4 k4 = quad[q];
       const unsigned int i = (unsigned int)(4 * q - mis);
-      unsigned int part = 0u;   // (rows are shorter than 2^30)
-      if (k4.x > k1) part += i;
-      if (k4.y > k1) part += i + 1u;
-      if (k4.z > k1) part += i + 2u;
-      if (k4.w > k1) part += i + 3u;
-      isum += part;
+      add_indices_above<kHeld>(isum, i, k4.x, k4.y, k4.z, k4.w, k1);   // (rows that shared memory holds are short)
       if (!ties && ((k4.x - k0 <= span) | (k4.y - k0 <= span) | (k4.z - k0 <= span) | (k4.w - k0 <= span))) {
         list_key(i, k4.x);
         list_key(i + 1, k4.y);

@@ -3,6 +3,7 @@ header declares; argument validation that needs no GPU; the binding fails loudly
 import ctypes
 import os
 import re
+import subprocess
 
 import pytest
 
@@ -114,3 +115,33 @@ def test_accumulator_phases_take_arrivals_of_their_own_tile_only():
             assert phase[bar] == tile, "an arrival of tile %d counts for tile %d of %s" % (tile, phase[bar], bar)
             todo.append(tuple(n + (r == role) for r, n in enumerate(state)))
     assert (len(helper), len(helper), len(commit)) in seen
+
+
+def test_index_sums_of_the_longest_rows(tmp_path):
+    """The sum of the indices whose keys lie above a limit, at both ends of the indices
+    that a row of up to 2^31 - 1 keys has, or one of up to 2^30."""
+    source = tmp_path / "sums.cc"
+    source.write_text("""
+#include <cstdio>
+#include <initializer_list>
+#include "index_sum.cuh"
+template <bool kShort>
+void print(unsigned int i) {
+  for (unsigned int m = 0; m < 16; ++m) {
+    unsigned long long sum = 5;
+    restkv::add_indices_above<kShort>(sum, i, 7 + (m & 1), 7 + (m >> 1 & 1), 7 + (m >> 2 & 1), 7 + (m >> 3), 7);
+    std::printf("%u %u %llu\\n", i, m, sum);
+  }
+}
+int main() {
+  for (unsigned int i : {0u, 1u, (1u << 30) - 4u}) print<true>(i);
+  for (unsigned int i : {0u, 1u, (1u << 30) - 4u, (1u << 30) - 1u, 1u << 30, 0x7FFFFFF8u, 0x7FFFFFFBu}) print<false>(i);
+}
+""")
+    program = tmp_path / "sums"
+    subprocess.run(["g++", "-std=c++17", "-I", rk_build.CSRC, "-o", str(program), str(source)], check=True)
+    lines = subprocess.run([str(program)], check=True, capture_output=True, text=True).stdout.split("\n")[:-1]
+    assert len(lines) == 10 * 16
+    for line in lines:
+        i, m, total = (int(x) for x in line.split())
+        assert total == 5 + sum(i + k for k in range(4) if m >> k & 1), line
