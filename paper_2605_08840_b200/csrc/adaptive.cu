@@ -273,11 +273,10 @@ cudaError_t launch_row_sums(const Problem& p, const Workspace& ws, int budget, i
     return launch_chained(row_sums_kernel<512, true, 3>, dim3((unsigned int)(rows < 3 * sm_count ? rows : 3 * sm_count)), 512, buffers * room, st,
                           rows, p.n, Bp, ws.I_raw, buffers, ws.adaptive_sums, dev_status);
   }
-  if (room <= (size_t)kRsHalfSmem) {
-    const int buffers = 2 * room <= (size_t)kRsHalfSmem ? 2 : 1;
-    return launch_chained(row_sums_kernel<512, true, 2>, dim3((unsigned int)(rows < 2 * sm_count ? rows : 2 * sm_count)), 512, buffers * room, st,
-                          rows, p.n, Bp, ws.I_raw, buffers, ws.adaptive_sums, dev_status);
-  }
+  // (one buffer: rows that two would fit are here only where each block has a single row)
+  if (room <= (size_t)kRsHalfSmem)
+    return launch_chained(row_sums_kernel<512, true, 2>, dim3((unsigned int)(rows < 2 * sm_count ? rows : 2 * sm_count)), 512, room, st,
+                          rows, p.n, Bp, ws.I_raw, 1, ws.adaptive_sums, dev_status);
   const bool held = room <= (size_t)kRsMaxSmem;
   const int buffers = 2 * room <= (size_t)kRsMaxSmem ? 2 : held ? 1 : 0;
   return launch_chained(held ? row_sums_kernel<1024, true, 1> : row_sums_kernel<1024, false, 1>, dim3((unsigned int)(rows < sm_count ? rows : sm_count)), 1024,

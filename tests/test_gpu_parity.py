@@ -509,9 +509,8 @@ def test_selection_kernel_edges(handle, spec):
                                   (1023, 40, 30), (11772, 900), (11773, 900, 25), (23548, 900, 25), (23549, 900), (25001, 900, 13),
                                   (51300, 2000, 7)])
 def test_adaptive_window_row_lengths(handle, spec):
-    """The index sums behind the adaptive window: rows that begin anywhere within 16 bytes, of a few keys, with two buffers and
-    one in small blocks (to 11772 and 23548 keys), two, one and none in large ones (to 25596 and 51196 keys and beyond), and more
-    rows than there are blocks, so that a block's buffers are filled again."""
+    """The index sums behind the adaptive window: rows that begin anywhere within 16 bytes, of a few keys, in small blocks (to 23548
+    keys), with two buffers, one and none in large ones (to 25596 and 51196 keys and beyond)."""
     n, budget = spec[:2]
     batch = spec[2] if len(spec) > 2 else 1
     for seed in range(n, n + 20):   # (of a few keys, front and rear may keep the same ones)
