@@ -530,10 +530,17 @@ def test_adaptive_window_row_lengths(handle, spec):
     assert np.array_equal(run.pool_used.cpu().numpy()[settled], ref.pool[settled])
 
 
-@pytest.mark.parametrize("spec", [(7292, 300, 25), (7293, 300, 13), (14588, 500, 25), (14589, 500, 13)])
-def test_adaptive_window_three_blocks(handle, spec):
-    """Rows on either side of what two buffers (7292 keys) and one (14588) of three blocks per SM take, more of them than blocks."""
-    test_adaptive_window_row_lengths(handle, spec)
+@pytest.mark.parametrize("spec", [(1023, 40, 6), (7292, 300, 6), (7293, 300, 3), (14588, 500, 3), (14589, 500, 2), (23548, 900, 2),
+                                  (23549, 900, 2), (25596, 900, 2), (25597, 900, 1), (51196, 900, 1)])
+def test_adaptive_window_buffers_are_filled_again(handle, spec):
+    """Rows of either side of each limit (two buffers and one of three blocks per SM to 7292 and 14588 keys, one of two blocks to 23548,
+    two and one of a single block to 25596 and 51196), a few more of them than the device has buffers, so that each kind is filled again."""
+    import torch
+    n, budget, buffers_per_sm = spec
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    batch = buffers_per_sm * sms // 24 + 1   # 24 rows of indicators a sequence
+    assert 24 * batch > buffers_per_sm * sms
+    test_adaptive_window_row_lengths(handle, (n, budget, batch))
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
