@@ -530,6 +530,13 @@ def test_adaptive_window_row_lengths(handle, spec):
     assert np.array_equal(run.pool_used.cpu().numpy()[settled], ref.pool[settled])
 
 
+@pytest.mark.parametrize("spec", [(7292, 300, 25), (7293, 300, 13), (14588, 500, 25), (14589, 500, 13)])
+def test_adaptive_window_three_blocks(handle, spec):
+    """Rows on either side of what two buffers (7292 keys) and one (14588) of three blocks per SM take, a row or two to
+    a block."""
+    test_adaptive_window_row_lengths(handle, spec)
+
+
 @pytest.mark.parametrize("spec", [(1023, 40, 6), (7292, 300, 6), (7293, 300, 3), (14588, 500, 3), (14589, 500, 2), (23548, 900, 2),
                                   (23549, 900, 2), (25596, 900, 2), (25597, 900, 1), (51196, 900, 1)])
 def test_adaptive_window_buffers_are_filled_again(handle, spec):
