@@ -493,6 +493,13 @@ def test_fp32_pass2_rows_per_thread(handle, heads_w, n):
     full_check(handle, make_inputs(Case("rows", 1, 2 * group, 2, 64, n, w, min(n, 100), 5, 0, 0.9, "f32", 0, "normal", group * w + n)))
 
 
+@pytest.mark.parametrize("spec", [(1, 20000), (2, 9601), (4, 4737), (5, 4000)])
+def test_merge_of_many_partials(handle, spec):
+    """148, 74, 37 and 29 partials a head, all of them with rows: five, three, two and one for each lane that weighs them."""
+    heads, n = spec
+    full_check(handle, make_inputs(Case("partials", 1, 4 * heads, heads, 128, n, 32, 200, 5, 0, 0.9, "bf16", 0, "planted", n)))
+
+
 # ------------------------------------------------------------------ unit: select, compact, decode
 @pytest.mark.parametrize("spec", [(1, 1, 1, 1), (1, 31, 7, 5), (2, 255, 254, 7), (3, 1025, 40, 33), (2, 8160, 3000, 7), (2, 8161, 3000, 5),
                                   (20, 8161, 77, 7), (40, 9000, 700, 3), (160, 1500, 64, 7), (150, 26001, 100, 5),
