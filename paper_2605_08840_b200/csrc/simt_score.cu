@@ -547,16 +547,25 @@ cudaError_t pass2(const Problem& p, const Workspace& ws, const void* Q, const vo
   // do not fit shared memory (8 were slower even for 1024 rows of 2 heads, one block per SM: 33.8 against 28.6 us)
   const bool wide = (long long)(p.n + 31) / 32 * p.BH >= 296 && floats(32, 64, 64) * sizeof(float) <= 220 * 1024;
   const int tb = wide ? 32 : 16;
-  // four rows per thread where there are more than 64 (fewer would leave half a step to do for nothing) and two blocks of a step of
-  // 128 fit an SM: 1500 rows of 2 heads 33.4 -> 32.4 us, 1024 rows no difference; not with 32 tokens, whose 16 pairs per thread take
-  // the registers of the second block on the SM (4 sequences of 5000 rows 164 -> 191 us)
-  const bool tall = !wide && p.R > 64 && floats(tb, 128, 128) * sizeof(float) <= 110 * 1024;
-  const int step = tall ? 128 : 64, all = (p.R + step - 1) / step * step;
+  const dim3 grid((p.n + tb - 1) / tb, p.BH);
+  const long long blocks = (long long)grid.x * grid.y;
   // all rows of Q and O stay in shared memory where two blocks of that size fit an SM
-  const int held = floats(tb, step, all) * sizeof(float) <= 110 * 1024 ? all : step;
+  auto held_rows = [&](int step) {
+    const int all = (p.R + step - 1) / step * step;
+    return floats(tb, step, all) * sizeof(float) <= 110 * 1024 ? all : step;
+  };
+  // four rows per thread where two blocks of a step of 128 fit an SM: 1500 rows of 2 heads 33.4 -> 32.4 us, 1024 rows no difference.  Not
+  // where half of the last step or more would be done for nothing (up to 64 query rows, and 129 to 192 of 1500 tokens 41 -> 44.7 us), nor
+  // where a step of 64 takes so little shared memory that three blocks fit an SM and all are under way at once, which two are not (256 of
+  // 3000 69.3 -> 79 us), nor with 32 tokens, whose 16 pairs per thread take the registers of the second block on the SM (4 sequences of
+  // 5000 rows 164 -> 191 us)
+  const bool once_by_threes = blocks > 2 * 148 && blocks <= 3 * 148 && floats(tb, 64, held_rows(64)) * sizeof(float) <= 73 * 1024;
+  const bool tall = !wide && (p.R - 1) % 128 >= 64 && !once_by_threes && floats(tb, 128, 128) * sizeof(float) <= 110 * 1024;
+  const int step = tall ? 128 : 64, held = held_rows(step);
   auto kernel = wide ? simt_pass2_kernel<T, 32, 2> : tall ? simt_pass2_kernel<T, 16, 4> : simt_pass2_kernel<T, 16, 2>;
-  return chain(kernel, dim3((p.n + tb - 1) / tb, p.BH), kThreads, floats(tb, step, held) * sizeof(float), st, p, (const T*)Q, (const T*)K,
-               (const T*)V, ws.fin_m, ws.fin_l, ws.O_f32, ema_decay, ws.I_hat, I_raw, held);
+  const size_t smem = floats(tb, step, held) * sizeof(float);
+  return chain(kernel, grid, kThreads, smem, st, p, (const T*)Q, (const T*)K, (const T*)V, ws.fin_m, ws.fin_l, ws.O_f32, ema_decay,
+               ws.I_hat, I_raw, held);
 }
 
 }  // namespace

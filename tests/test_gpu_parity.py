@@ -493,6 +493,21 @@ def test_fp32_pass2_rows_per_thread(handle, heads_w, n):
     full_check(handle, make_inputs(Case("rows", 1, 2 * group, 2, 64, n, w, min(n, 100), 5, 0, 0.9, "f32", 0, "normal", group * w + n)))
 
 
+@pytest.mark.parametrize("heads_w", [(1, 128), (1, 129), (3, 64), (1, 193), (4, 64)])
+@pytest.mark.parametrize("group_max", [0, 1])
+def test_fp32_pass2_rows_left_for_the_last_step(handle, heads_w, group_max):
+    """Query rows that leave none, one, 64, 65 and 128 for a second step of 128, where 64 and fewer go by steps of 64."""
+    group, w = heads_w
+    inp = make_inputs(Case("half", 1, 2 * group, 2, 64, 1100, w, 100, 5, 0, 0.9, "f32", 0, "normal", group * w))
+    variant_check(handle, inp, (0, 0, 0, group_max), path=rk.PATH_AUTO)
+
+
+@pytest.mark.parametrize("n", [1184, 1185, 2368, 2369, 3552, 3553])
+def test_fp32_pass2_blocks_and_sms(handle, n):
+    """Blocks of 16 tokens on either side of one, two and three for each of 148 SMs, 256 query rows."""
+    full_check(handle, make_inputs(Case("sms", 1, 8, 2, 64, n, 64, 100, 5, 0, 0.9, "f32", 0, "normal", n)))
+
+
 @pytest.mark.parametrize("spec", [(1, 20000), (2, 9601), (4, 4737), (5, 4000)])
 def test_merge_of_many_partials(handle, spec):
     """148, 74, 37 and 29 partials a head, all of them with rows: five, three, two and one for each lane that weighs them."""
