@@ -22,6 +22,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kP1Tile = 32;   // tokens per tile of pass 1
 constexpr int kP1Rows = 64;   // query rows per block of pass 1
+constexpr size_t kAlone = 116 * 1024;   // more shared memory than two blocks of an SM can have
 
 __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
   const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
@@ -200,8 +201,10 @@ __global__ void __launch_bounds__(kThreads) simt_pass1_kernel(Problem p, const T
 
 // ------------------------------------------------------------------------------------------------
 // Combine the token splits.  grid (R, BH), block 128: one block per query row; warp w adds up splits w, w + 4, ..., lane =
-// four dims (two times four where d > 128); the four sums are added in a fixed order.
-__global__ void __launch_bounds__(128) combine_kernel(int R, int d, int splits, const float* __restrict__ part_m,
+// four dims (two times four where d > 128); the four sums are added in a fixed order.  (96 registers: with the 128 that the compiler
+// takes by itself the blocks that wait fill an SM's, so that pass 2's begin late and unevenly; 1500 rows 33.0 -> 32.3 us, with 72
+// 1024 rows 26.7 -> 27.7.)
+__global__ void __launch_bounds__(128, 5) combine_kernel(int R, int d, int splits, const float* __restrict__ part_m,
                                                       const float* __restrict__ part_l, const float* __restrict__ part_O,
                                                       float* __restrict__ fin_m, float* __restrict__ fin_l,
                                                       float* __restrict__ O_f32) {
@@ -563,7 +566,10 @@ cudaError_t pass2(const Problem& p, const Workspace& ws, const void* Q, const vo
   const bool tall = !wide && (p.R - 1) % 128 >= 64 && !once_by_threes && floats(tb, 128, 128) * sizeof(float) <= 110 * 1024;
   const int step = tall ? 128 : 64, held = held_rows(step);
   auto kernel = wide ? simt_pass2_kernel<T, 32, 2> : tall ? simt_pass2_kernel<T, 16, 4> : simt_pass2_kernel<T, 16, 2>;
-  const size_t smem = floats(tb, step, held) * sizeof(float);
+  size_t smem = floats(tb, step, held) * sizeof(float);
+  // where there is an SM for every block, none shares one: an SM on which the blocks of the combine end early would take two of them
+  // (160 query rows of 1024 tokens 38.2 -> 35.3 us)
+  if (blocks <= 148 && smem < kAlone) smem = kAlone;
   return chain(kernel, grid, kThreads, smem, st, p, (const T*)Q, (const T*)K, (const T*)V, ws.fin_m, ws.fin_l, ws.O_f32, ema_decay,
                ws.I_hat, I_raw, held);
 }
