@@ -216,8 +216,9 @@ __device__ __forceinline__ void load_stage_c(const Ctx& cx, const CUtensorMap* t
 // ||v||^2 of row `row` of a [128 x 128] bf16 tile (two 128-byte-swizzled boxes, in which 16-byte chunk c of row r sits at chunk
 // c ^ (r & 7)).  Every instruction counts twice here: one warp does it for a tile while sixteen others use the issue slots.  One fma
 // per element that takes the bf16 as it is (its square is exact), four sums, and three loads in flight, which is what 32 registers
-// hold: 1.8 k cycles a tile beside busy workers, 2.6 k with two loads and 2.3 k with four in flight, 5.6 k with a shift, a mask and
-// a packed fma per pair, which had become what phase A waited for (and 0.6 k of each tile from given statistics).
+// hold: 1.8 k cycles a tile in a kernel of its own beside busy workers, where two loads in flight took 2.6 k, four 2.3 k, and a shift, a
+// mask and a packed fma per pair 5.6 k.  In the score kernel that last form took 4.5 k (trace of one CTA), which had become what phase A
+// waited for (and 0.6 k of each tile from given statistics).
 __device__ __forceinline__ float row_square_sum(uint32_t tile, int row) {
   const uint32_t at = tile + (uint32_t)(row >> 3) * 1024u + (uint32_t)(row & 7) * (128u + 16u);
   constexpr int kDepth = 3;
@@ -1305,9 +1306,9 @@ __device__ void phase_c_worker(const Ctx& cx, const FusedArgs& a, int bh, int ti
           const f32x2 nt = f2_mul(f2_make(sv[2 * q], sv[2 * q + 1]), nc2);
           f32x2 Iq;
           if (kEq7) {
-            // 1/A; one pair in four on the FMA pipe (1/A beyond 2^126 squares to infinity below either way): batch of 8
-            // x 32768 544 -> 531 us, 131072 266 -> 263 us (power-limited clock); with every other pair no better, and from given statistics
-            // (no pass 1, so less to wait for) slower
+            // 1/A; one pair in four on the FMA pipe (1/A beyond 2^126 squares to infinity below either way): 8 x 32768 rows 511.1 ->
+            // 507.2 us, 131072 246.9 -> 245.6, 16384 54.8 -> 54.0, under the projection no difference; with every other pair no better,
+            // and from given statistics (no pass 1, so less to wait for) slower
             const f32x2 u2 = (!from_lse && (q & 3) == 3) ? exp2_fma(f2_make(fminf(f2_lo(nt), 126.f), fminf(f2_hi(nt), 126.f)))
                                      : f2_make(ex2_approx(f2_lo(nt)), ex2_approx(f2_hi(nt)));
             const f32x2 um = f2_add(u2, m1);                                                       // 1/A - 1
